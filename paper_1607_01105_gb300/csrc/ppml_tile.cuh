@@ -222,6 +222,65 @@ __device__ __forceinline__ Parab<T> flat_parabola(T q) {
 // dpv = th (P+V+ - P-V-), dv = th (V+ - V-).  hook(p) is called before step p = -1..18
 // reads position p, and with p = 19 after the last step; positions below p - 3 are no
 // longer read at that point (step p reads positions p, p - 2 and p - 3).
+//
+// FP32: the parabolas in deviation form (LineF32), the steady steps p = 3..18 as a loop
+// unrolled by two (a small body for the instruction cache).
+template <bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
+__device__ __forceinline__ void sweep_eulerian_dev(VF v, PF pr, RF r, float gamma, float th,
+                                                   EF emit, HF hook) {
+  LineF32<FLAT> lv, lp;
+  hook(-1);
+  lv.start(v(-3), v(-2), v(-1));
+  lp.start(pr(-3), pr(-2), pr(-1));
+  hook(0);
+  lv.push(v(0));
+  lp.push(pr(0));
+  hook(1);
+  lv.push(v(1));
+  lp.push(pr(1));
+  // cell p-3 (the face's left cell): values, parabolas and sqrt(rho), rho sqrt(rho), p sqrt(rho)
+  float vl = lv.q2, pl = lp.q2;
+  DevParab Vl = lv.P, Pl = lp.P;
+  const float r0 = r(-1);
+  float sl = sqrt_approx(r0), Al = r0 * sl, Bl = pl * sl;
+  float Vp = 0.0f, Pp = 0.0f;
+  auto face = [&](int p, float& V, float& P) {  // after position p: the face of p-3 and p-2
+    hook(p);
+    lv.push(v(p));
+    lp.push(pr(p));
+    const float rc = r(p - 2), sc = sqrt_approx(rc);
+    const float Ac = rc * sc, Bc = lp.q2 * sc;
+    // face_constants_f32 from the carried products
+    const float A = Al + Ac, lam = sqrt_approx(gamma * (Bl + Bc) * rcp_approx(A));
+    const float Z = lam * A * rcp_approx(sl + sc);
+    const DevWeights w = dev_weights(lam * th);
+    const float vls = dev_right(vl, Vl, w), vrs = dev_left(lv.q2, lv.P, w);
+    const float pls = dev_right(pl, Pl, w), prs = dev_left(lp.q2, lp.P, w);
+    V = 0.5f * ((vls + vrs) + (pls - prs) * rcp_approx(Z));
+    P = 0.5f * ((pls + prs) + Z * (vls - vrs));
+    vl = lv.q2;
+    pl = lp.q2;
+    Vl = lv.P;
+    Pl = lp.P;
+    sl = sc;
+    Al = Ac;
+    Bl = Bc;
+  };
+  face(2, Vp, Pp);
+#pragma unroll 2
+  for (int p = 3; p <= TB + 2; p++) {
+    float V, P;
+    face(p, V, P);
+    emit(p - 3, th * (P - Pp), th * (P * V - Pp * Vp), th * (V - Vp));
+    Vp = V;
+    Pp = P;
+  }
+  hook(TB + 3);
+}
+
+// The same sweep with the parabolas in face values: FP64 (every expression in the checker's
+// order) and double-float FP32 states (whose low parts record the rounding of exactly these
+// expressions).
 template <typename T, bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
 __device__ __forceinline__ void sweep_eulerian(VF v, PF pr, RF r, T gamma, T th, double tau,
                                                double h, EF emit, HF hook) {
@@ -410,15 +469,80 @@ __device__ __forceinline__ void stage_box_fast(T* box, const T* __restrict__ src
 }
 
 // Face velocities as the sweeps read them.  FP64: v^ itself (the flux and the Courant
-// number are formed as the checker forms them).  FP32: w = v^ th / 2 (th = tau / h), so
-// that |w| is half the Courant number y and w times the upwind state is half of th times
-// the flux (both exact rescalings of v^ th): the per-field products by th disappear, the
-// sweeps accumulate half divergences and the update subtracts twice their sum.
-__device__ __forceinline__ float vh_stored(float v, float th) { return v * (0.5f * th); }
+// number are formed as the checker forms them).  FP32: w = v^ th (th = tau / h), so that
+// |w| is the Courant number y and w times the upwind state is th times the flux: the
+// per-field products by th disappear.  Double-float states (DF): half of that, as the
+// face-value form reads it.
+template <bool DF>
+__device__ __forceinline__ float vh_stored(float v, float th) {
+  return v * (DF ? 0.5f * th : th);
+}
+template <bool DF>
 __device__ __forceinline__ double vh_stored(double v, double) { return v; }
 // The flux divergence summed over axes from what the sweeps accumulated (exact).
-__device__ __forceinline__ float divergence_sum(float half_sum) { return 2.0f * half_sum; }
+template <bool DF>
+__device__ __forceinline__ float divergence_sum(float sum) { return DF ? 2.0f * sum : sum; }
+template <bool DF>
 __device__ __forceinline__ double divergence_sum(double sum) { return sum; }
+
+// One line of the FP32 Lagrangian stage for any axis, on the deviation form of the parabola
+// (LineF32).  Field values: core[p cs] for p in [0, 16), halo[h SLP] for the positions
+// -3..-1 (h = 0..2) and 16..18 (h = 3..5).  Face velocities vh[c TN], c = 0..16 (face
+// between cells c-1 and c).  When position p arrives, the slope at p-1, the deviations of
+// the face p-3/2, the parabola of cell p-2 and the flux through face p-5/2 are formed; the
+// warm-up positions are peeled and the steady state is a loop unrolled by four.  MODE 0:
+// acc = div; 1: acc += div; 2: dst[c gs] = core - (acc + div) for c < nvalid (acc only if
+// have_acc).  CS: the core stride of the sweep axis as a compile-time constant (immediate
+// shared-memory offsets).
+template <int MODE, bool FLAT, int CS>
+__device__ __forceinline__ void lag_line_dev(const float* core, const float* halo,
+                                             const float* vh, float* acc, bool have_acc,
+                                             float* __restrict__ dst, long long gs, int nvalid) {
+  constexpr int cs = CS;
+  LineF32<FLAT> ln;
+  ln.start(halo[0], halo[SLP], halo[2 * SLP]);
+  ln.push(core[0]);
+  ln.push(core[cs]);
+  DevParab Pl = ln.P;  // cell -1
+  float ql = ln.q2;
+  ln.push(core[2 * cs]);
+  float Fp = upwind_flux_f32(vh[0], ql, Pl, ln.q2, ln.P);
+  ql = ln.q2;
+  Pl = ln.P;
+  // steady state: position c + 3 arrives, cell c is finished
+  auto step = [&](float qnew, float w, int c) {
+    ln.push(qnew);
+    const float F = upwind_flux_f32(w, ql, Pl, ln.q2, ln.P);  // face between c and c+1
+    const float d = F - Fp;  // th (F+ - F-)
+    const int o = c * cs;
+    if (MODE == 0)
+      acc[o] = d;
+    else if (MODE == 1)
+      acc[o] = acc[o] + d;
+    else if (c < nvalid)
+      dst[gs * c] = ql - (have_acc ? acc[o] + d : d);
+    Fp = F;
+    ql = ln.q2;
+    Pl = ln.P;
+  };
+  // inputs one step ahead: position c + 3 and face c + 1 of step c are loaded in step c - 1
+  float q_in = core[3 * cs], v_in = vh[TN];
+#pragma unroll 4
+  for (int c = 0; c < TB - 4; c++) {
+    const float q = q_in, v = v_in;
+    q_in = core[(c + 4) * cs];
+    v_in = vh[(c + 2) * TN];
+    step(q, v, c);
+  }
+#pragma unroll 1
+  for (int c = TB - 4; c < TB - 1; c++) {
+    const float q = q_in, v = v_in;
+    q_in = halo[(c - TB + 7) * SLP];  // positions 16..18
+    v_in = vh[(c + 2) * TN];          // faces 14..16
+    step(q, v, c);
+  }
+  step(q_in, v_in, TB - 1);
+}
 
 // FP32 flux through a face of eq. fluxonlagrangestage from w = v^ th / 2: w times the
 // upwind state, the left cell's mean over its right fraction y when w >= 0, else the right
@@ -436,7 +560,9 @@ __device__ __forceinline__ float half_flux_f32(float w, float R_l, float D_l, fl
   return w * fmaf(c1, D, fmaf(c2, S, base));
 }
 
-// One line of the Lagrangian stage for any axis.  Field values: core[p cs] for p in
+// One line of the Lagrangian stage for any axis with the parabola in face values: FP64 (every
+// expression in the checker's order) and double-float FP32 states (whose low parts record
+// the rounding of exactly these expressions).  Field values: core[p cs] for p in
 // [0, 16), halo[h SLP] for the positions -3..-1 (h = 0..2) and 16..18 (h = 3..5).  Face
 // velocities vh[c TN], c = 0..16 (face between cells c-1 and c).  MODE 0: acc = div;
 // 1: acc += div; 2: dst[c gs] = core - (acc + div) for c < nvalid (acc only if have_acc).
@@ -513,7 +639,7 @@ __device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* 
     } else if (MODE == 1) {
       acc[o] = acc[o] + d;
     } else if (c < nvalid) {
-      const T upd = divergence_sum(have_acc ? acc[o] + d : d);
+      const T upd = divergence_sum<DF>(have_acc ? acc[o] + d : d);
       if constexpr (DF) {
         if (dstlo) {
           float hi, lo;
@@ -673,12 +799,12 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
     T vh0[TB + 1];
     line_face_velocities(vbox(0), rbox, 0, a, b, one_point, vh0);
 #pragma unroll
-    for (int q = 0; q <= TB; q++) S.vh[0][q][tid] = vh_stored(vh0[q], th[0]);
+    for (int q = 0; q <= TB; q++) S.vh[0][q][tid] = vh_stored<DF>(vh0[q], th[0]);
   }
 #pragma unroll
   for (int q = 0; q <= TB; q++) {
-    if (act[1]) S.vh[1][q][tid] = vh_stored(vh1[q], th[1]);
-    if (act[2]) S.vh[2][q][tid] = vh_stored(vh2[q], th[2]);
+    if (act[1]) S.vh[1][q][tid] = vh_stored<DF>(vh1[q], th[1]);
+    if (act[2]) S.vh[2][q][tid] = vh_stored<DF>(vh2[q], th[2]);
   }
   __syncthreads();
 
@@ -801,7 +927,10 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
         constexpr int M = decltype(mode_c)::value;
         constexpr bool FL = decltype(flat_c)::value;
         constexpr int C = decltype(cs_c)::value;
-        if constexpr (M == 2)
+        if constexpr (sizeof(T) == 4 && !DF)
+          lag_line_dev<M, FL, C>(core, halo, vhl, acc, mode == 1, A.out[f] + zline0, g.nxy,
+                                 nvalid_z);
+        else if constexpr (M == 2)
           lag_line<T, 2, FL, DF, C>(core, halo, vhl, th[2], tau, A.h[2], acc, mode == 1,
                                     A.out[f] + zline0, g.nxy, nvalid_z, srclo, dstlo);
         else
@@ -829,7 +958,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
       for (int c = 0; c < nvalid_z; c++) {
         const int o = acc_at(a, b, c);
         const long long idx = zline0 + g.nxy * c;
-        const T upd = mode == 1 ? divergence_sum(S.acc[o]) : T(0);
+        const T upd = mode == 1 ? divergence_sum<DF>(S.acc[o]) : T(0);
         if constexpr (DF) {
           if (f < 5) {
             float hi, lo;
@@ -1128,10 +1257,17 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
     };
     auto pq = [&](int p) { return gm1 * S.p[slab_at(p, a, b)]; };
     auto rq = [&](int p) { return S.r[slab_at(p, a, b)]; };
+    auto sweep = [&](auto flat_c) {
+      constexpr bool FL = decltype(flat_c)::value;
+      if constexpr (sizeof(T) == 4 && !DF)
+        sweep_eulerian_dev<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
+      else
+        sweep_eulerian<T, FL>(vq, pq, rq, gamma, th[ax], tau, A.h[ax], emit, hook);
+    };
     if (A.flags & PPML_FIRST_ORDER)
-      sweep_eulerian<T, true>(vq, pq, rq, gamma, th[ax], tau, A.h[ax], emit, hook);
+      sweep(BoolC<true>());
     else
-      sweep_eulerian<T, false>(vq, pq, rq, gamma, th[ax], tau, A.h[ax], emit, hook);
+      sweep(BoolC<false>());
     first = false;
     __syncthreads();
   }
