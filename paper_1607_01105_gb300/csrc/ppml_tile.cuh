@@ -1313,57 +1313,100 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
     }
     return;
   }
-  for (int c = 0; c < TB; c++) {
-    if (!in_domain(g, tg, a, b, c)) continue;
-    const int gi = tg.i0 + a, gj = tg.j0 + b, gk = tg.k0 + c;
-    const long long idx = (long long)gi + (long long)g.n[0] * gj + g.nxy * gk;
-    const T rho0 = A.u[0][idx];
-    const T ei0 = A.u[5][idx];
-    const T dpvs = first ? T(0) : S.apv[acc_at(a, b, c)];
-    const T dvs = first ? T(0) : S.av[acc_at(a, b, c)];
-    T en = A.u[4][idx] - dpvs;
-    T den = dpvs;  // DF: the whole FP32 decrement of rho E, added to the pair once
-    if (A.phi) {
-      GridGeom gp = g;  // Phi: zero-gradient at reflecting walls and inflow faces, as at outflow
-      for (int q = 0; q < 6; q++)
-        if (gp.bc[q] == 2 || gp.bc[q] == 3 || gp.bc[q] == PPML_BC_INFLOW) gp.bc[q] = 0;
-      T m[3] = {A.out[1][idx], A.out[2][idx], A.out[3][idx]};
-      const T m0[3] = {A.u[1][idx], A.u[2][idx], A.u[3][idx]};
+  if (!in_domain(g, tg, a, b, 0)) return;
+  const int nvalid = min(TB, g.n[2] - tg.k0);
+  // Phi's neighbours of the thread's column as offsets from the cell (zero-gradient at every
+  // face but periodic ones, where they wrap): the x and y ones are the same for the whole
+  // column, the z ones are its own last and next cell, so a cell costs five loads of Phi and
+  // no boundary arithmetic but the column's ends.
+  long long pxm = 0, pxp = 0, pym = 0, pyp = 0;
+  if (A.phi) {
+    const int gi = tg.i0 + a, gj = tg.j0 + b;
+    auto step = [](int c, int n, int bc, int dir) {  // neighbour's coordinate minus c
+      const int q = c + dir;
+      if ((unsigned)q < (unsigned)n) return dir;
+      return bc == PPML_BC_PERIODIC ? (dir < 0 ? n - 1 : 1 - n) : 0;
+    };
+    const long long nx = g.n[0];
+    pxm = step(gi, g.n[0], g.bc[0], -1);
+    pxp = step(gi, g.n[0], g.bc[1], 1);
+    pym = nx * step(gj, g.n[1], g.bc[2], -1);
+    pyp = nx * step(gj, g.n[1], g.bc[3], 1);
+  }
+  constexpr int GB = sizeof(T) == 4 ? 4 : 2;  // cells whose loads are in flight together
 #pragma unroll 1
-      for (int ax = 0; ax < 3; ax++) {
-        if (!act[ax]) continue;
-        const int di = ax == 0, dj = ax == 1, dk = ax == 2;
-        const T pp = load_bc(A.phi, -1, gi + di, gj + dj, gk + dk, gp);
-        const T pm = load_bc(A.phi, -1, gi - di, gj - dj, gk - dk, gp);
-        const T grad = (pp - pm) / T(2.0 * A.h[ax]);
-        if constexpr (DF) {
-          float hi, lo;
-          df_sub(m[ax], A.outlo[1 + ax][idx], T(tau) * rho0 * grad, hi, lo);
-          m[ax] = hi;
-          A.outlo[1 + ax][idx] = lo;
-          den += T(tau) * m0[ax] * grad;
-        } else {
-          m[ax] -= T(tau) * rho0 * grad;
-          en -= T(tau) * m0[ax] * grad;
+  for (int c0 = 0; c0 < nvalid; c0 += GB) {
+    T r0[GB], e0[GB], ei0[GB], m[GB][3], m0[GB][3], pd[GB][3];
+    float el[GB], ml[GB][3];
+#pragma unroll
+    for (int q = 0; q < GB; q++) {
+      const int c = min(c0 + q, nvalid - 1);
+      const long long idx = zline0e + g.nxy * c;
+      r0[q] = A.u[0][idx];
+      e0[q] = A.u[4][idx];
+      ei0[q] = A.u[5][idx];
+      if constexpr (DF) el[q] = A.ulo[4][idx];
+      if (A.phi) {
+        const int gk = tg.k0 + c;
+        const long long zm = gk > 0 ? -g.nxy
+                                    : (g.bc[4] == PPML_BC_PERIODIC ? g.nxy * (g.n[2] - 1) : 0);
+        const long long zp = gk < g.n[2] - 1
+                                 ? g.nxy
+                                 : (g.bc[5] == PPML_BC_PERIODIC ? g.nxy * (1 - g.n[2]) : 0);
+        const T* f = A.phi + idx;
+        pd[q][0] = f[pxp] - f[pxm];
+        pd[q][1] = f[pyp] - f[pym];
+        pd[q][2] = f[zp] - f[zm];
+#pragma unroll
+        for (int ax = 0; ax < 3; ax++) {
+          m[q][ax] = A.out[1 + ax][idx];
+          m0[q][ax] = A.u[1 + ax][idx];
+          if constexpr (DF) ml[q][ax] = A.outlo[1 + ax][idx];
         }
       }
-      A.out[1][idx] = m[0];
-      A.out[2][idx] = m[1];
-      A.out[3][idx] = m[2];
     }
-    if (A.out[0]) {
-      A.out[0][idx] = rho0;
-      if constexpr (DF) A.outlo[0][idx] = A.ulo[0][idx];
+#pragma unroll
+    for (int q = 0; q < GB; q++) {
+      const int c = c0 + q;
+      if (c >= nvalid) break;
+      const long long idx = zline0e + g.nxy * c;
+      const T dpvs = first ? T(0) : S.apv[acc_at(a, b, c)];
+      const T dvs = first ? T(0) : S.av[acc_at(a, b, c)];
+      T en = e0[q] - dpvs;
+      T den = dpvs;  // DF: the whole FP32 decrement of rho E, added to the pair once
+      if (A.phi) {
+#pragma unroll
+        for (int ax = 0; ax < 3; ax++) {
+          if (act[ax]) {
+            const T grad = pd[q][ax] / T(2.0 * A.h[ax]);
+            if constexpr (DF) {
+              float hi, lo;
+              df_sub(m[q][ax], ml[q][ax], T(tau) * r0[q] * grad, hi, lo);
+              m[q][ax] = hi;
+              A.outlo[1 + ax][idx] = lo;
+              den += T(tau) * m0[q][ax] * grad;
+            } else {
+              m[q][ax] -= T(tau) * r0[q] * grad;
+              en -= T(tau) * m0[q][ax] * grad;
+            }
+          }
+          A.out[1 + ax][idx] = m[q][ax];
+        }
+      }
+      if (A.out[0]) {
+        A.out[0][idx] = r0[q];
+        if constexpr (DF) A.outlo[0][idx] = A.ulo[0][idx];
+      }
+      if constexpr (DF) {
+        float hi, lo;
+        df_sub(e0[q], el[q], den, hi, lo);
+        A.out[4][idx] = hi;
+        A.outlo[4][idx] = lo;
+      } else {
+        A.out[4][idx] = en;
+      }
+      A.out[5][idx] = eps_update(ei0[q], gm1, dvs);
     }
-    if constexpr (DF) {
-      float hi, lo;
-      df_sub(A.u[4][idx], A.ulo[4][idx], den, hi, lo);
-      A.out[4][idx] = hi;
-      A.outlo[4][idx] = lo;
-    } else {
-      A.out[4][idx] = en;
-    }
-    A.out[5][idx] = eps_update(ei0, gm1, dvs);
   }
 }
 
