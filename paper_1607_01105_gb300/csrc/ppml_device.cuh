@@ -389,6 +389,53 @@ __device__ __forceinline__ void df_split(double x, float& hi, float& lo) {
   lo = (float)(x - (double)hi);
 }
 
+// A value of a host-formed table as a kernel of either precision reads it: the double
+// itself, or its float pair (hi, lo).
+struct FloatPair {
+  float x, y;
+};
+template <typename T>
+struct TableOf {
+  using type = double;
+};
+template <>
+struct TableOf<float> {
+  using type = FloatPair;
+};
+
+// c / (1 - p t) of the Poisson symbols: p the product of two tables, t the third.  In float
+// pairs every product and the difference keep about 2^-46, so 1 - p t of the smoothest mode
+// of N points, about (4/3)(pi / N)^2, keeps 30 bits at N = 512, more than the float
+// amplitude it scales; the quotient takes one Newton correction.  (FP64 would take some 15
+// instructions at one per 19 cycles and SM.)
+__device__ __forceinline__ double table_product(double a, double b) { return a * b; }
+__device__ __forceinline__ FloatPair table_product(FloatPair a, FloatPair b) {
+  const float p = a.x * b.x;
+  const float e = fmaf(a.x, b.x, -p) + fmaf(a.x, b.y, a.y * b.x);
+  FloatPair r;
+  r.x = p + e;
+  r.y = (p - r.x) + e;
+  return r;
+}
+__device__ __forceinline__ double over_one_minus(double c, double p, double t) {
+  return c / (1.0 - p * t);
+}
+__device__ __forceinline__ FloatPair over_one_minus(FloatPair c, FloatPair p, FloatPair t) {
+  const float q = p.x * t.x;
+  const float qe = fmaf(p.x, t.x, -q) + fmaf(p.x, t.y, p.y * t.x);
+  float d, de;
+  two_sum(1.0f, -q, d, de);
+  const float l = de - qe;
+  const float dh = d + l, dl = (d - dh) + l;  // 1 - p t
+  const float r = rcp_approx(dh);
+  FloatPair f;
+  f.x = c.x * r;
+  f.y = (fmaf(-f.x, dh, c.x) + fmaf(-f.x, dl, c.y)) * r;
+  return f;
+}
+__device__ __forceinline__ double scaled(double v, double f) { return v * f; }
+__device__ __forceinline__ float scaled(float v, FloatPair f) { return fmaf(v, f.x, v * f.y); }
+
 // rho eps = (eh + el) - |m|^2 / (2 rho) with rho = rh + rl and m_a = mh_a + ml_a, in
 // double-float (about 44 significant bits), rounded once to float.  Sec. 1.4 (dense
 // branch) on double-float totals: the error of the difference does not grow with the
@@ -520,30 +567,9 @@ struct GridGeom {
   long long nxy, ncell;
 };
 
-// Linear index of possibly out-of-domain cell (i, j, k) after boundary mapping; bit a of
-// flips is set when axis a was mirrored (the a-momentum changes sign there).
-__device__ __forceinline__ long long map_cell(int i, int j, int k, const GridGeom& g, int& flips) {
-  int f0, f1, f2;
-  const int ii = bc_map(i, g.n[0], g.bc[0], g.bc[1], f0);
-  const int jj = bc_map(j, g.n[1], g.bc[2], g.bc[3], f1);
-  const int kk = bc_map(k, g.n[2], g.bc[4], g.bc[5], f2);
-  flips = f0 | (f1 << 1) | (f2 << 2);
-  return (long long)ii + (long long)g.n[0] * jj + g.nxy * kk;
-}
-
 // Sign of field f (0..5; -1 for a scalar) at a cell reached through the mirrors in flips.
 __device__ __forceinline__ bool field_flipped(int f, int flips) {
   return f >= 1 && f <= 3 && ((flips >> (f - 1)) & 1);
-}
-
-// Value of field `f` at possibly out-of-domain cell (i, j, k), with the momentum component
-// normal to a reflecting wall negated.
-template <typename T>
-__device__ __forceinline__ T load_bc(const T* __restrict__ q, int f, int i, int j, int k,
-                                     const GridGeom& g) {
-  int fl;
-  T v = __ldg(q + map_cell(i, j, k, g, fl));
-  return field_flipped(f, fl) ? -v : v;
 }
 
 }  // namespace ppml

@@ -487,6 +487,15 @@ extern "C" int ppml_free_grid(ppml_grid* g) {
   return PPML_OK;
 }
 
+double ppml_table_value(double x, bool f64) {
+  if (f64) return x;
+  const float hi = (float)x;
+  const float pair[2] = {hi, (float)(x - (double)hi)};
+  double r;
+  memcpy(&r, pair, sizeof(r));
+  return r;
+}
+
 extern "C" int ppml_poisson_periodic(ppml_grid* g, const void* rho, void* phi, double G,
                                      void* stream) {
   ppml_clear_error();
@@ -511,7 +520,7 @@ extern "C" int ppml_poisson_periodic(ppml_grid* g, const void* rho, void* phi, d
     for (int a = 0; a < 3; a++)
       for (int k = 0; k < len[a]; k++) {
         const double s = sin(M_PI * (double)k / (double)n[a]);
-        tab.push_back(1.0 - (2.0 / 3.0) * s * s);
+        tab.push_back(ppml_table_value(1.0 - (2.0 / 3.0) * s * s, f64));
       }
     if (cudaMemcpy(g->tables, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice) !=
         cudaSuccess)
@@ -528,11 +537,9 @@ extern "C" int ppml_poisson_periodic(ppml_grid* g, const void* rho, void* phi, d
   if (r != CUFFT_SUCCESS) return ppml_fail(PPML_E_CUDA, "cuFFT forward failed (%d)", (int)r);
   const double h = g->d.h[0];
   const double coef = -(2.0 / 3.0) * M_PI * G * h * h / ((double)n[0] * n[1] * n[2]);
-  const double* tx = g->tables;
-  const double* ty = tx + mx;
-  const double* tz = ty + n[1];
-  int rc = f64 ? launch_poisson_symbol<double>(g->spec, tx, ty, tz, mx, n[1], n[2], coef, st)
-               : launch_poisson_symbol<float>(g->spec, tx, ty, tz, mx, n[1], n[2], coef, st);
+  const double c = ppml_table_value(coef, f64);
+  int rc = f64 ? launch_poisson_symbol<double>(g->spec, g->tables, mx, n[1], n[2], c, st)
+               : launch_poisson_symbol<float>(g->spec, g->tables, mx, n[1], n[2], c, st);
   if (rc) return rc;
   r = f64 ? cufftExecZ2D(g->fft_inv, (cufftDoubleComplex*)g->spec, (cufftDoubleReal*)phi)
           : cufftExecC2R(g->fft_inv, (cufftComplex*)g->spec, (cufftReal*)phi);

@@ -30,3 +30,7 @@ struct FourierState;
 int ppml_fourier_run(FourierState** state, const ppml_grid_desc* d, const void* rho, double r_f,
                      int m_max, double* a_out, cudaStream_t st);
 void ppml_fourier_free(FourierState* s);
+
+// x as a kernel's table holds it (TableOf in ppml_device.cuh): a double (f64), or its float
+// pair (hi, lo) in a double's storage.
+double ppml_table_value(double x, bool f64);

@@ -94,34 +94,44 @@ int launch_diag<PPML_REAL>(const MarchArgs<PPML_REAL>& A, int nblk, cudaStream_t
 
 namespace {
 // Multiply the half spectrum (R2C layout: kx in [0, nx/2], ky, kz) by the inverse symbol of
-// the 27-point stencil; tables hold 1 - (2/3) sin^2(pi k / N) per axis.
+// the 27-point stencil, coef / (1 - tx ty tz); tables hold 1 - (2/3) sin^2(pi k / N) per axis
+// (FP32 grids: as float pairs, coef too).  A warp takes one row of kx at a time, so tz ty is
+// formed once per row.  512^3 FP32: 1986 us with an FP64 division per value.
 template <typename T>
-__global__ void poisson_symbol_kernel(T* spec, const double* __restrict__ tx,
-                                      const double* __restrict__ ty,
-                                      const double* __restrict__ tz, int mx, int ny, int nz,
-                                      double coef) {
-  const long long n = (long long)mx * ny * nz;
-  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < n;
-       idx += (long long)gridDim.x * blockDim.x) {
-    const int kx = (int)(idx % mx);
-    const long long r = idx / mx;
-    const int ky = (int)(r % ny), kz = (int)(r / ny);
-    const double den = 1.0 - tz[kz] * ty[ky] * tx[kx];
-    const double f = idx == 0 ? 0.0 : coef / den;
-    spec[2 * idx] = (T)(spec[2 * idx] * f);
-    spec[2 * idx + 1] = (T)(spec[2 * idx + 1] * f);
+__global__ void __launch_bounds__(256) poisson_symbol_kernel(T* spec, const double* __restrict__ tab,
+                                                             int mx, int ny, int nz, double coef) {
+  using V = typename TableOf<T>::type;
+  using T2 = std::conditional_t<sizeof(T) == 8, double2, float2>;
+  static_assert(sizeof(V) == sizeof(double), "a table value fills a double's storage");
+  T2* const s = reinterpret_cast<T2*>(spec);
+  const V* const tx = reinterpret_cast<const V*>(tab);
+  const V* const ty = tx + mx;
+  const V* const tz = ty + ny;
+  const V c = *reinterpret_cast<const V*>(&coef);
+  const int lane = threadIdx.x & 31;
+  const long long rows = (long long)ny * nz;
+  const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
+  for (long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < rows;
+       row += warps) {
+    const V tzy = table_product(tz[row / ny], ty[row % ny]);
+    for (int kx = lane; kx < mx; kx += 32) {
+      const V f = over_one_minus(c, tzy, tx[kx]);
+      T2 v = s[row * mx + kx];
+      v.x = scaled(v.x, f);
+      v.y = scaled(v.y, f);
+      if (row == 0 && kx == 0) v.x = v.y = T(0);  // the k = 0 mode
+      s[row * mx + kx] = v;
+    }
   }
 }
 }  // namespace
 
 template <>
-int launch_poisson_symbol<PPML_REAL>(void* spec, const double* tx, const double* ty,
-                                     const double* tz, int mx, int ny, int nz, double coef,
-                                     cudaStream_t st) {
-  const long long n = (long long)mx * ny * nz;
-  const int blocks = (int)((n + 255) / 256 < 4096 ? (n + 255) / 256 : 4096);
-  poisson_symbol_kernel<PPML_REAL><<<blocks, 256, 0, st>>>((PPML_REAL*)spec, tx, ty, tz, mx, ny, nz,
-                                                           coef);
+int launch_poisson_symbol<PPML_REAL>(void* spec, const double* tab, int mx, int ny, int nz,
+                                     double coef, cudaStream_t st) {
+  const long long rows = (long long)ny * nz;
+  const int blocks = (int)((rows + 7) / 8 < 152 * 8 ? (rows + 7) / 8 : 152 * 8);
+  poisson_symbol_kernel<PPML_REAL><<<blocks, 256, 0, st>>>((PPML_REAL*)spec, tab, mx, ny, nz, coef);
   return ppml_check_launch("poisson_symbol_kernel");
 }
 

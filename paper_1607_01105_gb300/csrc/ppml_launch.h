@@ -19,8 +19,8 @@ int launch_lagrangian(const MarchArgs<T>& A, int nblk, cudaStream_t st);
 template <typename T>
 int launch_diag(const MarchArgs<T>& A, int nblk, cudaStream_t st);
 template <typename T>
-int launch_poisson_symbol(void* spec, const double* tx, const double* ty, const double* tz, int mx,
-                          int ny, int nz, double coef, cudaStream_t st);
+int launch_poisson_symbol(void* spec, const double* tab, int mx, int ny, int nz, double coef,
+                          cudaStream_t st);
 // Batched 1D problems: the vacuum thresholds of all ninst instances (instance = CTA index),
 // then one CTA per instance of order[0 .. ninst), or one cluster of two CTAs per work item
 // of items[0 .. nitems) (nlmax: the largest half of a split instance, nmax: the largest
@@ -52,9 +52,8 @@ int launch_finalize(const Partial* P, int nblk, DevScalars* S, double cfl, doubl
   template <>                                                                                \
   int launch_diag<R>(const MarchArgs<R>& A, int nblk, cudaStream_t st);                       \
   template <>                                                                                \
-  int launch_poisson_symbol<R>(void* spec, const double* tx, const double* ty,                 \
-                               const double* tz, int mx, int ny, int nz, double coef,          \
-                               cudaStream_t st);                                               \
+  int launch_poisson_symbol<R>(void* spec, const double* tab, int mx, int ny, int nz,          \
+                               double coef, cudaStream_t st);                                  \
   template <>                                                                                \
   int launch_batch_vacuum<R>(const R* rho, InstDev* inst, int ninst, cudaStream_t st);        \
   template <>                                                                                \

@@ -27,7 +27,10 @@
 #include <vector>
 
 #include "../../include/ppml.h"
+#include "ppml_device.cuh"
 #include "ppml_internal.h"
+
+using namespace ppml;
 
 namespace {
 
@@ -45,26 +48,39 @@ __device__ __forceinline__ double centre(int i, int n, double h) {
 }
 
 // Stage 1a: per-block FP64 partial moments of the masses rho h^3, fixed block count and a
-// fixed-shape tree, so the result does not depend on scheduling.
+// fixed-shape tree, so the result does not depend on scheduling.  A warp takes one row
+// (j, k) at a time and sums rho, rho x, rho x^2 over it (each lane its own cells); y and z
+// are the same for the whole row, so the seven moments cost seven more operations per lane
+// and row instead of about 25 FP64 operations per cell (128^3: 136 us before).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ rho, Dims D,
                                                           double h, double* __restrict__ part) {
   double acc[kMoments] = {0, 0, 0, 0, 0, 0, 0};
   const double vol = h * h * h;
-  for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < D.ncell;
-       idx += (long long)gridDim.x * kThreads) {
-    const int i = (int)(idx % D.n[0]);
-    const long long r = idx / D.n[0];
+  const int lane = threadIdx.x & 31;
+  const long long rows = (long long)D.n[1] * D.n[2];
+  const long long warps = (long long)gridDim.x * (kThreads / 32);
+  for (long long r = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r < rows;
+       r += warps) {
     const int j = (int)(r % D.n[1]), k = (int)(r / D.n[1]);
-    const double x = centre(i, D.n[0], h), y = centre(j, D.n[1], h), z = centre(k, D.n[2], h);
-    const double m = (double)rho[idx] * vol;
-    acc[0] += m;
-    acc[1] += (z * z + y * y) * m;
-    acc[2] += (x * x + z * z) * m;
-    acc[3] += (x * x + y * y) * m;
-    acc[4] += x * y * m;
-    acc[5] += x * z * m;
-    acc[6] += y * z * m;
+    double m0 = 0.0, m1 = 0.0, m2 = 0.0;
+    for (int i = lane; i < D.n[0]; i += 32) {
+      const double x = centre(i, D.n[0], h), m = (double)rho[r * D.n[0] + i], mx = m * x;
+      m0 += m;
+      m1 += mx;
+      m2 += mx * x;
+    }
+    const double y = centre(j, D.n[1], h), z = centre(k, D.n[2], h);
+    m0 *= vol;
+    m1 *= vol;
+    m2 *= vol;
+    acc[0] += m0;
+    acc[1] += (z * z + y * y) * m0;
+    acc[2] += m2 + z * z * m0;
+    acc[3] += m2 + y * y * m0;
+    acc[4] += y * m1;
+    acc[5] += z * m1;
+    acc[6] += y * z * m0;
   }
   __shared__ double s[kMoments][kThreads];
 #pragma unroll
@@ -110,128 +126,206 @@ __device__ double shell_potential(const double* __restrict__ mom, double x, doub
   return -G * mom[0] / r - 0.5 * G * (mom[1] + mom[2] + mom[3] - 3.0 * I0) / (r2 * r);
 }
 
+// Stage 1c: the potential on the shell of cells around the grid, each shell cell once (a
+// boundary cell's stencil meets up to 19 of them, and consecutive threads of the right-hand
+// side are mostly not boundary cells).  Layout of the (nx+2)(ny+2)(nz+2) box's surface: the
+// two z planes, then per inner z the two y rows, then the two x columns.
+__host__ __device__ __forceinline__ long long shell_cells(const Dims& D) {
+  const long long X = D.n[0] + 2, Y = D.n[1] + 2;
+  return 2 * X * Y + (long long)D.n[2] * (2 * X + 2 * D.n[1]);
+}
+// Index of shell cell (i, j, k), each in -1 .. n.
+__device__ __forceinline__ long long shell_at(const Dims& D, int i, int j, int k) {
+  const long long X = D.n[0] + 2, Y = D.n[1] + 2;
+  if (k < 0 || k >= D.n[2]) return (k < 0 ? 0 : X * Y) + X * (j + 1) + (i + 1);
+  const long long base = 2 * X * Y + (long long)k * (2 * X + 2 * D.n[1]);
+  if (j < 0 || j >= D.n[1]) return base + (j < 0 ? 0 : X) + (i + 1);
+  return base + 2 * X + (i < 0 ? 0 : D.n[1]) + j;
+}
+__global__ void __launch_bounds__(kThreads) shell_kernel(Dims D, double h, double G,
+                                                         const double* __restrict__ mom,
+                                                         double* __restrict__ shell) {
+  const long long n = shell_cells(D), X = D.n[0] + 2, Y = D.n[1] + 2;
+  for (long long q = (long long)blockIdx.x * kThreads + threadIdx.x; q < n;
+       q += (long long)gridDim.x * kThreads) {
+    int i, j, k;
+    if (q < 2 * X * Y) {
+      k = q < X * Y ? -1 : D.n[2];
+      const int r = (int)(q % (X * Y));
+      j = r / (int)X - 1;
+      i = r % (int)X - 1;
+    } else {
+      const int per = 2 * (int)X + 2 * D.n[1];
+      k = (int)((q - 2 * X * Y) / per);
+      const int r = (int)((q - 2 * X * Y) % per);
+      if (r < 2 * (int)X) {
+        j = r < (int)X ? -1 : D.n[1];
+        i = r % (int)X - 1;
+      } else {
+        i = r - 2 * (int)X < D.n[1] ? -1 : D.n[0];
+        j = (r - 2 * (int)X) % D.n[1];
+      }
+    }
+    shell[q] = shell_potential(mom, centre(i, D.n[0], h), centre(j, D.n[1], h),
+                               centre(k, D.n[2], h), G);
+  }
+}
+
+// rho + D7 rho / 12 of a cell from its value and the sum of its six neighbours.  FP32 grids
+// take it as a float pair (rho / 2 + sum / 12 with the sum in TwoSum): FP64 would cost
+// about 20 FP64 instructions per cell, at one per 19 cycles and SM.
+struct SourcePair {
+  float hi, lo;
+};
+__device__ __forceinline__ void pair_add(SourcePair& s, float x) {
+  const float t = s.hi + x, b = t - s.hi;
+  s.lo += (s.hi - (t - b)) + (x - b);
+  s.hi = t;
+}
+
 // Right-hand side: 4 pi G h^2 (rho [+ D7 rho / 12]) minus the stencil weights times the
 // shell values next to boundary cells.  Written into the potential array (the work array).
+// One row of x per warp pass.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho, T* __restrict__ out,
                                                        Dims D, double h, double G,
-                                                       const double* __restrict__ mom, int printed) {
+                                                       const double* __restrict__ shell, int printed) {
   const double c = 4.0 * M_PI * G * h * h;
-  for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < D.ncell;
-       idx += (long long)gridDim.x * kThreads) {
-    const int i = (int)(idx % D.n[0]);
-    const long long r = idx / D.n[0];
-    const int j = (int)(r % D.n[1]), k = (int)(r / D.n[1]);
-    const double rc = (double)rho[idx];
-    double src = rc;
-    if (!printed) {
-      double lap = -6.0 * rc;
-      if (i > 0) lap += (double)rho[idx - 1];
-      if (i < D.n[0] - 1) lap += (double)rho[idx + 1];
-      if (j > 0) lap += (double)rho[idx - D.n[0]];
-      if (j < D.n[1] - 1) lap += (double)rho[idx + D.n[0]];
-      if (k > 0) lap += (double)rho[idx - D.nxy];
-      if (k < D.n[2] - 1) lap += (double)rho[idx + D.nxy];
-      src = rc + lap / 12.0;
+  const float ch = (float)c, cl = (float)(c - (double)ch);
+  const float c12h = (float)(c / 12.0), c12l = (float)(c / 12.0 - (double)c12h);
+  const int lane = threadIdx.x & 31;
+  const long long rows = (long long)D.n[1] * D.n[2];
+  const long long warps = (long long)gridDim.x * (kThreads / 32);
+  for (long long row = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows;
+       row += warps) {
+    const int j = (int)(row % D.n[1]), k = (int)(row / D.n[1]);
+    const bool edge_row = j == 0 || k == 0 || j == D.n[1] - 1 || k == D.n[2] - 1;
+    for (int i = lane; i < D.n[0]; i += 32) {
+      const long long idx = row * D.n[0] + i;
+      const bool edge = edge_row || i == 0 || i == D.n[0] - 1;
+      const T rc = rho[idx];
+      T nb[6];  // rho = 0 outside the grid
+      if (!printed) {
+        nb[0] = i > 0 ? rho[idx - 1] : T(0);
+        nb[1] = i < D.n[0] - 1 ? rho[idx + 1] : T(0);
+        nb[2] = j > 0 ? rho[idx - D.n[0]] : T(0);
+        nb[3] = j < D.n[1] - 1 ? rho[idx + D.n[0]] : T(0);
+        nb[4] = k > 0 ? rho[idx - D.nxy] : T(0);
+        nb[5] = k < D.n[2] - 1 ? rho[idx + D.nxy] : T(0);
+      }
+      double v;
+      if (sizeof(T) == 4 && !edge) {
+        // c (rho / 2 + sum / 12), the products to 2^-46
+        if (printed) {
+          out[idx] = fmaf((float)rc, ch, (float)rc * cl);
+          continue;
+        }
+        SourcePair s = {6.0f * (float)rc, 0.0f};
+        s.lo = fmaf(6.0f, (float)rc, -s.hi);
+#pragma unroll
+        for (int q = 0; q < 6; q++) pair_add(s, (float)nb[q]);
+        const float p = s.hi * c12h;
+        out[idx] = p + (fmaf(s.hi, c12h, -p) + fmaf(s.hi, c12l, s.lo * c12h));
+        continue;
+      }
+      double src = (double)rc;
+      if (!printed) {
+        double lap = -6.0 * src;
+#pragma unroll
+        for (int q = 0; q < 6; q++) lap += (double)nb[q];
+        src = src + lap / 12.0;
+      }
+      v = c * src;
+      if (edge) {
+        for (int dz = -1; dz <= 1; dz++)
+          for (int dy = -1; dy <= 1; dy++)
+            for (int dx = -1; dx <= 1; dx++) {
+              const int ii = i + dx, jj = j + dy, kk = k + dz;
+              const bool outside = ii < 0 || jj < 0 || kk < 0 || ii >= D.n[0] || jj >= D.n[1] ||
+                                   kk >= D.n[2];
+              if (!outside) continue;
+              const int nnz = (dx != 0) + (dy != 0) + (dz != 0);
+              const double w = nnz == 1 ? 4.0 / 9.0 : (nnz == 2 ? 1.0 / 9.0 : 1.0 / 36.0);
+              v -= w * shell[shell_at(D, ii, jj, kk)];
+            }
+      }
+      out[idx] = (T)v;
     }
-    double v = c * src;
-    const bool edge = i == 0 || j == 0 || k == 0 || i == D.n[0] - 1 || j == D.n[1] - 1 ||
-                      k == D.n[2] - 1;
-    if (edge) {
-      for (int dz = -1; dz <= 1; dz++)
-        for (int dy = -1; dy <= 1; dy++)
-          for (int dx = -1; dx <= 1; dx++) {
-            const int ii = i + dx, jj = j + dy, kk = k + dz;
-            const bool outside = ii < 0 || jj < 0 || kk < 0 || ii >= D.n[0] || jj >= D.n[1] ||
-                                 kk >= D.n[2];
-            if (!outside) continue;
-            const int nnz = (dx != 0) + (dy != 0) + (dz != 0);
-            const double w = nnz == 1 ? 4.0 / 9.0 : (nnz == 2 ? 1.0 / 9.0 : 1.0 / 36.0);
-            v -= w * shell_potential(mom, centre(ii, D.n[0], h), centre(jj, D.n[1], h),
-                                     centre(kk, D.n[2], h), G);
-          }
-    }
-    out[idx] = (T)v;
   }
 }
 
 // Odd extension of every line along `axis` to M = 2 (N + 1) points:
 // (0, w_0 .. w_{N-1}, 0, -w_{N-1} .. -w_0).  Layout of the extension: axis 0 line-major
 // (line * M + p); axes 1 and 2 position-major (p * B + b), b the line's index over the
-// other two axes in memory order, so both the gather and the store are coalesced.
+// other two axes in memory order, so both the gather and the store are coalesced.  A warp
+// takes one contiguous row of the extension at a time (axis 0: a line; else, of position p,
+// the lines of one row of x), so no per-value index division is left (128^3: 16 us with
+// them, three quarters of it the divisions).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) dst_pack_kernel(const T* __restrict__ w, T* __restrict__ ext,
                                                             Dims D, int axis) {
-  const int N = D.n[axis];
+  const int N = D.n[axis], nx = D.n[0];
   const int M = 2 * (N + 1);
-  const long long B = D.ncell / N;
-  const long long total = (long long)M * B;
-  for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < total;
-       idx += (long long)gridDim.x * kThreads) {
-    long long line;
-    int p;
+  const int lane = threadIdx.x & 31;
+  const int other = axis == 0 ? 0 : D.n[axis == 1 ? 2 : 1];  // rows of x per position
+  const long long rows = axis == 0 ? (long long)D.n[1] * D.n[2] : (long long)M * other;
+  const long long warps = (long long)gridDim.x * (kThreads / 32);
+  for (long long row = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows;
+       row += warps) {
     if (axis == 0) {
-      line = idx / M;
-      p = (int)(idx % M);
+      for (int p = lane; p < M; p += 32) {
+        const int q = p <= N ? p - 1 : 2 * N + 1 - p;  // position along the axis, 0..N-1
+        const T v = p == 0 || p == N + 1 ? T(0) : w[row * N + q];
+        ext[row * M + p] = p <= N ? v : -v;
+      }
     } else {
-      p = (int)(idx / B);
-      line = idx % B;
+      const int p = (int)(row / other), r = (int)(row % other);
+      const int q = p <= N ? p - 1 : 2 * N + 1 - p;
+      const bool zero = p == 0 || p == N + 1;
+      const T* src = w + (axis == 1 ? (long long)r * D.nxy + (long long)q * nx
+                                    : (long long)q * D.nxy + (long long)r * nx);
+      T* dst = ext + row * nx;
+      for (int i = lane; i < nx; i += 32) {
+        const T v = zero ? T(0) : src[i];
+        dst[i] = p <= N ? v : -v;
+      }
     }
-    T v = T(0);
-    if (p != 0 && p != N + 1) {
-      const int q = p <= N ? p - 1 : 2 * N + 1 - p;  // position along the axis, 0..N-1
-      long long src;
-      if (axis == 0)
-        src = line * D.n[0] + q;
-      else if (axis == 1)
-        src = (line / D.n[0]) * D.nxy + (long long)q * D.n[0] + line % D.n[0];
-      else
-        src = (long long)q * D.nxy + line;
-      v = p <= N ? w[src] : -w[src];
-    }
-    ext[idx] = v;
   }
 }
 
-// Sine amplitudes back into the work array: S_k = -Im(Y_k) / 2, k = q + 1.
+// Sine amplitudes back into the work array: S_k = -Im(Y_k) / 2, k = q + 1 (the halving is
+// exact).  `tab` non-NULL (the last axis of the forward transform): also divided by the
+// eigenvalue 6 (prod - 1), with the inverse transform's scale folded in: times
+// c / (1 - tz ty tx), c = -scale / 6 (a table value, as tab's).  A warp takes one row of x.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) dst_unpack_kernel(const T* __restrict__ spec,
-                                                              T* __restrict__ w, Dims D, int axis) {
-  const int N = D.n[axis];
+                                                              T* __restrict__ w, Dims D, int axis,
+                                                              const double* __restrict__ tab,
+                                                              double coef) {
+  using V = typename TableOf<T>::type;
+  const V* const tx = reinterpret_cast<const V*>(tab);
+  const V* const ty = tx + D.n[0];
+  const V* const tz = ty + D.n[1];
+  const V c = *reinterpret_cast<const V*>(&coef);
+  const int nx = D.n[0], N = D.n[axis];
   const long long B = D.ncell / N;
   const long long half = N + 2;  // M / 2 + 1 complex values per line
-  for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < D.ncell;
-       idx += (long long)gridDim.x * kThreads) {
-    const int i = (int)(idx % D.n[0]);
-    const long long r = idx / D.n[0];
-    const int j = (int)(r % D.n[1]), k = (int)(r / D.n[1]);
-    long long ci;
-    if (axis == 0)
-      ci = r * half + (i + 1);
-    else if (axis == 1)
-      ci = (long long)(j + 1) * B + (long long)k * D.n[0] + i;
-    else
-      ci = (long long)(k + 1) * B + (long long)j * D.n[0] + i;
-    w[idx] = (T)(-0.5 * (double)spec[2 * ci + 1]);
-  }
-}
-
-// Divide the sine amplitudes by the eigenvalue 6 (prod - 1), with the inverse transform's
-// scale prod_a 2 / (N_a + 1) folded in.
-template <typename T>
-__global__ void __launch_bounds__(kThreads) iso_symbol_kernel(T* __restrict__ w, Dims D,
-                                                              const double* __restrict__ tab,
-                                                              double scale) {
-  const double* tx = tab;
-  const double* ty = tx + D.n[0];
-  const double* tz = ty + D.n[1];
-  for (long long idx = (long long)blockIdx.x * kThreads + threadIdx.x; idx < D.ncell;
-       idx += (long long)gridDim.x * kThreads) {
-    const int i = (int)(idx % D.n[0]);
-    const long long r = idx / D.n[0];
-    const int j = (int)(r % D.n[1]), k = (int)(r / D.n[1]);
-    const double lam = 6.0 * (tz[k] * ty[j] * tx[i] - 1.0);
-    w[idx] = (T)((double)w[idx] * (scale / lam));
+  const int lane = threadIdx.x & 31;
+  const long long rows = (long long)D.n[1] * D.n[2];
+  const long long warps = (long long)gridDim.x * (kThreads / 32);
+  for (long long row = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows;
+       row += warps) {
+    const int j = (int)(row % D.n[1]), k = (int)(row / D.n[1]);
+    const long long ci = axis == 0 ? row * half + 1
+                                   : (axis == 1 ? (long long)(j + 1) * B + (long long)k * nx
+                                                : (long long)(k + 1) * B + (long long)j * nx);
+    V tzy = V();
+    if (tab) tzy = table_product(tz[k], ty[j]);
+    for (int i = lane; i < nx; i += 32) {
+      T v = T(-0.5) * spec[2 * (ci + i) + 1];
+      if (tab) v = scaled(v, over_one_minus(c, tzy, tx[i]));
+      w[row * nx + i] = v;
+    }
   }
 }
 
@@ -252,6 +346,7 @@ struct PoissonIso {
   double* part;
   double* mom;
   double* tab;
+  double* shell;  // the potential on the cells around the grid
 };
 
 void ppml_iso_free(PoissonIso* s) {
@@ -262,6 +357,7 @@ void ppml_iso_free(PoissonIso* s) {
   if (s->part) cudaFree(s->part);
   if (s->mom) cudaFree(s->mom);
   if (s->tab) cudaFree(s->tab);
+  if (s->shell) cudaFree(s->shell);
   delete s;
 }
 
@@ -274,6 +370,8 @@ static int iso_create(const ppml_grid_desc* d, PoissonIso** out) {
   const bool f64 = d->dtype == PPML_F64;
   const size_t elt = f64 ? sizeof(double) : sizeof(float);
   const long long ncell = (long long)d->nx * d->ny * d->nz;
+  Dims D;
+  for (int a = 0; a < 3; a++) D.n[a] = s->n[a];
   size_t ext_n = 0, spec_n = 0;
   for (int a = 0; a < 3; a++) {
     const long long N = s->n[a], B = ncell / N;
@@ -284,7 +382,8 @@ static int iso_create(const ppml_grid_desc* d, PoissonIso** out) {
       cudaMalloc(&s->spec, spec_n * 2 * elt) != cudaSuccess ||
       cudaMalloc(&s->part, sizeof(double) * kMoments * kMaxMomentBlocks) != cudaSuccess ||
       cudaMalloc(&s->mom, sizeof(double) * kMoments) != cudaSuccess ||
-      cudaMalloc(&s->tab, sizeof(double) * (size_t)(s->n[0] + s->n[1] + s->n[2])) != cudaSuccess) {
+      cudaMalloc(&s->tab, sizeof(double) * (size_t)(s->n[0] + s->n[1] + s->n[2])) != cudaSuccess ||
+      cudaMalloc(&s->shell, sizeof(double) * (size_t)shell_cells(D)) != cudaSuccess) {
     cudaGetLastError();
     ppml_iso_free(s);
     return ppml_fail(PPML_E_NOMEM, "isolated Poisson buffers (%zu + %zu elements)", ext_n,
@@ -294,7 +393,7 @@ static int iso_create(const ppml_grid_desc* d, PoissonIso** out) {
   for (int a = 0; a < 3; a++)
     for (int q = 0; q < s->n[a]; q++) {
       const double sn = sin(M_PI * (double)(q + 1) / (2.0 * (double)(s->n[a] + 1)));
-      tab.push_back(1.0 - (2.0 / 3.0) * sn * sn);
+      tab.push_back(ppml_table_value(1.0 - (2.0 / 3.0) * sn * sn, f64));
     }
   if (cudaMemcpy(s->tab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice) !=
       cudaSuccess) {
@@ -332,10 +431,13 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   if (rc) return rc;
   moment_final_kernel<<<1, kThreads, 0, st>>>(s->part, nb, s->mom);
   if ((rc = ppml_check_launch("moment_final_kernel"))) return rc;
-  rhs_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, h, G, s->mom, printed);
+  shell_kernel<<<blocks_for(shell_cells(D)), kThreads, 0, st>>>(D, h, G, s->mom, s->shell);
+  if ((rc = ppml_check_launch("shell_kernel"))) return rc;
+  rhs_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, h, G, s->shell, printed);
   if ((rc = ppml_check_launch("rhs_kernel"))) return rc;
   double scale = 1.0;
   for (int a = 0; a < 3; a++) scale *= 2.0 / (double)(D.n[a] + 1);
+  const double symbol = ppml_table_value(-scale / 6.0, sizeof(T) == sizeof(double));
   for (int pass = 0; pass < 2; pass++) {
     for (int a = 0; a < 3; a++) {
       const long long total = 2LL * (D.n[a] + 1) * (D.ncell / D.n[a]);
@@ -349,12 +451,9 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
       else
         r = cufftExecR2C(s->plan[a], (cufftReal*)s->ext, (cufftComplex*)s->spec);
       if (r != CUFFT_SUCCESS) return ppml_fail(PPML_E_CUDA, "cuFFT sine transform failed (%d)", (int)r);
-      dst_unpack_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>((const T*)s->spec, phi, D, a);
+      dst_unpack_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(
+          (const T*)s->spec, phi, D, a, pass == 0 && a == 2 ? s->tab : nullptr, symbol);
       if ((rc = ppml_check_launch("dst_unpack_kernel"))) return rc;
-    }
-    if (pass == 0) {
-      iso_symbol_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(phi, D, s->tab, scale);
-      if ((rc = ppml_check_launch("iso_symbol_kernel"))) return rc;
     }
   }
   return PPML_OK;
