@@ -64,7 +64,10 @@ __device__ __forceinline__ void fill_ghosts_1d(T* q, int n) {
 template <typename T>
 __device__ __forceinline__ T template_1d(T v) {
   const T four = v + v + v + v;
-  return four / T(16) + four / T(8) + v / T(4);
+  if constexpr (sizeof(T) == 8)
+    return f64::scale<-4>(four) + f64::scale<-3>(four) + f64::scale<-2>(v);
+  else
+    return four / T(16) + four / T(8) + v / T(4);
 }
 
 // Parabolas of two quantities along a contiguous run of faces, streamed (Appendix Steps 1-3):
@@ -481,14 +484,14 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
     }
   }
   // Upwind Lagrangian fluxes of one field at the own faces 0 .. nl (Sec. 1.3)
-  auto lagrangian_fluxes = [&](const T* q, double dt, T th) {
+  auto lagrangian_fluxes = [&](const T* q, const AxisStep<T>& ks) {
     auto qq = [&](int c) { return q[c + G]; };
     for (int f0 = tid * run; f0 <= nl; f0 += NTHREADS * run) {
       const int f1 = min(f0 + run - 1, nl);
       stream_faces<T>(qq, f0, f1, [&](int f, const Parab<T>& PL, const Parab<T>& PR) {
         const T vh = FA[f + FO];
-        const T y = Prec<T>::courant(tabs(vh), dt, I.h, th);
-        FB[f + FO] = vh >= T(0) ? vh * avg_right(PL.R, PL.D, PL.S, y)
+        const T y = Prec<T>::courant(tabs(vh), ks);
+        FB[f + FO] = nonnegative(vh) ? vh * avg_right(PL.R, PL.D, PL.S, y)
                                 : vh * avg_left(PR.L, PR.D, PR.S, y);
       });
     }
@@ -508,6 +511,7 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
     else
       go = block_cfl_step<T>(vm, cm, bad, cfl, I, red, dt, th);
     if (!go) break;
+    const AxisStep<T> ks(dt, I.h, th);
     // Eulerian stage: faces fa .. fb; each thread streams one run of consecutive faces
     {
       auto vq = [&](int k) { return vel_of(M[k + G], R[k + G]); };
@@ -516,7 +520,11 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
         const int f1 = min(f0 + run_e - 1, P.fb);
         // rho and sqrt(rho) of the face's left cell, carried from the previous face
         T r_l = R[f0 - 1 + G], s_l = T(0);
-        if constexpr (sizeof(T) == 4) s_l = sqrt_approx(r_l);
+        RootWeights w_l = {0, 0, 0};  // FP64
+        if constexpr (sizeof(T) == 4)
+          s_l = sqrt_approx(r_l);
+        else
+          w_l = root_weights(r_l, pq(f0 - 1));
         stream_faces2<T>(vq, pq, f0, f1,
                          [&](int f, T, T, const Parab<T>& vL, const Parab<T>& vR, T pl, T pr,
                              const Parab<T>& pL, const Parab<T>& pR) {
@@ -535,8 +543,10 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
             Pf = 0.5f * (pls + prs) + 0.5f * Z * (vls - vrs);
           } else {
             T lam, Z;
-            face_constants(rl, rr, pl, pr, gamma, lam, Z);
-            const T y = Prec<T>::courant(lam, dt, I.h, th);
+            const RootWeights wr = root_weights(rr, pr);
+            face_constants(w_l, wr, gamma, lam, Z);
+            w_l = wr;
+            const T y = Prec<T>::courant(lam, ks);
             riemann_vp(avg_right(vL.R, vL.D, vL.S, y), avg_left(vR.L, vR.D, vR.S, y),
                        avg_right(pL.R, pL.D, pL.S, y), avg_left(pR.L, pR.D, pR.S, y), Z, V, Pf);
           }
@@ -604,7 +614,7 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
           const float vh = (vt_r * s_r + vt_l * s_l) * rcp_approx(s_r + s_l);
           vt_l = vt_r;
           s_l = s_r;
-          const float y = Prec<float>::courant(tabs(vh), dt, I.h, th);
+          const float y = Prec<float>::courant(tabs(vh), ks);
           float F[4];
 #pragma unroll
           for (int j = 0; j < 4; j++)
@@ -710,13 +720,13 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
 #pragma unroll 1
       for (int k = 0; k < 3; k++) {
         T* q = fields[k];
-        lagrangian_fluxes(q, dt, th);
+        lagrangian_fluxes(q, ks);
         __syncthreads();
         for (int c = tid; c < nl; c += NTHREADS)
           q[c + G] = q[c + G] - th * (FB[c + 1 + FO] - FB[c + FO]);
         __syncthreads();
       }
-      lagrangian_fluxes(Ei, dt, th);
+      lagrangian_fluxes(Ei, ks);
       __syncthreads();
       // rho eps update, then the Sec. 1.4 energy consistency, on the same cells
       vm = T(0);

@@ -17,27 +17,46 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "ppml_f64.cuh"
+
 namespace ppml {
 
 template <typename T>
 struct Prec;
 
+// Constants of a sweep along one axis: tau, h, th = tau / h (and FP64: 1 / h).
+template <typename T>
+struct AxisStep;
+
+template <>
+struct AxisStep<float> {
+  float th;
+  __device__ __forceinline__ AxisStep(double, double, float th_) : th(th_) {}
+};
+template <>
+struct AxisStep<double> {
+  double th, tau;
+  f64::Divisor h;
+  __device__ __forceinline__ AxisStep(double tau_, double h_, double th_)
+      : th(th_), tau(tau_), h(f64::divisor(h_)) {}
+};
+
 template <>
 struct Prec<float> {
+  static __device__ __forceinline__ float half(float x) { return 0.5f * x; }
   static __device__ __forceinline__ float two_thirds(float y) { return y * (2.0f / 3.0f); }
   // Courant number of a signal speed s: s * tau / h with th = tau / h precomputed.
-  static __device__ __forceinline__ float courant(float s, double /*tau*/, double /*h*/,
-                                                  float th) {
-    return s * th;
+  static __device__ __forceinline__ float courant(float s, const AxisStep<float>& k) {
+    return s * k.th;
   }
 };
 
 template <>
 struct Prec<double> {
-  static __device__ __forceinline__ double two_thirds(double y) { return 2.0 * y / 3.0; }
-  static __device__ __forceinline__ double courant(double s, double tau, double h,
-                                                   double /*th*/) {
-    return s * tau / h;
+  static __device__ __forceinline__ double half(double x) { return f64::half(x); }
+  static __device__ __forceinline__ double two_thirds(double y) { return f64::div3(f64::twice(y)); }
+  static __device__ __forceinline__ double courant(double s, const AxisStep<double>& k) {
+    return f64::divide(s * k.tau, k.h);
   }
 };
 
@@ -46,8 +65,10 @@ struct Parab {
   T L, R, D, S;  // q^L, q^R, Delta q = q^R - q^L, q^(6)
 };
 
-template <typename T>
-__device__ __forceinline__ T tabs(T x) { return x < T(0) ? -x : x; }
+__device__ __forceinline__ float tabs(float x) { return x < 0.0f ? -x : x; }
+__device__ __forceinline__ double tabs(double x) { return fabs(x); }
+__device__ __forceinline__ bool nonnegative(float x) { return x >= 0.0f; }
+__device__ __forceinline__ bool nonnegative(double x) { return f64::hi_word(x) >= 0; }
 
 // Appendix, Step 1: limited slope delta_m q_i.  Branch-free: min(|dq|, 2 min(|r|, |l|))
 // equals min(|dq|, 2|r|, 2|l|) exactly (doubling is exact), and r l > 0 implies q is
@@ -59,11 +80,8 @@ __device__ __forceinline__ T tabs(T x) { return x < T(0) ? -x : x; }
 template <typename T>
 __device__ __forceinline__ T limited_slope(T qm, T q0, T qp) {
   const T r = qp - q0, l = q0 - qm;
-  if constexpr (sizeof(T) == 8) {  // FP64: evaluate only what is used (same values)
-    const T dq = T(0.5) * (qp - qm);
-    if (!(r * l > T(0))) return T(0);
-    const T m = fmin(fabs(dq), T(2) * fmin(fabs(r), fabs(l)));
-    return copysign(m, dq);
+  if constexpr (sizeof(T) == 8) {
+    return f64::slope(l, r, qp - qm);
   } else {
     const T dq2 = qp - qm;
     const T m2 = fmin(fabs(dq2), T(4) * fmin(fabs(r), fabs(l)));
@@ -77,7 +95,7 @@ __device__ __forceinline__ T limited_slope(T qm, T q0, T qp) {
 template <typename T>
 __device__ __forceinline__ T face_value(T q0, T q1, T d0, T d1) {
   if constexpr (sizeof(T) == 8)
-    return T(0.5) * (q0 + q1) - (d1 - d0) / 6.0;
+    return f64::half(q0 + q1) - f64::div6(d1 - d0);
   else
     return T(0.5) * (q0 + q1) - (d1 - d0) * (1.0f / 12.0f);
 }
@@ -88,15 +106,32 @@ __device__ __forceinline__ T face_value(T q0, T q1, T d0, T d1) {
 // sequential form (flat test first, then at most one fix).
 template <typename T>
 __device__ __forceinline__ Parab<T> parabola(T q0, T L, T R) {
-  const bool flat = (L - q0) * (q0 - R) <= T(0);
-  if (sizeof(T) == 8 && flat) {  // FP64: skip the overshoot tests of a flattened cell
+  if constexpr (sizeof(T) == 8) {
     Parab<T> p;
-    p.L = q0;
-    p.R = q0;
-    p.D = q0 - q0;
-    p.S = T(6) * (q0 - T(0.5) * (q0 + q0));
+    if (f64::product_nonpositive(L - q0, q0 - R)) {  // flat: q0 - q0 = 0 for finite q0
+      p.L = q0;
+      p.R = q0;
+      p.D = T(0);
+      p.S = T(0);
+      if (f64::exponent(q0) == 0x7ffu) p.D = p.S = q0 - q0;
+      return p;
+    }
+    p.L = L;
+    p.R = R;
+    p.D = R - L;
+    p.S = T(6) * (q0 - f64::half(L + R));
+    const int o = f64::overshoot(p.D, p.S);
+    if (o != 0) {
+      if (o > 0)
+        p.L = T(3) * q0 - f64::twice(R);
+      else
+        p.R = T(3) * q0 - f64::twice(L);
+      p.D = p.R - p.L;
+      p.S = T(6) * (q0 - f64::half(p.L + p.R));
+    }
     return p;
   }
+  const bool flat = (L - q0) * (q0 - R) <= T(0);
   const T D = R - L;
   const T S = T(6) * (q0 - T(0.5) * (L + R));
   // at most one fix: D S > D D >= 0 >= -(D D) excludes D S < -(D D)
@@ -116,22 +151,33 @@ __device__ __forceinline__ Parab<T> parabola(T q0, T L, T R) {
 // the cell (q_L(-lambda t), y = lambda t / h) ...
 template <typename T>
 __device__ __forceinline__ T avg_right(T R, T D, T S, T y) {
-  return R - T(0.5) * y * (D - S * (T(1) - Prec<T>::two_thirds(y)));
+  return R - Prec<T>::half(y) * (D - S * (T(1) - Prec<T>::two_thirds(y)));
 }
 // ... and over its left fraction y (q_R(lambda t)).
 template <typename T>
 __device__ __forceinline__ T avg_left(T L, T D, T S, T y) {
-  return L + T(0.5) * y * (D + S * (T(1) - Prec<T>::two_thirds(y)));
+  return L + Prec<T>::half(y) * (D + S * (T(1) - Prec<T>::two_thirds(y)));
 }
 
 // Sec. 1.1/1.2: face constants of the acoustic Riemann problem from the adjacent cell
-// values: lambda = sqrt(gamma p^/rho^) and the impedance Z = rho^ lambda.
-template <typename T>
-__device__ __forceinline__ void face_constants(T rl, T rr, T pl, T pr, T gamma, T& lam, T& Z) {
-  const T sl = sqrt(rl), sr = sqrt(rr);
-  const T A = rl * sl + rr * sr;  // rho_L^{3/2} + rho_R^{3/2}
-  const T B = pl * sl + pr * sr;  // p_L sqrt(rho_L) + p_R sqrt(rho_R)
-  const T S = sl + sr;
+// values: lambda = sqrt(gamma p^/rho^) and the impedance Z = rho^ lambda (FP64; sl, sr the
+// square roots of rl, rr, and ws the products rho sqrt(rho), p sqrt(rho) of a cell, each
+// formed once per cell by the caller).
+struct RootWeights {
+  double s, a, b;  // sqrt(rho), rho sqrt(rho), p sqrt(rho)
+};
+__device__ __forceinline__ RootWeights root_weights(double rho, double p) {
+  RootWeights w;
+  w.s = sqrt(rho);
+  w.a = rho * w.s;
+  w.b = p * w.s;
+  return w;
+}
+__device__ __forceinline__ void face_constants(const RootWeights& l, const RootWeights& r,
+                                               double gamma, double& lam, double& Z) {
+  const double A = l.a + r.a;  // rho_L^{3/2} + rho_R^{3/2}
+  const double B = l.b + r.b;  // p_L sqrt(rho_L) + p_R sqrt(rho_R)
+  const double S = l.s + r.s;
   lam = sqrt(gamma * B / A);
   Z = sqrt(gamma * A * B / (S * S));
 }
@@ -146,16 +192,17 @@ __device__ __forceinline__ T upwind_state(bool from_left, T R_l, T D_l, T S_l, T
   const T D = from_left ? D_l : D_r;
   const T S = from_left ? S_l : S_r;
   const T t = S * (T(1) - Prec<T>::two_thirds(y));
-  const T u = from_left ? D - t : D + t;
-  const T w = T(0.5) * y * u;
-  return from_left ? R_l - w : L_r + w;
+  // (an addition of the negated term is the subtraction)
+  const T u = D + (from_left ? -t : t);
+  const T w = Prec<T>::half(y) * u;
+  return (from_left ? R_l : L_r) + (from_left ? -w : w);
 }
 
 // eqs. lowriemannvelocity / lowriemannpressure from the four characteristic averages.
-template <typename T>
-__device__ __forceinline__ void riemann_vp(T vls, T vrs, T pls, T prs, T Z, T& V, T& P) {
-  V = T(0.5) * (vls + vrs) + (pls - prs) / (T(2) * Z);
-  P = T(0.5) * (pls + prs) + T(0.5) * Z * (vls - vrs);
+__device__ __forceinline__ void riemann_vp(double vls, double vrs, double pls, double prs,
+                                           double Z, double& V, double& P) {
+  V = f64::half(vls + vrs) + (pls - prs) / f64::twice(Z);
+  P = f64::half(pls + prs) + f64::half(Z) * (vls - vrs);
 }
 
 // Sec. 1.4: energy consistency of one cell, in double.  u = {rho, mx, my, mz, rhoE, rhoeps}.

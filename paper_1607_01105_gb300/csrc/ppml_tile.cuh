@@ -282,14 +282,16 @@ __device__ __forceinline__ void sweep_eulerian_dev(VF v, PF pr, RF r, float gamm
 // order) and double-float FP32 states (whose low parts record the rounding of exactly these
 // expressions).
 template <typename T, bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
-__device__ __forceinline__ void sweep_eulerian(VF v, PF pr, RF r, T gamma, T th, double tau,
-                                               double h, EF emit, HF hook) {
+__device__ __forceinline__ void sweep_eulerian(VF v, PF pr, RF r, T gamma,
+                                               const AxisStep<T>& ks, EF emit, HF hook) {
+  const T th = ks.th;
   T va = v(-3), vb = v(-2), pa = pr(-3), pb = pr(-2);
   T dva = T(0), fva = T(0), dpa = T(0), fpa = T(0);
   T vR = T(0), vD = T(0), vS = T(0), pR = T(0), pD = T(0), pS = T(0);
   T Vp = T(0), Pp = T(0);
   T rprev = T(0), pprev = T(0);  // rho, p of cell p-3
   T sprev = T(0);                // FP32: sqrt(rho) of cell p-3
+  RootWeights wprev = {0, 0, 0};  // FP64: the root weights of cell p-3
   // step p; WARM: one of the first four steps (p constant), which skip the parts whose
   // inputs have not arrived; in FP32 the steady steps p = 3..18 run as a loop unrolled by
   // two (a smaller body for the instruction cache)
@@ -322,17 +324,20 @@ __device__ __forceinline__ void sweep_eulerian(VF v, PF pr, RF r, T gamma, T th,
           Pp = P;
         }
         sprev = sc;
-      } else if (!W || p >= 2) {
-        // face between cells p-3 and p-2
+      } else {
+        const RootWeights wc = root_weights(rc, pa);
+        if (!W || p >= 2) {  // face between cells p-3 and p-2
         T lam, Z;
-        face_constants(rprev, rc, pprev, pa, gamma, lam, Z);
-        const T y = Prec<T>::courant(lam, tau, h, th);
+        face_constants(wprev, wc, gamma, lam, Z);
+        const T y = Prec<T>::courant(lam, ks);
         T V, P;
         riemann_vp(avg_right(vR, vD, vS, y), avg_left(Pv.L, Pv.D, Pv.S, y),
                    avg_right(pR, pD, pS, y), avg_left(Pq.L, Pq.D, Pq.S, y), Z, V, P);
         if (!W || p >= 3) emit(p - 3, th * (P - Pp), th * (P * V - Pp * Vp), th * (V - Vp));
         Vp = V;
         Pp = P;
+        }
+        wprev = wc;
       }
       vR = Pv.R;
       vD = Pv.D;
@@ -573,8 +578,8 @@ __device__ __forceinline__ float half_flux_f32(float w, float R_l, float D_l, fl
 // update is added in double-float (dst the high part, dstlo the low part).  CS: the core
 // stride of the sweep axis as a compile-time constant (immediate shared-memory offsets).
 template <typename T, int MODE, bool FLAT, bool DF, int CS>
-__device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* vh, T th,
-                                         double tau, double h, T* acc, bool have_acc,
+__device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* vh,
+                                         const AxisStep<T>& ks, T* acc, bool have_acc,
                                          T* __restrict__ dst, long long gs, int nvalid,
                                          const T* __restrict__ srclo = nullptr,
                                          T* __restrict__ dstlo = nullptr) {
@@ -608,8 +613,8 @@ __device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* 
     Fp = half_flux_f32(vh[0], PR, PD, PS, P.L, P.D, P.S);
   } else {
     const T v = vh[0];
-    const T y = Prec<T>::courant(tabs(v), tau, h, th);
-    Fp = v * upwind_state(v >= T(0), PR, PD, PS, P.L, P.D, P.S, y);
+    const T y = Prec<T>::courant(tabs(v), ks);
+    Fp = v * upwind_state(nonnegative(v), PR, PD, PS, P.L, P.D, P.S, y);
   }
   PR = P.R;
   PD = P.D;
@@ -629,9 +634,9 @@ __device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* 
       F = half_flux_f32(vv, PR, PD, PS, Pn.L, Pn.D, Pn.S);
       d = F - Fp;  // half of th (F+ - F-)
     } else {
-      const T yy = Prec<T>::courant(tabs(vv), tau, h, th);
-      F = vv * upwind_state(vv >= T(0), PR, PD, PS, Pn.L, Pn.D, Pn.S, yy);
-      d = th * (F - Fp);
+      const T yy = Prec<T>::courant(tabs(vv), ks);
+      F = vv * upwind_state(nonnegative(vv), PR, PD, PS, Pn.L, Pn.D, Pn.S, yy);
+      d = ks.th * (F - Fp);
     }
     const int o = c * cs;
     if (MODE == 0) {
@@ -702,8 +707,11 @@ __device__ __forceinline__ void line_face_velocities(const T* vb, const T* rb, i
     const int o = base + p * s_ax;
     const T corners = vb[o + s_b + s_c] + vb[o + s_b - s_c] + vb[o - s_b + s_c] + vb[o - s_b - s_c];
     const T edges = vb[o + s_b] + vb[o - s_b] + vb[o + s_c] + vb[o - s_c];
-    const T vt = one_point ? vb[o] : corners / T(16) + edges / T(8) + vb[o] / T(4);
-    T sq;
+    T vt, sq;
+    if constexpr (sizeof(T) == 4)
+      vt = one_point ? vb[o] : corners / T(16) + edges / T(8) + vb[o] / T(4);
+    else
+      vt = one_point ? vb[o] : f64::scale<-4>(corners) + f64::scale<-3>(edges) + f64::scale<-2>(vb[o]);
     if constexpr (sizeof(T) == 4) {
       sq = sqrt_approx(rb[o]);
       if (p >= 0) out[p] = (vt * sq + vt_prev * sq_prev) * rcp_approx(sq + sq_prev);
@@ -921,6 +929,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
       T* dstlo = DF && f < 5 ? A.outlo[f] + zline0 : nullptr;
       const T* core = &S.fld[cb];
       T* acc = &S.acc[cb];
+      const AxisStep<T> ks(tau, A.h[ax], th[ax]);
       // one instantiation per (axis, mode): x is always the first sweep (mode 0), y the
       // first or the second, z the last (MODE 2: finish into the output)
       auto sweep = [&](auto mode_c, auto flat_c, auto cs_c) {
@@ -931,11 +940,10 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
           lag_line_dev<M, FL, C>(core, halo, vhl, acc, mode == 1, A.out[f] + zline0, g.nxy,
                                  nvalid_z);
         else if constexpr (M == 2)
-          lag_line<T, 2, FL, DF, C>(core, halo, vhl, th[2], tau, A.h[2], acc, mode == 1,
+          lag_line<T, 2, FL, DF, C>(core, halo, vhl, ks, acc, mode == 1,
                                     A.out[f] + zline0, g.nxy, nvalid_z, srclo, dstlo);
         else
-          lag_line<T, M, FL, false, C>(core, halo, vhl, th[ax], tau, A.h[ax], acc, false,
-                                       nullptr, 0, 0);
+          lag_line<T, M, FL, false, C>(core, halo, vhl, ks, acc, false, nullptr, 0, 0);
       };
       auto sweep_ax = [&](auto flat_c) {
         if (ax == 2)
@@ -1262,7 +1270,7 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
       if constexpr (sizeof(T) == 4 && !DF)
         sweep_eulerian_dev<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
       else
-        sweep_eulerian<T, FL>(vq, pq, rq, gamma, th[ax], tau, A.h[ax], emit, hook);
+        sweep_eulerian<T, FL>(vq, pq, rq, gamma, AxisStep<T>(tau, A.h[ax], th[ax]), emit, hook);
     };
     if (A.flags & PPML_FIRST_ORDER)
       sweep(BoolC<true>());
