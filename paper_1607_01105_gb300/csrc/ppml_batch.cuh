@@ -403,6 +403,8 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
   T* const fields[7] = {R, M, E, Ei, RL, ML, EL};
   const int tid = threadIdx.x;
   const T gamma = T(gamma_d), gm1 = T(gamma_d - 1.0);
+  f64::Divisor hdiv = {};  // FP64: the cell size as a divisor
+  if constexpr (sizeof(T) == 8) hdiv = f64::divisor(I.h);
   // faces per streamed run: one run per thread covers the pass's faces; at least 9 (the
   // stream reads 3 extra cells on each side of its run) and odd, so that the runs of the
   // 32 lanes of a warp start on 32 different banks
@@ -442,8 +444,9 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
       v = fabsf(m * ir);
       cs = sqrt_approx(gamma * p * ir);
     } else {
-      const T vx = m / r, vy = T(0) / r, vz = T(0) / r;
-      v = sqrt(vx * vx + vy * vy + vz * vz);
+      // |v| = sqrt(vx^2 + 0 + 0), which is |vx| exactly while the square is a normal number
+      const T vx = f64::over(m, r);
+      v = f64::is_zero(vx) || f64::moderate(vx) ? fabs(vx) : sqrt(vx * vx);
       cs = sqrt(gamma * p / r);
     }
     vm = valid ? fmax(vm, v) : vm;
@@ -490,9 +493,12 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
       const int f1 = min(f0 + run - 1, nl);
       stream_faces<T>(qq, f0, f1, [&](int f, const Parab<T>& PL, const Parab<T>& PR) {
         const T vh = FA[f + FO];
-        const T y = Prec<T>::courant(tabs(vh), ks);
-        FB[f + FO] = nonnegative(vh) ? vh * avg_right(PL.R, PL.D, PL.S, y)
-                                : vh * avg_left(PR.L, PR.D, PR.S, y);
+        if constexpr (sizeof(T) == 8) {  // (FP32 forms all four fluxes in one pass, below)
+          const bool left = f64::hi_word(vh) >= 0;
+          const f64::Weights k = f64::weights(courant(tabs(vh), ks));
+          FB[f + FO] = vh * f64::average(left, left ? PL.R : PR.L, left ? PL.D : PR.D,
+                                         left ? PL.S : PR.S, k);
+        }
       });
     }
   };
@@ -511,7 +517,7 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
     else
       go = block_cfl_step<T>(vm, cm, bad, cfl, I, red, dt, th);
     if (!go) break;
-    const AxisStep<T> ks(dt, I.h, th);
+    const AxisStep<T> ks(dt, hdiv, th);
     // Eulerian stage: faces fa .. fb; each thread streams one run of consecutive faces
     {
       auto vq = [&](int k) { return vel_of(M[k + G], R[k + G]); };
@@ -546,9 +552,10 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
             const RootWeights wr = root_weights(rr, pr);
             face_constants(w_l, wr, gamma, lam, Z);
             w_l = wr;
-            const T y = Prec<T>::courant(lam, ks);
-            riemann_vp(avg_right(vL.R, vL.D, vL.S, y), avg_left(vR.L, vR.D, vR.S, y),
-                       avg_right(pL.R, pL.D, pL.S, y), avg_left(pR.L, pR.D, pR.S, y), Z, V, Pf);
+            const f64::Weights k = f64::weights(courant(lam, ks));
+            riemann_vp(f64::average(true, vL.R, vL.D, vL.S, k), f64::average(false, vR.L, vR.D, vR.S, k),
+                       f64::average(true, pL.R, pL.D, pL.S, k), f64::average(false, pR.L, pR.D, pR.S, k),
+                       Z, V, Pf);
           }
           FA[f + FO] = V;
           FB[f + FO] = Pf;
@@ -614,7 +621,7 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
           const float vh = (vt_r * s_r + vt_l * s_l) * rcp_approx(s_r + s_l);
           vt_l = vt_r;
           s_l = s_r;
-          const float y = Prec<float>::courant(tabs(vh), ks);
+          const float y = courant(tabs(vh), ks);
           float F[4];
 #pragma unroll
           for (int j = 0; j < 4; j++)

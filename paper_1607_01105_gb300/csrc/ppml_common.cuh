@@ -211,7 +211,7 @@ struct FieldSums<double> {
   }
   __device__ __forceinline__ void add(const double u[6]) {
 #pragma unroll
-    for (int f = 0; f < 6; f++) s[f] += u[f];
+    for (int f = 0; f < 6; f++) s[f] = f64::plus(s[f], u[f]);
   }
   __device__ __forceinline__ void get(double out[6]) const {
 #pragma unroll
@@ -238,6 +238,88 @@ __device__ __forceinline__ void cell_speeds(const T u[6], T gamma, T gm1, T& vma
     nbad++;
   }
 }
+
+// The CFL maxima of an FP64 tile without five divisions and roots per cell: every cell's
+// speeds are bounded in float (RoughSpeeds: upper bounds), the largest lower bounds of the
+// tile are taken, and only cells whose upper bound reaches them are evaluated exactly
+// (ExactSpeeds, in cell_speeds' operations).  Values outside 2^-60 .. 2^60 have no float
+// bound: their cells are always evaluated.
+struct RoughSpeeds {
+  float v, c;  // upper bounds; v = 0: at rest exactly; negative: not a physical cell
+};
+constexpr float kRoughUp = 1.00002f, kRoughDown = 0.99998f;  // truncations and approximations
+
+__device__ __forceinline__ float truncated_float(double x) {  // x in float range or zero
+  const unsigned h = (unsigned)f64::hi_word(x), l = (unsigned)f64::lo_word(x);
+  if ((h << 1) == 0u) return 0.0f;
+  return __uint_as_float((h & 0x80000000u) | (((h & 0x7fffffffu) - (896u << 20)) << 3) | (l >> 29));
+}
+__device__ __forceinline__ bool rough_range(double x) { return f64::exponent(x) - 963u <= 120u; }
+
+__device__ __forceinline__ void rough_speeds(const double u[6], float ggm1, RoughSpeeds& r,
+                                             float& vlow, float& clow,
+                                             unsigned long long& nbad) {
+  bool ok = f64::positive(u[0]) && f64::positive(u[5]);
+#pragma unroll
+  for (int f = 0; f < 6; f++) ok = ok && f64::finite(u[f]);
+  if (!ok) {
+    nbad++;
+    r.v = r.c = -1.0f;
+    return;
+  }
+  bool in = rough_range(u[0]) && rough_range(u[5]);
+  bool rest = true;
+#pragma unroll
+  for (int f = 1; f <= 3; f++) {
+    const bool z = f64::is_zero(u[f]);
+    rest = rest && z;
+    in = in && (z || rough_range(u[f]));
+  }
+  if (!in) {
+    r.v = rest ? 0.0f : __int_as_float(0x7f800000);
+    r.c = __int_as_float(0x7f800000);
+    return;
+  }
+  const float ir = rcp_approx(truncated_float(u[0]));
+  const float c = sqrt_approx(ggm1 * truncated_float(u[5]) * ir);
+  float v = 0.0f;
+  if (!rest) {
+    const float mx = truncated_float(u[1]), my = truncated_float(u[2]), mz = truncated_float(u[3]);
+    v = sqrt_approx(mx * mx + my * my + mz * mz) * ir;
+  }
+  r.v = v * kRoughUp;
+  r.c = c * kRoughUp;
+  vlow = fmaxf(vlow, v * kRoughDown);
+  clow = fmaxf(clow, c * kRoughDown);
+}
+
+__device__ __forceinline__ float warp_max(float x) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) x = fmaxf(x, __shfl_xor_sync(0xffffffffu, x, o));
+  return x;
+}
+
+struct ExactSpeeds {
+  double rho = 0.0, ei = 0.0;  // the last evaluated sound speed's cell (equal cells: equal speed)
+  double last[4] = {0.0, 0.0, 0.0, 0.0};
+  __device__ __forceinline__ void add(const double u[6], double gamma, double gm1, bool need_v,
+                                      bool need_c, double& vmax, double& cmax) {
+    if (need_v && !(f64::same_bits(u[0], last[0]) && f64::same_bits(u[1], last[1]) &&
+                    f64::same_bits(u[2], last[2]) && f64::same_bits(u[3], last[3]))) {
+#pragma unroll
+      for (int f = 0; f < 4; f++) last[f] = u[f];
+      const double vx = f64::over(u[1], u[0]), vy = f64::over(u[2], u[0]), vz = f64::over(u[3], u[0]);
+      const double v = sqrt(vx * vx + vy * vy + vz * vz);
+      vmax = fmax(vmax, v);
+    }
+    if (need_c && !(f64::same_bits(u[0], rho) && f64::same_bits(u[5], ei))) {
+      rho = u[0];
+      ei = u[5];
+      const double p = gm1 * u[5];
+      cmax = fmax(cmax, sqrt(gamma * p / u[0]));
+    }
+  }
+};
 
 // FP32 form for the stage kernels: one approximate reciprocal of rho, |v| = |m| / rho.
 __device__ __forceinline__ void cell_speeds_f32(const float u[6], float gamma, float gm1,

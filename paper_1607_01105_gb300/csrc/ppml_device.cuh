@@ -21,9 +21,6 @@
 
 namespace ppml {
 
-template <typename T>
-struct Prec;
-
 // Constants of a sweep along one axis: tau, h, th = tau / h (and FP64: 1 / h).
 template <typename T>
 struct AxisStep;
@@ -31,34 +28,21 @@ struct AxisStep;
 template <>
 struct AxisStep<float> {
   float th;
-  __device__ __forceinline__ AxisStep(double, double, float th_) : th(th_) {}
+  __device__ __forceinline__ AxisStep(double, const f64::Divisor&, float th_) : th(th_) {}
 };
 template <>
 struct AxisStep<double> {
   double th, tau;
   f64::Divisor h;
-  __device__ __forceinline__ AxisStep(double tau_, double h_, double th_)
-      : th(th_), tau(tau_), h(f64::divisor(h_)) {}
+  __device__ __forceinline__ AxisStep(double tau_, const f64::Divisor& h_, double th_)
+      : th(th_), tau(tau_), h(h_) {}
 };
 
-template <>
-struct Prec<float> {
-  static __device__ __forceinline__ float half(float x) { return 0.5f * x; }
-  static __device__ __forceinline__ float two_thirds(float y) { return y * (2.0f / 3.0f); }
-  // Courant number of a signal speed s: s * tau / h with th = tau / h precomputed.
-  static __device__ __forceinline__ float courant(float s, const AxisStep<float>& k) {
-    return s * k.th;
-  }
-};
-
-template <>
-struct Prec<double> {
-  static __device__ __forceinline__ double half(double x) { return f64::half(x); }
-  static __device__ __forceinline__ double two_thirds(double y) { return f64::div3(f64::twice(y)); }
-  static __device__ __forceinline__ double courant(double s, const AxisStep<double>& k) {
-    return f64::divide(s * k.tau, k.h);
-  }
-};
+// Courant number s tau / h of a signal speed s (FP32: with th = tau / h precomputed).
+__device__ __forceinline__ float courant(float s, const AxisStep<float>& k) { return s * k.th; }
+__device__ __forceinline__ double courant(double s, const AxisStep<double>& k) {
+  return f64::divide(s * k.tau, k.h);
+}
 
 template <typename T>
 struct Parab {
@@ -67,8 +51,11 @@ struct Parab {
 
 __device__ __forceinline__ float tabs(float x) { return x < 0.0f ? -x : x; }
 __device__ __forceinline__ double tabs(double x) { return fabs(x); }
-__device__ __forceinline__ bool nonnegative(float x) { return x >= 0.0f; }
-__device__ __forceinline__ bool nonnegative(double x) { return f64::hi_word(x) >= 0; }
+// Sums and differences whose second operand is often zero in FP64 (f64::plus, minus).
+__device__ __forceinline__ float sub_term(float a, float b) { return a - b; }
+__device__ __forceinline__ double sub_term(double a, double b) { return f64::minus(a, b); }
+__device__ __forceinline__ float add_term(float a, float b) { return a + b; }
+__device__ __forceinline__ double add_term(double a, double b) { return f64::plus(a, b); }
 
 // Appendix, Step 1: limited slope delta_m q_i.  Branch-free: min(|dq|, 2 min(|r|, |l|))
 // equals min(|dq|, 2|r|, 2|l|) exactly (doubling is exact), and r l > 0 implies q is
@@ -79,10 +66,11 @@ __device__ __forceinline__ bool nonnegative(double x) { return f64::hi_word(x) >
 // (every scaling exact), which face_value expects: the halving is folded into its 1/6.
 template <typename T>
 __device__ __forceinline__ T limited_slope(T qm, T q0, T qp) {
-  const T r = qp - q0, l = q0 - qm;
   if constexpr (sizeof(T) == 8) {
-    return f64::slope(l, r, qp - qm);
+    const T r = f64::diff(qp, q0), l = f64::diff(q0, qm);
+    return f64::slope(l, r, qm, qp);
   } else {
+    const T r = qp - q0, l = q0 - qm;
     const T dq2 = qp - qm;
     const T m2 = fmin(fabs(dq2), T(4) * fmin(fabs(r), fabs(l)));
     return r * l > T(0) ? copysign(m2, dq2) : T(0);
@@ -95,7 +83,7 @@ __device__ __forceinline__ T limited_slope(T qm, T q0, T qp) {
 template <typename T>
 __device__ __forceinline__ T face_value(T q0, T q1, T d0, T d1) {
   if constexpr (sizeof(T) == 8)
-    return f64::half(q0 + q1) - f64::div6(d1 - d0);
+    return f64::face(q0, q1, d0, d1);
   else
     return T(0.5) * (q0 + q1) - (d1 - d0) * (1.0f / 12.0f);
 }
@@ -108,27 +96,9 @@ template <typename T>
 __device__ __forceinline__ Parab<T> parabola(T q0, T L, T R) {
   if constexpr (sizeof(T) == 8) {
     Parab<T> p;
-    if (f64::product_nonpositive(L - q0, q0 - R)) {  // flat: q0 - q0 = 0 for finite q0
-      p.L = q0;
-      p.R = q0;
-      p.D = T(0);
-      p.S = T(0);
-      if (f64::exponent(q0) == 0x7ffu) p.D = p.S = q0 - q0;
-      return p;
-    }
     p.L = L;
     p.R = R;
-    p.D = R - L;
-    p.S = T(6) * (q0 - f64::half(L + R));
-    const int o = f64::overshoot(p.D, p.S);
-    if (o != 0) {
-      if (o > 0)
-        p.L = T(3) * q0 - f64::twice(R);
-      else
-        p.R = T(3) * q0 - f64::twice(L);
-      p.D = p.R - p.L;
-      p.S = T(6) * (q0 - f64::half(p.L + p.R));
-    }
+    f64::parabola(q0, p.L, p.R, p.D, p.S);
     return p;
   }
   const bool flat = (L - q0) * (q0 - R) <= T(0);
@@ -148,15 +118,13 @@ __device__ __forceinline__ Parab<T> parabola(T q0, T L, T R) {
 }
 
 // Appendix, characteristic integrals: mean of the parabola over the right fraction y of
-// the cell (q_L(-lambda t), y = lambda t / h) ...
-template <typename T>
-__device__ __forceinline__ T avg_right(T R, T D, T S, T y) {
-  return R - Prec<T>::half(y) * (D - S * (T(1) - Prec<T>::two_thirds(y)));
+// the cell (q_L(-lambda t), y = lambda t / h; FP64: f64::average) ...
+__device__ __forceinline__ float avg_right(float R, float D, float S, float y) {
+  return R - 0.5f * y * (D - S * (1.0f - y * (2.0f / 3.0f)));
 }
 // ... and over its left fraction y (q_R(lambda t)).
-template <typename T>
-__device__ __forceinline__ T avg_left(T L, T D, T S, T y) {
-  return L + Prec<T>::half(y) * (D + S * (T(1) - Prec<T>::two_thirds(y)));
+__device__ __forceinline__ float avg_left(float L, float D, float S, float y) {
+  return L + 0.5f * y * (D + S * (1.0f - y * (2.0f / 3.0f)));
 }
 
 // Sec. 1.1/1.2: face constants of the acoustic Riemann problem from the adjacent cell
@@ -173,6 +141,10 @@ __device__ __forceinline__ RootWeights root_weights(double rho, double p) {
   w.b = p * w.s;
   return w;
 }
+// A cell between whose faces nothing varies: rho and p positive, mid-range.
+__device__ __forceinline__ bool plain_gas(double rho, double p) {
+  return f64::hi_word(rho) >= 0 && f64::hi_word(p) >= 0 && f64::moderate(rho) && f64::moderate(p);
+}
 __device__ __forceinline__ void face_constants(const RootWeights& l, const RootWeights& r,
                                                double gamma, double& lam, double& Z) {
   const double A = l.a + r.a;  // rho_L^{3/2} + rho_R^{3/2}
@@ -180,22 +152,6 @@ __device__ __forceinline__ void face_constants(const RootWeights& l, const RootW
   const double S = l.s + r.s;
   lam = sqrt(gamma * B / A);
   Z = sqrt(gamma * A * B / (S * S));
-}
-
-// Upwind state of eq. fluxonlagrangestage: the left cell's mean over its right fraction y
-// when the face velocity is >= 0, else the right cell's mean over its left fraction y.
-// The selected operands go through one evaluation (same operations as avg_right /
-// avg_left).
-template <typename T>
-__device__ __forceinline__ T upwind_state(bool from_left, T R_l, T D_l, T S_l, T L_r, T D_r,
-                                          T S_r, T y) {
-  const T D = from_left ? D_l : D_r;
-  const T S = from_left ? S_l : S_r;
-  const T t = S * (T(1) - Prec<T>::two_thirds(y));
-  // (an addition of the negated term is the subtraction)
-  const T u = D + (from_left ? -t : t);
-  const T w = Prec<T>::half(y) * u;
-  return (from_left ? R_l : L_r) + (from_left ? -w : w);
 }
 
 // eqs. lowriemannvelocity / lowriemannpressure from the four characteristic averages.
@@ -209,8 +165,12 @@ __device__ __forceinline__ void riemann_vp(double vls, double vrs, double pls, d
 // Returns 1 if the cell took the vacuum branch.
 __device__ __forceinline__ int energy_correction(double u[6], double rho_vac) {
   const double rho = u[0];
-  const double m2 = u[1] * u[1] + u[2] * u[2] + u[3] * u[3];
-  if (rho < rho_vac && m2 > 0.0) {
+  if (f64::is_zero(u[1]) && f64::is_zero(u[2]) && f64::is_zero(u[3]) && f64::moderate(rho)) {
+    if (f64::positive(u[4])) u[5] = u[4];  // at rest: rho E - 0 / (2 rho)
+    return 0;
+  }
+  const double m2 = f64::plus(f64::plus(u[1] * u[1], f64::times(u[2], u[2])), f64::times(u[3], u[3]));
+  if (f64::below(rho, rho_vac) && f64::positive(m2)) {
     const double de = u[4] - u[5];
     if (de < 0.0) {
       u[1] = u[2] = u[3] = 0.0;
@@ -225,8 +185,8 @@ __device__ __forceinline__ int energy_correction(double u[6], double rho_vac) {
     u[3] *= s;
     return 1;
   }
-  const double e = u[4] - m2 / (2.0 * rho);
-  if (e > 0.0) u[5] = e;
+  const double e = u[4] - m2 / f64::twice(rho);
+  if (f64::positive(e)) u[5] = e;
   return 0;
 }
 

@@ -24,24 +24,63 @@ __device__ __forceinline__ unsigned long long magnitude(double x) {
 __device__ __forceinline__ bool is_zero(double x) {
   return (((unsigned)hi_word(x) << 1) | (unsigned)lo_word(x)) == 0u;
 }
-// Plain operations that the compiler may not hoist out of the branch they stand in.
-__device__ __forceinline__ double plain_mul(double a, double b) {
-#ifdef __CUDA_ARCH__
-  double r;
-  asm volatile("mul.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-  return r;
-#else
-  return a * b;
-#endif
+__device__ __forceinline__ bool same_bits(double x, double y) {
+  return __double_as_longlong(x) == __double_as_longlong(y);
 }
-__device__ __forceinline__ double plain_div(double a, double b) {
+__device__ __forceinline__ bool finite(double x) { return exponent(x) != 0x7ffu; }
+__device__ __forceinline__ bool positive(double x) {  // x > 0
+  const long long b = __double_as_longlong(x);
+  return b > 0 && b <= 0x7ff0000000000000ll;
+}
+// x < b for a positive b
+__device__ __forceinline__ bool below(double x, double b) {
+  return __double_as_longlong(x) < __double_as_longlong(b) && magnitude(x) <= 0x7ff0000000000000ull;
+}
+// a normal number with room around it: products and quotients of a few such are normal
+__device__ __forceinline__ bool moderate(double x) { return exponent(x) - 623u <= 800u; }
+
+// Plain operations that the compiler does not hoist out of the branch they stand in (a
+// speculated FP64 instruction costs what the branch was to save).
 #ifdef __CUDA_ARCH__
-  double r;
-  asm volatile("div.rn.f64 %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));
-  return r;
+#define PPML_F64_PLAIN(name, op, expr)                                       \
+  __device__ __forceinline__ double name(double a, double b) {               \
+    double r;                                                                \
+    asm(op " %0, %1, %2;" : "=d"(r) : "d"(a), "d"(b));                       \
+    return r;                                                                \
+  }
 #else
-  return a / b;
+#define PPML_F64_PLAIN(name, op, expr) \
+  __device__ __forceinline__ double name(double a, double b) { return expr; }
 #endif
+PPML_F64_PLAIN(plain_add, "add.rn.f64", a + b)
+PPML_F64_PLAIN(plain_sub, "sub.rn.f64", a - b)
+PPML_F64_PLAIN(plain_mul, "mul.rn.f64", a * b)
+PPML_F64_PLAIN(plain_div, "div.rn.f64", a / b)
+#undef PPML_F64_PLAIN
+
+// Uniform and resting gas is common (ambient gas ahead of a blast, the transverse lines of
+// planar problems, planes of symmetry), and there most operands are equal or zero.  These
+// forms return the value of the plain operation without issuing it then (the sign of a zero
+// result may differ, which no later value depends on).
+__device__ __forceinline__ double diff(double a, double b) {  // a - b
+  if (same_bits(a, b) && finite(a)) return 0.0;
+  return plain_sub(a, b);
+}
+__device__ __forceinline__ double minus(double a, double b) {  // a - b, b often zero
+  if (is_zero(b)) return a;
+  return plain_sub(a, b);
+}
+__device__ __forceinline__ double plus(double a, double b) {  // a + b, b often zero
+  if (is_zero(b)) return a;
+  return plain_add(a, b);
+}
+__device__ __forceinline__ double times(double a, double b) {  // a b, b often zero
+  if (is_zero(b) && finite(a)) return 0.0;
+  return plain_mul(a, b);
+}
+__device__ __forceinline__ double over(double a, double b) {  // a / b, a often zero
+  if (is_zero(a) && moderate(b)) return a;
+  return plain_div(a, b);
 }
 
 // x 2^K by its exponent field where x and the result are normal.
@@ -117,17 +156,27 @@ __device__ __forceinline__ double divide(double x, const Divisor& d) {
   return plain_div(x, d.h);
 }
 
-// Appendix, Step 1 from the differences l = q0 - qm, r = qp - q0 and w = qp - qm: the
-// limited slope min(|w| / 2, 2 |l|, 2 |r|) with w's sign, 0 unless l r > 0 (then none of
+// Appendix, Step 1 from the differences l = q0 - qm, r = qp - q0: the limited slope
+// min(|w| / 2, 2 |l|, 2 |r|) with the sign of w = qp - qm, 0 unless l r > 0 (then none of
 // them is NaN and magnitudes order as integers).
-__device__ __forceinline__ double slope(double l, double r, double w) {
+__device__ __forceinline__ double slope(double l, double r, double qm, double qp) {
   if (!product_positive(r, l)) return 0.0;
+  const double w = plain_sub(qp, qm);
   const unsigned long long ml = magnitude(l), mr = magnitude(r);
   const double m2 = twice(__longlong_as_double((long long)(ml < mr ? ml : mr)));
   const double dq = half(w);
   const unsigned long long a = magnitude(dq), b = magnitude(m2), m = a < b ? a : b;
   return __longlong_as_double(
       (long long)(m | ((unsigned long long)__double_as_longlong(dq) & 0x8000000000000000ull)));
+}
+
+// Appendix, Step 1: the face value (q0 + q1) / 2 - (d1 - d0) / 6.
+__device__ __forceinline__ double face(double q0, double q1, double d0, double d1) {
+  if (is_zero(d0) && is_zero(d1)) {
+    if (same_bits(q0, q1) && exponent(q0) < 2046u) return q0;
+    return half(plain_add(q0, q1));
+  }
+  return plain_sub(half(plain_add(q0, q1)), div6(plain_sub(d1, d0)));
 }
 
 // Appendix, Steps 2-3: whether the unflattened parabola (D, S) overshoots: 1 if D S > D D
@@ -141,6 +190,48 @@ __device__ __forceinline__ int overshoot(double D, double S) {
     return (hi_word(D) ^ hi_word(S)) < 0 ? -1 : 1;
   const double ds = plain_mul(D, S), dd = plain_mul(D, D);
   return ds > dd ? 1 : (ds < -dd ? -1 : 0);
+}
+
+// Appendix, Steps 2-3: a cell's parabola (faces L, R, D = R - L and S = q^(6)) from its value
+// and its two unlimited faces, in place.
+__device__ __forceinline__ void parabola(double q0, double& L, double& R, double& D, double& S) {
+  if (product_nonpositive(diff(L, q0), diff(q0, R))) {  // flat
+    L = R = q0;
+    D = S = 0.0;  // q0 - q0 and 6 (q0 - q0)
+    if (!finite(q0)) D = S = plain_sub(q0, q0);
+    return;
+  }
+  D = plain_sub(R, L);
+  S = plain_mul(6.0, plain_sub(q0, half(plain_add(L, R))));
+  const int o = overshoot(D, S);
+  if (o != 0) {
+    if (o > 0)
+      L = plain_sub(plain_mul(3.0, q0), twice(R));
+    else
+      R = plain_sub(plain_mul(3.0, q0), twice(L));
+    D = plain_sub(R, L);
+    S = plain_mul(6.0, plain_sub(q0, half(plain_add(L, R))));
+  }
+}
+
+// What the characteristic averages read of a Courant number y: y / 2 and 1 - 2 y / 3.
+struct Weights {
+  double hy, w;
+};
+__device__ __forceinline__ Weights weights(double y) {
+  Weights k;
+  k.hy = half(y);
+  k.w = is_zero(y) ? 1.0 : plain_sub(1.0, div3(twice(y)));
+  return k;
+}
+// Average next to the right face of a cell (face value F = R, sgn -1: R - y/2 (D - S w)) or
+// to its left one (F = L, sgn +1: L + y/2 (D + S w)); adding a negated term is subtracting.
+__device__ __forceinline__ double average(bool right, double F, double D, double S,
+                                          const Weights& k) {
+  if (is_zero(D) && is_zero(S)) return F;
+  const double t = plain_mul(S, k.w);
+  const double u = plain_mul(k.hy, plain_add(D, right ? -t : t));
+  return plain_add(F, right ? -u : u);
 }
 
 }  // namespace f64

@@ -278,23 +278,21 @@ __device__ __forceinline__ void sweep_eulerian_dev(VF v, PF pr, RF r, float gamm
   hook(TB + 3);
 }
 
-// The same sweep with the parabolas in face values: FP64 (every expression in the checker's
-// order) and double-float FP32 states (whose low parts record the rounding of exactly these
-// expressions).
-template <typename T, bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
-__device__ __forceinline__ void sweep_eulerian(VF v, PF pr, RF r, T gamma,
-                                               const AxisStep<T>& ks, EF emit, HF hook) {
-  const T th = ks.th;
+// The same sweep with the parabolas in face values, for double-float states: their low parts
+// record the rounding of exactly these expressions.
+template <bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
+__device__ __forceinline__ void sweep_eulerian_faces(VF v, PF pr, RF r, float gamma, float th,
+                                                     EF emit, HF hook) {
+  using T = float;
   T va = v(-3), vb = v(-2), pa = pr(-3), pb = pr(-2);
   T dva = T(0), fva = T(0), dpa = T(0), fpa = T(0);
   T vR = T(0), vD = T(0), vS = T(0), pR = T(0), pD = T(0), pS = T(0);
   T Vp = T(0), Pp = T(0);
   T rprev = T(0), pprev = T(0);  // rho, p of cell p-3
-  T sprev = T(0);                // FP32: sqrt(rho) of cell p-3
-  RootWeights wprev = {0, 0, 0};  // FP64: the root weights of cell p-3
+  T sprev = T(0);                // sqrt(rho) of cell p-3
   // step p; WARM: one of the first four steps (p constant), which skip the parts whose
-  // inputs have not arrived; in FP32 the steady steps p = 3..18 run as a loop unrolled by
-  // two (a smaller body for the instruction cache)
+  // inputs have not arrived; the steady steps p = 3..18 run as a loop unrolled by two (a
+  // smaller body for the instruction cache)
   auto step = [&](int p, auto warm_c) {
     constexpr bool W = decltype(warm_c)::value;
     hook(p);
@@ -309,36 +307,20 @@ __device__ __forceinline__ void sweep_eulerian(VF v, PF pr, RF r, T gamma,
       const Parab<T> Pv = FLAT ? flat_parabola(va) : parabola(va, fva, fvn);  // cell p-2
       const Parab<T> Pq = FLAT ? flat_parabola(pa) : parabola(pa, fpa, fpn);
       const T rc = r(p - 2);
-      if constexpr (sizeof(T) == 4) {
-        const float sc = sqrt_approx(rc);
-        if (!W || p >= 2) {  // face between cells p-3 and p-2
-          float lam, Z, hrz;
-          face_constants_f32(rprev, rc, sprev, sc, pprev, pa, gamma, lam, Z, hrz);
-          const float y = lam * th;
-          const float vls = avg_right(vR, vD, vS, y), vrs = avg_left(Pv.L, Pv.D, Pv.S, y);
-          const float pls = avg_right(pR, pD, pS, y), prs = avg_left(Pq.L, Pq.D, Pq.S, y);
-          const float V = 0.5f * (vls + vrs) + (pls - prs) * hrz;
-          const float P = 0.5f * (pls + prs) + 0.5f * Z * (vls - vrs);
-          if (!W || p >= 3) emit(p - 3, th * (P - Pp), th * (P * V - Pp * Vp), th * (V - Vp));
-          Vp = V;
-          Pp = P;
-        }
-        sprev = sc;
-      } else {
-        const RootWeights wc = root_weights(rc, pa);
-        if (!W || p >= 2) {  // face between cells p-3 and p-2
-        T lam, Z;
-        face_constants(wprev, wc, gamma, lam, Z);
-        const T y = Prec<T>::courant(lam, ks);
-        T V, P;
-        riemann_vp(avg_right(vR, vD, vS, y), avg_left(Pv.L, Pv.D, Pv.S, y),
-                   avg_right(pR, pD, pS, y), avg_left(Pq.L, Pq.D, Pq.S, y), Z, V, P);
+      const float sc = sqrt_approx(rc);
+      if (!W || p >= 2) {  // face between cells p-3 and p-2
+        float lam, Z, hrz;
+        face_constants_f32(rprev, rc, sprev, sc, pprev, pa, gamma, lam, Z, hrz);
+        const float y = lam * th;
+        const float vls = avg_right(vR, vD, vS, y), vrs = avg_left(Pv.L, Pv.D, Pv.S, y);
+        const float pls = avg_right(pR, pD, pS, y), prs = avg_left(Pq.L, Pq.D, Pq.S, y);
+        const float V = 0.5f * (vls + vrs) + (pls - prs) * hrz;
+        const float P = 0.5f * (pls + prs) + 0.5f * Z * (vls - vrs);
         if (!W || p >= 3) emit(p - 3, th * (P - Pp), th * (P * V - Pp * Vp), th * (V - Vp));
         Vp = V;
         Pp = P;
-        }
-        wprev = wc;
       }
+      sprev = sc;
       vR = Pv.R;
       vD = Pv.D;
       vS = Pv.S;
@@ -359,12 +341,122 @@ __device__ __forceinline__ void sweep_eulerian(VF v, PF pr, RF r, T gamma,
   };
 #pragma unroll
   for (int p = -1; p < 3; p++) step(p, BoolC<true>());
-  if constexpr (sizeof(T) == 4) {
 #pragma unroll 2
-    for (int p = 3; p <= TB + 2; p++) step(p, BoolC<false>());
-  } else {  // FP64 is bound by its FP64 pipe, not by instruction fetch: fully unrolled
-#pragma unroll
-    for (int p = 3; p <= TB + 2; p++) step(p, BoolC<false>());
+  for (int p = 3; p <= TB + 2; p++) step(p, BoolC<false>());
+  hook(TB + 3);
+}
+
+// FP64 line pipeline, every expression in the checker's order: push(q) takes the next
+// position p; then q2 is the value and L, R, D, S the parabola of cell p - 2.  FLAT: the
+// first-order variant.
+template <bool FLAT>
+struct LineF64 {
+  double q2, q1, qn;  // values at p-2, p-1, p
+  double d;           // difference between p and p-1
+  double s;           // limited slope of p-1
+  double f;           // face between p-2 and p-1
+  double L, R, D, S;
+  __device__ __forceinline__ void start(double a, double b, double c) {
+    q2 = a;
+    q1 = b;
+    qn = c;
+    d = f64::diff(c, b);
+    s = FLAT ? 0.0 : f64::slope(f64::diff(b, a), d, a, c);
+    f = L = R = D = S = 0.0;
+  }
+  __device__ __forceinline__ void push(double q) {
+    if constexpr (FLAT) {
+      L = R = q1;
+    } else {
+      const double dn = f64::diff(q, qn);
+      const double sn = f64::slope(d, dn, q1, q);
+      const double fn = f64::face(q1, qn, s, sn);
+      L = f;
+      R = fn;
+      f64::parabola(q1, L, R, D, S);
+      d = dn;
+      s = sn;
+      f = fn;
+    }
+    q2 = q1;
+    q1 = qn;
+    qn = q;
+  }
+};
+
+// The Eulerian sweep in FP64, every expression in the checker's order.  Where neither side of
+// a face varies, the face solution is the cells' own (v, p) and the impedance and the wave
+// speed, three square roots and two divisions, are not needed.  Rolled: the FP64 pipe binds
+// it and the branches make a long body.
+template <bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
+__device__ __forceinline__ void sweep_eulerian_f64(VF v, PF pr, RF r, double gamma,
+                                                   const AxisStep<double>& ks, EF emit, HF hook) {
+  LineF64<FLAT> lv, lp;
+  hook(-1);
+  lv.start(v(-3), v(-2), v(-1));
+  lp.start(pr(-3), pr(-2), pr(-1));
+  hook(0);
+  lv.push(v(0));
+  lp.push(pr(0));
+  hook(1);
+  lv.push(v(1));
+  lp.push(pr(1));
+  // the face's left cell: right faces and parabolas, rho, p, root weights (when formed)
+  double vR = lv.R, vD = lv.D, vS = lv.S, pR = lp.R, pD = lp.D, pS = lp.S;
+  double rl = r(-1), pl = lp.q2;
+  RootWeights wl = {0, 0, 0};
+  bool have_wl = false, have_pv = false;
+  double Vp = 0.0, Pp = 0.0, PVp = 0.0;
+#pragma unroll 1
+  for (int p = 2; p <= TB + 2; p++) {
+    hook(p);
+    lv.push(v(p));
+    lp.push(pr(p));
+    const double rc = r(p - 2);
+    const bool uniform =
+        f64::is_zero(vD) && f64::is_zero(vS) && f64::is_zero(lv.D) && f64::is_zero(lv.S) &&
+        f64::is_zero(pD) && f64::is_zero(pS) && f64::is_zero(lp.D) && f64::is_zero(lp.S) &&
+        f64::same_bits(vR, lv.L) && f64::same_bits(pR, lp.L) && f64::exponent(vR) < 2046u &&
+        plain_gas(rl, pl) && plain_gas(rc, lp.q2);
+    double V, P;
+    if (uniform) {
+      V = vR;
+      P = pR;
+      have_wl = false;
+    } else {
+      if (!have_wl) wl = root_weights(rl, pl);
+      const RootWeights wc = root_weights(rc, lp.q2);
+      double lam, Z;
+      face_constants(wl, wc, gamma, lam, Z);
+      wl = wc;
+      have_wl = true;
+      const f64::Weights k = f64::weights(courant(lam, ks));
+      riemann_vp(f64::average(true, vR, vD, vS, k), f64::average(false, lv.L, lv.D, lv.S, k),
+                 f64::average(true, pR, pD, pS, k), f64::average(false, lp.L, lp.D, lp.S, k), Z, V,
+                 P);
+    }
+    if (p >= 3) {
+      if (f64::same_bits(P, Pp) && f64::same_bits(V, Vp) && f64::finite(P) && f64::finite(V)) {
+        emit(p - 3, 0.0, 0.0, 0.0);
+      } else {
+        if (!have_pv) PVp = f64::times(Pp, Vp);
+        const double PV = f64::times(P, V);
+        emit(p - 3, f64::times(ks.th, f64::diff(P, Pp)), f64::times(ks.th, f64::diff(PV, PVp)),
+             f64::times(ks.th, f64::diff(V, Vp)));
+        PVp = PV;
+        have_pv = true;
+      }
+    }
+    Vp = V;
+    Pp = P;
+    vR = lv.R;
+    vD = lv.D;
+    vS = lv.S;
+    pR = lp.R;
+    pD = lp.D;
+    pS = lp.S;
+    rl = rc;
+    pl = lp.q2;
   }
   hook(TB + 3);
 }
@@ -565,9 +657,9 @@ __device__ __forceinline__ float half_flux_f32(float w, float R_l, float D_l, fl
   return w * fmaf(c1, D, fmaf(c2, S, base));
 }
 
-// One line of the Lagrangian stage for any axis with the parabola in face values: FP64 (every
-// expression in the checker's order) and double-float FP32 states (whose low parts record
-// the rounding of exactly these expressions).  Field values: core[p cs] for p in
+// One line of the Lagrangian stage for any axis with the parabola in face values, for
+// double-float states: their low parts record the rounding of exactly these expressions.
+// Field values: core[p cs] for p in
 // [0, 16), halo[h SLP] for the positions -3..-1 (h = 0..2) and 16..18 (h = 3..5).  Face
 // velocities vh[c TN], c = 0..16 (face between cells c-1 and c).  MODE 0: acc = div;
 // 1: acc += div; 2: dst[c gs] = core - (acc + div) for c < nvalid (acc only if have_acc).
@@ -577,12 +669,13 @@ __device__ __forceinline__ float half_flux_f32(float w, float R_l, float D_l, fl
 // non-NULL the field is a double-float value whose low part srclo[c gs] is read and the
 // update is added in double-float (dst the high part, dstlo the low part).  CS: the core
 // stride of the sweep axis as a compile-time constant (immediate shared-memory offsets).
-template <typename T, int MODE, bool FLAT, bool DF, int CS>
-__device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* vh,
-                                         const AxisStep<T>& ks, T* acc, bool have_acc,
-                                         T* __restrict__ dst, long long gs, int nvalid,
-                                         const T* __restrict__ srclo = nullptr,
-                                         T* __restrict__ dstlo = nullptr) {
+template <int MODE, bool FLAT, bool DF, int CS>
+__device__ __forceinline__ void lag_line_faces(const float* core, const float* halo,
+                                               const float* vh, float* acc, bool have_acc,
+                                               float* __restrict__ dst, long long gs, int nvalid,
+                                               const float* __restrict__ srclo = nullptr,
+                                               float* __restrict__ dstlo = nullptr) {
+  using T = float;
   constexpr int cs = CS;
   T qa = halo[0], qb = halo[SLP];  // q(p-2), q(p-1)
   T qn = halo[2 * SLP];            // p = -1
@@ -608,14 +701,7 @@ __device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* 
   dn = limited_slope(qa, qb, qn);
   fn = face_value(qa, qb, da, dn);
   P = FLAT ? flat_parabola(qa) : parabola(qa, fa, fn);  // cell 0
-  T Fp;
-  if constexpr (sizeof(T) == 4) {
-    Fp = half_flux_f32(vh[0], PR, PD, PS, P.L, P.D, P.S);
-  } else {
-    const T v = vh[0];
-    const T y = Prec<T>::courant(tabs(v), ks);
-    Fp = v * upwind_state(nonnegative(v), PR, PD, PS, P.L, P.D, P.S, y);
-  }
+  T Fp = half_flux_f32(vh[0], PR, PD, PS, P.L, P.D, P.S);
   PR = P.R;
   PD = P.D;
   PS = P.S;
@@ -629,22 +715,15 @@ __device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* 
     const T dnn = limited_slope(qa, qb, qnew);
     const T fnn = face_value(qa, qb, da, dnn);
     const Parab<T> Pn = FLAT ? flat_parabola(qa) : parabola(qa, fa, fnn);  // cell c+1
-    T F, d;  // through the face between cells c and c+1
-    if constexpr (sizeof(T) == 4) {
-      F = half_flux_f32(vv, PR, PD, PS, Pn.L, Pn.D, Pn.S);
-      d = F - Fp;  // half of th (F+ - F-)
-    } else {
-      const T yy = Prec<T>::courant(tabs(vv), ks);
-      F = vv * upwind_state(nonnegative(vv), PR, PD, PS, Pn.L, Pn.D, Pn.S, yy);
-      d = ks.th * (F - Fp);
-    }
+    // through the face between cells c and c+1; d: half of th (F+ - F-)
+    const T F = half_flux_f32(vv, PR, PD, PS, Pn.L, Pn.D, Pn.S), d = F - Fp;
     const int o = c * cs;
     if (MODE == 0) {
       acc[o] = d;
     } else if (MODE == 1) {
       acc[o] = acc[o] + d;
     } else if (c < nvalid) {
-      const T upd = divergence_sum<DF>(have_acc ? acc[o] + d : d);
+      const T upd = 2.0f * (have_acc ? acc[o] + d : d);
       if constexpr (DF) {
         if (dstlo) {
           float hi, lo;
@@ -687,8 +766,47 @@ __device__ __forceinline__ void lag_line(const T* core, const T* halo, const T* 
   step(q_in, v_in, TB - 1);
 }
 
+// One line of the FP64 Lagrangian stage (arguments as lag_line_faces'; th = tau / h, fw the
+// faces' weights of the characteristic averages), every expression in the checker's order.
+template <int MODE, bool FLAT, int CS>
+__device__ __forceinline__ void lag_line_f64(const double* core, const double* halo,
+                                             const double* vh, const f64::Weights* fw, double th,
+                                             double* acc, bool have_acc, double* __restrict__ dst,
+                                             long long gs, int nvalid) {
+  constexpr int cs = CS;
+  LineF64<FLAT> ln;
+  ln.start(halo[0], halo[SLP], halo[2 * SLP]);
+  ln.push(core[0]);
+  ln.push(core[cs]);
+  double Rl = ln.R, Dl = ln.D, Sl = ln.S, ql = ln.q2, Fp = 0.0;  // the face's left cell
+#pragma unroll 1
+  for (int c = -1; c < TB; c++) {  // position c + 3 arrives, cell c is finished
+    const double v = vh[(c + 1) * TN];
+    const f64::Weights k = fw[c + 1];
+    ln.push(c + 3 < TB ? core[(c + 3) * cs] : halo[(c - TB + 6) * SLP]);
+    const bool left = f64::hi_word(v) >= 0;  // upwind side (eq. fluxonlagrangestage)
+    const double st = f64::average(left, left ? Rl : ln.L, left ? Dl : ln.D, left ? Sl : ln.S, k);
+    const double F = f64::is_zero(v) && f64::finite(st) ? 0.0 : f64::plain_mul(v, st);
+    if (c >= 0) {
+      const double d = f64::times(th, f64::diff(F, Fp));
+      const int o = c * cs;
+      if (MODE == 0)
+        acc[o] = d;
+      else if (MODE == 1)
+        acc[o] = f64::plus(acc[o], d);
+      else if (c < nvalid)
+        dst[gs * c] = f64::minus(ql, have_acc ? f64::plus(acc[o], d) : d);
+    }
+    ql = ln.q2;
+    Fp = F;
+    Rl = ln.R;
+    Dl = ln.D;
+    Sl = ln.S;
+  }
+}
+
 // Face velocities v^ of line (a, b) along axis ax (faces 0..16, face c between cells c-1
-// and c) from the dense 18^3 boxes of v_ax and rho: the 9-point template in the plane normal
+// and c) from the dense 18^3 boxes of v_ax and sqrt(rho): the 9-point template in the plane normal
 // to ax (eq. veltemplate; the cell's own v in the one-point variant) and the sqrt(rho)
 // weighted average of the two adjacent cells (eq. modspaceaveragevelocitylagrange).
 template <typename T>
@@ -705,21 +823,37 @@ __device__ __forceinline__ void line_face_velocities(const T* vb, const T* rb, i
 #pragma unroll
   for (int p = -1; p <= TB; p++) {
     const int o = base + p * s_ax;
-    const T corners = vb[o + s_b + s_c] + vb[o + s_b - s_c] + vb[o - s_b + s_c] + vb[o - s_b - s_c];
-    const T edges = vb[o + s_b] + vb[o - s_b] + vb[o + s_c] + vb[o - s_c];
-    T vt, sq;
-    if constexpr (sizeof(T) == 4)
-      vt = one_point ? vb[o] : corners / T(16) + edges / T(8) + vb[o] / T(4);
-    else
-      vt = one_point ? vb[o] : f64::scale<-4>(corners) + f64::scale<-3>(edges) + f64::scale<-2>(vb[o]);
+    const T sq = rb[o];
     if constexpr (sizeof(T) == 4) {
-      sq = sqrt_approx(rb[o]);
+      const T corners = vb[o + s_b + s_c] + vb[o + s_b - s_c] + vb[o - s_b + s_c] + vb[o - s_b - s_c];
+      const T edges = vb[o + s_b] + vb[o - s_b] + vb[o + s_c] + vb[o - s_c];
+      const T vt = one_point ? vb[o] : corners / T(16) + edges / T(8) + vb[o] / T(4);
       if (p >= 0) out[p] = (vt * sq + vt_prev * sq_prev) * rcp_approx(sq + sq_prev);
+      vt_prev = vt;
     } else {
-      sq = sqrt(rb[o]);
-      if (p >= 0) out[p] = (vt * sq + vt_prev * sq_prev) / (sq + sq_prev);
+      const T v0 = vb[o];
+      T vt = v0;
+      if (!one_point) {
+        const T c0 = vb[o + s_b + s_c], c1 = vb[o + s_b - s_c], c2 = vb[o - s_b + s_c],
+                c3 = vb[o - s_b - s_c], e0 = vb[o + s_b], e1 = vb[o - s_b], e2 = vb[o + s_c],
+                e3 = vb[o - s_c];
+        if (!(f64::is_zero(v0) && f64::is_zero(c0) && f64::is_zero(c1) && f64::is_zero(c2) &&
+              f64::is_zero(c3) && f64::is_zero(e0) && f64::is_zero(e1) && f64::is_zero(e2) &&
+              f64::is_zero(e3)))  // gas at rest: 0
+          vt = f64::plain_add(
+              f64::plain_add(
+                  f64::scale<-4>(f64::plain_add(f64::plain_add(f64::plain_add(c0, c1), c2), c3)),
+                  f64::scale<-3>(f64::plain_add(f64::plain_add(f64::plain_add(e0, e1), e2), e3))),
+              f64::scale<-2>(v0));
+      }
+      const T prod = f64::times(sq, vt);  // vt_prev carries the last cell's
+      const T num = f64::plus(prod, vt_prev);
+      if (p >= 0)
+        out[p] = f64::is_zero(num) && f64::moderate(sq) && f64::moderate(sq_prev)
+                     ? num
+                     : f64::plain_div(num, f64::plain_add(sq, sq_prev));
+      vt_prev = prod;
     }
-    vt_prev = vt;
     sq_prev = sq;
   }
 }
@@ -755,6 +889,8 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
   }
   __shared__ TileMaps maps;
   if (!fast_async) build_maps(maps, g, tg);  // ordered by the barrier below
+  __shared__ f64::Divisor hdiv[3];  // FP64: the cell sizes as divisors
+  if (sizeof(T) == 8 && tid < 3) hdiv[tid] = f64::divisor(A.h[tid]);  // (barrier below)
   double stc[4];
   cta_step_constants(A.dt_dev, A.dt_host, A.h, stc);
   const double tau = stc[0];
@@ -792,10 +928,12 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
 #pragma unroll
       for (int ax = 0; ax < 3; ax++)
         if (act[ax]) vbox(ax)[it] = vbox(ax)[it] * ir;
+      rbox[it] = sqrt_approx(r);  // the Roe weight
     } else {
 #pragma unroll
       for (int ax = 0; ax < 3; ax++)
-        if (act[ax]) vbox(ax)[it] = vbox(ax)[it] / r;
+        if (act[ax]) vbox(ax)[it] = f64::over(vbox(ax)[it], r);
+      rbox[it] = sqrt(r);
     }
   }
   __syncthreads();
@@ -803,17 +941,27 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
   if (act[1]) line_face_velocities(vbox(1), rbox, 1, a, b, one_point, vh1);
   if (act[2]) line_face_velocities(vbox(2), rbox, 2, a, b, one_point, vh2);
   __syncthreads();  // the y and z boxes are read; the face-velocity space is free
+  // FP64: the faces' weights of the characteristic averages, formed once for the six fields
+  // (thread-private, in local memory: they stay in the L1 and L2 caches)
+  f64::Weights fweights[sizeof(T) == 8 ? 3 : 1][sizeof(T) == 8 ? TB + 1 : 1];
+  auto store_vh = [&](int ax, const T* v) {
+#pragma unroll
+    for (int q = 0; q <= TB; q++) {
+      S.vh[ax][q][tid] = vh_stored<DF>(v[q], th[ax]);
+      if constexpr (sizeof(T) == 8) {
+        const AxisStep<T> ks(tau, hdiv[ax], th[ax]);
+        fweights[ax][q] = f64::is_zero(v[q]) ? f64::Weights{0.0, 1.0}
+                                             : f64::weights(courant(tabs(v[q]), ks));
+      }
+    }
+  };
   if (act[0]) {
     T vh0[TB + 1];
     line_face_velocities(vbox(0), rbox, 0, a, b, one_point, vh0);
-#pragma unroll
-    for (int q = 0; q <= TB; q++) S.vh[0][q][tid] = vh_stored<DF>(vh0[q], th[0]);
+    store_vh(0, vh0);
   }
-#pragma unroll
-  for (int q = 0; q <= TB; q++) {
-    if (act[1]) S.vh[1][q][tid] = vh_stored<DF>(vh1[q], th[1]);
-    if (act[2]) S.vh[2][q][tid] = vh_stored<DF>(vh2[q], th[2]);
-  }
+  if (act[1]) store_vh(1, vh1);
+  if (act[2]) store_vh(2, vh2);
   __syncthreads();
 
   // ---- per field: stage, sweep x, y (into acc), z (finish into the output)
@@ -929,21 +1077,21 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
       T* dstlo = DF && f < 5 ? A.outlo[f] + zline0 : nullptr;
       const T* core = &S.fld[cb];
       T* acc = &S.acc[cb];
-      const AxisStep<T> ks(tau, A.h[ax], th[ax]);
       // one instantiation per (axis, mode): x is always the first sweep (mode 0), y the
       // first or the second, z the last (MODE 2: finish into the output)
       auto sweep = [&](auto mode_c, auto flat_c, auto cs_c) {
         constexpr int M = decltype(mode_c)::value;
         constexpr bool FL = decltype(flat_c)::value;
         constexpr int C = decltype(cs_c)::value;
-        if constexpr (sizeof(T) == 4 && !DF)
-          lag_line_dev<M, FL, C>(core, halo, vhl, acc, mode == 1, A.out[f] + zline0, g.nxy,
+        T* const dst = A.out[f] + zline0;  // (written by the z sweep)
+        if constexpr (sizeof(T) == 8)
+          lag_line_f64<M, FL, C>(core, halo, vhl, fweights[ax], th[ax], acc, mode == 1, dst, g.nxy,
                                  nvalid_z);
-        else if constexpr (M == 2)
-          lag_line<T, 2, FL, DF, C>(core, halo, vhl, ks, acc, mode == 1,
-                                    A.out[f] + zline0, g.nxy, nvalid_z, srclo, dstlo);
+        else if constexpr (!DF)
+          lag_line_dev<M, FL, C>(core, halo, vhl, acc, mode == 1, dst, g.nxy, nvalid_z);
         else
-          lag_line<T, M, FL, false, C>(core, halo, vhl, ks, acc, false, nullptr, 0, 0);
+          lag_line_faces<M, FL, DF && M == 2, C>(core, halo, vhl, acc, mode == 1, dst, g.nxy,
+                                                 nvalid_z, srclo, dstlo);
       };
       auto sweep_ax = [&](auto flat_c) {
         if (ax == 2)
@@ -976,7 +1124,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
             continue;
           }
         }
-        A.out[f][idx] = S.fld[o] - upd;
+        A.out[f][idx] = sub_term(S.fld[o], upd);
       }
     }
   }
@@ -987,6 +1135,8 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
   T vmax = T(0), cmax = T(0);
   unsigned long long nvac = 0, nbad = 0;
   const float rho_vac_up = __double2float_ru(A.rho_vac);
+  RoughSpeeds rough[sizeof(T) == 8 ? TB : 1];  // FP64: bounds of the cells' speeds
+  float vlow = 0.0f, clow = 0.0f;
   // groups of FB cells: all loads of a group are issued before its first store.  The
   // correction changes m only in vacuum cells, so only those store m back.
   constexpr int FB = 4;
@@ -1053,7 +1203,33 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
       if constexpr (sizeof(T) == 4)
         cell_speeds_f32(u[q], gamma, gm1, vmax, cmax, nbad);
       else
-        cell_speeds<T>(u[q], gamma, gm1, vmax, cmax, nbad);
+        rough_speeds(u[q], (float)A.gamma * (float)(A.gamma - 1.0), rough[c0 + q], vlow, clow, nbad);
+    }
+  }
+  if constexpr (sizeof(T) == 8) {
+    // exact speeds of the cells that can hold the tile's maxima (rough_speeds)
+    __shared__ float low[TN / 32][2];
+    vlow = warp_max(vlow);
+    clow = warp_max(clow);
+    if ((tid & 31) == 0) {
+      low[tid >> 5][0] = vlow;
+      low[tid >> 5][1] = clow;
+    }
+    __syncthreads();
+    for (int q = 0; q < TN / 32; q++) {
+      vlow = fmaxf(vlow, low[q][0]);
+      clow = fmaxf(clow, low[q][1]);
+    }
+    ExactSpeeds ex;
+#pragma unroll 1
+    for (int c = 0; c < nvalid_z; c++) {
+      const bool nv = rough[c].v > 0.0f && rough[c].v >= vlow, nc = rough[c].c >= clow;
+      if (nv || nc) {
+        T u[6];
+#pragma unroll
+        for (int f = 0; f < 6; f++) u[f] = A.out[f][zline0 + g.nxy * c];
+        ex.add(u, gamma, gm1, nv, nc, vmax, cmax);
+      }
     }
   }
   if constexpr (sizeof(T) == 4) {
@@ -1080,7 +1256,8 @@ __device__ __forceinline__ float eps_update(float ei, float gm1, float dv) {
   return fmaf(-(gm1 * ei), dv, ei);
 }
 __device__ __forceinline__ double eps_update(double ei, double gm1, double dv) {
-  return ei - gm1 * ei * dv;
+  if (f64::is_zero(dv) && f64::finite(ei)) return ei;
+  return f64::plain_sub(ei, f64::plain_mul(f64::plain_mul(gm1, ei), dv));
 }
 
 template <typename T>
@@ -1110,6 +1287,8 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
   const bool tin = INF && tile_inflow(g, tg);  // some copy of this tile reads an inflow ghost
   __shared__ TileMaps maps;
   build_maps(maps, g, tg);  // ordered by the barrier below
+  __shared__ f64::Divisor hdiv[3];  // FP64: the cell sizes as divisors
+  if (sizeof(T) == 8 && tid < 3) hdiv[tid] = f64::divisor(A.h[tid]);  // (barrier below)
   double stc[4];
   cta_step_constants(A.dt_dev, A.dt_host, A.h, stc);
   const double tau = stc[0];
@@ -1242,8 +1421,8 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
     T* const om = A.out[1 + ax] + gbase;
     auto emit = [&](int c, T dm, T dpv, T dv) {
       const int ai = acc0 + c * acs;
-      S.apv[ai] = first ? dpv : S.apv[ai] + dpv;
-      S.av[ai] = first ? dv : S.av[ai] + dv;
+      S.apv[ai] = first ? dpv : add_term(S.apv[ai], dpv);
+      S.av[ai] = first ? dv : add_term(S.av[ai], dv);
       if (c < nvalid) {
         const long long off = gst * c;
         if constexpr (DF) {
@@ -1252,7 +1431,7 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
           om[off] = hi;
           A.outlo[1 + ax][gbase + off] = lo;
         } else {
-          om[off] = S.m[slab_at(c, a, b)] - dm;
+          om[off] = sub_term(S.m[slab_at(c, a, b)], dm);
         }
       }
     };
@@ -1261,16 +1440,28 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
       if constexpr (sizeof(T) == 4)
         return S.m[o] * rcp_approx(S.r[o]);
       else
-        return S.m[o] / S.r[o];
+        return f64::over(S.m[o], S.r[o]);
     };
-    auto pq = [&](int p) { return gm1 * S.p[slab_at(p, a, b)]; };
+    T last_e = T(0), last_p = T(0);  // FP64: a position's pressure, kept for an equal next one
+    auto pq = [&](int p) {
+      const T e = S.p[slab_at(p, a, b)];
+      if constexpr (sizeof(T) == 4) {
+        return gm1 * e;
+      } else {
+        if (!f64::same_bits(e, last_e)) last_p = f64::plain_mul(gm1, e);
+        last_e = e;
+        return last_p;
+      }
+    };
     auto rq = [&](int p) { return S.r[slab_at(p, a, b)]; };
     auto sweep = [&](auto flat_c) {
       constexpr bool FL = decltype(flat_c)::value;
-      if constexpr (sizeof(T) == 4 && !DF)
-        sweep_eulerian_dev<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
+      if constexpr (sizeof(T) == 8)
+        sweep_eulerian_f64<FL>(vq, pq, rq, gamma, AxisStep<T>(tau, hdiv[ax], th[ax]), emit, hook);
+      else if constexpr (DF)
+        sweep_eulerian_faces<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
       else
-        sweep_eulerian<T, FL>(vq, pq, rq, gamma, AxisStep<T>(tau, A.h[ax], th[ax]), emit, hook);
+        sweep_eulerian_dev<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
     };
     if (A.flags & PPML_FIRST_ORDER)
       sweep(BoolC<true>());
@@ -1314,7 +1505,7 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
           A.out[4][idx] = hi;
           A.outlo[4][idx] = lo;
         } else {
-          A.out[4][idx] = en[q] - S.apv[ai];
+          A.out[4][idx] = sub_term(en[q], S.apv[ai]);
         }
         A.out[5][idx] = eps_update(ei[q], gm1, S.av[ai]);
       }
@@ -1380,7 +1571,7 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
       const long long idx = zline0e + g.nxy * c;
       const T dpvs = first ? T(0) : S.apv[acc_at(a, b, c)];
       const T dvs = first ? T(0) : S.av[acc_at(a, b, c)];
-      T en = e0[q] - dpvs;
+      T en = sub_term(e0[q], dpvs);
       T den = dpvs;  // DF: the whole FP32 decrement of rho E, added to the pair once
       if (A.phi) {
 #pragma unroll

@@ -58,9 +58,44 @@ int main() {
     CHECK("divide", divide(x, divisor(std::fabs(y))), x / std::fabs(y));
     CHECK("positive", product_positive(x, y), x * y > 0.0);
     CHECK("nonpositive", product_nonpositive(x, y), x * y <= 0.0);
-    const double l = y - x, r = z - y, w = z - x, dq = 0.5 * w;
+    const double l = y - x, r = z - y, dq = 0.5 * (z - x);
     const double m = std::fmin(std::fabs(dq), 2.0 * std::fmin(std::fabs(r), std::fabs(l)));
-    CHECK("slope", slope(l, r, w), r * l > 0.0 ? std::copysign(m, dq) : 0.0);
+    CHECK("slope", slope(l, r, x, z), r * l > 0.0 ? std::copysign(m, dq) : 0.0);
+    // equal up to the sign of a zero
+    CHECK("diff", diff(x, y) + 0.0, (x - y) + 0.0);
+    CHECK("plus", plus(x, n % 9 ? y : 0.0) + 0.0, (x + (n % 9 ? y : 0.0)) + 0.0);
+    CHECK("minus", minus(x, n % 9 ? y : 0.0) + 0.0, (x - (n % 9 ? y : 0.0)) + 0.0);
+    CHECK("times", times(x, n % 9 ? y : 0.0) + 0.0, (x * (n % 9 ? y : 0.0)) + 0.0);
+    CHECK("over", over(n % 9 ? x : 0.0, y) + 0.0, ((n % 9 ? x : 0.0) / y) + 0.0);
+    CHECK("positive value", positive(x), x > 0.0);
+    CHECK("below", below(x, 1.5), x < 1.5);
+    const double d0 = n % 2 ? 0.0 : r, d1 = n % 2 ? 0.0 : l, yy = n % 6 == 3 ? x : y;
+    CHECK("face", face(x, yy, d0, d1) + 0.0, (0.5 * (x + yy) - (d1 - d0) / 6.0) + 0.0);
+    {
+      double L = 0.5 * (x + y) - l / 6.0, R = 0.5 * (y + z) - r / 6.0, D, S;  // cell value y
+      const double L0 = L, R0 = R;
+      parabola(y, L, R, D, S);
+      double Ln = L0, Rn = R0;
+      if ((L0 - y) * (y - R0) <= 0.0) {
+        Ln = Rn = y;
+      } else {
+        const double d = R0 - L0, q6 = 6.0 * (y - 0.5 * (L0 + R0));
+        if (d * q6 > d * d) Ln = 3.0 * y - 2.0 * R0;
+        else if (d * q6 < -(d * d)) Rn = 3.0 * y - 2.0 * L0;
+      }
+      const double Dn = Rn - Ln, Sn = 6.0 * (y - 0.5 * (Ln + Rn));
+      const bool huge = std::fabs(y) > 8e307;  // y + y overflows
+      if (!huge) {
+        CHECK("parabola L", L, Ln);
+        CHECK("parabola R", R, Rn);
+        CHECK("parabola D", D + 0.0, Dn + 0.0);
+        CHECK("parabola S", S + 0.0, Sn + 0.0);
+        const double c = 0.3;
+        const Weights k = weights(c);
+        CHECK("right average", average(true, R, D, S, k) + 0.0, (Rn - 0.5 * c * (Dn - Sn * (1.0 - 2.0 * c / 3.0))) + 0.0);
+        CHECK("left average", average(false, L, D, S, k) + 0.0, (Ln + 0.5 * c * (Dn + Sn * (1.0 - 2.0 * c / 3.0))) + 0.0);
+      }
+    }
     CHECK("overshoot", overshoot(x, y), x * y > x * x ? 1 : (x * y < -(x * x) ? -1 : 0));
   }
   printf("%d wrong\n", bad);
