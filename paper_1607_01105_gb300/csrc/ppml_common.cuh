@@ -19,7 +19,18 @@ struct Partial {
 struct DevScalars {
   double t, dt, vmax, cmax, sums[6];
   long long steps, n_vac, n_bad;
-  unsigned flags, pad;
+  unsigned flags;
+  unsigned arrived;  // CTAs of the running Lagrangian launch that have stored their partial
+};
+
+// What the partials of a state become: mode 0, the device scalars S of a state; 1, the same
+// after a step; 2, the maxima, sums and counts in red[PPML_REDUCE_LEN] (a slab's share, for
+// an all-reduce over the slabs).
+struct Finalize {
+  DevScalars* S;
+  double* red;
+  double cfl, hmin, vol, t_end;
+  int mode;
 };
 
 template <typename T>
@@ -42,6 +53,12 @@ struct MarchArgs {
   int tile_order;         // launch order of the tiles (TileOrder)
   int any_reflect;       // a reflecting wall exists (its sign flips need register copies)
   int flags;             // PPML_FIRST_ORDER, PPML_VHAT_1PT
+  Finalize fin;          // of the Lagrangian stage's partials
+  // FP32 with three active axes: the tiles' face velocities (ppml_tile_f32.cuh), room for
+  // face_tiles tiles; a launch covers the blocks from tile_first on, and the array's first
+  // tile is face_first (set by the launcher where the tiles take several launches)
+  T* face;
+  int face_tiles, tile_first, face_first;
   const T* inflow;       // [face][field]: the prescribed ghost states of inflow faces
   int any_inflow;        // an inflow face exists (selects the kernels that read them)
 };
@@ -69,6 +86,31 @@ __device__ __forceinline__ void cta_step_constants(const double* dt_dev, double 
 
 // ------------------------------------------------------------------ block reduction
 
+// The warps' shares folded in a fixed order into out[slot], a thread of the first warp per
+// quantity (one thread folding all eight took 13 k cycles of 64 dependent FP64 operations at
+// the end of every tile).  The stores are ordered before the warp's return.
+template <int NW>
+__device__ __forceinline__ void fold_warps(const double (*sh)[8], const unsigned long long (*shc)[2],
+                                           Partial* out, int slot) {
+  const int q = threadIdx.x;
+  if (q < 6) {
+    double v = 0.0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) v += sh[w][q];
+    out[slot].s[q] = v;
+  } else if (q < 8) {  // nonnegative: ordered as integers
+    unsigned long long m = 0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) m = max(m, (unsigned long long)__double_as_longlong(sh[w][q]));
+    (q == 6 ? out[slot].vmax : out[slot].cmax) = __longlong_as_double((long long)m);
+  } else if (q < 10) {
+    unsigned long long n = 0;
+#pragma unroll
+    for (int w = 0; w < NW; w++) n += shc[w][q - 8];
+    (q == 8 ? out[slot].nvac : out[slot].nbad) = n;
+  }
+}
+
 // Writes the CTA's partial to out[slot].
 template <int NTHREADS>
 __device__ __forceinline__ void block_reduce_store(double s[6], double vmax, double cmax,
@@ -95,22 +137,7 @@ __device__ __forceinline__ void block_reduce_store(double s[6], double vmax, dou
     shc[w][1] = nbad;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Partial p;
-    for (int f = 0; f < 6; f++) p.s[f] = 0.0;
-    p.vmax = 0.0;
-    p.cmax = 0.0;
-    p.nvac = 0;
-    p.nbad = 0;
-    for (int q = 0; q < NTHREADS / 32; q++) {
-      for (int f = 0; f < 6; f++) p.s[f] += sh[q][f];
-      p.vmax = fmax(p.vmax, sh[q][6]);
-      p.cmax = fmax(p.cmax, sh[q][7]);
-      p.nvac += shc[q][0];
-      p.nbad += shc[q][1];
-    }
-    out[slot] = p;
-  }
+  fold_warps<NTHREADS / 32>(sh, shc, out, slot);
 }
 
 // (hi, lo) += (bh, bl) in double-float (TwoSum of the high parts, then renormalised).
@@ -159,22 +186,128 @@ __device__ __forceinline__ void block_reduce_store_f32(const float hi_in[6], con
     shc[w][1] = nbad;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    Partial p;
-    for (int f = 0; f < 6; f++) p.s[f] = 0.0;
-    p.vmax = 0.0;
-    p.cmax = 0.0;
-    p.nvac = 0;
-    p.nbad = 0;
-    for (int q = 0; q < NTHREADS / 32; q++) {
-      for (int f = 0; f < 6; f++) p.s[f] += sh[q][f];
-      p.vmax = fmax(p.vmax, sh[q][6]);
-      p.cmax = fmax(p.cmax, sh[q][7]);
-      p.nvac += shc[q][0];
-      p.nbad += shc[q][1];
-    }
-    out[slot] = p;
+  fold_warps<NTHREADS / 32>(sh, shc, out, slot);
+}
+
+// The device scalars from the maxima, sums (times the cell volume) and counts of a state:
+// advance: the state ends a step of tau (t += tau, clipped to t_end; steps + 1).  Then the
+// next CFL step (Sec. 1.1) clipped to the remaining time, and the flags.
+__device__ __forceinline__ void apply_scalars(DevScalars* S, double vmax, double cmax,
+                                              const double* sums, double nvac, double nbad,
+                                              int advance, double tau, double cfl, double hmin,
+                                              double t_end) {
+  double tn = S->t;
+  if (advance) {
+    tn = S->t + tau;
+    if (t_end > 0.0 && tn > t_end) tn = t_end;
+    S->t = tn;
+    S->steps += 1;
+    S->n_vac = (long long)nvac;
   }
+  S->vmax = vmax;
+  S->cmax = cmax;
+  for (int f = 0; f < 6; f++) S->sums[f] = sums[f];
+  S->n_bad = (long long)nbad;
+  double dt = cfl * hmin / (vmax + cmax);
+  if (t_end > 0.0 && dt > t_end - tn) dt = t_end - tn;
+  if (!(dt > 0.0)) {
+    dt = 0.0;
+    S->flags |= 2u;  // PPML_FLAG_DT_ZERO
+  }
+  S->dt = dt;
+  if (nbad > 0.0) S->flags |= 1u;  // PPML_FLAG_NONPHYSICAL
+}
+
+// Reduce nblk partials with one CTA of at least eight warps in an order that depends on nblk
+// alone: a warp per sum (lane l takes partials l, l + 32, ..), one for the two maxima, one
+// for the counts, so no FP64 lane idles (a tree over threads that each hold all eight values
+// spent 12 us on 256 partials).  The partials may come from other CTAs of the same launch
+// (read past L1).  tau: the step taken (mode 1).
+__device__ __forceinline__ void finalize_cta(const Partial* P, int nblk, const Finalize& F,
+                                             double tau) {
+  __shared__ double res[8];
+  __shared__ unsigned long long cnt[2];
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  constexpr int IN = 16;  // loads in flight per lane (the tail of the launch is their latency)
+  if (w < 6) {
+    double s = 0.0;
+    for (int b0 = lane; b0 < nblk; b0 += 32 * IN) {
+      double x[IN];
+#pragma unroll
+      for (int q = 0; q < IN; q++)
+        x[q] = b0 + 32 * q < nblk ? __ldcg(&P[b0 + 32 * q].s[w]) : 0.0;
+#pragma unroll
+      for (int q = 0; q < IN; q++) s = f64::plus(s, x[q]);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
+    if (lane == 0) res[w] = s * F.vol;
+  } else if (w == 6) {  // maxima: nonnegative, so they order as integers
+    unsigned long long v = 0, c = 0;
+#pragma unroll 8
+    for (int b = lane; b < nblk; b += 32) {
+      v = max(v, (unsigned long long)__double_as_longlong(__ldcg(&P[b].vmax)));
+      c = max(c, (unsigned long long)__double_as_longlong(__ldcg(&P[b].cmax)));
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      v = max(v, __shfl_down_sync(0xffffffffu, v, o));
+      c = max(c, __shfl_down_sync(0xffffffffu, c, o));
+    }
+    if (lane == 0) {
+      res[6] = __longlong_as_double((long long)v);
+      res[7] = __longlong_as_double((long long)c);
+    }
+  } else if (w == 7) {
+    unsigned long long nv = 0, nb = 0;
+#pragma unroll 8
+    for (int b = lane; b < nblk; b += 32) {
+      nv += __ldcg(&P[b].nvac);
+      nb += __ldcg(&P[b].nbad);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      nv += __shfl_down_sync(0xffffffffu, nv, o);
+      nb += __shfl_down_sync(0xffffffffu, nb, o);
+    }
+    if (lane == 0) {
+      cnt[0] = nv;
+      cnt[1] = nb;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x != 0) return;
+  if (F.mode == 2) {
+    F.red[0] = res[6];
+    F.red[1] = res[7];
+    for (int f = 0; f < 6; f++) F.red[2 + f] = res[f];
+    F.red[8] = (double)cnt[0];
+    F.red[9] = (double)cnt[1];
+    return;
+  }
+  apply_scalars(F.S, res[6], res[7], res, (double)cnt[0], (double)cnt[1], F.mode == 1, tau, F.cfl,
+                F.hmin, F.t_end);
+}
+
+// End of a CTA of the Lagrangian stage whose first warp has stored its partial: the CTA that
+// arrives last of nblk reduces them all.  The counter is zero between launches.
+__device__ __forceinline__ void finalize_last(const Partial* P, int nblk, const Finalize& F,
+                                              double tau) {
+  __shared__ bool last;
+  if (threadIdx.x < 32) {  // the partial's stores (fold_warps), visible before the arrival
+    __threadfence();
+    __syncwarp();
+  }
+  if (threadIdx.x == 0) {
+    const unsigned n = atomicAdd(&F.S->arrived, 1u);
+    last = n == (unsigned)nblk - 1u;
+    if (last) {
+      F.S->arrived = 0u;
+      __threadfence();
+    }
+  }
+  __syncthreads();
+  if (last) finalize_cta(P, nblk, F, tau);
 }
 
 // Running per-thread sums of the six output fields: compensated float for the FP32

@@ -7,8 +7,8 @@
 //   lagrangian_tile    Sec. 1.3/1.4: 9-point velocity template, Roe-weighted face velocity,
 //                      upwind parabola fluxes of all six fields, unsplit update, energy
 //                      correction; per-CTA partial maxima and sums of U^{n+1}
-//   finalize_kernel    deterministic reduction of the partials -> device-resident CFL step
-//                      (Sec. 1.1), FP64 sums, time and flags
+//                      the last CTA to finish reduces them in a fixed order -> device-resident
+//                      CFL step (Sec. 1.1), FP64 sums, time and flags (finalize_cta)
 // No host synchronization inside a step, so consecutive steps can be captured in a CUDA
 // graph (the step size stays on the device).
 #include <cuda_runtime.h>
@@ -29,87 +29,13 @@ using namespace ppml;
 
 namespace {
 
-constexpr int kFinThreads = 512;
+constexpr int kFinThreads = 256;
 
-// The device scalars from the maxima, sums (times the cell volume) and counts of a state:
-// advance: the state ends a step of tau (t += tau, clipped to t_end; steps + 1).  Then the
-// next CFL step (Sec. 1.1) clipped to the remaining time, and the flags.
-__device__ void apply_scalars(DevScalars* S, double vmax, double cmax, const double* sums,
-                              double nvac, double nbad, int advance, double tau, double cfl,
-                              double hmin, double t_end) {
-  double tn = S->t;
-  if (advance) {
-    tn = S->t + tau;
-    if (t_end > 0.0 && tn > t_end) tn = t_end;
-    S->t = tn;
-    S->steps += 1;
-    S->n_vac = (long long)nvac;
-  }
-  S->vmax = vmax;
-  S->cmax = cmax;
-  for (int f = 0; f < 6; f++) S->sums[f] = sums[f];
-  S->n_bad = (long long)nbad;
-  double dt = cfl * hmin / (vmax + cmax);
-  if (t_end > 0.0 && dt > t_end - tn) dt = t_end - tn;
-  if (!(dt > 0.0)) {
-    dt = 0.0;
-    S->flags |= PPML_FLAG_DT_ZERO;
-  }
-  S->dt = dt;
-  if (nbad > 0.0) S->flags |= PPML_FLAG_NONPHYSICAL;
-}
-
-// Reduce nblk partials in a fixed order (independent of scheduling).  mode 0: diagnostics
-// of a state into the device scalars; 1: after a step; 2: only write the maxima, sums and
-// counts to red[PPML_REDUCE_LEN] (a slab's share, for an all-reduce across slabs).
-__global__ void __launch_bounds__(kFinThreads)
-    finalize_kernel(const Partial* __restrict__ P, int nblk, DevScalars* S, double cfl,
-                    double hmin, double vol, double t_end, int mode, const double* dt_dev,
-                    double dt_host, double* red) {
-  __shared__ double sh[kFinThreads][8];
-  __shared__ unsigned long long shc[kFinThreads][2];
-  const int t = threadIdx.x;
-  double tau = 0.0;
-  if (t == 0 && mode == 1) tau = dt_dev ? *dt_dev : dt_host;
-  double s[6] = {0, 0, 0, 0, 0, 0}, vmax = 0.0, cmax = 0.0;
-  unsigned long long nvac = 0, nbad = 0;
-  for (int b = t; b < nblk; b += kFinThreads) {
-    for (int f = 0; f < 6; f++) s[f] += P[b].s[f];
-    vmax = fmax(vmax, P[b].vmax);
-    cmax = fmax(cmax, P[b].cmax);
-    nvac += P[b].nvac;
-    nbad += P[b].nbad;
-  }
-  for (int f = 0; f < 6; f++) sh[t][f] = s[f];
-  sh[t][6] = vmax;
-  sh[t][7] = cmax;
-  shc[t][0] = nvac;
-  shc[t][1] = nbad;
-  __syncthreads();
-  for (int w = kFinThreads / 2; w > 0; w >>= 1) {
-    if (t < w) {
-      for (int f = 0; f < 6; f++) sh[t][f] += sh[t + w][f];
-      sh[t][6] = fmax(sh[t][6], sh[t + w][6]);
-      sh[t][7] = fmax(sh[t][7], sh[t + w][7]);
-      shc[t][0] += shc[t + w][0];
-      shc[t][1] += shc[t + w][1];
-    }
-    __syncthreads();
-  }
-  if (t == 0) {
-    double sums[6];
-    for (int f = 0; f < 6; f++) sums[f] = sh[0][f] * vol;
-    if (mode == 2) {
-      red[0] = sh[0][6];
-      red[1] = sh[0][7];
-      for (int f = 0; f < 6; f++) red[2 + f] = sums[f];
-      red[8] = (double)shc[0][0];
-      red[9] = (double)shc[0][1];
-      return;
-    }
-    apply_scalars(S, sh[0][6], sh[0][7], sums, (double)shc[0][0], (double)shc[0][1], mode == 1,
-                  tau, cfl, hmin, t_end);
-  }
+// Reduce nblk partials (finalize_cta): mode 0, the diagnostics of a state into the device
+// scalars; 2, only into red (a slab's share).  The stage kernels reduce their own partials.
+__global__ void __launch_bounds__(kFinThreads) finalize_kernel(const Partial* P, int nblk,
+                                                               Finalize f) {
+  finalize_cta(P, nblk, f, 0.0);
 }
 
 // The device scalars from an all-reduced red[PPML_REDUCE_LEN] (slab decomposition).
@@ -123,15 +49,10 @@ __global__ void apply_reduced_kernel(const double* __restrict__ red, DevScalars*
 
 }  // namespace
 
-namespace ppml {
-int launch_finalize(const Partial* P, int nblk, DevScalars* S, double cfl, double hmin, double vol,
-                    double t_end, int mode, const double* dt_dev, double dt_host, cudaStream_t st,
-                    double* red) {
-  finalize_kernel<<<1, kFinThreads, 0, st>>>(P, nblk, S, cfl, hmin, vol, t_end, mode, dt_dev,
-                                             dt_host, red);
+static int launch_finalize(const Partial* P, int nblk, const Finalize& f, cudaStream_t st) {
+  finalize_kernel<<<1, kFinThreads, 0, st>>>(P, nblk, f);
   return ppml_check_launch("finalize_kernel");
 }
-}  // namespace ppml
 
 struct ppml_grid {
   ppml_grid_desc d;
@@ -140,6 +61,7 @@ struct ppml_grid {
   void* ustar[6];  // [0] unused (rho is not changed by the Eulerian stage)
   void* ustar_lo[5];  // FP32: low parts of U*'s m and rho E ([0] unused)
   Partial* partials;
+  float* face;   // FP32 with three active axes: face velocities of every tile
   void* inflow;  // 36 values of the state's type: the inflow faces' ghost states [face][field]
   int nblk_march, nblk_diag, npartials;  // tiles (partials of a step), diagnostics blocks
   int tiles_x, tiles_y, tiles_z;
@@ -260,6 +182,18 @@ static int check_state_type(const ppml_grid_desc* d, const ppml_state* u, const 
 
 namespace {
 
+Finalize make_finalize(const ppml_grid* g, int mode, double* red) {
+  Finalize f;
+  f.S = g->dev;
+  f.red = red;
+  f.cfl = g->d.cfl;
+  f.hmin = g->hmin;
+  f.vol = g->vol;
+  f.t_end = g->d.t_end;
+  f.mode = mode;
+  return f;
+}
+
 template <typename T>
 MarchArgs<T> make_args(const ppml_grid* g, double dt_host, const double* dt_dev) {
   MarchArgs<T> A;
@@ -279,6 +213,9 @@ MarchArgs<T> make_args(const ppml_grid* g, double dt_host, const double* dt_dev)
   for (int q = 0; q < 6; q++) A.any_reflect |= g->d.bc[q] == PPML_BC_REFLECT;
   A.flags = g->d.flags;
   A.inflow = (const T*)g->inflow;
+  A.fin = make_finalize(g, 0, nullptr);
+  A.face = (T*)g->face;
+  A.face_tiles = g->nblk_march;
   A.any_inflow = 0;
   for (int q = 0; q < 6; q++) A.any_inflow |= g->d.bc[q] == PPML_BC_INFLOW;
   return A;
@@ -291,8 +228,7 @@ int run_diag(ppml_grid* g, const ppml_state* u, cudaStream_t st) {
   for (int f = 0; f < 5; f++) A.ulo[f] = (const T*)u->lo[f];
   int rc = launch_diag<T>(A, g->nblk_diag, st);
   if (rc) return rc;
-  return launch_finalize(g->partials, g->nblk_diag, g->dev, g->d.cfl, g->hmin, g->vol,
-                         g->d.t_end, 0, nullptr, 0.0, st, nullptr);
+  return launch_finalize(g->partials, g->nblk_diag, make_finalize(g, 0, nullptr), st);
 }
 
 template <typename T>
@@ -356,12 +292,12 @@ int run_step(ppml_grid* g, const ppml_state* uin, ppml_state* uout, const T* phi
     for (int f = 1; f < 5; f++) L.ulo[f] = (const T*)g->ustar_lo[f];
     for (int f = 0; f < 5; f++) L.outlo[f] = (T*)uout->lo[f];
   }
+  L.fin = make_finalize(g, 1, nullptr);
   rc = launch_lagrangian<T>(L, g->nblk_launch, st);
-  if (rc) return rc;
-  if (ev) cudaEventRecord(ev[2], st);
-  rc = launch_finalize(g->partials, g->nblk_march, g->dev, g->d.cfl, g->hmin, g->vol,
-                       g->d.t_end, 1, dt_dev, dt_host, st, nullptr);
-  if (ev) cudaEventRecord(ev[3], st);
+  if (ev) {  // (the Lagrangian kernel's last CTA finalizes: no launch of its own)
+    cudaEventRecord(ev[2], st);
+    cudaEventRecord(ev[3], st);
+  }
   return rc;
 }
 
@@ -421,6 +357,12 @@ extern "C" int ppml_init_grid(const ppml_grid_desc* d, const ppml_state* u0, voi
       return ppml_fail(PPML_E_NOMEM, "cudaMalloc of U* low parts (%zu bytes) failed", fbytes);
     }
   }
+  if (d->dtype == PPML_F32 && d->nx > 1 && d->ny > 1 && d->nz > 1 &&
+      cudaMalloc(&g->face, kFaceBytes * (size_t)g->nblk_march) != cudaSuccess) {
+    ppml_free_grid(g);
+    return ppml_fail(PPML_E_NOMEM, "cudaMalloc of the face velocities (%zu bytes) failed",
+                     kFaceBytes * (size_t)g->nblk_march);
+  }
   if (cudaMalloc(&g->partials, sizeof(Partial) * (size_t)g->npartials) != cudaSuccess ||
       cudaMalloc(&g->dev, sizeof(DevScalars)) != cudaSuccess ||
       cudaMalloc(&g->inflow, 36 * g->elt) != cudaSuccess) {
@@ -469,6 +411,7 @@ extern "C" int ppml_free_grid(ppml_grid* g) {
   for (int f = 0; f < 5; f++)
     if (g->ustar_lo[f]) cudaFree(g->ustar_lo[f]);
   if (g->partials) cudaFree(g->partials);
+  if (g->face) cudaFree(g->face);
   if (g->inflow) cudaFree(g->inflow);
   if (g->dev) cudaFree(g->dev);
   if (g->ev) {
@@ -873,8 +816,7 @@ extern "C" int ppml_local_reduce(ppml_grid* g, const ppml_state* u, double* red,
   rc = g->d.dtype == PPML_F64 ? launch_diag<double>(A64, g->nblk_diag, st)
                               : launch_diag<float>(A32, g->nblk_diag, st);
   if (rc) return rc;
-  return launch_finalize(g->partials, g->nblk_diag, g->dev, g->d.cfl, g->hmin, g->vol,
-                         g->d.t_end, 2, nullptr, 0.0, st, red);
+  return launch_finalize(g->partials, g->nblk_diag, make_finalize(g, 2, red), st);
 }
 
 extern "C" int ppml_lagrangian_stage(ppml_grid* g, const ppml_state* u_star, ppml_state* u_out,
@@ -896,6 +838,7 @@ extern "C" int ppml_lagrangian_stage(ppml_grid* g, const ppml_state* u_star, ppm
       L.u[f] = (const double*)u_star->f[f];
       L.out[f] = (double*)u_out->f[f];
     }
+    L.fin = make_finalize(g, 2, red);
     rc = launch_lagrangian<double>(L, g->nblk_launch, st);
   } else {
     MarchArgs<float> L = make_args<float>(g, dt, dt_dev);
@@ -908,11 +851,10 @@ extern "C" int ppml_lagrangian_stage(ppml_grid* g, const ppml_state* u_star, ppm
         L.ulo[f] = (const float*)u_star->lo[f];
         L.outlo[f] = (float*)u_out->lo[f];
       }
+    L.fin = make_finalize(g, 2, red);
     rc = launch_lagrangian<float>(L, g->nblk_launch, st);
   }
-  if (rc) return rc;
-  return launch_finalize(g->partials, g->nblk_march, g->dev, g->d.cfl, g->hmin, g->vol,
-                         g->d.t_end, 2, dt_dev, dt, st, red);
+  return rc;
 }
 
 extern "C" int ppml_apply_reduced(ppml_grid* g, const double* red, int advance, double dt,

@@ -1,3 +1,41 @@
 // FP32 instantiation of the stencil kernels (FMA contraction on).
+#include "ppml_tile_f32.cuh"
+
+namespace ppml {
+namespace {
+
+cudaError_t prepare_sweeps(float) {
+  cudaError_t e = cudaFuncSetAttribute(lagrangian_sweep_f32<false>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       (int)sizeof(SweepSmem));
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(lagrangian_sweep_f32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(SweepSmem));
+  return e;
+}
+
+// Lagrangian stage of plain float states with three active axes: face velocities, then the
+// sweeps; in several launches where the face array does not hold every tile (the
+// allocation-free step).  False: not such a state, nothing launched.
+bool launch_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
+  if (!A.face || A.g.n[0] == 1 || A.g.n[1] == 1 || A.g.n[2] == 1) return false;
+  MarchArgs<float> B = A;
+  const int per = A.face_tiles >= nblk || A.tile_order != 0 ? nblk : A.face_tiles;
+  for (int first = 0; first < nblk; first += per) {
+    const int n = nblk - first < per ? nblk - first : per;
+    B.tile_first = first;
+    B.face_first = first;
+    face_velocity_f32<<<n, FV_THREADS, 0, st>>>(B);
+    if (A.flags & PPML_FIRST_ORDER)
+      lagrangian_sweep_f32<true><<<n, TN, sizeof(SweepSmem), st>>>(B);
+    else
+      lagrangian_sweep_f32<false><<<n, TN, sizeof(SweepSmem), st>>>(B);
+  }
+  return true;
+}
+
+}  // namespace
+}  // namespace ppml
+
 #define PPML_REAL float
 #include "ppml_kern_impl.cuh"

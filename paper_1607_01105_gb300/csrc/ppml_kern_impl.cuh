@@ -6,6 +6,10 @@
 
 namespace ppml {
 
+// Kernels of their own for plain float states (ppml_kern_f32.cu); FP64 has none.
+inline bool launch_sweeps(const MarchArgs<double>&, int, cudaStream_t) { return false; }
+inline cudaError_t prepare_sweeps(double) { return cudaSuccess; }
+
 namespace {
 // CTAs per SM the march kernels are compiled for (register budget per thread)
 template <typename T>
@@ -45,6 +49,7 @@ cudaError_t set_stage_smem() {
 template <>
 int prepare_kernels<PPML_REAL>() {
   cudaError_t e = set_stage_smem<false>();
+  if (e == cudaSuccess) e = prepare_sweeps(PPML_REAL(0));
   if (e == cudaSuccess && kHasDF) e = set_stage_smem<kHasDF>();
   if (e != cudaSuccess) return ppml_fail(PPML_E_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   return PPML_OK;
@@ -73,6 +78,7 @@ int launch_lagrangian<PPML_REAL>(const MarchArgs<PPML_REAL>& A, int nblk, cudaSt
   constexpr int MB = MinBlocks<PPML_REAL>::value;
   constexpr size_t SM = sizeof(LagTileSmem<PPML_REAL>);
   const bool df = kHasDF && A.outlo[0];
+  if (!df && launch_sweeps(A, nblk, st)) return ppml_check_launch("lagrangian_sweep_f32");
   if (A.any_inflow) {
     if (df)
       lagrangian_tile<PPML_REAL, MB, kHasDF, true><<<nblk, TN, SM, st>>>(A);

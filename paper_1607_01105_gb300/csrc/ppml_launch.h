@@ -10,6 +10,9 @@
 
 namespace ppml {
 
+// Bytes of a tile's face velocities (FP32 Lagrangian stage; FACE_TILE in ppml_tile_f32.cuh).
+constexpr size_t kFaceBytes = 3 * (TB + 1) * TN * sizeof(float);
+
 template <typename T>
 int prepare_kernels();  // opt-in shared-memory sizes; call outside stream capture
 template <typename T>
@@ -35,11 +38,6 @@ template <typename T>
 int launch_batch_cluster(T* rho, T* m, T* en, T* ei, BatchLo<T> lo, InstDev* inst,
                          const int2* items, double gamma, double cfl, int max_steps, int nlmax,
                          int nmax, int nitems, size_t smem, int threads, cudaStream_t st);
-
-// Deterministic reduction of per-CTA partials into the step scalars (ppml_grid.cu).
-int launch_finalize(const Partial* P, int nblk, DevScalars* S, double cfl, double hmin, double vol,
-                    double t_end, int mode, const double* dt_dev, double dt_host, cudaStream_t st,
-                    double* red);
 
 // explicit specializations live in ppml_kern_f32.cu / ppml_kern_f64.cu
 #define PPML_DECLARE_LAUNCHERS(R)                                                            \

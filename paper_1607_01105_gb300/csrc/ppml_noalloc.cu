@@ -32,7 +32,11 @@ constexpr size_t kUstarBytes = 5ull * PPML_NOALLOC_MAX_CELLS * sizeof(double);
 // partial tiles per axis.
 constexpr size_t kMaxPartials = PPML_NOALLOC_MAX_CELLS / 16 + 4096;
 constexpr size_t kPartialBytes = kMaxPartials * sizeof(Partial);
-constexpr size_t kScratchBytes = kUstarBytes + kPartialBytes + sizeof(DevScalars);
+// FP32: the face velocities of a launch's tiles (64^3 cells are 64 tiles; thin grids of more
+// tiles take several launches).
+constexpr int kFaceTiles = 64;
+constexpr size_t kFaceOffset = (kUstarBytes + kPartialBytes + sizeof(DevScalars) + 255) / 256 * 256;
+constexpr size_t kScratchBytes = kFaceOffset + kFaceTiles * kFaceBytes;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -90,6 +94,10 @@ int step_noalloc(const ppml_grid_desc* d, const ppml_state* u_in, ppml_state* u_
   const int tiles_z = (d->nz + TB - 1) / TB;
   A.tiles_z = tiles_z;
   A.tile_order = 0;
+  if (sizeof(T) == 4) {
+    A.face = (T*)(scratch + kFaceOffset);
+    A.face_tiles = kFaceTiles;
+  }
   const int nblk = A.tiles_x * A.tiles_y * tiles_z;
   if ((size_t)nblk > kMaxPartials)
     return ppml_fail(PPML_E_INVAL, "grid needs %d tiles (the fixed buffer holds %zu)", nblk,
@@ -114,10 +122,14 @@ int step_noalloc(const ppml_grid_desc* d, const ppml_state* u_in, ppml_state* u_
     A.u[f] = f == 0 ? (const T*)u_in->f[0] : ustar + (size_t)(f - 1) * ncell;
     A.out[f] = (T*)u_out->f[f];
   }
+  A.fin.S = S;
+  A.fin.red = nullptr;
+  A.fin.cfl = d->cfl;
+  A.fin.hmin = hmin;
+  A.fin.vol = d->h[0] * d->h[1] * d->h[2];
+  A.fin.t_end = 0.0;
+  A.fin.mode = 1;
   rc = launch_lagrangian<T>(A, nblk, st);
-  if (rc) return rc;
-  rc = launch_finalize(partials, nblk, S, d->cfl, hmin, d->h[0] * d->h[1] * d->h[2], 0.0, 1,
-                       nullptr, dt, st, nullptr);
   if (rc) return rc;
   if (out9) {
     DevScalars hs;

@@ -69,9 +69,9 @@ __host__ __device__ __forceinline__ long long order_blocks(int order, int tx, in
   return (long long)((tx + sx - 1) / sx * sx) * ((ty + sy - 1) / sy * sy) * ((tz + sz - 1) / sz * sz);
 }
 
-__device__ __forceinline__ TileGeom tile_geom(const GridGeom& g, const int tiles[3], int order) {
+__device__ __forceinline__ TileGeom tile_geom(const GridGeom& g, const int tiles[3], int order,
+                                              int b) {  // b: the block's place in the order
   TileGeom t;
-  int b = blockIdx.x;
   int tc[3];
   if (order == 1) {
     tc[2] = b % tiles[2];
@@ -869,7 +869,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
   const bool act[3] = {g.n[0] > 1, g.n[1] > 1, g.n[2] > 1};
   const int tid = threadIdx.x, a = tid % TB, b = tid / TB;
   const int tiles[3] = {A.tiles_x, A.tiles_y, A.tiles_z};
-  const TileGeom tg = tile_geom(g, tiles, A.tile_order);
+  const TileGeom tg = tile_geom(g, tiles, A.tile_order, blockIdx.x);
   if (!tg.valid) return;  // a padding block of a blocked order (uniform over the CTA)
   const bool async_ok = !A.any_reflect;  // reflecting walls flip signs: copy through registers
   const bool fast_async = async_ok && tg.fast;
@@ -1246,6 +1246,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
     sums.get(sd);
     block_reduce_store<TN>(sd, (double)vmax, (double)cmax, nvac, nbad, A.partials, tg.id);
   }
+  finalize_last(A.partials, tiles[0] * tiles[1] * tiles[2], A.fin, tau);
 }
 
 // ====================================================================== Eulerian stage
@@ -1281,7 +1282,7 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
   const bool act[3] = {g.n[0] > 1, g.n[1] > 1, g.n[2] > 1};
   const int tid = threadIdx.x, a = tid % TB, b = tid / TB;
   const int tiles[3] = {A.tiles_x, A.tiles_y, A.tiles_z};
-  const TileGeom tg = tile_geom(g, tiles, A.tile_order);
+  const TileGeom tg = tile_geom(g, tiles, A.tile_order, blockIdx.x);
   if (!tg.valid) return;  // a padding block of a blocked order (uniform over the CTA)
   const bool async_ok = !A.any_reflect;  // reflecting walls flip signs: copy through registers
   const bool tin = INF && tile_inflow(g, tg);  // some copy of this tile reads an inflow ghost

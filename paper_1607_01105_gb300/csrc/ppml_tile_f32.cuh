@@ -1,0 +1,515 @@
+// FP32 Lagrangian stage of grids with three active axes (plain float states), in two kernels:
+//
+//   face_velocity_f32   eqs. veltemplate and modspaceaveragevelocitylagrange: the Courant
+//                       velocities w = v^ tau/h of every face of every 16^3 tile, into a
+//                       scratch array in the order the sweeps read it
+//   lagrangian_sweep_f32  eqs. fluxonlagrangestage, genlagrange, the energy consistency of
+//                       Sec. 1.4, the CFL maxima and sums
+//
+// Why two: one kernel that holds the velocity boxes, the face velocities of its lines, a
+// field with its halos and an accumulator fills 105 KB of shared memory, two CTAs of eight
+// warps per SM, and waits for staging with nothing beside it (issue slots 52 % busy).  With
+// the velocities coming from L2 in coalesced rows the sweeps need 70 KB for two fields at a
+// time, so three CTAs share an SM, the weights of a face are formed once for two fields, and
+// no staging phase is left: the z sweep reads its columns from global memory itself, a few
+// positions ahead, and leaves them in shared memory for the x and y sweeps.
+#pragma once
+#include "ppml_tile.cuh"
+
+namespace ppml {
+
+// Face velocities of a tile: [axis][face 0..16][line], line a + 16 b of that axis.
+constexpr int FACE_AXIS = (TB + 1) * TN;
+constexpr int FACE_TILE = 3 * FACE_AXIS;
+
+// Tile maps with 32-bit offsets (a grid has fewer than 2^31 cells), as TileMaps.
+struct TileMaps32 {
+  int off[3][TW];
+  int flip[3][TW];    // the axis is mirrored there
+  int inflow[3][TW];  // the inflow face whose ghost region the coordinate lies in, or -1
+};
+__device__ __forceinline__ void build_maps32(TileMaps32& M, const GridGeom& g, const TileGeom& t) {
+  for (int e = threadIdx.x; e < 3 * TW; e += blockDim.x) {
+    const int ax = e / TW, c = e % TW - TH;
+    const int o = ax == 0 ? t.i0 : (ax == 1 ? t.j0 : t.k0);
+    const int gc = o + c, n = g.n[ax];
+    int fl;
+    const int m = bc_map(gc, n, g.bc[2 * ax], g.bc[2 * ax + 1], fl);
+    M.off[ax][c + TH] = m * (ax == 0 ? 1 : (ax == 1 ? g.n[0] : (int)g.nxy));
+    M.flip[ax][c + TH] = fl;
+    M.inflow[ax][c + TH] = gc < 0 && g.bc[2 * ax] == PPML_BC_INFLOW
+                               ? 2 * ax
+                               : (gc >= n && g.bc[2 * ax + 1] == PPML_BC_INFLOW ? 2 * ax + 1 : -1);
+  }
+}
+
+// ------------------------------------------------------------------------ face velocities
+
+constexpr int FV_W = TB + 2;                 // columns -1..16 along x and y
+constexpr int FV_THREADS = 352;              // 18 x 18 columns in eleven warps
+constexpr int FV_PLANE = FV_W * FV_W;
+
+// A CTA marches the planes k = -1..16 of its tile; thread (i, j) owns a column.  The 9-point
+// template is (1 2 1)/4 x (1 2 1)/4: across z and y (v_x) or z and x (v_y) the in-plane part
+// is summed from shared memory and the z part from the thread's last planes; v_z takes nine
+// values of its plane.  Products with the Roe weight sqrt(rho) of plane k - 1 then meet their
+// neighbours through shared memory, remapped so that each face row is stored contiguously.
+// One plane of loads is in flight ahead.
+template <bool SPECIAL>  // mirrored or prescribed ghosts may occur
+__device__ __forceinline__ void face_velocity_tile(const MarchArgs<float>& A, const TileGeom& tg,
+                                                   const TileMaps32& M, const float th[3],
+                                                   float (*vel)[3][FV_PLANE], float (*prod)[FV_PLANE],
+                                                   float* __restrict__ face) {
+  const int t = threadIdx.x;
+  const bool col = t < FV_PLANE;
+  const int i = col ? t % FV_W - 1 : 0, j = col ? t / FV_W - 1 : 0;
+  const bool in_i = i >= 0 && i < TB, in_j = j >= 0 && j < TB;
+  const bool one_point = (A.flags & PPML_VHAT_1PT) != 0;
+  const int base = M.off[0][i + TH] + M.off[1][j + TH];
+  const bool fx = SPECIAL && M.flip[0][i + TH], fy = SPECIAL && M.flip[1][j + TH];
+  int inf_xy = -1;
+  if (SPECIAL) {
+    inf_xy = M.inflow[1][j + TH];
+    if (inf_xy < 0) inf_xy = M.inflow[0][i + TH];
+  }
+  auto load = [&](int k, float q[4]) {
+    const int o = base + M.off[2][k + TH];
+#pragma unroll
+    for (int f = 0; f < 4; f++) q[f] = __ldg(A.u[f] + o);
+    if (SPECIAL) {
+      if (fx) q[1] = -q[1];
+      if (fy) q[2] = -q[2];
+      if (M.flip[2][k + TH]) q[3] = -q[3];
+      int face_in = M.inflow[2][k + TH];  // the later axis decides
+      if (face_in < 0) face_in = inf_xy;
+      if (face_in >= 0)
+#pragma unroll
+        for (int f = 0; f < 4; f++) q[f] = __ldg(A.inflow + 6 * face_in + f);
+    }
+  };
+  float next[4] = {1.0f, 0.0f, 0.0f, 0.0f};
+  if (col) load(-1, next);
+  float ax0 = 0.0f, ax1 = 0.0f, by0 = 0.0f, by1 = 0.0f;  // in-plane sums of planes k-2, k-1
+  float vx1 = 0.0f, vy1 = 0.0f, sq1 = 1.0f, pz1 = 0.0f;  // of plane k-1
+  const int me = t;
+#pragma unroll 2
+  for (int k = -1; k <= TB; k++) {
+    const float ir = rcp_approx(next[0]), sq = sqrt_approx(next[0]);
+    const float vx = next[1] * ir, vy = next[2] * ir, vz = next[3] * ir;
+    float* const px = vel[k & 1][0];
+    float* const py = vel[k & 1][1];
+    float* const pz = vel[k & 1][2];
+    if (col) {
+      px[me] = vx;
+      py[me] = vy;
+      pz[me] = vz;
+      if (k < TB) load(k + 1, next);
+    }
+    __syncthreads();
+    // (k = -1: only the sums of the plane)
+    float ax = 4.0f * vx, by = 4.0f * vy, vt = vz;
+    if (col && !one_point) {
+      if (in_j) ax = 2.0f * vx + (px[me - FV_W] + px[me + FV_W]);
+      if (in_i) by = 2.0f * vy + (py[me - 1] + py[me + 1]);
+      if (in_i && in_j)
+        vt = 0.25f * vz + 0.125f * ((pz[me - 1] + pz[me + 1]) + (pz[me - FV_W] + pz[me + FV_W])) +
+             0.0625f * ((pz[me - FV_W - 1] + pz[me - FV_W + 1]) +
+                        (pz[me + FV_W - 1] + pz[me + FV_W + 1]));
+    }
+    const float pzk = vt * sq;
+    if (k >= 0 && in_i && in_j && col)  // face between k-1 and k
+      face[2 * FACE_AXIS + k * TN + i + TB * j] = th[2] * ((pzk + pz1) * rcp_approx(sq + sq1));
+    if (k >= 1) {  // plane k - 1 is complete
+      if (col) {
+        const float tx = one_point ? vx1 : 0.0625f * (2.0f * ax1 + (ax0 + ax));
+        const float ty = one_point ? vy1 : 0.0625f * (2.0f * by1 + (by0 + by));
+        prod[0][me] = tx * sq1;
+        prod[1][me] = ty * sq1;
+        prod[2][me] = sq1;
+      }
+      __syncthreads();
+      if (t < (TB + 1) * TB) {
+        const int l = t % TB, f = t / TB;  // line, face
+        const int ex = (l + 1) * FV_W + f;  // x face f of row y = l: cells f-1 and f
+        const float wx = (prod[0][ex] + prod[0][ex + 1]) * rcp_approx(prod[2][ex] + prod[2][ex + 1]);
+        face[f * TN + l + TB * (k - 1)] = th[0] * wx;
+        const int ey = f * FV_W + l + 1;  // y face f of column x = l
+        const float wy =
+            (prod[1][ey] + prod[1][ey + FV_W]) * rcp_approx(prod[2][ey] + prod[2][ey + FV_W]);
+        face[FACE_AXIS + f * TN + l + TB * (k - 1)] = th[1] * wy;
+      }
+    }
+    ax0 = ax1;
+    ax1 = ax;
+    by0 = by1;
+    by1 = by;
+    vx1 = vx;
+    vy1 = vy;
+    sq1 = sq;
+    pz1 = pzk;
+  }
+}
+
+__global__ void __launch_bounds__(FV_THREADS, 4) face_velocity_f32(MarchArgs<float> A) {
+  __shared__ float vel[2][3][FV_PLANE];
+  __shared__ float prod[3][FV_PLANE];
+  __shared__ TileMaps32 maps;
+  const int tiles[3] = {A.tiles_x, A.tiles_y, A.tiles_z};
+  const TileGeom tg = tile_geom(A.g, tiles, A.tile_order, A.tile_first + blockIdx.x);
+  if (!tg.valid) return;
+  build_maps32(maps, A.g, tg);
+  double stc[4];
+  cta_step_constants(A.dt_dev, A.dt_host, A.h, stc);  // (a barrier: the maps are built)
+  const float th[3] = {(float)stc[1], (float)stc[2], (float)stc[3]};
+  float* const face = A.face + (size_t)(tg.id - A.face_first) * FACE_TILE;
+  if (!tg.fast && (A.any_reflect || A.any_inflow))
+    face_velocity_tile<true>(A, tg, maps, th, vel, prod, face);
+  else
+    face_velocity_tile<false>(A, tg, maps, th, vel, prod, face);
+}
+
+// ----------------------------------------------------------------------------- the sweeps
+
+// Two fields at once: packed additions, multiplications and FMAs (one issue slot for two).
+__device__ __forceinline__ unsigned long long as_u64(float2 v) {
+  return *reinterpret_cast<unsigned long long*>(&v);
+}
+__device__ __forceinline__ float2 as_f2(unsigned long long v) {
+  return *reinterpret_cast<float2*>(&v);
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
+  return as_f2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+  unsigned long long r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
+  return as_f2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+  unsigned long long r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)), "l"(as_u64(c)));
+  return as_f2(r);
+}
+__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.0f), a); }
+
+// LineF32 for two fields.
+template <bool FLAT>
+struct LinePair {
+  float2 q2, q1, qn, d, s, l2;
+  float2 Pl, Pr;  // doubled deviations of cell p - 2
+  static __device__ __forceinline__ float2 half_slope(float2 l, float2 r) {
+    const float2 c = mul2(add2(l, r), both(0.25f));
+    return make_float2(min_xs(c.x, fmaxf(min_xs(l.x, r.x), 0.0f)),
+                       min_xs(c.y, fmaxf(min_xs(l.y, r.y), 0.0f)));
+  }
+  __device__ __forceinline__ void start(float2 a, float2 b, float2 c) {
+    q2 = a;
+    q1 = b;
+    qn = c;
+    Pl = Pr = l2 = both(0.0f);
+    d = sub2(c, b);
+    s = half_slope(sub2(b, a), d);
+  }
+  __device__ __forceinline__ void push(float2 q) {
+    if constexpr (!FLAT) {
+      const float2 dn = sub2(q, qn);
+      const float2 sn = half_slope(d, dn);
+      const float2 e = sub2(sn, s);
+      const float2 r2 = fma2(e, both(-2.0f / 3.0f), d);
+      const float2 t = make_float2(max_nan(min_xs_nan(l2.x, r2.x), 0.0f),
+                                   max_nan(min_xs_nan(l2.y, r2.y), 0.0f));
+      const float2 m = add2(t, t);
+      Pl = make_float2(min_xs_nan(l2.x, m.x), min_xs_nan(l2.y, m.y));
+      Pr = make_float2(min_xs_nan(r2.x, m.x), min_xs_nan(r2.y, m.y));
+      l2 = fma2(e, both(2.0f / 3.0f), d);
+      d = dn;
+      s = sn;
+    }
+    q2 = q1;
+    q1 = qn;
+    qn = q;
+  }
+};
+
+// upwind_flux_f32 for two fields.
+__device__ __forceinline__ float2 upwind_flux_pair(float w, float2 ql, float2 Ll, float2 Lr,
+                                                   float2 qr, float2 Rl, float2 Rr) {
+  const DevWeights c = dev_weights(fabsf(w));
+  const bool left = w >= 0.0f;
+  const float2 q = make_float2(left ? ql.x : qr.x, left ? ql.y : qr.y);
+  const float2 x = make_float2(left ? Lr.x : -Rl.x, left ? Lr.y : -Rl.y);
+  const float2 y = make_float2(left ? Ll.x : -Rr.x, left ? Ll.y : -Rr.y);
+  return mul2(both(w), fma2(both(c.a), x, fma2(both(c.b), y, q)));
+}
+
+// One line of two fields: q(p) for the positions -3..18 (called in order, each once), w(c) the
+// face velocities 0..16 (in order); emit(c, d, qc) for the cells c = 0..15 with
+// d = th (F+ - F-).  ahead() is called before the last four steps: the place to issue the
+// loads that the next sweep starts with.
+template <bool FLAT, typename QF, typename WF, typename EF, typename AF>
+__device__ __forceinline__ void lag_line_pair(QF q, WF w, EF emit, AF ahead) {
+  LinePair<FLAT> ln;
+  {
+    const float2 a = q(-3), b = q(-2), c = q(-1);
+    ln.start(a, b, c);
+  }
+  ln.push(q(0));
+  ln.push(q(1));
+  float2 ql = ln.q2, Ll = ln.Pl, Lr = ln.Pr;
+  ln.push(q(2));
+  float2 Fp = upwind_flux_pair(w(0), ql, Ll, Lr, ln.q2, ln.Pl, ln.Pr);
+  ql = ln.q2;
+  Ll = ln.Pl;
+  Lr = ln.Pr;
+  auto step = [&](int c) {
+    ln.push(q(c + 3));
+    const float2 F = upwind_flux_pair(w(c + 1), ql, Ll, Lr, ln.q2, ln.Pl, ln.Pr);
+    emit(c, sub2(F, Fp), ql);
+    Fp = F;
+    ql = ln.q2;
+    Ll = ln.Pl;
+    Lr = ln.Pr;
+  };
+#pragma unroll 1
+  for (int c0 = 0; c0 < TB - 4; c0 += 4) {
+#pragma unroll
+    for (int k = 0; k < 4; k++) step(c0 + k);
+  }
+  ahead();
+#pragma unroll
+  for (int c = TB - 4; c < TB; c++) step(c);
+}
+
+struct SweepSmem {
+  float2 core[ACC];  // two fields, pitches 17 and 272: every sweep's 8-byte accesses of a
+  float2 acc[ACC];   // half warp fall on 16 different bank pairs
+};
+
+// The sweeps of a tile, two fields at a time.  The z sweep reads the thread's column from
+// global memory four positions ahead and leaves the core, and what its divergence leaves of
+// the fields, in shared memory; the x sweep subtracts its divergence there; the y sweep
+// finishes into the output, rows of x.  The x and y lines of a warp lie in the warp's own two
+// z planes, so between them only the warp meets.  Each sweep issues the first loads of the
+// next (halos, face velocities) before its last four steps.
+// SPECIAL: mirrored or prescribed ghosts may occur.
+template <bool FLAT, bool SPECIAL>
+__device__ __forceinline__ void sweep_tile(const MarchArgs<float>& A, const TileGeom& tg,
+                                           const TileMaps32& maps, SweepSmem& S,
+                                           const float* __restrict__ face, int out0, int nvalid) {
+  const GridGeom& g = A.g;
+  const int a = threadIdx.x % TB, b = threadIdx.x / TB, nx = g.n[0];
+  // the thread's lines: z (x = a, y = b), x (y = a, z = b), y (x = a, z = b)
+  const int zbase = maps.off[0][a + TH] + maps.off[1][b + TH];
+  const int xbase = maps.off[1][a + TH] + maps.off[2][b + TH];
+  const int ybase = maps.off[0][a + TH] + maps.off[2][b + TH];
+  // cells of the core beyond the domain's x and y ends are ghosts to the x and y sweeps:
+  // columns there carry the mirrors and prescribed states of those axes
+  const bool col_fx = SPECIAL && maps.flip[0][a + TH], col_fy = SPECIAL && maps.flip[1][b + TH];
+  int col_in = -1;
+  if (SPECIAL) {
+    col_in = maps.inflow[1][b + TH];
+    if (col_in < 0) col_in = maps.inflow[0][a + TH];
+  }
+  // fields f, f + 1 at position p of the line with offset base along ax, through the maps
+  auto fetch = [&](int f, int ax, int base, int p) {
+    const int o = base + maps.off[ax][p + TH];
+    float2 v = make_float2(__ldg(A.u[f] + o), __ldg(A.u[f + 1] + o));
+    if (SPECIAL) {
+      if (maps.flip[ax][p + TH]) {
+        if (f == 1 + ax) v.x = -v.x;
+        if (f == ax) v.y = -v.y;
+      }
+      int in = maps.inflow[ax][p + TH];
+      if (ax == 2) {
+        if (col_fx && f == 0) v.y = -v.y;  // m_x
+        if (col_fy && f == 2) v.x = -v.x;  // m_y
+        if (in < 0) in = col_in;           // (the later axis decides)
+      }
+      if (in >= 0) v = make_float2(__ldg(A.inflow + 6 * in + f), __ldg(A.inflow + 6 * in + f + 1));
+    }
+    return v;
+  };
+  const float* const wx = face;
+  const float* const wy = face + FACE_AXIS;
+  const float* const wz = face + 2 * FACE_AXIS;
+  float2 ring[4], halo[6];
+  float wr[4], wn[4];  // face velocities: ring of the running sweep, first four of the next
+  auto first_w = [&](const float* w) {
+#pragma unroll
+    for (int c = 0; c < 4; c++) wn[c] = __ldg(w + c * TN);
+  };
+  auto take_w = [&]() {
+#pragma unroll
+    for (int c = 0; c < 4; c++) wr[c] = wn[c];
+  };
+  auto ring_w = [&](const float* w, int c) {
+    const float v = wr[c & 3];
+    if (c + 4 <= TB) wr[c & 3] = __ldg(w + (c + 4) * TN);
+    return v;
+  };
+  auto first_z = [&](int f) {
+#pragma unroll
+    for (int p = 0; p < 4; p++) ring[p] = fetch(f, 2, zbase, p - TH);
+    first_w(wz);
+  };
+  auto low_halo = [&](int f, int ax, int base) {  // positions -3..-1
+#pragma unroll
+    for (int h = 0; h < 3; h++) halo[h] = fetch(f, ax, base, h - 3);
+    first_w(ax == 0 ? wx : wy);
+  };
+  auto high_halo = [&](int f, int ax, int base) {  // positions 16..18
+#pragma unroll
+    for (int h = 3; h < 6; h++) halo[h] = fetch(f, ax, base, TB + h - 3);
+  };
+  auto line_q = [&](const float2* core, int stride, int p) {  // x and y lines
+    if (p < 0) return halo[p < -2 ? 0 : (p < -1 ? 1 : 2)];
+    if (p < TB) return core[p * stride];
+    return p == TB ? halo[3] : (p == TB + 1 ? halo[4] : halo[5]);
+  };
+  first_z(0);
+#pragma unroll 1
+  for (int f = 0; f < 6; f += 2) {
+    {  // z
+      float2* const core = &S.core[acc_at(a, b, 0)];
+      float2* const acc = &S.acc[acc_at(a, b, 0)];
+      take_w();
+      lag_line_pair<FLAT>(
+          [&](int p) {
+            const float2 v = ring[(p + 3) & 3];
+            if (p + 4 < TB + TH) ring[(p + 3) & 3] = fetch(f, 2, zbase, p + 4);
+            if (p >= 0 && p < TB) core[p * APP] = v;
+            return v;
+          },
+          [&](int c) { return ring_w(wz, c); },
+          [&](int c, float2 d, float2 q) { acc[c * APP] = sub2(q, d); },
+          [&]() {
+            low_halo(f, 0, xbase);
+            high_halo(f, 0, xbase);
+          });
+    }
+    __syncthreads();
+    {  // x
+      const float2* const core = &S.core[acc_at(0, a, b)];
+      float2* const acc = &S.acc[acc_at(0, a, b)];
+      take_w();
+      lag_line_pair<FLAT>([&](int p) { return line_q(core, 1, p); },
+                          [&](int c) { return ring_w(wx, c); },
+                          [&](int c, float2 d, float2) { acc[c] = sub2(acc[c], d); },
+                          [&]() { low_halo(f, 1, ybase); });
+    }
+    high_halo(f, 1, ybase);
+    __syncwarp();
+    {  // y
+      const float2* const core = &S.core[acc_at(a, 0, b)];
+      const float2* const acc = &S.acc[acc_at(a, 0, b)];
+      float* const o0 = A.out[f] + out0;
+      float* const o1 = A.out[f + 1] + out0;
+      take_w();
+      lag_line_pair<FLAT>([&](int p) { return line_q(core, ARP, p); },
+                          [&](int c) { return ring_w(wy, c); },
+                          [&](int c, float2 d, float2) {
+                            if (c < nvalid) {
+                              const float2 v = sub2(acc[c * ARP], d);
+                              o0[(size_t)c * nx] = v.x;
+                              o1[(size_t)c * nx] = v.y;
+                            }
+                          },
+                          [&]() {
+                            if (f < 4) first_z(f + 2);
+                          });
+    }
+    __syncthreads();  // the next z sweep writes the core and the accumulator
+  }
+}
+
+template <bool FLAT>
+__global__ void __launch_bounds__(TN, 3) lagrangian_sweep_f32(MarchArgs<float> A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  SweepSmem& S = *reinterpret_cast<SweepSmem*>(smem_raw);
+  __shared__ TileMaps32 maps;
+  const GridGeom& g = A.g;
+  const int tid = threadIdx.x, a = tid % TB, b = tid / TB;
+  const int tiles[3] = {A.tiles_x, A.tiles_y, A.tiles_z};
+  const TileGeom tg = tile_geom(g, tiles, A.tile_order, A.tile_first + blockIdx.x);
+  if (!tg.valid) return;  // a padding block of a blocked order (uniform over the CTA)
+  build_maps32(maps, g, tg);
+  __syncthreads();
+  const float* const face = A.face + (size_t)(tg.id - A.face_first) * FACE_TILE + tid;
+  const bool line_ok = tg.i0 + a < g.n[0] && tg.k0 + b < g.n[2];
+  const int nvalid = line_ok ? min(TB, g.n[1] - tg.j0) : 0;
+  const int nx = g.n[0];
+  const int out0 = (tg.i0 + a) + nx * tg.j0 + (int)g.nxy * (tg.k0 + b);
+  if (!tg.fast && (A.any_reflect || A.any_inflow))
+    sweep_tile<FLAT, true>(A, tg, maps, S, face, out0, nvalid);
+  else
+    sweep_tile<FLAT, false>(A, tg, maps, S, face, out0, nvalid);
+
+  // ---- energy correction (Sec. 1.4), CFL maxima and sums of the thread's y line
+  FieldSums<float> sums;
+  sums.init();
+  float vmax = 0.0f, cmax = 0.0f;
+  unsigned long long nvac = 0, nbad = 0;
+  const float gamma = (float)A.gamma, gm1 = (float)(A.gamma - 1.0);
+  const float rho_vac_up = __double2float_ru(A.rho_vac);
+  constexpr int FB = 2;  // cells at a time, the next ones' loads in flight
+  float nu[FB][6];
+  auto load = [&](int c0) {
+#pragma unroll
+    for (int q = 0; q < FB; q++) {
+      const size_t idx = out0 + (size_t)min(c0 + q, nvalid - 1) * nx;
+#pragma unroll
+      for (int f = 0; f < 6; f++) nu[q][f] = A.out[f][idx];
+    }
+  };
+  if (nvalid > 0) load(0);
+#pragma unroll 1
+  for (int c0 = 0; c0 < nvalid; c0 += FB) {
+    float u[FB][6];
+#pragma unroll
+    for (int q = 0; q < FB; q++)
+#pragma unroll
+      for (int f = 0; f < 6; f++) u[q][f] = nu[q][f];
+    if (c0 + FB < nvalid) load(c0 + FB);
+    bool vac[FB], any_vac = false;
+#pragma unroll
+    for (int q = 0; q < FB; q++) {
+      vac[q] = c0 + q < nvalid && vacuum_cell_f32(u[q], rho_vac_up);
+      any_vac |= vac[q];
+      const float e = dense_eps_f32(u[q]);
+      u[q][5] = vac[q] ? u[q][5] : e;
+    }
+    if (any_vac) {
+#pragma unroll
+      for (int q = 0; q < FB; q++)
+        if (vac[q]) {
+          vacuum_correct_f32(u[q], A.rho_vac);
+          nvac++;
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < FB; q++) {
+      if (c0 + q >= nvalid) break;
+      const size_t idx = out0 + (size_t)(c0 + q) * nx;
+      if (vac[q]) {
+#pragma unroll
+        for (int f = 1; f <= 3; f++) A.out[f][idx] = u[q][f];
+      }
+      A.out[5][idx] = u[q][5];
+      sums.add(u[q]);
+      cell_speeds_f32(u[q], gamma, gm1, vmax, cmax, nbad);
+    }
+  }
+  float hi[6], lo[6];
+#pragma unroll
+  for (int f = 0; f < 6; f++) {
+    hi[f] = sums.s[f].hi;
+    lo[f] = sums.s[f].lo;
+  }
+  block_reduce_store_f32<TN>(hi, lo, vmax, cmax, (unsigned)nvac, (unsigned)nbad, A.partials, tg.id);
+  finalize_last(A.partials, tiles[0] * tiles[1] * tiles[2], A.fin, read_tau(A.dt_dev, A.dt_host));
+}
+
+}  // namespace ppml
