@@ -11,14 +11,46 @@ cudaError_t prepare_sweeps(float) {
   if (e == cudaSuccess)
     e = cudaFuncSetAttribute(lagrangian_sweep_f32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)sizeof(SweepSmem));
+  auto euler = [&](auto kernel) {
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)sizeof(EulerSmem));
+  };
+  euler(eulerian_sweep_f32<false, false>);
+  euler(eulerian_sweep_f32<false, true>);
+  euler(eulerian_sweep_f32<true, false>);
+  euler(eulerian_sweep_f32<true, true>);
   return e;
+}
+
+bool three_axes(const MarchArgs<float>& A) {
+  return A.g.n[0] > 1 && A.g.n[1] > 1 && A.g.n[2] > 1;
+}
+
+// Eulerian stage of plain float states with three active axes.  False: not such a state.
+bool launch_euler_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
+  if (!three_axes(A)) return false;
+  constexpr size_t SM = sizeof(EulerSmem);
+  const bool flat = (A.flags & PPML_FIRST_ORDER) != 0;
+  if (A.phi) {
+    if (flat)
+      eulerian_sweep_f32<true, true><<<nblk, TN, SM, st>>>(A);
+    else
+      eulerian_sweep_f32<false, true><<<nblk, TN, SM, st>>>(A);
+  } else {
+    if (flat)
+      eulerian_sweep_f32<true, false><<<nblk, TN, SM, st>>>(A);
+    else
+      eulerian_sweep_f32<false, false><<<nblk, TN, SM, st>>>(A);
+  }
+  return true;
 }
 
 // Lagrangian stage of plain float states with three active axes: face velocities, then the
 // sweeps; in several launches where the face array does not hold every tile (the
 // allocation-free step).  False: not such a state, nothing launched.
 bool launch_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
-  if (!A.face || A.g.n[0] == 1 || A.g.n[1] == 1 || A.g.n[2] == 1) return false;
+  if (!A.face || !three_axes(A)) return false;
   MarchArgs<float> B = A;
   const int per = A.face_tiles >= nblk || A.tile_order != 0 ? nblk : A.face_tiles;
   for (int first = 0; first < nblk; first += per) {

@@ -7,6 +7,7 @@
 namespace ppml {
 
 // Kernels of their own for plain float states (ppml_kern_f32.cu); FP64 has none.
+inline bool launch_euler_sweeps(const MarchArgs<double>&, int, cudaStream_t) { return false; }
 inline bool launch_sweeps(const MarchArgs<double>&, int, cudaStream_t) { return false; }
 inline cudaError_t prepare_sweeps(double) { return cudaSuccess; }
 
@@ -60,6 +61,7 @@ int launch_eulerian<PPML_REAL>(const MarchArgs<PPML_REAL>& A, int nblk, cudaStre
   constexpr int MB = MinBlocks<PPML_REAL>::value;
   constexpr size_t SM = sizeof(EulTileSmem<PPML_REAL>);
   const bool df = kHasDF && A.outlo[1];
+  if (!df && launch_euler_sweeps(A, nblk, st)) return ppml_check_launch("eulerian_sweep_f32");
   if (A.any_inflow) {
     if (df)
       eulerian_tile<PPML_REAL, MB, kHasDF, true><<<nblk, TN, SM, st>>>(A);

@@ -1,4 +1,8 @@
-// FP32 Lagrangian stage of grids with three active axes (plain float states), in two kernels:
+// FP32 stages of grids with three active axes (plain float states), 16^3 tiles:
+//
+//   eulerian_sweep_f32  the Eulerian stage (Sec. 1.1/1.2), with the gravity source terms
+//
+// and the Lagrangian stage in two kernels:
 //
 //   face_velocity_f32   eqs. veltemplate and modspaceaveragevelocitylagrange: the Courant
 //                       velocities w = v^ tau/h of every face of every 16^3 tile, into a
@@ -273,7 +277,7 @@ __device__ __forceinline__ void lag_line_pair(QF q, WF w, EF emit, AF ahead) {
     Ll = ln.Pl;
     Lr = ln.Pr;
   };
-#pragma unroll 1
+#pragma unroll
   for (int c0 = 0; c0 < TB - 4; c0 += 4) {
 #pragma unroll
     for (int k = 0; k < 4; k++) step(c0 + k);
@@ -289,9 +293,9 @@ struct SweepSmem {
 };
 
 // The sweeps of a tile, two fields at a time.  The z sweep reads the thread's column from
-// global memory four positions ahead and leaves the core, and what its divergence leaves of
-// the fields, in shared memory; the x sweep subtracts its divergence there; the y sweep
-// finishes into the output, rows of x.  The x and y lines of a warp lie in the warp's own two
+// global memory eight positions ahead and leaves the core and its divergence in shared
+// memory; the x sweep adds its divergence there; the y sweep finishes into the output, rows
+// of x.  The x and y lines of a warp lie in the warp's own two
 // z planes, so between them only the warp meets.  Each sweep issues the first loads of the
 // next (halos, face velocities) before its last four steps.
 // SPECIAL: mirrored or prescribed ghosts may occur.
@@ -335,7 +339,7 @@ __device__ __forceinline__ void sweep_tile(const MarchArgs<float>& A, const Tile
   const float* const wx = face;
   const float* const wy = face + FACE_AXIS;
   const float* const wz = face + 2 * FACE_AXIS;
-  float2 ring[4], halo[6];
+  float2 ring[8], halo[6], yhalo[6];
   float wr[4], wn[4];  // face velocities: ring of the running sweep, first four of the next
   auto first_w = [&](const float* w) {
 #pragma unroll
@@ -352,7 +356,7 @@ __device__ __forceinline__ void sweep_tile(const MarchArgs<float>& A, const Tile
   };
   auto first_z = [&](int f) {
 #pragma unroll
-    for (int p = 0; p < 4; p++) ring[p] = fetch(f, 2, zbase, p - TH);
+    for (int p = 0; p < 8; p++) ring[p] = fetch(f, 2, zbase, p - TH);
     first_w(wz);
   };
   auto low_halo = [&](int f, int ax, int base) {  // positions -3..-1
@@ -378,18 +382,20 @@ __device__ __forceinline__ void sweep_tile(const MarchArgs<float>& A, const Tile
       take_w();
       lag_line_pair<FLAT>(
           [&](int p) {
-            const float2 v = ring[(p + 3) & 3];
-            if (p + 4 < TB + TH) ring[(p + 3) & 3] = fetch(f, 2, zbase, p + 4);
+            const float2 v = ring[(p + 3) & 7];
+            if (p + 8 < TB + TH) ring[(p + 3) & 7] = fetch(f, 2, zbase, p + 8);
             if (p >= 0 && p < TB) core[p * APP] = v;
             return v;
           },
           [&](int c) { return ring_w(wz, c); },
-          [&](int c, float2 d, float2 q) { acc[c * APP] = sub2(q, d); },
+          [&](int c, float2 d, float2) { acc[c * APP] = d; },
           [&]() {
             low_halo(f, 0, xbase);
             high_halo(f, 0, xbase);
           });
     }
+#pragma unroll
+    for (int h = 0; h < 6; h++) yhalo[h] = fetch(f, 1, ybase, h < 3 ? h - 3 : TB + h - 3);
     __syncthreads();
     {  // x
       const float2* const core = &S.core[acc_at(0, a, b)];
@@ -397,10 +403,11 @@ __device__ __forceinline__ void sweep_tile(const MarchArgs<float>& A, const Tile
       take_w();
       lag_line_pair<FLAT>([&](int p) { return line_q(core, 1, p); },
                           [&](int c) { return ring_w(wx, c); },
-                          [&](int c, float2 d, float2) { acc[c] = sub2(acc[c], d); },
-                          [&]() { low_halo(f, 1, ybase); });
+                          [&](int c, float2 d, float2) { acc[c] = add2(acc[c], d); },
+                          [&]() { first_w(wy); });
     }
-    high_halo(f, 1, ybase);
+#pragma unroll
+    for (int h = 0; h < 6; h++) halo[h] = yhalo[h];
     __syncwarp();
     {  // y
       const float2* const core = &S.core[acc_at(a, 0, b)];
@@ -410,9 +417,9 @@ __device__ __forceinline__ void sweep_tile(const MarchArgs<float>& A, const Tile
       take_w();
       lag_line_pair<FLAT>([&](int p) { return line_q(core, ARP, p); },
                           [&](int c) { return ring_w(wy, c); },
-                          [&](int c, float2 d, float2) {
+                          [&](int c, float2 d, float2 qc) {
                             if (c < nvalid) {
-                              const float2 v = sub2(acc[c * ARP], d);
+                              const float2 v = sub2(qc, add2(acc[c * ARP], d));
                               o0[(size_t)c * nx] = v.x;
                               o1[(size_t)c * nx] = v.y;
                             }
@@ -426,7 +433,7 @@ __device__ __forceinline__ void sweep_tile(const MarchArgs<float>& A, const Tile
 }
 
 template <bool FLAT>
-__global__ void __launch_bounds__(TN, 3) lagrangian_sweep_f32(MarchArgs<float> A) {
+__global__ void __launch_bounds__(TN, 2) lagrangian_sweep_f32(MarchArgs<float> A) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   SweepSmem& S = *reinterpret_cast<SweepSmem*>(smem_raw);
   __shared__ TileMaps32 maps;
@@ -510,6 +517,314 @@ __global__ void __launch_bounds__(TN, 3) lagrangian_sweep_f32(MarchArgs<float> A
   }
   block_reduce_store_f32<TN>(hi, lo, vmax, cmax, (unsigned)nvac, (unsigned)nbad, A.partials, tg.id);
   finalize_last(A.partials, tiles[0] * tiles[1] * tiles[2], A.fin, read_tau(A.dt_dev, A.dt_host));
+}
+
+// ------------------------------------------------------------------------- Eulerian stage
+
+struct EulerSmem {
+  float2 re[ACC];   // (rho, rho eps) of the tile
+  float mx[ACC];    // m_x of the tile, then its update
+  float2 acc[ACC];  // sums over axes of th (PV+ - PV-) and th (V+ - V-)
+};
+
+// One line of the Eulerian stage, (v, p) as a packed pair of lines: q(p, v, r) gives the pair
+// (v_a, p) and rho at the positions p = -3..18 (called in order, each once).  emit(c, dm, dpv,
+// dv) as in sweep_eulerian_dev.  ahead(): before the last four steps.
+template <bool FLAT, typename QF, typename EF, typename AF>
+__device__ __forceinline__ void euler_line_pair(QF q, float gamma, float th, EF emit, AF ahead) {
+  LinePair<FLAT> ln;
+  float r1, r2, rn, skip;  // rho at p-1, p-2, p
+  {
+    float2 a, b, c;
+    q(-3, a, skip);
+    q(-2, b, skip);
+    q(-1, c, r2);
+    ln.start(a, b, c);
+  }
+  {
+    float2 v;
+    q(0, v, r1);
+    ln.push(v);
+    q(1, v, rn);
+    ln.push(v);
+  }
+  // cell p-3 (the face's left cell): values, deviations, sqrt(rho), rho sqrt(rho), p sqrt(rho)
+  float2 ql = ln.q2, Ll = ln.Pl, Lr = ln.Pr;
+  float sl = sqrt_approx(r2), Al = r2 * sl, Bl = ql.y * sl;
+  r2 = r1;
+  r1 = rn;
+  float Vp = 0.0f, Pp = 0.0f;
+  auto face = [&](int p, float& V, float& P) {  // after position p: the face of p-3 and p-2
+    float2 v;
+    q(p, v, rn);
+    ln.push(v);
+    const float sc = sqrt_approx(r2), Ac = r2 * sc, Bc = ln.q2.y * sc;
+    const float A = Al + Ac, lam = sqrt_approx(gamma * (Bl + Bc) * rcp_approx(A));
+    const float Z = lam * A * rcp_approx(sl + sc);
+    const DevWeights w = dev_weights(lam * th);
+    const float2 right = fma2(both(w.a), Lr, fma2(both(w.b), Ll, ql));
+    const float2 left = fma2(both(-w.a), ln.Pl, fma2(both(-w.b), ln.Pr, ln.q2));
+    const float2 sum = add2(right, left), dif = sub2(right, left);
+    V = 0.5f * fmaf(dif.y, rcp_approx(Z), sum.x);
+    P = 0.5f * fmaf(dif.x, Z, sum.y);
+    ql = ln.q2;
+    Ll = ln.Pl;
+    Lr = ln.Pr;
+    sl = sc;
+    Al = Ac;
+    Bl = Bc;
+    r2 = r1;
+    r1 = rn;
+  };
+  face(2, Vp, Pp);
+  auto step = [&](int c) {
+    float V, P;
+    face(c + 3, V, P);
+    emit(c, th * (P - Pp), th * (P * V - Pp * Vp), th * (V - Vp));
+    Vp = V;
+    Pp = P;
+  };
+#pragma unroll 1
+  for (int c0 = 0; c0 < TB - 4; c0 += 4) {
+#pragma unroll
+    for (int k = 0; k < 4; k++) step(c0 + k);
+  }
+  ahead();
+#pragma unroll
+  for (int c = TB - 4; c < TB; c++) step(c);
+}
+
+// The Eulerian stage of a tile.  The z sweep reads rho, rho eps and m_z of the thread's column
+// from global memory, stores m_z's update and leaves (rho, rho eps), m_x and its pressure-work
+// and divergence terms in shared memory; the x sweep reads the core there and leaves m_x's
+// update in place; the y sweep reads m_y in rows of x, adds its terms and stores m_x, m_y,
+// rho E and rho eps, all in rows of x.  One CTA barrier: the x and y lines of a warp lie in
+// its own two z planes.  PHI: the gravity source terms, each where its momentum is at hand.
+// SPECIAL: mirrored or prescribed ghosts may occur.
+template <bool FLAT, bool PHI, bool SPECIAL>
+__device__ __forceinline__ void euler_tile(const MarchArgs<float>& A, const TileGeom& tg,
+                                           const TileMaps32& maps, EulerSmem& S,
+                                           const float th[3], float tau) {
+  const GridGeom& g = A.g;
+  const int a = threadIdx.x % TB, b = threadIdx.x / TB, nx = g.n[0], nxy = (int)g.nxy;
+  const float gamma = (float)A.gamma, gm1 = (float)(A.gamma - 1.0);
+  const int zbase = maps.off[0][a + TH] + maps.off[1][b + TH];
+  const int xbase = maps.off[1][a + TH] + maps.off[2][b + TH];
+  const int ybase = maps.off[0][a + TH] + maps.off[2][b + TH];
+  // ghost cells of the core beyond the domain's x and y ends (see sweep_tile)
+  const bool col_fx = SPECIAL && maps.flip[0][a + TH];
+  int col_in = -1;
+  if (SPECIAL) {
+    col_in = maps.inflow[1][b + TH];
+    if (col_in < 0) col_in = maps.inflow[0][a + TH];
+  }
+  // rho, m_ax and rho eps at position p of the line with offset base along ax
+  auto fetch = [&](int ax, int base, int p) {
+    const int o = base + maps.off[ax][p + TH];
+    float3 v = make_float3(__ldg(A.u[0] + o), __ldg(A.u[1 + ax] + o), __ldg(A.u[5] + o));
+    if (SPECIAL) {
+      if (maps.flip[ax][p + TH]) v.y = -v.y;
+      int in = maps.inflow[ax][p + TH];
+      if (ax == 2 && in < 0) in = col_in;
+      if (in >= 0)
+        v = make_float3(__ldg(A.inflow + 6 * in), __ldg(A.inflow + 6 * in + 1 + ax),
+                        __ldg(A.inflow + 6 * in + 5));
+    }
+    return v;
+  };
+  auto fetch_mx = [&](int p) {  // m_x of the column's cell p of the core
+    float m = __ldg(A.u[1] + (zbase + maps.off[2][p + TH]));
+    if (SPECIAL) {
+      if (col_fx) m = -m;
+      int in = maps.inflow[2][p + TH];
+      if (in < 0) in = col_in;
+      if (in >= 0) m = __ldg(A.inflow + 6 * in + 1);
+    }
+    return m;
+  };
+  // Phi's neighbour along ax at coordinate c (domain) in direction dir, as an offset: wraps at
+  // periodic faces, zero-gradient at the others
+  auto phi_step = [&](int ax, int c, int dir) {
+    const int n = g.n[ax], q = c + dir, st = ax == 0 ? 1 : (ax == 1 ? nx : nxy);
+    if ((unsigned)q < (unsigned)n) return dir * st;
+    return g.bc[2 * ax + (dir > 0)] == PPML_BC_PERIODIC ? -dir * (n - 1) * st : 0;
+  };
+  float3 ring[4], halo[6], yhalo[6];
+  float mring[4];
+  // ---- z
+  {
+    float2* const re = &S.re[acc_at(a, b, 0)];
+    float* const mx = &S.mx[acc_at(a, b, 0)];
+    float2* const acc = &S.acc[acc_at(a, b, 0)];
+    const bool ok = tg.i0 + a < nx && tg.j0 + b < g.n[1];
+    const int nvalid = ok ? min(TB, g.n[2] - tg.k0) : 0;
+    const int o0 = (tg.i0 + a) + nx * (tg.j0 + b) + nxy * tg.k0;
+    float* const om = A.out[3] + o0;
+    const float rg = PHI ? tau / (float)(2.0 * A.h[2]) : 0.0f;
+    float m1 = 0.0f, m2 = 0.0f, m3 = 0.0f, mn = 0.0f;  // m_z at p-1, p-2, p-3, p
+    float d1 = 0.0f, d2 = 0.0f, d3 = 0.0f, dn = 0.0f;  // rho there (PHI)
+#pragma unroll
+    for (int p = 0; p < 4; p++) ring[p] = fetch(2, zbase, p - TH);
+#pragma unroll
+    for (int p = 0; p < 4; p++) mring[p] = fetch_mx(p);
+    euler_line_pair<FLAT>(
+        [&](int p, float2& v, float& r) {
+          const float3 u = ring[(p + 3) & 3];
+          if (p + 4 < TB + TH) ring[(p + 3) & 3] = fetch(2, zbase, p + 4);
+          if (p >= 0 && p < TB) {
+            re[p * APP] = make_float2(u.x, u.z);
+            mx[p * APP] = mring[p & 3];
+            if (p + 4 < TB) mring[p & 3] = fetch_mx(p + 4);
+          }
+          v = make_float2(u.y * rcp_approx(u.x), gm1 * u.z);
+          r = u.x;
+          m3 = m2;
+          m2 = m1;
+          m1 = mn;
+          mn = u.y;
+          if (PHI) {
+            d3 = d2;
+            d2 = d1;
+            d1 = dn;
+            dn = u.x;
+          }
+        },
+        gamma, th[2],
+        [&](int c, float dm, float dpv, float dv) {
+          if (PHI && c < nvalid) {
+            const float* const f = A.phi + o0 + (size_t)c * nxy;
+            const float gr = (__ldg(f + phi_step(2, tg.k0 + c, 1)) - __ldg(f + phi_step(2, tg.k0 + c, -1))) * rg;
+            dm = fmaf(d3, gr, dm);
+            dpv = fmaf(m3, gr, dpv);
+          }
+          acc[c * APP] = make_float2(dpv, dv);
+          if (c < nvalid) om[(size_t)c * nxy] = m3 - dm;
+        },
+        [&]() {
+#pragma unroll
+          for (int h = 0; h < 6; h++) halo[h] = fetch(0, xbase, h < 3 ? h - 3 : TB + h - 3);
+        });
+  }
+#pragma unroll
+  for (int h = 0; h < 6; h++) yhalo[h] = fetch(1, ybase, h < 3 ? h - 3 : TB + h - 3);
+  __syncthreads();
+  const bool yok = tg.i0 + a < nx && tg.k0 + b < g.n[2];
+  const int nvalid = yok ? min(TB, g.n[1] - tg.j0) : 0;
+  const int o0 = (tg.i0 + a) + nx * tg.j0 + nxy * (tg.k0 + b);  // the y line's first cell
+  auto my_at = [&](int p) { return __ldg(A.u[2] + (ybase + maps.off[1][p + TH])); };
+  float ering[4];
+  // ---- x
+  {
+    const float2* const re = &S.re[acc_at(0, a, b)];
+    float* const mx = &S.mx[acc_at(0, a, b)];
+    float2* const acc = &S.acc[acc_at(0, a, b)];
+    euler_line_pair<FLAT>(
+        [&](int p, float2& v, float& r) {
+          float3 u;
+          if (p < 0 || p >= TB) {
+            u = p < 0 ? halo[p < -2 ? 0 : (p < -1 ? 1 : 2)]
+                      : (p == TB ? halo[3] : (p == TB + 1 ? halo[4] : halo[5]));
+          } else {
+            const float2 q = re[p];
+            u = make_float3(q.x, mx[p], q.y);
+          }
+          v = make_float2(u.y * rcp_approx(u.x), gm1 * u.z);
+          r = u.x;
+        },
+        gamma, th[0],
+        [&](int c, float dm, float dpv, float dv) {
+          acc[c] = add2(acc[c], make_float2(dpv, dv));
+          mx[c] = mx[c] - dm;
+        },
+        [&]() {
+#pragma unroll
+          for (int p = 0; p < 4; p++) {
+            mring[p] = my_at(p);
+            ering[p] = p < nvalid ? __ldg(A.u[4] + o0 + (size_t)p * nx) : 0.0f;
+          }
+        });
+  }
+#pragma unroll
+  for (int h = 0; h < 6; h++) halo[h] = yhalo[h];
+  __syncwarp();
+  // ---- y
+  {
+    const float2* const re = &S.re[acc_at(a, 0, b)];
+    const float* const mx = &S.mx[acc_at(a, 0, b)];
+    const float2* const acc = &S.acc[acc_at(a, 0, b)];
+    const float rgx = PHI ? tau / (float)(2.0 * A.h[0]) : 0.0f;
+    const float rgy = PHI ? tau / (float)(2.0 * A.h[1]) : 0.0f;
+    const int pxm = PHI ? phi_step(0, tg.i0 + a, -1) : 0, pxp = PHI ? phi_step(0, tg.i0 + a, 1) : 0;
+    float m1 = 0.0f, m2 = 0.0f, m3 = 0.0f, mn = 0.0f;  // m_y at p-1, p-2, p-3, p
+    euler_line_pair<FLAT>(
+        [&](int p, float2& v, float& r) {
+          float3 u;
+          if (p < 0 || p >= TB) {
+            u = p < 0 ? halo[p < -2 ? 0 : (p < -1 ? 1 : 2)]
+                      : (p == TB ? halo[3] : (p == TB + 1 ? halo[4] : halo[5]));
+          } else {
+            const float2 q = re[p * ARP];
+            float m = mring[p & 3];
+            if (SPECIAL) {  // core cells beyond the domain's y end are ghosts of this sweep
+              if (maps.flip[1][p + TH]) m = -m;
+              const int in = maps.inflow[1][p + TH];
+              if (in >= 0) m = __ldg(A.inflow + 6 * in + 2);
+            }
+            if (p + 4 < TB) mring[p & 3] = my_at(p + 4);
+            u = make_float3(q.x, m, q.y);
+          }
+          v = make_float2(u.y * rcp_approx(u.x), gm1 * u.z);
+          r = u.x;
+          m3 = m2;
+          m2 = m1;
+          m1 = mn;
+          mn = u.y;
+        },
+        gamma, th[1],
+        [&](int c, float dm, float dpv, float dv) {
+          const float en = ering[c & 3];
+          if (c + 4 < nvalid) ering[c & 3] = __ldg(A.u[4] + o0 + (size_t)(c + 4) * nx);
+          if (c < nvalid) {
+            const float2 s = acc[c * ARP], q = re[c * ARP];
+            const size_t o = o0 + (size_t)c * nx;
+            float m = mx[c * ARP];
+            if (PHI) {
+              const float* const f = A.phi + o;
+              const int j = tg.j0 + c;
+              const float gy = (__ldg(f + phi_step(1, j, 1)) - __ldg(f + phi_step(1, j, -1))) * rgy;
+              const float gx = (__ldg(f + pxp) - __ldg(f + pxm)) * rgx;
+              dm = fmaf(q.x, gy, dm);
+              dpv = fmaf(m3, gy, dpv);
+              m = fmaf(-q.x, gx, m);
+              dpv = fmaf(__ldg(A.u[1] + o), gx, dpv);
+            }
+            A.out[1][o] = m;
+            A.out[2][o] = m3 - dm;
+            A.out[4][o] = en - (s.x + dpv);
+            A.out[5][o] = eps_update(q.y, gm1, s.y + dv);
+            if (A.out[0]) A.out[0][o] = q.x;
+          }
+        },
+        [&]() {});
+  }
+}
+
+template <bool FLAT, bool PHI>
+__global__ void __launch_bounds__(TN, 2) eulerian_sweep_f32(MarchArgs<float> A) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  EulerSmem& S = *reinterpret_cast<EulerSmem*>(smem_raw);
+  __shared__ TileMaps32 maps;
+  const int tiles[3] = {A.tiles_x, A.tiles_y, A.tiles_z};
+  const TileGeom tg = tile_geom(A.g, tiles, A.tile_order, blockIdx.x);
+  if (!tg.valid) return;  // a padding block of a blocked order (uniform over the CTA)
+  build_maps32(maps, A.g, tg);
+  double stc[4];
+  cta_step_constants(A.dt_dev, A.dt_host, A.h, stc);  // (a barrier: the maps are built)
+  const float th[3] = {(float)stc[1], (float)stc[2], (float)stc[3]};
+  if (!tg.fast && (A.any_reflect || A.any_inflow))
+    euler_tile<FLAT, PHI, true>(A, tg, maps, S, th, (float)stc[0]);
+  else
+    euler_tile<FLAT, PHI, false>(A, tg, maps, S, th, (float)stc[0]);
 }
 
 }  // namespace ppml
