@@ -79,6 +79,14 @@ int plan_batch(ppml_batch* b) {
   int dev = 0, maxsm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&maxsm, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+  // plain FP32 instances hold eight padded arrays (advance_part_f32), a few values more than
+  // the documented size that decides whether an instance fits; the kernels' own static
+  // shared memory leaves that much of its 1 KB
+  const size_t launch =
+      b->dtype == PPML_F64
+          ? smem
+          : std::max(smem, 8 * elt * (size_t)std::max(n_split ? nlmax + 2 * kPairHalo : 0,
+                                                      nmax ? nmax + 2 * kBatchGhost : 0));
   if (smem + 1024 > (size_t)maxsm)
     return ppml_fail(PPML_E_INVAL,
                      "largest instance needs %zu bytes of shared memory (> %d): %d cells on one "
@@ -108,7 +116,7 @@ int plan_batch(ppml_batch* b) {
   b->n_split = n_split;
   b->nlmax = nlmax;
   b->nmax = nmax;
-  b->smem = smem;
+  b->smem = launch;
   b->smem_df = smem_df;
   b->max_smem = maxsm;
   return PPML_OK;
@@ -121,7 +129,7 @@ int launch_typed_t(ppml_batch* b, void* const state[4], void* const lo[3], InstD
   BatchLo<T> L;
   for (int q = 0; q < 3; q++) L.p[q] = lo ? (T*)lo[q] : nullptr;
   const size_t smem = lo ? b->smem_df : b->smem;
-  if (smem + 1024 > (size_t)b->max_smem)
+  if (lo && smem + 1024 > (size_t)b->max_smem)
     return ppml_fail(PPML_E_INVAL,
                      "with low parts the largest instance needs %zu bytes of shared memory (> %d)",
                      smem, b->max_smem);

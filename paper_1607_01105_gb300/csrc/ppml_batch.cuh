@@ -17,6 +17,7 @@
 #include <cooperative_groups.h>
 
 #include "ppml_device.cuh"
+#include "ppml_pair.cuh"
 
 namespace ppml {
 
@@ -41,6 +42,15 @@ __device__ __forceinline__ unsigned cluster_rank() {
 }
 // barrier of all threads of the cluster (release / acquire of the cluster's shared memory)
 __device__ __forceinline__ void cluster_sync() { cooperative_groups::this_cluster().sync(); }
+
+// CTAs per SM the stepping kernels are compiled for.  FP64 fills its pipe better with two
+// (64 registers a thread: 192 instances of 128..2048 cells, 16 steps, 5.95 -> 5.27 ms); plain
+// FP32 loses more to spills than it gains (512 instances: 3.31 -> 4.35 ms).
+template <typename T, int NTHREADS>
+constexpr int kBatchCtas = sizeof(T) == 8 && NTHREADS == 512 ? 2 : 1;
+
+// Doubles of a CTA's reduction scratch (block_cfl_step, cfl_decide).
+constexpr int kBatchRed = 70;
 
 struct InstDev {
   long long off;  // first cell in the packed arrays
@@ -289,6 +299,60 @@ __device__ __forceinline__ bool block_cfl_step(T a, T b, bool bad, double cfl, I
 }
 
 
+// The keeper of a plain FP32 instance's time: the first lane of the last warp, which has the
+// fewest cells (or none) to stream.
+template <int NTHREADS>
+__device__ __forceinline__ bool keeps_time() {
+  return threadIdx.x == NTHREADS - 32;
+}
+
+// CFL step of a plain FP32 instance on one CTA, as block_cfl_step with one barrier: after it
+// every warp folds the warps' maxima itself and, while the step is clearly shorter than what
+// remains of the run (a float lower bound that the keeper published during the last step),
+// takes tau / h = cfl / (max|v| + max c) from them; the keeper advances the instance's time
+// beside the Eulerian stage.  Otherwise (near t_end, at it, or a non-physical state) the keeper
+// decides as cfl_decide does, behind a second barrier.  sh + 69: the lower bound.
+template <int NTHREADS>
+__device__ __forceinline__ bool block_cfl_step_f32(float a, float b, bool bad, double cfl,
+                                                   InstDev& I, double* sh, float& th) {
+  warp_maxima<float>(a, b, sh);
+  const bool any_bad = __syncthreads_or(bad) != 0;
+  const float* const shT = reinterpret_cast<const float*>(sh);
+  float* const rem_low = reinterpret_cast<float*>(sh + 69);
+  const float rem = *rem_low;
+  constexpr int NW = NTHREADS / 32;
+  const int lane = threadIdx.x & 31;
+  float A = lane < NW ? shT[lane] : 0.0f, B = lane < NW ? shT[32 + lane] : 0.0f;
+#pragma unroll
+  for (int o = NW / 2; o > 0; o >>= 1) {
+    A = fmaxf(A, __shfl_xor_sync(0xffffffffu, A, o));
+    B = fmaxf(B, __shfl_xor_sync(0xffffffffu, B, o));
+  }
+  A = __shfl_sync(0xffffffffu, A, 0);
+  B = __shfl_sync(0xffffffffu, B, 0);
+  const float q = (float)cfl / (A + B);
+  if (!any_bad && q > 0.0f && 1.001f * q * (float)I.h < rem) {  // (false for NaN)
+    th = q;
+    if (keeps_time<NTHREADS>()) {
+      I.t += (double)q * I.h;
+      I.steps += 1;
+      // (read after the next barrier; this step's reads of it lie before the Eulerian
+      // stage's barrier, so it is written behind that one by the caller)
+    }
+    return true;
+  }
+  __syncthreads();  // every thread has read the bound and the maxima
+  if (keeps_time<NTHREADS>()) cfl_decide<float>(A, B, any_bad, cfl, I, sh);
+  __syncthreads();
+  th = *reinterpret_cast<const float*>(sh + 66);
+  return *reinterpret_cast<const int*>(sh + 68) != 0;
+}
+template <int NTHREADS>
+__device__ __forceinline__ void publish_remaining(const InstDev& I, double* sh) {
+  if (keeps_time<NTHREADS>())
+    *reinterpret_cast<float*>(sh + 69) = __double2float_rd(I.t_end - I.t);
+}
+
 // Vacuum threshold of every instance (Sec. 1.4: a fraction of the mean density; the
 // fraction is stored negated until this kernel has run): the instance's mean initial
 // density from a fixed 256-thread reduction, so the threshold does not depend on the CTA
@@ -370,6 +434,190 @@ __device__ __forceinline__ bool pair_cfl_step(T a, T b, bool bad, double cfl, In
   dt = sh[64];
   th = *reinterpret_cast<const T*>(sh + 66);
   return *reinterpret_cast<const int*>(sh + 68) != 0;
+}
+
+// One CTA's part of a plain FP32 instance advanced for up to max_steps steps (as
+// advance_part, below).  A thread owns a run of consecutive cells and streams them twice per
+// step on packed line pairs: the Eulerian stage with (v, p), finishing each cell as its right
+// face arrives, then the Lagrangian stage with (rho, m) and (rho E, rho eps), the energy
+// consistency and the next step's CFL maxima.  The stages write other arrays than they read
+// (state -> U* -> state; rho alternates), so nothing but one barrier stands between them and
+// no face values go through shared memory; the face between two runs is formed by both of
+// its threads from the same values.  Per step: one CTA barrier and the CFL reduction's (five
+// with face arrays and separate update passes; 512 instances of 128..4096 cells, 128 steps:
+// 4.43 ms then).
+// Shared memory: eight arrays of `stride` floats, cells at index G + c.
+template <int NTHREADS, bool PAIR>
+__device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, float* __restrict__ g_m,
+                                                 float* __restrict__ g_en, float* __restrict__ g_ei,
+                                                 InstDev& I, const Part P, float* smem, int stride,
+                                                 double gamma_d, double cfl, int max_steps,
+                                                 double* red, float* xslot) {
+  constexpr int G = PAIR ? kPairHalo : kBatchGhost;
+  const int nl = P.nl, tid = threadIdx.x;
+  float* R = smem + G;  // rho of the state; the next state's goes to Rn
+  float* Rn = R + stride;
+  float* const M = Rn + stride;
+  float* const E = M + stride;
+  float* const Ei = E + stride;
+  float* const Ms = Ei + stride;  // U*
+  float* const Es = Ms + stride;
+  float* const Is = Es + stride;
+  const float gamma = (float)gamma_d, gm1 = (float)(gamma_d - 1.0);
+  const float rho_vac_up = __double2float_ru(I.rho_vac);  // set by batch_vacuum_kernel
+  // odd runs: the runs of a warp's lanes start on 32 different banks.  As many threads as
+  // there are cells: the start-up of six cells is repeated more often by short runs, but the
+  // step is bound by its latency (256 cells, 128 steps: runs of one cell 304 us, of three 376,
+  // of five 480; 512 instances: 3.31, 3.31 and 3.37 ms)
+  const int run_e = ((P.cb - P.ca + NTHREADS - 1) / NTHREADS) | 1;
+  const int run = ((nl + NTHREADS - 1) / NTHREADS) | 1;
+  // a value of cell c with the outflow ghosts that repeat it at the instance's ends
+  auto put = [&](float* q, int c, float v) {
+    q[c] = v;
+    if (P.gl && c == 0) q[-1] = q[-2] = q[-3] = v;
+    if (P.gr && c == nl - 1) q[nl] = q[nl + 1] = q[nl + 2] = v;
+  };
+  float vm = 0.0f, cm = 0.0f;
+  bool bad = false;
+  auto cfl_cell = [&](float r, float m, float en, float ei) {
+    const bool ok = r > 0.0f && ei > 0.0f && isfinite(r) && isfinite(m) && isfinite(en) &&
+                    isfinite(ei);
+    bad = bad || !ok;
+    const float ir = rcp_approx(r);
+    vm = fmaxf(vm, fabsf(m * ir));
+    cm = fmaxf(cm, sqrt_approx(gamma * (gm1 * ei) * ir));
+  };
+  const long long off = I.off + P.lo;
+  for (int c = tid; c < nl; c += NTHREADS) {
+    const float r = g_rho[off + c], m = g_m[off + c], en = g_en[off + c], ei = g_ei[off + c];
+    put(R, c, r);
+    put(M, c, m);
+    put(E, c, en);
+    put(Ei, c, ei);
+    cfl_cell(r, m, en, ei);
+  }
+  if constexpr (PAIR) {  // the initial halo: the partner's first cells, from the state
+    const int h0 = P.gl ? nl : -kPairHalo;  // local index of the halo's first cell
+    if (tid < kPairHalo) {
+      const long long gi = off + h0 + tid;
+      R[h0 + tid] = g_rho[gi];
+      M[h0 + tid] = g_m[gi];
+      E[h0 + tid] = g_en[gi];
+      Ei[h0 + tid] = g_ei[gi];
+    }
+  }
+  if constexpr (!PAIR) publish_remaining<NTHREADS>(I, red);  // (the CFL step's barrier follows)
+  for (int s = 0; s < max_steps; s++) {
+    float th;
+    bool go;
+    if constexpr (PAIR) {
+      double dt;
+      float* const fields[4] = {R - G, M - G, E - G, Ei - G};
+      go = pair_cfl_step<float, 4>(vm, cm, bad, cfl, I, red, xslot, s & 1, P, fields, dt, th);
+    } else {
+      go = block_cfl_step_f32<NTHREADS>(vm, cm, bad, cfl, I, red, th);
+    }
+    if (!go) break;
+    // Eulerian stage of the cells ca .. cb-1
+    for (int c0 = P.ca + tid * run_e; c0 < P.cb; c0 += NTHREADS * run_e) {
+      const int c1 = min(c0 + run_e, P.cb);  // faces c0 .. c1
+      auto vp = [&](int k) { return make_float2(M[k] * rcp_approx(R[k]), gm1 * Ei[k]); };
+      LinePair<false> ln;
+      ln.start(vp(c0 - 3), vp(c0 - 2), vp(c0 - 1));
+      ln.push(vp(c0));
+      ln.push(vp(c0 + 1));
+      FaceCell left{ln.q2, ln.Pl, ln.Pr};
+      face_roots(left, R[c0 - 1]);
+      float Vp = 0.0f, Pp = 0.0f;
+#pragma unroll 2
+      for (int f = c0; f <= c1; f++) {
+        ln.push(vp(f + 2));
+        FaceCell right{ln.q2, ln.Pl, ln.Pr};  // cell f
+        face_roots(right, R[f]);
+        float V, Pf;
+        acoustic_face(left, right, gamma, th, V, Pf);
+        if (f > c0) {
+          const int c = f - 1;
+          const float ei = Ei[c];
+          put(Ms, c, M[c] - th * (Pf - Pp));
+          put(Es, c, E[c] - th * (Pf * V - Pp * Vp));
+          put(Is, c, ei - gm1 * ei * (th * (V - Vp)));
+        }
+        Vp = V;
+        Pp = Pf;
+        left = right;
+      }
+    }
+    __syncthreads();
+    if constexpr (!PAIR) publish_remaining<NTHREADS>(I, red);
+    // Lagrangian stage of the own cells, Sec. 1.4 and the next step's CFL maxima
+    vm = 0.0f;
+    cm = 0.0f;
+    for (int c0 = tid * run; c0 < nl; c0 += NTHREADS * run) {
+      const int c1 = min(c0 + run, nl);  // faces c0 .. c1
+      auto rm = [&](int k) { return make_float2(R[k], Ms[k]); };
+      auto ee = [&](int k) { return make_float2(Es[k], Is[k]); };
+      LinePair<false> la, lb;
+      la.start(rm(c0 - 3), rm(c0 - 2), rm(c0 - 1));
+      lb.start(ee(c0 - 3), ee(c0 - 2), ee(c0 - 1));
+      la.push(rm(c0));
+      lb.push(ee(c0));
+      la.push(rm(c0 + 1));
+      lb.push(ee(c0 + 1));
+      // cell f-1: values, deviations, sqrt(rho), v sqrt(rho)
+      float2 qa = la.q2, La = la.Pl, Ra = la.Pr, qb = lb.q2, Lb = lb.Pl, Rb = lb.Pr;
+      float sl = sqrt_approx(qa.x), wl = qa.y * rcp_approx(qa.x) * sl;
+      float2 Fa = both(0.0f), Fb = both(0.0f);
+#pragma unroll 2
+      for (int f = c0; f <= c1; f++) {
+        la.push(rm(f + 2));
+        lb.push(ee(f + 2));
+        // v^ (Sec. 1.3: in 1D the template is the cell's own v), as the Courant velocity
+        const float sr = sqrt_approx(la.q2.x), wr = la.q2.y * rcp_approx(la.q2.x) * sr;
+        const float w = (wr + wl) * rcp_approx(sr + sl) * th;
+        const DevWeights k = dev_weights(fabsf(w));
+        const float2 Ga = upwind_flux_pair(w, k, qa, La, Ra, la.q2, la.Pl, la.Pr);
+        const float2 Gb = upwind_flux_pair(w, k, qb, Lb, Rb, lb.q2, lb.Pl, lb.Pr);
+        if (f > c0) {
+          const int c = f - 1;
+          const float2 na = sub2(qa, sub2(Ga, Fa)), nb = sub2(qb, sub2(Gb, Fb));
+          float u[6] = {na.x, na.y, 0.0f, 0.0f, nb.x, nb.y};
+          const bool vac = vacuum_cell_f32(u, rho_vac_up);
+          const float e = dense_eps_f32(u);
+          if (vac)
+            vacuum_correct_f32(u, I.rho_vac);
+          else
+            u[5] = e;
+          put(Rn, c, u[0]);
+          put(M, c, u[1]);
+          put(E, c, u[4]);
+          put(Ei, c, u[5]);
+          cfl_cell(u[0], u[1], u[4], u[5]);
+        }
+        Fa = Ga;
+        Fb = Gb;
+        qa = la.q2;
+        La = la.Pl;
+        Ra = la.Pr;
+        qb = lb.q2;
+        Lb = lb.Pl;
+        Rb = lb.Pr;
+        sl = sr;
+        wl = wr;
+      }
+    }
+    float* const t = R;
+    R = Rn;
+    Rn = t;
+  }
+  if constexpr (PAIR) cluster_sync();  // the partner may still read this CTA's slot
+  __syncthreads();
+  for (int c = tid; c < nl; c += NTHREADS) {
+    g_rho[off + c] = R[c];
+    g_m[off + c] = M[c];
+    g_en[off + c] = E[c];
+    g_ei[off + c] = Ei[c];
+  }
 }
 
 // One CTA's part of an instance advanced for up to max_steps steps (Sec. 1 in 1D).  PAIR:
@@ -774,7 +1022,7 @@ struct BatchLo {
 };
 
 template <typename T, int NTHREADS, bool DF>
-__global__ void __launch_bounds__(NTHREADS, 1) batch_kernel(T* __restrict__ g_rho,
+__global__ void __launch_bounds__(NTHREADS, kBatchCtas<T, NTHREADS>) batch_kernel(T* __restrict__ g_rho,
                                                               T* __restrict__ g_m,
                                                               T* __restrict__ g_en,
                                                               T* __restrict__ g_ei, BatchLo<T> lo,
@@ -783,15 +1031,20 @@ __global__ void __launch_bounds__(NTHREADS, 1) batch_kernel(T* __restrict__ g_rh
                                                               double gamma_d, double cfl,
                                                               int max_steps, int nmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[80];
+  __shared__ double red[kBatchRed];
   const int id = order[blockIdx.x];
   InstDev I = inst[id];
   if (I.done) return;
   const Part P{I.n, 0, 0, I.n, 0, I.n, true, true};
-  advance_part<T, NTHREADS, false, DF>(g_rho, g_m, g_en, g_ei, lo.p, I, P, (T*)smem_raw,
-                                       nmax + 2 * kBatchGhost, nmax + 1, gamma_d, cfl, max_steps,
-                                       red, nullptr);
-  if (threadIdx.x == 0) {  // thread 0's copy holds the instance's time
+  if constexpr (sizeof(T) == 4 && !DF)
+    advance_part_f32<NTHREADS, false>(g_rho, g_m, g_en, g_ei, I, P, (T*)smem_raw,
+                                      nmax + 2 * kBatchGhost, gamma_d, cfl, max_steps, red, nullptr);
+  else
+    advance_part<T, NTHREADS, false, DF>(g_rho, g_m, g_en, g_ei, lo.p, I, P, (T*)smem_raw,
+                                         nmax + 2 * kBatchGhost, nmax + 1, gamma_d, cfl, max_steps,
+                                         red, nullptr);
+  // the time keeper's copy holds the instance's time
+  if (sizeof(T) == 4 && !DF ? keeps_time<NTHREADS>() : threadIdx.x == 0) {
     if (I.t >= I.t_end) I.done = 1;
     inst[id] = I;
   }
@@ -812,13 +1065,13 @@ constexpr int kItemSplit = -2;
 // decisions, so they meet the same cluster barriers; the CTAs of a two-instance item
 // never wait on each other.  A split instance needs n >= 2 kPairHalo.
 template <typename T, int NTHREADS, bool DF>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, kBatchCtas<T, NTHREADS>)
     batch_cluster_kernel(T* __restrict__ g_rho, T* __restrict__ g_m, T* __restrict__ g_en,
                          T* __restrict__ g_ei, BatchLo<T> lo, InstDev* __restrict__ inst,
                          const int2* __restrict__ items, double gamma_d, double cfl,
                          int max_steps, int nlmax, int nmax) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  __shared__ double red[80];
+  __shared__ double red[kBatchRed];
   __shared__ T xslot[2][kPairSlot];
   T* const* g_lo = lo.p;
   const int rank = (int)cluster_rank();
@@ -830,9 +1083,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     const int n = I.n, n0 = n / 2;
     const Part P = rank == 0 ? Part{n0, 0, 0, n0 + 3, 0, n0 + 3, true, false}
                              : Part{n - n0, n0, -3, n - n0, -3, n - n0, false, true};
-    advance_part<T, NTHREADS, true, DF>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
-                                    nlmax + 2 * kPairHalo, nlmax + 8, gamma_d, cfl, max_steps,
-                                    red, &xslot[0][0]);
+    if constexpr (sizeof(T) == 4 && !DF)
+      advance_part_f32<NTHREADS, true>(g_rho, g_m, g_en, g_ei, I, P, (T*)smem_raw,
+                                       nlmax + 2 * kPairHalo, gamma_d, cfl, max_steps, red,
+                                       &xslot[0][0]);
+    else
+      advance_part<T, NTHREADS, true, DF>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
+                                          nlmax + 2 * kPairHalo, nlmax + 8, gamma_d, cfl, max_steps,
+                                          red, &xslot[0][0]);
     if (rank == 0 && threadIdx.x == 0) {  // both CTAs hold the same time; rank 0 stores it
       if (I.t >= I.t_end) I.done = 1;
       inst[id] = I;
@@ -843,10 +1101,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, 1)
     InstDev I = inst[id];
     if (I.done) return;
     const Part P{I.n, 0, 0, I.n, 0, I.n, true, true};
-    advance_part<T, NTHREADS, false, DF>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
-                                     nmax + 2 * kBatchGhost, nmax + 1, gamma_d, cfl, max_steps,
-                                     red, nullptr);
-    if (threadIdx.x == 0) {
+    if constexpr (sizeof(T) == 4 && !DF)
+      advance_part_f32<NTHREADS, false>(g_rho, g_m, g_en, g_ei, I, P, (T*)smem_raw,
+                                        nmax + 2 * kBatchGhost, gamma_d, cfl, max_steps, red, nullptr);
+    else
+      advance_part<T, NTHREADS, false, DF>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
+                                           nmax + 2 * kBatchGhost, nmax + 1, gamma_d, cfl, max_steps,
+                                           red, nullptr);
+    if (sizeof(T) == 4 && !DF ? keeps_time<NTHREADS>() : threadIdx.x == 0) {
       if (I.t >= I.t_end) I.done = 1;
       inst[id] = I;
     }

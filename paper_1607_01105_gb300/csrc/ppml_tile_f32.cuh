@@ -18,6 +18,7 @@
 // no staging phase is left: the z sweep reads its columns from global memory itself, a few
 // positions ahead, and leaves them in shared memory for the x and y sweeps.
 #pragma once
+#include "ppml_pair.cuh"
 #include "ppml_tile.cuh"
 
 namespace ppml {
@@ -173,81 +174,6 @@ __global__ void __launch_bounds__(FV_THREADS, 4) face_velocity_f32(MarchArgs<flo
 }
 
 // ----------------------------------------------------------------------------- the sweeps
-
-// Two fields at once: packed additions, multiplications and FMAs (one issue slot for two).
-__device__ __forceinline__ unsigned long long as_u64(float2 v) {
-  return *reinterpret_cast<unsigned long long*>(&v);
-}
-__device__ __forceinline__ float2 as_f2(unsigned long long v) {
-  return *reinterpret_cast<float2*>(&v);
-}
-__device__ __forceinline__ float2 add2(float2 a, float2 b) {
-  unsigned long long r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
-  return as_f2(r);
-}
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
-  unsigned long long r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)));
-  return as_f2(r);
-}
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(as_u64(a)), "l"(as_u64(b)), "l"(as_u64(c)));
-  return as_f2(r);
-}
-__device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
-__device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.0f), a); }
-
-// LineF32 for two fields.
-template <bool FLAT>
-struct LinePair {
-  float2 q2, q1, qn, d, s, l2;
-  float2 Pl, Pr;  // doubled deviations of cell p - 2
-  static __device__ __forceinline__ float2 half_slope(float2 l, float2 r) {
-    const float2 c = mul2(add2(l, r), both(0.25f));
-    return make_float2(min_xs(c.x, fmaxf(min_xs(l.x, r.x), 0.0f)),
-                       min_xs(c.y, fmaxf(min_xs(l.y, r.y), 0.0f)));
-  }
-  __device__ __forceinline__ void start(float2 a, float2 b, float2 c) {
-    q2 = a;
-    q1 = b;
-    qn = c;
-    Pl = Pr = l2 = both(0.0f);
-    d = sub2(c, b);
-    s = half_slope(sub2(b, a), d);
-  }
-  __device__ __forceinline__ void push(float2 q) {
-    if constexpr (!FLAT) {
-      const float2 dn = sub2(q, qn);
-      const float2 sn = half_slope(d, dn);
-      const float2 e = sub2(sn, s);
-      const float2 r2 = fma2(e, both(-2.0f / 3.0f), d);
-      const float2 t = make_float2(max_nan(min_xs_nan(l2.x, r2.x), 0.0f),
-                                   max_nan(min_xs_nan(l2.y, r2.y), 0.0f));
-      const float2 m = add2(t, t);
-      Pl = make_float2(min_xs_nan(l2.x, m.x), min_xs_nan(l2.y, m.y));
-      Pr = make_float2(min_xs_nan(r2.x, m.x), min_xs_nan(r2.y, m.y));
-      l2 = fma2(e, both(2.0f / 3.0f), d);
-      d = dn;
-      s = sn;
-    }
-    q2 = q1;
-    q1 = qn;
-    qn = q;
-  }
-};
-
-// upwind_flux_f32 for two fields.
-__device__ __forceinline__ float2 upwind_flux_pair(float w, float2 ql, float2 Ll, float2 Lr,
-                                                   float2 qr, float2 Rl, float2 Rr) {
-  const DevWeights c = dev_weights(fabsf(w));
-  const bool left = w >= 0.0f;
-  const float2 q = make_float2(left ? ql.x : qr.x, left ? ql.y : qr.y);
-  const float2 x = make_float2(left ? Lr.x : -Rl.x, left ? Lr.y : -Rl.y);
-  const float2 y = make_float2(left ? Ll.x : -Rr.x, left ? Ll.y : -Rr.y);
-  return mul2(both(w), fma2(both(c.a), x, fma2(both(c.b), y, q)));
-}
 
 // One line of two fields: q(p) for the positions -3..18 (called in order, each once), w(c) the
 // face velocities 0..16 (in order); emit(c, d, qc) for the cells c = 0..15 with
@@ -548,9 +474,8 @@ __device__ __forceinline__ void euler_line_pair(QF q, float gamma, float th, EF 
     q(1, v, rn);
     ln.push(v);
   }
-  // cell p-3 (the face's left cell): values, deviations, sqrt(rho), rho sqrt(rho), p sqrt(rho)
-  float2 ql = ln.q2, Ll = ln.Pl, Lr = ln.Pr;
-  float sl = sqrt_approx(r2), Al = r2 * sl, Bl = ql.y * sl;
+  FaceCell left{ln.q2, ln.Pl, ln.Pr};  // cell p-3, the face's left cell
+  face_roots(left, r2);
   r2 = r1;
   r1 = rn;
   float Vp = 0.0f, Pp = 0.0f;
@@ -558,21 +483,10 @@ __device__ __forceinline__ void euler_line_pair(QF q, float gamma, float th, EF 
     float2 v;
     q(p, v, rn);
     ln.push(v);
-    const float sc = sqrt_approx(r2), Ac = r2 * sc, Bc = ln.q2.y * sc;
-    const float A = Al + Ac, lam = sqrt_approx(gamma * (Bl + Bc) * rcp_approx(A));
-    const float Z = lam * A * rcp_approx(sl + sc);
-    const DevWeights w = dev_weights(lam * th);
-    const float2 right = fma2(both(w.a), Lr, fma2(both(w.b), Ll, ql));
-    const float2 left = fma2(both(-w.a), ln.Pl, fma2(both(-w.b), ln.Pr, ln.q2));
-    const float2 sum = add2(right, left), dif = sub2(right, left);
-    V = 0.5f * fmaf(dif.y, rcp_approx(Z), sum.x);
-    P = 0.5f * fmaf(dif.x, Z, sum.y);
-    ql = ln.q2;
-    Ll = ln.Pl;
-    Lr = ln.Pr;
-    sl = sc;
-    Al = Ac;
-    Bl = Bc;
+    FaceCell right{ln.q2, ln.Pl, ln.Pr};
+    face_roots(right, r2);
+    acoustic_face(left, right, gamma, th, V, P);
+    left = right;
     r2 = r1;
     r1 = rn;
   };
