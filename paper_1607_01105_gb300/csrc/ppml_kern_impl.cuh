@@ -3,6 +3,7 @@
 #include "../../include/ppml.h"
 #include "ppml_internal.h"
 #include "ppml_launch.h"
+#include "ppml_thin.cuh"
 
 namespace ppml {
 
@@ -47,10 +48,54 @@ cudaError_t set_stage_smem() {
   return e;
 }
 
+namespace {
+// Grids with one or two active axes, plain states (ppml_thin.cuh).
+template <bool FLAT, bool TWO>
+void launch_thin_eulerian(const MarchArgs<PPML_REAL>& A, cudaStream_t st) {
+  ThinGeom t;
+  const int n = thin_tiles<ThinShape<PPML_REAL, TWO>>(A.g, t);
+  thin_eulerian<PPML_REAL, FLAT, TWO><<<n, THIN_NT, 0, st>>>(A);
+}
+template <bool FLAT, bool TWO>
+void launch_thin_lagrangian(const MarchArgs<PPML_REAL>& A, cudaStream_t st) {
+  using S = ThinShape<PPML_REAL, TWO>;
+  ThinGeom t;
+  const int n = thin_tiles<S>(A.g, t);
+  thin_lagrangian<PPML_REAL, FLAT, TWO>
+      <<<n, THIN_NT, sizeof(ThinLagSmem<PPML_REAL, S>), st>>>(A);
+}
+template <bool FLAT, bool TWO>
+cudaError_t prepare_thin() {
+  return cudaFuncSetAttribute(thin_lagrangian<PPML_REAL, FLAT, TWO>,
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              (int)sizeof(ThinLagSmem<PPML_REAL, ThinShape<PPML_REAL, TWO>>));
+}
+bool launch_thin(const MarchArgs<PPML_REAL>& A, bool eulerian, cudaStream_t st) {
+  if (!thin_grid(A.g) || (eulerian && A.phi)) return false;
+  const bool flat = (A.flags & PPML_FIRST_ORDER) != 0, two = thin_axes(A.g).axB >= 0;
+  if (eulerian) {
+    if (flat)
+      two ? launch_thin_eulerian<true, true>(A, st) : launch_thin_eulerian<true, false>(A, st);
+    else
+      two ? launch_thin_eulerian<false, true>(A, st) : launch_thin_eulerian<false, false>(A, st);
+  } else {
+    if (flat)
+      two ? launch_thin_lagrangian<true, true>(A, st) : launch_thin_lagrangian<true, false>(A, st);
+    else
+      two ? launch_thin_lagrangian<false, true>(A, st) : launch_thin_lagrangian<false, false>(A, st);
+  }
+  return true;
+}
+}  // namespace
+
 template <>
 int prepare_kernels<PPML_REAL>() {
   cudaError_t e = set_stage_smem<false>();
   if (e == cudaSuccess) e = prepare_sweeps(PPML_REAL(0));
+  if (e == cudaSuccess) e = prepare_thin<false, false>();
+  if (e == cudaSuccess) e = prepare_thin<false, true>();
+  if (e == cudaSuccess) e = prepare_thin<true, false>();
+  if (e == cudaSuccess) e = prepare_thin<true, true>();
   if (e == cudaSuccess && kHasDF) e = set_stage_smem<kHasDF>();
   if (e != cudaSuccess) return ppml_fail(PPML_E_CUDA, "cudaFuncSetAttribute: %s", cudaGetErrorString(e));
   return PPML_OK;
@@ -61,6 +106,7 @@ int launch_eulerian<PPML_REAL>(const MarchArgs<PPML_REAL>& A, int nblk, cudaStre
   constexpr int MB = MinBlocks<PPML_REAL>::value;
   constexpr size_t SM = sizeof(EulTileSmem<PPML_REAL>);
   const bool df = kHasDF && A.outlo[1];
+  if (!df && launch_thin(A, true, st)) return ppml_check_launch("thin_eulerian");
   if (!df && launch_euler_sweeps(A, nblk, st)) return ppml_check_launch("eulerian_sweep_f32");
   if (A.any_inflow) {
     if (df)
@@ -80,6 +126,7 @@ int launch_lagrangian<PPML_REAL>(const MarchArgs<PPML_REAL>& A, int nblk, cudaSt
   constexpr int MB = MinBlocks<PPML_REAL>::value;
   constexpr size_t SM = sizeof(LagTileSmem<PPML_REAL>);
   const bool df = kHasDF && A.outlo[0];
+  if (!df && launch_thin(A, false, st)) return ppml_check_launch("thin_lagrangian");
   if (!df && launch_sweeps(A, nblk, st)) return ppml_check_launch("lagrangian_sweep_f32");
   if (A.any_inflow) {
     if (df)
