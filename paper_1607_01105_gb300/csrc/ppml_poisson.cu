@@ -27,7 +27,7 @@
 #include <vector>
 
 #include "../../include/ppml.h"
-#include "ppml_device.cuh"
+#include "ppml_pair.cuh"
 #include "ppml_internal.h"
 
 using namespace ppml;
@@ -329,6 +329,166 @@ __global__ void __launch_bounds__(kThreads) dst_unpack_kernel(const T* __restric
   }
 }
 
+// ---------------------------------------------------- dense sine transforms (FP32)
+// A type-I sine transform along one axis of N <= kDenseMax points as a matrix product.  The
+// symmetry sin(pi j (N - i) / (N + 1)) = -+ sin(pi j (i + 1) / (N + 1)) halves it: the odd
+// j take the sums w_i + w_{N-1-i}, the even j the differences.  A CTA holds 64 lines and the
+// matrix in shared memory; a warp forms 16 outputs of one parity for two columns per lane,
+// on packed FMAs, summing blocks of 16 terms before adding them up (the rounding error of a
+// fast transform).  128^3: 134 M FMAs a pass, 3.4 us at the FMA peak, beside 16.8 MB of
+// traffic; the odd extension, the real transform of 2 (N + 1) points and the unpacking took
+// about 100 us a pass (258 = 2 3 43 is a poor length).  N^2 work: beyond kDenseMax the
+// matrix does not fit and the transform of the extension is used.
+constexpr int kDenseMax = 256;
+constexpr int kDenseCols = 64;
+constexpr int kDenseOut = 16;
+
+// The matrix in the order the warps read it: chunks of 16 outputs (first those of odd j, then
+// of even j), each [term][16], zero beyond the last output.
+struct DenseDims {
+  int N, terms[2], outs[2], chunks[2];
+};
+__host__ __device__ inline DenseDims dense_dims(int N) {
+  DenseDims d;
+  d.N = N;
+  d.terms[0] = d.outs[0] = (N + 1) / 2;
+  d.terms[1] = d.outs[1] = N / 2;
+  for (int q = 0; q < 2; q++) d.chunks[q] = (d.outs[q] + kDenseOut - 1) / kDenseOut;
+  return d;
+}
+__host__ __device__ inline int dense_matrix(const DenseDims& d) {
+  return kDenseOut * (d.chunks[0] * d.terms[0] + d.chunks[1] * d.terms[1]);
+}
+size_t dense_smem(int N) {
+  return sizeof(float) * ((size_t)dense_matrix(dense_dims(N)) + (size_t)N * kDenseCols);
+}
+
+// The transform of the 64 lines in D (D[i][column]), in place; matrix in Sm.  Barriers around.
+__device__ __forceinline__ void dense_sine(float* D, const float* Sm, const DenseDims& d) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int N = d.N, h = d.terms[1];
+  // sums to the first half, differences to the mirrored places (the middle one stays)
+  for (int e = threadIdx.x; e < h * kDenseCols; e += kThreads) {
+    const int i = e / kDenseCols, c = e % kDenseCols;
+    const float x = D[i * kDenseCols + c], y = D[(N - 1 - i) * kDenseCols + c];
+    D[i * kDenseCols + c] = x + y;
+    D[(N - 1 - i) * kDenseCols + c] = x - y;
+  }
+  __syncthreads();
+  // each warp's outputs stay in registers until every warp has read D
+  constexpr int kMaxChunks = (kDenseMax / kDenseOut + kThreads / 32 - 1) / (kThreads / 32);
+  float2 out[kMaxChunks][kDenseOut / 2][2];
+  const int chunks = d.chunks[0] + d.chunks[1];
+#pragma unroll
+  for (int r = 0; r < kMaxChunks; r++) {
+    const int ch = warp + r * (kThreads / 32);
+#pragma unroll
+    for (int q = 0; q < kDenseOut / 2; q++) out[r][q][0] = out[r][q][1] = make_float2(0.0f, 0.0f);
+    if (ch >= chunks) continue;
+    const bool odd = ch < d.chunks[0];
+    const int terms = d.terms[odd ? 0 : 1];
+    const float* m = Sm + kDenseOut * (odd ? ch * d.terms[0]
+                                           : d.chunks[0] * d.terms[0] +
+                                                 (ch - d.chunks[0]) * d.terms[1]);
+    const float* x = D + (odd ? 0 : (N - 1) * kDenseCols) + lane;
+    const int step = odd ? kDenseCols : -kDenseCols;
+    for (int i0 = 0; i0 < terms; i0 += 16) {
+      float2 acc[kDenseOut / 2][2];
+#pragma unroll
+      for (int q = 0; q < kDenseOut / 2; q++) acc[q][0] = acc[q][1] = make_float2(0.0f, 0.0f);
+      const int i1 = min(i0 + 16, terms);
+#pragma unroll 4
+      for (int i = i0; i < i1; i++) {
+        const float2 a = both(x[i * step]), b = both(x[i * step + 32]);
+        const float4* row = reinterpret_cast<const float4*>(m + i * kDenseOut);
+#pragma unroll
+        for (int q = 0; q < kDenseOut / 4; q++) {
+          const float4 w = row[q];
+          const float2 w0 = make_float2(w.x, w.y), w1 = make_float2(w.z, w.w);
+          acc[2 * q][0] = fma2(w0, a, acc[2 * q][0]);
+          acc[2 * q][1] = fma2(w0, b, acc[2 * q][1]);
+          acc[2 * q + 1][0] = fma2(w1, a, acc[2 * q + 1][0]);
+          acc[2 * q + 1][1] = fma2(w1, b, acc[2 * q + 1][1]);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kDenseOut / 2; q++) {
+        out[r][q][0] = add2(out[r][q][0], acc[q][0]);
+        out[r][q][1] = add2(out[r][q][1], acc[q][1]);
+      }
+    }
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kMaxChunks; r++) {
+    const int ch = warp + r * (kThreads / 32);
+    if (ch >= chunks) continue;
+    const bool odd = ch < d.chunks[0];
+    const int o0 = kDenseOut * (odd ? ch : ch - d.chunks[0]), outs = d.outs[odd ? 0 : 1];
+#pragma unroll
+    for (int q = 0; q < kDenseOut; q++) {
+      if (o0 + q >= outs) break;
+      float* row = D + (2 * (o0 + q) + (odd ? 0 : 1)) * kDenseCols + lane;  // output j - 1
+      row[0] = q & 1 ? out[r][q / 2][0].y : out[r][q / 2][0].x;
+      row[32] = q & 1 ? out[r][q / 2][1].y : out[r][q / 2][1].x;
+    }
+  }
+  __syncthreads();
+}
+
+// The lines along `axis`, 64 per CTA, transformed in place.  tab non-NULL (axis 2 only): the
+// amplitudes are divided by the operator's eigenvalue (see dst_unpack_kernel) and transformed
+// back at once.
+__global__ void __launch_bounds__(kThreads, 2) dense_sine_kernel(float* __restrict__ w,
+                                                              const float* __restrict__ matrix,
+                                                              Dims D, int axis,
+                                                              const double* __restrict__ tab,
+                                                              double coef) {
+  extern __shared__ __align__(16) float dense_mem[];
+  const DenseDims d = dense_dims(D.n[axis]);
+  const int nm = dense_matrix(d), N = d.N;
+  float* const Sm = dense_mem;
+  float* const X = dense_mem + nm;
+  const long long lines = D.ncell / N, l0 = (long long)blockIdx.x * kDenseCols;
+  for (int e = threadIdx.x; e < nm / 4; e += kThreads)
+    reinterpret_cast<float4*>(Sm)[e] = reinterpret_cast<const float4*>(matrix)[e];
+  const int cols = (int)(lines - l0 < kDenseCols ? lines - l0 : kDenseCols);
+  // axis 0: a warp reads lines of consecutive values; else threads take consecutive lines
+  const long long stride = axis == 1 ? D.n[0] : D.nxy;
+  const int col = threadIdx.x % kDenseCols;
+  const long long line = l0 + col;
+  const long long base = axis == 1 ? line / D.n[0] * D.nxy + line % D.n[0] : line;
+  auto each = [&](auto op) {
+    if (axis == 0) {
+      for (int c = threadIdx.x / 32; c < kDenseCols; c += kThreads / 32)
+        for (int i = threadIdx.x & 31; i < N; i += 32)
+          op(i, c, (l0 + c) * N + i, c < cols);
+    } else {
+      for (int i = threadIdx.x / kDenseCols; i < N; i += kThreads / kDenseCols)
+        op(i, col, base + i * stride, col < cols);
+    }
+  };
+  each([&](int i, int c, long long o, bool ok) { X[i * kDenseCols + c] = ok ? w[o] : 0.0f; });
+  __syncthreads();
+  dense_sine(X, Sm, d);
+  if (tab) {
+    const FloatPair* const tx = reinterpret_cast<const FloatPair*>(tab);
+    const FloatPair* const ty = tx + D.n[0];
+    const FloatPair* const tz = ty + D.n[1];
+    const FloatPair cf = *reinterpret_cast<const FloatPair*>(&coef);
+    if (col < cols) {
+      const FloatPair txy = table_product(ty[line / D.n[0]], tx[line % D.n[0]]);
+      for (int i = threadIdx.x / kDenseCols; i < N; i += kThreads / kDenseCols)
+        X[i * kDenseCols + col] = scaled(X[i * kDenseCols + col], over_one_minus(cf, txy, tz[i]));
+    }
+    __syncthreads();
+    dense_sine(X, Sm, d);
+  }
+  each([&](int i, int c, long long o, bool ok) {
+    if (ok) w[o] = X[i * kDenseCols + c];
+  });
+}
+
 int blocks_for(long long n) {
   const long long b = (n + kThreads - 1) / kThreads;
   return (int)(b < 152LL * 16 ? (b > 0 ? b : 1) : 152LL * 16);
@@ -347,6 +507,7 @@ struct PoissonIso {
   double* mom;
   double* tab;
   double* shell;  // the potential on the cells around the grid
+  float* sine[3];  // FP32 grids of at most kDenseMax points per axis: the sine matrices
 };
 
 void ppml_iso_free(PoissonIso* s) {
@@ -358,6 +519,8 @@ void ppml_iso_free(PoissonIso* s) {
   if (s->mom) cudaFree(s->mom);
   if (s->tab) cudaFree(s->tab);
   if (s->shell) cudaFree(s->shell);
+  for (int a = 0; a < 3; a++)
+    if (s->sine[a]) cudaFree(s->sine[a]);
   delete s;
 }
 
@@ -378,8 +541,11 @@ static int iso_create(const ppml_grid_desc* d, PoissonIso** out) {
     if ((size_t)(2 * (N + 1) * B) > ext_n) ext_n = (size_t)(2 * (N + 1) * B);
     if ((size_t)((N + 2) * B) > spec_n) spec_n = (size_t)((N + 2) * B);
   }
-  if (cudaMalloc(&s->ext, ext_n * elt) != cudaSuccess ||
-      cudaMalloc(&s->spec, spec_n * 2 * elt) != cudaSuccess ||
+  bool dense = !f64;
+  for (int a = 0; a < 3; a++) dense = dense && s->n[a] <= kDenseMax;
+  if (dense) ext_n = spec_n = 0;
+  if ((ext_n && cudaMalloc(&s->ext, ext_n * elt) != cudaSuccess) ||
+      (spec_n && cudaMalloc(&s->spec, spec_n * 2 * elt) != cudaSuccess) ||
       cudaMalloc(&s->part, sizeof(double) * kMoments * kMaxMomentBlocks) != cudaSuccess ||
       cudaMalloc(&s->mom, sizeof(double) * kMoments) != cudaSuccess ||
       cudaMalloc(&s->tab, sizeof(double) * (size_t)(s->n[0] + s->n[1] + s->n[2])) != cudaSuccess ||
@@ -401,7 +567,34 @@ static int iso_create(const ppml_grid_desc* d, PoissonIso** out) {
     return ppml_fail(PPML_E_CUDA, "isolated Poisson tables: %s",
                      cudaGetErrorString(cudaGetLastError()));
   }
-  for (int a = 0; a < 3; a++) {
+  for (int a = 0; a < 3 && dense; a++) {
+    const DenseDims d = dense_dims(s->n[a]);
+    std::vector<float> m((size_t)dense_matrix(d), 0.0f);
+    float* at = m.data();
+    for (int q = 0; q < 2; q++)
+      for (int ch = 0; ch < d.chunks[q]; ch++)
+        for (int i = 0; i < d.terms[q]; i++)
+          for (int o = 0; o < kDenseOut; o++, at++) {
+            const int k = ch * kDenseOut + o;  // output of this parity: j = 2 k + 1 + q
+            if (k < d.outs[q])
+              *at = (float)sin(M_PI * (double)((long long)(2 * k + 1 + q) * (i + 1) % (2LL * (d.N + 1))) /
+                               (double)(d.N + 1));
+          }
+    if (cudaMalloc(&s->sine[a], sizeof(float) * m.size()) != cudaSuccess) {
+      cudaGetLastError();
+      ppml_iso_free(s);
+      return ppml_fail(PPML_E_NOMEM, "isolated Poisson sine matrix (%zu elements)", m.size());
+    }
+    cudaError_t e = cudaMemcpy(s->sine[a], m.data(), sizeof(float) * m.size(), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(dense_sine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               (int)dense_smem(kDenseMax));
+    if (e != cudaSuccess) {
+      ppml_iso_free(s);
+      return ppml_fail(PPML_E_CUDA, "isolated Poisson sine matrix: %s", cudaGetErrorString(e));
+    }
+  }
+  for (int a = 0; a < 3 && !dense; a++) {
     int M = 2 * (s->n[a] + 1);
     int inembed[1] = {M}, onembed[1] = {M / 2 + 1};
     const int B = (int)(ncell / s->n[a]);
@@ -438,6 +631,20 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   double scale = 1.0;
   for (int a = 0; a < 3; a++) scale *= 2.0 / (double)(D.n[a] + 1);
   const double symbol = ppml_table_value(-scale / 6.0, sizeof(T) == sizeof(double));
+  if constexpr (sizeof(T) == sizeof(float)) {
+    if (s->sine[0]) {  // x, y, then z there and back, y, x
+      const int order[5] = {0, 1, 2, 1, 0};
+      for (int q = 0; q < 5; q++) {
+        const int a = order[q];
+        const long long lines = D.ncell / D.n[a];
+        dense_sine_kernel<<<(int)((lines + kDenseCols - 1) / kDenseCols), kThreads,
+                            dense_smem(D.n[a]), st>>>(phi, s->sine[a], D, a,
+                                                      q == 2 ? s->tab : nullptr, symbol);
+        if ((rc = ppml_check_launch("dense_sine_kernel"))) return rc;
+      }
+      return PPML_OK;
+    }
+  }
   for (int pass = 0; pass < 2; pass++) {
     for (int a = 0; a < 3; a++) {
       const long long total = 2LL * (D.n[a] + 1) * (D.ncell / D.n[a]);
