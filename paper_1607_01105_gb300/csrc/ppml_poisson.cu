@@ -95,6 +95,66 @@ __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ 
   if (threadIdx.x < kMoments) part[(size_t)blockIdx.x * kMoments + threadIdx.x] = s[threadIdx.x][0];
 }
 
+// The same on FP32 grids of at most kPairMax cells per axis, in float pairs: the centres are
+// half integers times h, so x', y' and their products are exact floats there, each term is a
+// product with its exact error, and the sums are TwoSum pairs (about 2^-45, far below the
+// float potential).  Blocks take planes; z enters once per plane and lane, in double.
+constexpr int kPairMax = 2048;
+struct PairSum {
+  float hi, lo;
+  __device__ __forceinline__ void add(float m, float c) {  // += m c
+    const float p = m * c, e = fmaf(m, c, -p);
+    float s, t;
+    two_sum(hi, p, s, t);
+    hi = s;
+    lo += t + e;
+  }
+  __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+__global__ void __launch_bounds__(kThreads) moment_pair_kernel(const float* __restrict__ rho, Dims D,
+                                                               double h, double* __restrict__ part) {
+  double acc[kMoments] = {0, 0, 0, 0, 0, 0, 0};
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double vol = h * h * h;
+  for (int k = blockIdx.x; k < D.n[2]; k += gridDim.x) {
+    PairSum s[6] = {};  // m, m x, m y, m x x, m y y, m x y
+    for (int j = warp; j < D.n[1]; j += kThreads / 32) {
+      const float y = (float)j + 0.5f - 0.5f * (float)D.n[1];
+      const float* row = rho + (long long)k * D.nxy + (long long)j * D.n[0];
+      for (int i = lane; i < D.n[0]; i += 32) {
+        const float x = (float)i + 0.5f - 0.5f * (float)D.n[0], m = row[i];
+        s[0].add(m, 1.0f);
+        s[1].add(m, x);
+        s[2].add(m, y);
+        s[3].add(m, x * x);
+        s[4].add(m, y * y);
+        s[5].add(m, x * y);
+      }
+    }
+    const double z = centre(k, D.n[2], h), m0 = vol * s[0].value(), mx = vol * h * s[1].value(),
+                 my = vol * h * s[2].value(), mxx = vol * h * h * s[3].value(),
+                 myy = vol * h * h * s[4].value(), mxy = vol * h * h * s[5].value();
+    acc[0] += m0;
+    acc[1] += z * z * m0 + myy;
+    acc[2] += mxx + z * z * m0;
+    acc[3] += mxx + myy;
+    acc[4] += mxy;
+    acc[5] += z * mx;
+    acc[6] += z * my;
+  }
+  __shared__ double sh[kMoments][kThreads];
+#pragma unroll
+  for (int q = 0; q < kMoments; q++) sh[q][threadIdx.x] = acc[q];
+  __syncthreads();
+  for (int w = kThreads / 2; w > 0; w >>= 1) {
+    if ((int)threadIdx.x < w)
+#pragma unroll
+      for (int q = 0; q < kMoments; q++) sh[q][threadIdx.x] += sh[q][threadIdx.x + w];
+    __syncthreads();
+  }
+  if (threadIdx.x < kMoments) part[(size_t)blockIdx.x * kMoments + threadIdx.x] = sh[threadIdx.x][0];
+}
+
 // Stage 1b: one block folds the partials in a fixed order.
 __global__ void __launch_bounds__(kThreads) moment_final_kernel(const double* __restrict__ part,
                                                                 int nblk, double* __restrict__ mom) {
@@ -183,74 +243,117 @@ __device__ __forceinline__ void pair_add(SourcePair& s, float x) {
   s.hi = t;
 }
 
-// Right-hand side: 4 pi G h^2 (rho [+ D7 rho / 12]) minus the stencil weights times the
-// shell values next to boundary cells.  Written into the potential array (the work array).
-// One row of x per warp pass.
+// Right-hand side 4 pi G h^2 (rho [+ D7 rho / 12]) of the cells away from the boundary, written
+// into the potential array (the work array); boundary cells are left to rhs_edge_kernel.  One
+// row of x per warp pass.
 template <typename T>
 __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho, T* __restrict__ out,
-                                                       Dims D, double h, double G,
-                                                       const double* __restrict__ shell, int printed) {
+                                                       Dims D, double h, double G, int printed) {
   const double c = 4.0 * M_PI * G * h * h;
   const float ch = (float)c, cl = (float)(c - (double)ch);
   const float c12h = (float)(c / 12.0), c12l = (float)(c / 12.0 - (double)c12h);
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, nx = D.n[0];
   const long long rows = (long long)D.n[1] * D.n[2];
   const long long warps = (long long)gridDim.x * (kThreads / 32);
   for (long long row = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows;
        row += warps) {
     const int j = (int)(row % D.n[1]), k = (int)(row / D.n[1]);
-    const bool edge_row = j == 0 || k == 0 || j == D.n[1] - 1 || k == D.n[2] - 1;
-    for (int i = lane; i < D.n[0]; i += 32) {
-      const long long idx = row * D.n[0] + i;
-      const bool edge = edge_row || i == 0 || i == D.n[0] - 1;
+    if (j == 0 || k == 0 || j == D.n[1] - 1 || k == D.n[2] - 1) continue;
+    for (int i = 1 + lane; i < nx - 1; i += 32) {
+      const long long idx = row * nx + i;
       const T rc = rho[idx];
-      T nb[6];  // rho = 0 outside the grid
-      if (!printed) {
-        nb[0] = i > 0 ? rho[idx - 1] : T(0);
-        nb[1] = i < D.n[0] - 1 ? rho[idx + 1] : T(0);
-        nb[2] = j > 0 ? rho[idx - D.n[0]] : T(0);
-        nb[3] = j < D.n[1] - 1 ? rho[idx + D.n[0]] : T(0);
-        nb[4] = k > 0 ? rho[idx - D.nxy] : T(0);
-        nb[5] = k < D.n[2] - 1 ? rho[idx + D.nxy] : T(0);
-      }
-      double v;
-      if (sizeof(T) == 4 && !edge) {
-        // c (rho / 2 + sum / 12), the products to 2^-46
-        if (printed) {
-          out[idx] = fmaf((float)rc, ch, (float)rc * cl);
-          continue;
-        }
-        SourcePair s = {6.0f * (float)rc, 0.0f};
-        s.lo = fmaf(6.0f, (float)rc, -s.hi);
-#pragma unroll
-        for (int q = 0; q < 6; q++) pair_add(s, (float)nb[q]);
-        const float p = s.hi * c12h;
-        out[idx] = p + (fmaf(s.hi, c12h, -p) + fmaf(s.hi, c12l, s.lo * c12h));
+      if (printed) {
+        if constexpr (sizeof(T) == 4)
+          out[idx] = fmaf(rc, ch, rc * cl);
+        else
+          out[idx] = c * rc;
         continue;
       }
-      double src = (double)rc;
-      if (!printed) {
-        double lap = -6.0 * src;
+      const T nb[6] = {rho[idx - 1],  rho[idx + 1],     rho[idx - nx],
+                       rho[idx + nx], rho[idx - D.nxy], rho[idx + D.nxy]};
+      if constexpr (sizeof(T) == 4) {
+        // c / 12 (6 rho + sum), the products to 2^-46
+        SourcePair s = {6.0f * rc, 0.0f};
+        s.lo = fmaf(6.0f, rc, -s.hi);
 #pragma unroll
-        for (int q = 0; q < 6; q++) lap += (double)nb[q];
-        src = src + lap / 12.0;
+        for (int q = 0; q < 6; q++) pair_add(s, nb[q]);
+        const float p = s.hi * c12h;
+        out[idx] = p + (fmaf(s.hi, c12h, -p) + fmaf(s.hi, c12l, s.lo * c12h));
+      } else {
+        double lap = -6.0 * rc;
+#pragma unroll
+        for (int q = 0; q < 6; q++) lap += nb[q];
+        out[idx] = c * (rc + lap / 12.0);
       }
-      v = c * src;
-      if (edge) {
-        for (int dz = -1; dz <= 1; dz++)
-          for (int dy = -1; dy <= 1; dy++)
-            for (int dx = -1; dx <= 1; dx++) {
-              const int ii = i + dx, jj = j + dy, kk = k + dz;
-              const bool outside = ii < 0 || jj < 0 || kk < 0 || ii >= D.n[0] || jj >= D.n[1] ||
-                                   kk >= D.n[2];
-              if (!outside) continue;
-              const int nnz = (dx != 0) + (dy != 0) + (dz != 0);
-              const double w = nnz == 1 ? 4.0 / 9.0 : (nnz == 2 ? 1.0 / 9.0 : 1.0 / 36.0);
-              v -= w * shell[shell_at(D, ii, jj, kk)];
-            }
-      }
-      out[idx] = (T)v;
     }
+  }
+}
+
+// The cells of the grid's boundary, a thread each (inside the rows of rhs_kernel they would
+// hold up warps of interior cells): the source as above with rho = 0 outside, in FP64, minus
+// the stencil weights times the shell values next to the cell.
+__host__ __device__ __forceinline__ long long edge_cells(const Dims& D) {
+  const long long nx = D.n[0], ny = D.n[1], nz = D.n[2];
+  const long long in_x = nx > 2 ? nx - 2 : 0, in_y = ny > 2 ? ny - 2 : 0, in_z = nz > 2 ? nz - 2 : 0;
+  return nx * ny * nz - in_x * in_y * in_z;
+}
+template <typename T>
+__global__ void __launch_bounds__(kThreads) rhs_edge_kernel(const T* __restrict__ rho,
+                                                            T* __restrict__ out, Dims D, double h,
+                                                            double G,
+                                                            const double* __restrict__ shell,
+                                                            int printed) {
+  const double c = 4.0 * M_PI * G * h * h;
+  const int nx = D.n[0], ny = D.n[1], nz = D.n[2];
+  const long long n = edge_cells(D);
+  const long long planes = (long long)(nz > 1 ? 2 : 1) * D.nxy;  // whole boundary planes first
+  const int per_rows = (ny > 1 ? 2 : 1) * nx, per = per_rows + (ny > 2 ? ny - 2 : 0) * (nx > 1 ? 2 : 1);
+  for (long long q = (long long)blockIdx.x * kThreads + threadIdx.x; q < n;
+       q += (long long)gridDim.x * kThreads) {
+    int i, j, k;
+    if (q < planes) {
+      k = q < D.nxy ? 0 : nz - 1;
+      j = (int)(q % D.nxy) / nx;
+      i = (int)(q % D.nxy) % nx;
+    } else {
+      const long long r = q - planes;
+      k = 1 + (int)(r / per);
+      const int e = (int)(r % per);
+      if (e < per_rows) {
+        j = e < nx ? 0 : ny - 1;
+        i = e % nx;
+      } else {
+        const int d = e - per_rows;
+        i = d < ny - 2 ? 0 : nx - 1;
+        j = 1 + d % (ny - 2);
+      }
+    }
+    const long long idx = (long long)k * D.nxy + (long long)j * nx + i;
+    const double rc = (double)rho[idx];
+    double src = rc;
+    if (!printed) {
+      double lap = -6.0 * rc;
+      if (i > 0) lap += (double)rho[idx - 1];
+      if (i < nx - 1) lap += (double)rho[idx + 1];
+      if (j > 0) lap += (double)rho[idx - nx];
+      if (j < ny - 1) lap += (double)rho[idx + nx];
+      if (k > 0) lap += (double)rho[idx - D.nxy];
+      if (k < nz - 1) lap += (double)rho[idx + D.nxy];
+      src = rc + lap / 12.0;
+    }
+    double v = c * src;
+    for (int dz = -1; dz <= 1; dz++)
+      for (int dy = -1; dy <= 1; dy++) {
+        const bool out_yz = j + dy < 0 || j + dy >= ny || k + dz < 0 || k + dz >= nz;
+        for (int dx = -1; dx <= 1; dx++) {
+          const int ii = i + dx;
+          if (!out_yz && ii >= 0 && ii < nx) continue;
+          const int nnz = (dx != 0) + (dy != 0) + (dz != 0);
+          const double w = nnz == 1 ? 4.0 / 9.0 : (nnz == 2 ? 1.0 / 9.0 : 1.0 / 36.0);
+          v -= w * shell[shell_at(D, ii, j + dy, k + dz)];
+        }
+      }
+    out[idx] = (T)v;
   }
 }
 
@@ -619,14 +722,23 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   D.nxy = (long long)D.n[0] * D.n[1];
   D.ncell = D.nxy * D.n[2];
   const int nb = blocks_for(D.ncell) < kMaxMomentBlocks ? blocks_for(D.ncell) : kMaxMomentBlocks;
-  moment_kernel<T><<<nb, kThreads, 0, st>>>(rho, D, h, s->part);
+  int blocks = nb;
+  if (sizeof(T) == sizeof(float) && D.n[0] <= kPairMax && D.n[1] <= kPairMax) {
+    blocks = D.n[2] < kMaxMomentBlocks ? D.n[2] : kMaxMomentBlocks;
+    moment_pair_kernel<<<blocks, kThreads, 0, st>>>((const float*)rho, D, h, s->part);
+  } else {
+    moment_kernel<T><<<nb, kThreads, 0, st>>>(rho, D, h, s->part);
+  }
   int rc = ppml_check_launch("moment_kernel");
   if (rc) return rc;
-  moment_final_kernel<<<1, kThreads, 0, st>>>(s->part, nb, s->mom);
+  moment_final_kernel<<<1, kThreads, 0, st>>>(s->part, blocks, s->mom);
   if ((rc = ppml_check_launch("moment_final_kernel"))) return rc;
   shell_kernel<<<blocks_for(shell_cells(D)), kThreads, 0, st>>>(D, h, G, s->mom, s->shell);
   if ((rc = ppml_check_launch("shell_kernel"))) return rc;
-  rhs_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, h, G, s->shell, printed);
+  rhs_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, h, G, printed);
+  if ((rc = ppml_check_launch("rhs_kernel"))) return rc;
+  rhs_edge_kernel<T><<<blocks_for(edge_cells(D)), kThreads, 0, st>>>(rho, phi, D, h, G, s->shell,
+                                                                     printed);
   if ((rc = ppml_check_launch("rhs_kernel"))) return rc;
   double scale = 1.0;
   for (int a = 0; a < 3; a++) scale *= 2.0 / (double)(D.n[a] + 1);
