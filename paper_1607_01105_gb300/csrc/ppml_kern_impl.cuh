@@ -54,21 +54,30 @@ template <bool FLAT, bool TWO>
 void launch_thin_eulerian(const MarchArgs<PPML_REAL>& A, cudaStream_t st) {
   ThinGeom t;
   const int n = thin_tiles<ThinShape<PPML_REAL, TWO>>(A.g, t);
-  thin_eulerian<PPML_REAL, FLAT, TWO><<<n, THIN_NT, 0, st>>>(A);
+  if constexpr (sizeof(PPML_REAL) == 8 && !TWO)
+    thin1d_eulerian_f64<FLAT><<<n, THIN_NT, 0, st>>>(A);
+  else
+    thin_eulerian<PPML_REAL, FLAT, TWO><<<n, THIN_NT, 0, st>>>(A);
 }
 template <bool FLAT, bool TWO>
 void launch_thin_lagrangian(const MarchArgs<PPML_REAL>& A, cudaStream_t st) {
   using S = ThinShape<PPML_REAL, TWO>;
   ThinGeom t;
   const int n = thin_tiles<S>(A.g, t);
-  thin_lagrangian<PPML_REAL, FLAT, TWO>
-      <<<n, THIN_NT, sizeof(ThinLagSmem<PPML_REAL, S>), st>>>(A);
+  if constexpr (sizeof(PPML_REAL) == 8 && !TWO)
+    thin1d_lagrangian_f64<FLAT><<<n, THIN_NT, 0, st>>>(A);
+  else
+    thin_lagrangian<PPML_REAL, FLAT, TWO>
+        <<<n, THIN_NT, sizeof(ThinLagSmem<PPML_REAL, S>), st>>>(A);
 }
 template <bool FLAT, bool TWO>
 cudaError_t prepare_thin() {
-  return cudaFuncSetAttribute(thin_lagrangian<PPML_REAL, FLAT, TWO>,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              (int)sizeof(ThinLagSmem<PPML_REAL, ThinShape<PPML_REAL, TWO>>));
+  if constexpr (sizeof(PPML_REAL) == 8 && !TWO)
+    return cudaSuccess;
+  else
+    return cudaFuncSetAttribute(thin_lagrangian<PPML_REAL, FLAT, TWO>,
+                                cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)sizeof(ThinLagSmem<PPML_REAL, ThinShape<PPML_REAL, TWO>>));
 }
 bool launch_thin(const MarchArgs<PPML_REAL>& A, bool eulerian, cudaStream_t st) {
   if (!thin_grid(A.g) || (eulerian && A.phi)) return false;

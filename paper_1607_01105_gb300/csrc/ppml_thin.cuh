@@ -532,4 +532,240 @@ __global__ void __launch_bounds__(THIN_NT) thin_lagrangian(MarchArgs<T> A) {
   finalize_last(A.partials, tiles, A.fin, stc[0]);
 }
 
+// ------------------------------------------------- FP64 grids with one active axis
+// One FP64 instruction of a lone warp takes 76 cycles, so even one cell's chain through a
+// line segment (seven positions of start-up for two quantities, two faces of 75 instructions)
+// is 25 us.  Here every quantity of the stage has its own pass over the CTA's 32 cells and
+// their ghosts, spread over (quantity, cell): the chain is one slope, one face, one parabola,
+// one face solve and one update (256 cells: 61 us a step with segments of one cell).
+
+struct Thin1dEuler {
+  static constexpr int L = 32, W = L + 2 * TH;  // positions -3 .. L+2 at index p + 3
+  double r[W], m[W], ei[W];
+  double q[2][W];             // v, p
+  RootWeights w[W];           // of the cells -1 .. L
+  double s[2][W], f[2][W];    // slopes; face p: between p-1 and p
+  double PL[2][W], PR[2][W], D[2][W], S[2][W];
+  double V[W], P[W];          // faces 0 .. L
+};
+
+template <bool FLAT>
+__global__ void __launch_bounds__(THIN_NT) thin1d_eulerian_f64(MarchArgs<double> A) {
+  using E = Thin1dEuler;
+  using S1 = ThinShape<double, false>;
+  static_assert(E::L == S1::LA, "cells of a CTA");
+  __shared__ E M;
+  __shared__ ThinMaps maps;
+  __shared__ f64::Divisor hdiv[3];
+  const GridGeom& g = A.g;
+  ThinGeom t;
+  thin_tiles<S1>(g, t);
+  t.a0 = (int)blockIdx.x * E::L;
+  build_thin_maps<S1>(maps, g, t);
+  if (threadIdx.x < 3) hdiv[threadIdx.x] = f64::divisor(A.h[threadIdx.x]);
+  double stc[4];
+  cta_step_constants(A.dt_dev, A.dt_host, A.h, stc);  // (a barrier)
+  const double gamma = A.gamma, gm1 = A.gamma - 1.0;
+  const int ax = t.axA, tid = threadIdx.x;
+  const AxisStep<double> ks(stc[0], hdiv[ax], stc[1 + ax]);
+  load_box<double, S1>(M.r, A, 0, t, maps);
+  load_box<double, S1>(M.m, A, 1 + ax, t, maps);
+  load_box<double, S1>(M.ei, A, 5, t, maps);
+  __syncthreads();
+  // v, p, root weights: 64 tasks per quantity, one warp pair each
+  const int job = tid / 64, c = tid % 64;
+  if (c < E::W) {
+    if (job == 0) M.q[0][c] = f64::over(M.m[c], M.r[c]);
+    if (job == 1) M.q[1][c] = f64::plain_mul(gm1, M.ei[c]);
+    if (job == 2 && c >= 2 && c < E::W - 2)
+      M.w[c] = root_weights(M.r[c], f64::plain_mul(gm1, M.ei[c]));
+  }
+  __syncthreads();
+  if (job < 2) {
+    double* const q = M.q[job];
+    // slopes of the cells -2 .. L+1
+    if (c >= 1 && c < E::W - 1)
+      M.s[job][c] = FLAT ? 0.0
+                         : f64::slope(f64::diff(q[c], q[c - 1]), f64::diff(q[c + 1], q[c]), q[c - 1],
+                                      q[c + 1]);
+  }
+  __syncthreads();
+  if (job < 2 && c >= 2 && c < E::W - 1)  // faces -1 .. L+1
+    M.f[job][c] = f64::face(M.q[job][c - 1], M.q[job][c], M.s[job][c - 1], M.s[job][c]);
+  __syncthreads();
+  if (job < 2 && c >= 2 && c < E::W - 2) {  // cells -1 .. L
+    const double q0 = M.q[job][c];
+    double Lf = M.f[job][c], Rf = M.f[job][c + 1], D = 0.0, S = 0.0;
+    if (FLAT)
+      Lf = Rf = q0;
+    else
+      f64::parabola(q0, Lf, Rf, D, S);
+    M.PL[job][c] = Lf;
+    M.PR[job][c] = Rf;
+    M.D[job][c] = D;
+    M.S[job][c] = S;
+  }
+  __syncthreads();
+  if (job == 0 && c >= TH && c <= TH + E::L) {  // face c - 3, between cells c-1 and c
+    double lam, Z;
+    face_constants(M.w[c - 1], M.w[c], gamma, lam, Z);
+    const f64::Weights k = f64::weights(courant(lam, ks));
+    riemann_vp(f64::average(true, M.PR[0][c - 1], M.D[0][c - 1], M.S[0][c - 1], k),
+               f64::average(false, M.PL[0][c], M.D[0][c], M.S[0][c], k),
+               f64::average(true, M.PR[1][c - 1], M.D[1][c - 1], M.S[1][c - 1], k),
+               f64::average(false, M.PL[1][c], M.D[1][c], M.S[1][c], k), Z, M.V[c], M.P[c]);
+  }
+  __syncthreads();
+  // updates: a thread per field and cell; cell i at index b
+  const int i = c, b = c + TH;
+  if (i < E::L && t.a0 + i < g.n[ax]) {
+    const long long o = t.a0 + i;  // (the only active axis: contiguous)
+    const double Vm = M.V[b], Vp = M.V[b + 1], Pm = M.P[b], Pp = M.P[b + 1];
+    if (job == 0) {
+#pragma unroll
+      for (int q = 0; q < 3; q++)
+        A.out[1 + q][o] = q == ax ? f64::minus(M.m[b], f64::times(ks.th, f64::diff(Pp, Pm)))
+                                  : A.u[1 + q][o];
+    } else if (job == 1) {
+      const double d = f64::diff(f64::times(Pp, Vp), f64::times(Pm, Vm));
+      A.out[4][o] = f64::minus(A.u[4][o], f64::times(ks.th, d));
+    } else if (job == 2) {
+      A.out[5][o] = eps_update(M.ei[b], gm1, f64::times(ks.th, f64::diff(Vp, Vm)));
+      if (A.out[0]) A.out[0][o] = M.r[b];
+    }
+  }
+}
+
+struct Thin1dLag {
+  static constexpr int L = 32, W = L + 2 * TH;
+  double u[6][W + 1];
+  double pr[W], sq[W];        // v sqrt(rho), sqrt(rho) of the cells -1 .. L
+  double v[W];                // v^ of the faces 0 .. L
+  f64::Weights k[W];
+  double s[6][W], f[6][W], PL[6][W], PR[6][W], D[6][W], S[6][W];
+  double F[6][W];
+  double n[6][L];             // the updated cells
+};
+
+template <bool FLAT>
+__global__ void __launch_bounds__(THIN_NT) thin1d_lagrangian_f64(MarchArgs<double> A) {
+  using E = Thin1dLag;
+  using S1 = ThinShape<double, false>;
+  __shared__ E M;
+  __shared__ ThinMaps maps;
+  __shared__ f64::Divisor hdiv[3];
+  const GridGeom& g = A.g;
+  ThinGeom t;
+  const int tiles = thin_tiles<S1>(g, t);
+  t.a0 = (int)blockIdx.x * E::L;
+  build_thin_maps<S1>(maps, g, t);
+  if (threadIdx.x < 3) hdiv[threadIdx.x] = f64::divisor(A.h[threadIdx.x]);
+  double stc[4];
+  cta_step_constants(A.dt_dev, A.dt_host, A.h, stc);  // (a barrier)
+  const double gamma = A.gamma, gm1 = A.gamma - 1.0;
+  const int ax = t.axA, tid = threadIdx.x;
+  const AxisStep<double> ks(stc[0], hdiv[ax], stc[1 + ax]);
+  const bool one_point = (A.flags & PPML_VHAT_1PT) != 0;
+#pragma unroll 1
+  for (int f = 0; f < 6; f++) load_box<double, S1>(M.u[f], A, f, t, maps);
+  __syncthreads();
+  // slopes of the fields (38 threads each), and beside them the velocities and Roe weights
+  // of the cells -1 .. L (the template of a cell whose transverse neighbours are itself)
+  for (int e = tid; e < 6 * E::W + (E::L + 2); e += THIN_NT) {
+    if (e < 6 * E::W) {
+      const int f = e / E::W, c = e % E::W;
+      const double* const q = M.u[f];
+      if (c >= 1 && c < E::W - 1)
+        M.s[f][c] = FLAT ? 0.0
+                         : f64::slope(f64::diff(q[c], q[c - 1]), f64::diff(q[c + 1], q[c]),
+                                      q[c - 1], q[c + 1]);
+    }
+  }
+  if (tid >= THIN_NT - 64 && tid - (THIN_NT - 64) < E::L + 2) {
+    const int c = tid - (THIN_NT - 64) + 2;
+    const double r = M.u[0][c], sq = sqrt(r);
+    const double v = f64::over(ax == 0 ? M.u[1][c] : (ax == 1 ? M.u[2][c] : M.u[3][c]), r);
+    // corners and edges of eq. veltemplate along an axis with its transverse ones inactive
+    const double four = v + v + v + v;
+    const double vt = one_point ? v
+                                : f64::scale<-4>(four) + f64::scale<-3>(four) + f64::scale<-2>(v);
+    M.sq[c] = sq;
+    M.pr[c] = vt * sq;
+  }
+  __syncthreads();
+  for (int e = tid; e < 6 * E::W; e += THIN_NT) {
+    const int f = e / E::W, c = e % E::W;
+    if (c >= 2 && c < E::W - 1)
+      M.f[f][c] = f64::face(M.u[f][c - 1], M.u[f][c], M.s[f][c - 1], M.s[f][c]);
+  }
+  if (tid >= THIN_NT - 64 && tid - (THIN_NT - 64) <= E::L) {
+    const int c = tid - (THIN_NT - 64) + TH;  // face c - 3
+    const ThinFace<double> w = thin_face(M.pr[c - 1], M.pr[c], M.sq[c - 1], M.sq[c], ks);
+    M.v[c] = w.v;
+    M.k[c] = w.k;
+  }
+  __syncthreads();
+  for (int e = tid; e < 6 * E::W; e += THIN_NT) {
+    const int f = e / E::W, c = e % E::W;
+    if (c < 2 || c >= E::W - 2) continue;
+    const double q0 = M.u[f][c];
+    double Lf = M.f[f][c], Rf = M.f[f][c + 1], D = 0.0, S = 0.0;
+    if (FLAT)
+      Lf = Rf = q0;
+    else
+      f64::parabola(q0, Lf, Rf, D, S);
+    M.PL[f][c] = Lf;
+    M.PR[f][c] = Rf;
+    M.D[f][c] = D;
+    M.S[f][c] = S;
+  }
+  __syncthreads();
+  for (int e = tid; e < 6 * (E::L + 1); e += THIN_NT) {
+    const int f = e / (E::L + 1), c = e % (E::L + 1) + TH;
+    const double v = M.v[c];
+    const bool left = f64::hi_word(v) >= 0;
+    const int o = left ? c - 1 : c;
+    const double st = f64::average(left, left ? M.PR[f][o] : M.PL[f][o], M.D[f][o], M.S[f][o], M.k[c]);
+    M.F[f][c] = f64::is_zero(v) && f64::finite(st) ? 0.0 : f64::plain_mul(v, st);
+  }
+  __syncthreads();
+  for (int e = tid; e < 6 * E::L; e += THIN_NT) {
+    const int f = e / E::L, i = e % E::L, b = i + TH;
+    M.n[f][i] = f64::minus(M.u[f][b], f64::times(ks.th, f64::diff(M.F[f][b + 1], M.F[f][b])));
+  }
+  __syncthreads();
+  // a cell per thread of the first warp: energy correction, CFL maxima; sums over the warp
+  FieldSums<double> sums;
+  sums.init();
+  double vmax = 0.0, cmax = 0.0;
+  unsigned long long nvac = 0, nbad = 0;
+  static_assert(E::L == 32, "the cells are one warp's");
+  if (tid < 32) {
+    double u[6];
+    RoughSpeeds rough = {-1.0f, -1.0f};
+    float vlow = 0.0f, clow = 0.0f;
+    if (t.a0 + tid < g.n[ax]) {
+      const long long o = t.a0 + tid;
+#pragma unroll
+      for (int f = 0; f < 6; f++) u[f] = M.n[f][tid];
+      nvac = correct_energy<double>(u, A.rho_vac);
+#pragma unroll
+      for (int f = 0; f < 6; f++) A.out[f][o] = u[f];
+      sums.add(u);
+      rough_speeds(u, (float)A.gamma * (float)(A.gamma - 1.0), rough, vlow, clow, nbad);
+    }
+    vlow = warp_max(vlow);
+    clow = warp_max(clow);
+    const bool nv = rough.v > 0.0f && rough.v >= vlow, nc = rough.c >= clow;
+    if (nv || nc) {
+      ExactSpeeds ex;
+      ex.add(u, gamma, gm1, nv, nc, vmax, cmax);
+    }
+  }
+  double sd[6];
+  sums.get(sd);
+  block_reduce_store<THIN_NT>(sd, vmax, cmax, nvac, nbad, A.partials, blockIdx.x);
+  finalize_last(A.partials, tiles, A.fin, stc[0]);
+}
+
 }  // namespace ppml

@@ -367,6 +367,12 @@ struct LineF64 {
   __device__ __forceinline__ void push(double q) {
     if constexpr (FLAT) {
       L = R = q1;
+    } else if (f64::same_bits(q, qn) && f64::same_bits(qn, q1) && f64::same_bits(f, q1) &&
+               f64::is_zero(s) && f64::exponent(q) < 2046u) {
+      // nothing varies here: the slopes are zero, the faces the value (a branch of its own,
+      // as the forms below would each find that out: 256^3 blast, most of it ambient gas)
+      L = R = q1;
+      D = S = d = 0.0;
     } else {
       const double dn = f64::diff(q, qn);
       const double sn = f64::slope(d, dn, q1, q);
