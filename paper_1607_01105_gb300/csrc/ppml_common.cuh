@@ -67,17 +67,17 @@ __device__ __forceinline__ double read_tau(const double* dt_dev, double dt_host)
   return dt_dev ? *dt_dev : dt_host;
 }
 
-// The step size and tau / h per axis, formed by one thread of the CTA (three FP64
-// divisions per CTA instead of per thread) and shared.  Contains a CTA barrier.
+// The step size and tau / h per axis, formed by one thread of the CTA per axis (a division of
+// a lone thread is ten dependent FP64 instructions of 76 cycles) and shared.  Contains a CTA
+// barrier.
 __device__ __forceinline__ void cta_step_constants(const double* dt_dev, double dt_host,
                                                    const double h[3], double out[4]) {
   __shared__ double s[4];
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 3) {
     const double tau = read_tau(dt_dev, dt_host);
-    s[0] = tau;
-    s[1] = tau / h[0];
-    s[2] = tau / h[1];
-    s[3] = tau / h[2];
+    const double ha = threadIdx.x == 0 ? h[0] : (threadIdx.x == 1 ? h[1] : h[2]);
+    if (threadIdx.x == 0) s[0] = tau;
+    s[1 + threadIdx.x] = tau / ha;
   }
   __syncthreads();
 #pragma unroll
@@ -96,7 +96,7 @@ __device__ __forceinline__ void fold_warps(const double (*sh)[8], const unsigned
   if (q < 6) {
     double v = 0.0;
 #pragma unroll
-    for (int w = 0; w < NW; w++) v += sh[w][q];
+    for (int w = 0; w < NW; w++) v = f64::plus(v, sh[w][q]);
     out[slot].s[q] = v;
   } else if (q < 8) {  // nonnegative: ordered as integers
     unsigned long long m = 0;
@@ -122,9 +122,12 @@ __device__ __forceinline__ void block_reduce_store(double s[6], double vmax, dou
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
 #pragma unroll
-    for (int f = 0; f < 6; f++) s[f] += __shfl_down_sync(0xffffffffu, s[f], o);
-    vmax = fmax(vmax, __shfl_down_sync(0xffffffffu, vmax, o));
-    cmax = fmax(cmax, __shfl_down_sync(0xffffffffu, cmax, o));
+    for (int f = 0; f < 6; f++) s[f] = f64::plus(s[f], __shfl_down_sync(0xffffffffu, s[f], o));
+    // nonnegative: ordered as integers
+    vmax = __longlong_as_double(max(__double_as_longlong(vmax),
+                                    __double_as_longlong(__shfl_down_sync(0xffffffffu, vmax, o))));
+    cmax = __longlong_as_double(max(__double_as_longlong(cmax),
+                                    __double_as_longlong(__shfl_down_sync(0xffffffffu, cmax, o))));
     nvac += __shfl_down_sync(0xffffffffu, nvac, o);
     nbad += __shfl_down_sync(0xffffffffu, nbad, o);
   }
