@@ -471,18 +471,19 @@ __device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, floa
   // of five 480; 512 instances: 3.31, 3.31 and 3.37 ms)
   const int run_e = ((P.cb - P.ca + NTHREADS - 1) / NTHREADS) | 1;
   const int run = ((nl + NTHREADS - 1) / NTHREADS) | 1;
-  // a value of cell c with the outflow ghosts that repeat it at the instance's ends
-  auto put = [&](float* q, int c, float v) {
-    q[c] = v;
+  // whether the cells c0 .. c1-1 hold an end of the instance, and the outflow ghosts that
+  // repeat an end cell's value
+  auto at_end = [&](int c0, int c1) { return (P.gl && c0 <= 0) || (P.gr && c1 >= nl); };
+  auto ghosts = [&](float* q, int c, float v) {
     if (P.gl && c == 0) q[-1] = q[-2] = q[-3] = v;
     if (P.gr && c == nl - 1) q[nl] = q[nl + 1] = q[nl + 2] = v;
   };
   float vm = 0.0f, cm = 0.0f;
   bool bad = false;
   auto cfl_cell = [&](float r, float m, float en, float ei) {
-    const bool ok = r > 0.0f && ei > 0.0f && isfinite(r) && isfinite(m) && isfinite(en) &&
-                    isfinite(ei);
-    bad = bad || !ok;
+    // rho, rho eps > 0 and all four finite (NaN fails the comparisons)
+    const float top = max_nan(max_nan(r, ei), max_nan(fabsf(m), fabsf(en)));
+    bad = bad || !(fminf(r, ei) > 0.0f && top < __int_as_float(0x7f800000));
     const float ir = rcp_approx(r);
     vm = fmaxf(vm, fabsf(m * ir));
     cm = fmaxf(cm, sqrt_approx(gamma * (gm1 * ei) * ir));
@@ -490,10 +491,16 @@ __device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, floa
   const long long off = I.off + P.lo;
   for (int c = tid; c < nl; c += NTHREADS) {
     const float r = g_rho[off + c], m = g_m[off + c], en = g_en[off + c], ei = g_ei[off + c];
-    put(R, c, r);
-    put(M, c, m);
-    put(E, c, en);
-    put(Ei, c, ei);
+    R[c] = r;
+    M[c] = m;
+    E[c] = en;
+    Ei[c] = ei;
+    if (at_end(c, c + 1)) {
+      ghosts(R, c, r);
+      ghosts(M, c, m);
+      ghosts(E, c, en);
+      ghosts(Ei, c, ei);
+    }
     cfl_cell(r, m, en, ei);
   }
   if constexpr (PAIR) {  // the initial halo: the partner's first cells, from the state
@@ -521,6 +528,7 @@ __device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, floa
     // Eulerian stage of the cells ca .. cb-1
     for (int c0 = P.ca + tid * run_e; c0 < P.cb; c0 += NTHREADS * run_e) {
       const int c1 = min(c0 + run_e, P.cb);  // faces c0 .. c1
+      const bool end = at_end(c0, c1);
       auto vp = [&](int k) { return make_float2(M[k] * rcp_approx(R[k]), gm1 * Ei[k]); };
       LinePair<false> ln;
       ln.start(vp(c0 - 3), vp(c0 - 2), vp(c0 - 1));
@@ -539,9 +547,16 @@ __device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, floa
         if (f > c0) {
           const int c = f - 1;
           const float ei = Ei[c];
-          put(Ms, c, M[c] - th * (Pf - Pp));
-          put(Es, c, E[c] - th * (Pf * V - Pp * Vp));
-          put(Is, c, ei - gm1 * ei * (th * (V - Vp)));
+          const float ms = M[c] - th * (Pf - Pp), es = E[c] - th * (Pf * V - Pp * Vp),
+                      is = ei - gm1 * ei * (th * (V - Vp));
+          Ms[c] = ms;
+          Es[c] = es;
+          Is[c] = is;
+          if (end) {
+            ghosts(Ms, c, ms);
+            ghosts(Es, c, es);
+            ghosts(Is, c, is);
+          }
         }
         Vp = V;
         Pp = Pf;
@@ -555,6 +570,7 @@ __device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, floa
     cm = 0.0f;
     for (int c0 = tid * run; c0 < nl; c0 += NTHREADS * run) {
       const int c1 = min(c0 + run, nl);  // faces c0 .. c1
+      const bool end = at_end(c0, c1);
       auto rm = [&](int k) { return make_float2(R[k], Ms[k]); };
       auto ee = [&](int k) { return make_float2(Es[k], Is[k]); };
       LinePair<false> la, lb;
@@ -581,18 +597,25 @@ __device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, floa
         if (f > c0) {
           const int c = f - 1;
           const float2 na = sub2(qa, sub2(Ga, Fa)), nb = sub2(qb, sub2(Gb, Fb));
-          float u[6] = {na.x, na.y, 0.0f, 0.0f, nb.x, nb.y};
-          const bool vac = vacuum_cell_f32(u, rho_vac_up);
-          const float e = dense_eps_f32(u);
-          if (vac)
+          const float e = internal_energy_1d(na.x, na.y, nb.x);
+          float m = na.y, ei = e > 0.0f ? e : nb.y;
+          if (na.x < rho_vac_up && m * m > 0.0f) {
+            float u[6] = {na.x, m, 0.0f, 0.0f, nb.x, nb.y};
             vacuum_correct_f32(u, I.rho_vac);
-          else
-            u[5] = e;
-          put(Rn, c, u[0]);
-          put(M, c, u[1]);
-          put(E, c, u[4]);
-          put(Ei, c, u[5]);
-          cfl_cell(u[0], u[1], u[4], u[5]);
+            m = u[1];
+            ei = u[5];
+          }
+          Rn[c] = na.x;
+          M[c] = m;
+          E[c] = nb.x;
+          Ei[c] = ei;
+          if (end) {
+            ghosts(Rn, c, na.x);
+            ghosts(M, c, m);
+            ghosts(E, c, nb.x);
+            ghosts(Ei, c, ei);
+          }
+          cfl_cell(na.x, m, nb.x, ei);
         }
         Fa = Ga;
         Fb = Gb;

@@ -375,6 +375,17 @@ __device__ __forceinline__ float internal_energy_ff(float rho, float mx, float m
   return d + (de - ql);
 }
 
+// The same with one momentum component (the operations that are left when the others are 0).
+__device__ __forceinline__ float internal_energy_1d(float rho, float m, float en) {
+  const float hi = m * m, lo = fmaf(m, m, -hi);
+  const float r2 = 2.0f * rho, ir2 = rcp_approx(r2);
+  const float q = hi * ir2;
+  const float ql = (fmaf(-q, r2, hi) + lo) * ir2;
+  float d, de;
+  two_sum(en, -q, d, de);
+  return d + (de - ql);
+}
+
 // ------------------------------------------------------------ double-float state values
 // A field stored as an unevaluated float pair (hi, lo), |lo| <= ulp(hi) / 2, carries about
 // 48 significant bits.  The FP32 path keeps rho, m and rho E this way when the caller
