@@ -221,7 +221,8 @@ __device__ __forceinline__ void face_constants_f32(float rl, float rr, float sl,
 }
 
 // ------------------------------------------------- FP32 parabolas in deviation form
-// The FP32 kernels carry a cell's parabola as its two face deviations from the cell value,
+// The plain FP32 kernels (line pipelines in ppml_pair.cuh) carry a cell's parabola as its two
+// face deviations from the cell value,
 // l = q0 - q^L and r = q^R - q0 (stored doubled), instead of (q^L, q^R, Delta q, q^(6)):
 //   * the monotonicity step (Appendix, Steps 2-3) reads, with Delta q = l + r and
 //     q^(6) = 3 (l - r): flat where l r <= 0, else l <- min(|l|, 2|r|) and
@@ -251,26 +252,6 @@ __device__ __forceinline__ float max_nan(float a, float b) {
   return r;
 }
 
-// Half of the limited slope (Step 1) from the differences to the left and right cells:
-// min(|l + r| / 4, |l|, |r|) with their common sign, 0 where the signs differ.
-__device__ __forceinline__ float half_slope_f32(float l, float r) {
-  const float t = fmaxf(min_xs(l, r), 0.0f);
-  return min_xs(0.25f * (l + r), t);
-}
-
-struct DevParab {
-  float l2, r2;  // 2 (q0 - q^L), 2 (q^R - q0)
-};
-
-__device__ __forceinline__ DevParab monotone_f32(float l2, float r2) {
-  const float t = max_nan(min_xs_nan(l2, r2), 0.0f);
-  const float m = t + t;
-  DevParab P;
-  P.l2 = min_xs_nan(l2, m);
-  P.r2 = min_xs_nan(r2, m);
-  return P;
-}
-
 // Weights of the deviations at Courant number y, halved for the doubled deviations.
 struct DevWeights {
   float a, b;  // (1-y)^2 / 2, y (1-y) / 2
@@ -282,67 +263,6 @@ __device__ __forceinline__ DevWeights dev_weights(float y) {
   w.b = hz * y;
   return w;
 }
-// Averages next to a cell's right and left face.
-__device__ __forceinline__ float dev_right(float q, const DevParab& P, const DevWeights& w) {
-  return fmaf(w.a, P.r2, fmaf(w.b, P.l2, q));
-}
-__device__ __forceinline__ float dev_left(float q, const DevParab& P, const DevWeights& w) {
-  return fmaf(-w.a, P.l2, fmaf(-w.b, P.r2, q));
-}
-
-// th times the flux of eq. fluxonlagrangestage through a face, w = v^ th: w times the left
-// cell's average when w >= 0, else the right cell's.
-__device__ __forceinline__ float upwind_flux_f32(float w, float ql, const DevParab& Pl, float qr,
-                                                 const DevParab& Pr) {
-  const DevWeights c = dev_weights(fabsf(w));
-  const bool from_left = w >= 0.0f;
-  const float q = from_left ? ql : qr;
-  const float x = from_left ? Pl.r2 : -Pr.l2;
-  const float y = from_left ? Pl.l2 : -Pr.r2;
-  return w * fmaf(c.a, x, fmaf(c.b, y, q));
-}
-
-// Line pipeline of the deviation form: push(q) takes the next position p; then q2 is the
-// value and P the parabola of cell p - 2.  FLAT: the first-order variant (no deviations).
-template <bool FLAT>
-struct LineF32 {
-  float q1, q2;   // values at p-1... after push: at p, p-... see push
-  float qn;       // value at p
-  float d;        // difference between p and p-1
-  float s;        // half slope of p-1
-  float l2;       // doubled left deviation of p-1
-  DevParab P;     // parabola of p-2
-  // the first three positions of the line
-  __device__ __forceinline__ void start(float a, float b, float c) {
-    q2 = a;
-    q1 = b;
-    qn = c;
-    P.l2 = P.r2 = l2 = 0.0f;
-    d = c - b;
-    s = half_slope_f32(b - a, d);
-  }
-  __device__ __forceinline__ void push(float q) {
-    if constexpr (FLAT) {
-      q2 = q1;
-      q1 = qn;
-      qn = q;
-    } else {
-      const float dn = q - qn;
-      const float sn = half_slope_f32(d, dn);  // of the previous position
-      // face between the two positions before q: doubled deviations d -+ (2/3)(sn - s)
-      const float e = sn - s;
-      const float r2 = fmaf(e, -2.0f / 3.0f, d);
-      P = monotone_f32(l2, r2);
-      l2 = fmaf(e, 2.0f / 3.0f, d);
-      q2 = q1;
-      q1 = qn;
-      qn = q;
-      d = dn;
-      s = sn;
-    }
-  }
-};
-
 // ---------------------------------------------------------- compensated FP32 helpers
 // Error-free transformations (Knuth TwoSum; FMA-based TwoProduct).  Used where the
 // paper's quantity is a small difference of large totals so that the FP32 path keeps

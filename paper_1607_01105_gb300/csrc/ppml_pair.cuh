@@ -31,11 +31,16 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
 __device__ __forceinline__ float2 both(float x) { return make_float2(x, x); }
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return fma2(b, both(-1.0f), a); }
 
-// LineF32 for two fields.
+// Line pipeline of the deviation form for two quantities: push(q) takes the next position p;
+// then q2 is the values and Pl, Pr the doubled deviations 2 (q0 - q^L), 2 (q^R - q0) of cell
+// p - 2.  FLAT: the first-order variant (no deviations).
 template <bool FLAT>
 struct LinePair {
-  float2 q2, q1, qn, d, s, l2;
-  float2 Pl, Pr;  // doubled deviations of cell p - 2
+  float2 q2, q1, qn;  // values at p-2, p-1, p
+  float2 d, s, l2;    // difference p-1 .. p, half slope and doubled left deviation of p-1
+  float2 Pl, Pr;
+  // half of the limited slope (Step 1): min(|l + r| / 4, |l|, |r|) with the differences'
+  // common sign, 0 where their signs differ
   static __device__ __forceinline__ float2 half_slope(float2 l, float2 r) {
     const float2 c = mul2(add2(l, r), both(0.25f));
     return make_float2(min_xs(c.x, fmaxf(min_xs(l.x, r.x), 0.0f)),
@@ -53,6 +58,7 @@ struct LinePair {
     if constexpr (!FLAT) {
       const float2 dn = sub2(q, qn);
       const float2 sn = half_slope(d, dn);
+      // face between the two positions before q: doubled deviations d -+ (2/3)(sn - s)
       const float2 e = sub2(sn, s);
       const float2 r2 = fma2(e, both(-2.0f / 3.0f), d);
       const float2 t = make_float2(max_nan(min_xs_nan(l2.x, r2.x), 0.0f),
@@ -70,7 +76,8 @@ struct LinePair {
   }
 };
 
-// upwind_flux_f32 for two fields, c = dev_weights(|w|).
+// th times the flux of eq. fluxonlagrangestage of two fields through a face, w = v^ th and
+// c = dev_weights(|w|): w times the left cell's average when w >= 0, else the right cell's.
 __device__ __forceinline__ float2 upwind_flux_pair(float w, const DevWeights& c, float2 ql, float2 Ll,
                                                    float2 Lr, float2 qr, float2 Rl, float2 Rr) {
   const bool left = w >= 0.0f;

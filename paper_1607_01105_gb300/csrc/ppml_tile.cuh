@@ -1,4 +1,6 @@
-// Tiled line-sweep kernels of one PPML step (Kulikov & Vorobyov, arXiv:1607.01105).
+// Tiled line-sweep kernels of one PPML step (Kulikov & Vorobyov, arXiv:1607.01105): FP64 and
+// double-float states (plain FP32 states have kernels of their own, ppml_tile_f32.cuh and
+// ppml_thin.cuh, which also take FP64 grids of one or two active axes).
 //
 // A CTA of 256 threads owns a 16^3 tile.  Thread t = a + 16 b owns one line per axis
 // (x line (j, k) = (a, b); y line (i, k) = (a, b); z line (i, j) = (a, b)).  Each line is
@@ -223,63 +225,9 @@ __device__ __forceinline__ Parab<T> flat_parabola(T q) {
 // reads position p, and with p = 19 after the last step; positions below p - 3 are no
 // longer read at that point (step p reads positions p, p - 2 and p - 3).
 //
-// FP32: the parabolas in deviation form (LineF32), the steady steps p = 3..18 as a loop
-// unrolled by two (a small body for the instruction cache).
-template <bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
-__device__ __forceinline__ void sweep_eulerian_dev(VF v, PF pr, RF r, float gamma, float th,
-                                                   EF emit, HF hook) {
-  LineF32<FLAT> lv, lp;
-  hook(-1);
-  lv.start(v(-3), v(-2), v(-1));
-  lp.start(pr(-3), pr(-2), pr(-1));
-  hook(0);
-  lv.push(v(0));
-  lp.push(pr(0));
-  hook(1);
-  lv.push(v(1));
-  lp.push(pr(1));
-  // cell p-3 (the face's left cell): values, parabolas and sqrt(rho), rho sqrt(rho), p sqrt(rho)
-  float vl = lv.q2, pl = lp.q2;
-  DevParab Vl = lv.P, Pl = lp.P;
-  const float r0 = r(-1);
-  float sl = sqrt_approx(r0), Al = r0 * sl, Bl = pl * sl;
-  float Vp = 0.0f, Pp = 0.0f;
-  auto face = [&](int p, float& V, float& P) {  // after position p: the face of p-3 and p-2
-    hook(p);
-    lv.push(v(p));
-    lp.push(pr(p));
-    const float rc = r(p - 2), sc = sqrt_approx(rc);
-    const float Ac = rc * sc, Bc = lp.q2 * sc;
-    // face_constants_f32 from the carried products
-    const float A = Al + Ac, lam = sqrt_approx(gamma * (Bl + Bc) * rcp_approx(A));
-    const float Z = lam * A * rcp_approx(sl + sc);
-    const DevWeights w = dev_weights(lam * th);
-    const float vls = dev_right(vl, Vl, w), vrs = dev_left(lv.q2, lv.P, w);
-    const float pls = dev_right(pl, Pl, w), prs = dev_left(lp.q2, lp.P, w);
-    V = 0.5f * ((vls + vrs) + (pls - prs) * rcp_approx(Z));
-    P = 0.5f * ((pls + prs) + Z * (vls - vrs));
-    vl = lv.q2;
-    pl = lp.q2;
-    Vl = lv.P;
-    Pl = lp.P;
-    sl = sc;
-    Al = Ac;
-    Bl = Bc;
-  };
-  face(2, Vp, Pp);
-#pragma unroll 2
-  for (int p = 3; p <= TB + 2; p++) {
-    float V, P;
-    face(p, V, P);
-    emit(p - 3, th * (P - Pp), th * (P * V - Pp * Vp), th * (V - Vp));
-    Vp = V;
-    Pp = P;
-  }
-  hook(TB + 3);
-}
-
-// The same sweep with the parabolas in face values, for double-float states: their low parts
-// record the rounding of exactly these expressions.
+// FP32, the parabolas in face values: double-float states, whose low parts record the rounding
+// of exactly these expressions (and one- and two-axis grids with gravity; plain states of
+// three axes have eulerian_sweep_f32, of fewer thin_eulerian).
 template <bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
 __device__ __forceinline__ void sweep_eulerian_faces(VF v, PF pr, RF r, float gamma, float th,
                                                      EF emit, HF hook) {
@@ -572,80 +520,15 @@ __device__ __forceinline__ void stage_box_fast(T* box, const T* __restrict__ src
 }
 
 // Face velocities as the sweeps read them.  FP64: v^ itself (the flux and the Courant
-// number are formed as the checker forms them).  FP32: w = v^ th (th = tau / h), so that
-// |w| is the Courant number y and w times the upwind state is th times the flux: the
-// per-field products by th disappear.  Double-float states (DF): half of that, as the
-// face-value form reads it.
-template <bool DF>
-__device__ __forceinline__ float vh_stored(float v, float th) {
-  return v * (DF ? 0.5f * th : th);
-}
-template <bool DF>
+// number are formed as the checker forms them).  FP32: w = v^ th / 2 (th = tau / h), so
+// that |w| is half the Courant number y and w times the upwind state is half of th times
+// the flux (both exact rescalings of v^ th): the per-field products by th disappear, the
+// sweeps accumulate half divergences and the update subtracts twice their sum.
+__device__ __forceinline__ float vh_stored(float v, float th) { return v * (0.5f * th); }
 __device__ __forceinline__ double vh_stored(double v, double) { return v; }
 // The flux divergence summed over axes from what the sweeps accumulated (exact).
-template <bool DF>
-__device__ __forceinline__ float divergence_sum(float sum) { return DF ? 2.0f * sum : sum; }
-template <bool DF>
+__device__ __forceinline__ float divergence_sum(float half_sum) { return 2.0f * half_sum; }
 __device__ __forceinline__ double divergence_sum(double sum) { return sum; }
-
-// One line of the FP32 Lagrangian stage for any axis, on the deviation form of the parabola
-// (LineF32).  Field values: core[p cs] for p in [0, 16), halo[h SLP] for the positions
-// -3..-1 (h = 0..2) and 16..18 (h = 3..5).  Face velocities vh[c TN], c = 0..16 (face
-// between cells c-1 and c).  When position p arrives, the slope at p-1, the deviations of
-// the face p-3/2, the parabola of cell p-2 and the flux through face p-5/2 are formed; the
-// warm-up positions are peeled and the steady state is a loop unrolled by four.  MODE 0:
-// acc = div; 1: acc += div; 2: dst[c gs] = core - (acc + div) for c < nvalid (acc only if
-// have_acc).  CS: the core stride of the sweep axis as a compile-time constant (immediate
-// shared-memory offsets).
-template <int MODE, bool FLAT, int CS>
-__device__ __forceinline__ void lag_line_dev(const float* core, const float* halo,
-                                             const float* vh, float* acc, bool have_acc,
-                                             float* __restrict__ dst, long long gs, int nvalid) {
-  constexpr int cs = CS;
-  LineF32<FLAT> ln;
-  ln.start(halo[0], halo[SLP], halo[2 * SLP]);
-  ln.push(core[0]);
-  ln.push(core[cs]);
-  DevParab Pl = ln.P;  // cell -1
-  float ql = ln.q2;
-  ln.push(core[2 * cs]);
-  float Fp = upwind_flux_f32(vh[0], ql, Pl, ln.q2, ln.P);
-  ql = ln.q2;
-  Pl = ln.P;
-  // steady state: position c + 3 arrives, cell c is finished
-  auto step = [&](float qnew, float w, int c) {
-    ln.push(qnew);
-    const float F = upwind_flux_f32(w, ql, Pl, ln.q2, ln.P);  // face between c and c+1
-    const float d = F - Fp;  // th (F+ - F-)
-    const int o = c * cs;
-    if (MODE == 0)
-      acc[o] = d;
-    else if (MODE == 1)
-      acc[o] = acc[o] + d;
-    else if (c < nvalid)
-      dst[gs * c] = ql - (have_acc ? acc[o] + d : d);
-    Fp = F;
-    ql = ln.q2;
-    Pl = ln.P;
-  };
-  // inputs one step ahead: position c + 3 and face c + 1 of step c are loaded in step c - 1
-  float q_in = core[3 * cs], v_in = vh[TN];
-#pragma unroll 4
-  for (int c = 0; c < TB - 4; c++) {
-    const float q = q_in, v = v_in;
-    q_in = core[(c + 4) * cs];
-    v_in = vh[(c + 2) * TN];
-    step(q, v, c);
-  }
-#pragma unroll 1
-  for (int c = TB - 4; c < TB - 1; c++) {
-    const float q = q_in, v = v_in;
-    q_in = halo[(c - TB + 7) * SLP];  // positions 16..18
-    v_in = vh[(c + 2) * TN];          // faces 14..16
-    step(q, v, c);
-  }
-  step(q_in, v_in, TB - 1);
-}
 
 // FP32 flux through a face of eq. fluxonlagrangestage from w = v^ th / 2: w times the
 // upwind state, the left cell's mean over its right fraction y when w >= 0, else the right
@@ -953,7 +836,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
   auto store_vh = [&](int ax, const T* v) {
 #pragma unroll
     for (int q = 0; q <= TB; q++) {
-      S.vh[ax][q][tid] = vh_stored<DF>(v[q], th[ax]);
+      S.vh[ax][q][tid] = vh_stored(v[q], th[ax]);
       if constexpr (sizeof(T) == 8) {
         const AxisStep<T> ks(tau, hdiv[ax], th[ax]);
         fweights[ax][q] = f64::is_zero(v[q]) ? f64::Weights{0.0, 1.0}
@@ -1093,8 +976,6 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
         if constexpr (sizeof(T) == 8)
           lag_line_f64<M, FL, C>(core, halo, vhl, fweights[ax], th[ax], acc, mode == 1, dst, g.nxy,
                                  nvalid_z);
-        else if constexpr (!DF)
-          lag_line_dev<M, FL, C>(core, halo, vhl, acc, mode == 1, dst, g.nxy, nvalid_z);
         else
           lag_line_faces<M, FL, DF && M == 2, C>(core, halo, vhl, acc, mode == 1, dst, g.nxy,
                                                  nvalid_z, srclo, dstlo);
@@ -1120,7 +1001,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
       for (int c = 0; c < nvalid_z; c++) {
         const int o = acc_at(a, b, c);
         const long long idx = zline0 + g.nxy * c;
-        const T upd = mode == 1 ? divergence_sum<DF>(S.acc[o]) : T(0);
+        const T upd = mode == 1 ? divergence_sum(S.acc[o]) : T(0);
         if constexpr (DF) {
           if (f < 5) {
             float hi, lo;
@@ -1465,10 +1346,8 @@ __global__ void __launch_bounds__(TN, MINB) eulerian_tile(MarchArgs<T> A) {
       constexpr bool FL = decltype(flat_c)::value;
       if constexpr (sizeof(T) == 8)
         sweep_eulerian_f64<FL>(vq, pq, rq, gamma, AxisStep<T>(tau, hdiv[ax], th[ax]), emit, hook);
-      else if constexpr (DF)
-        sweep_eulerian_faces<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
       else
-        sweep_eulerian_dev<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
+        sweep_eulerian_faces<FL>(vq, pq, rq, gamma, th[ax], emit, hook);
     };
     if (A.flags & PPML_FIRST_ORDER)
       sweep(BoolC<true>());

@@ -455,7 +455,7 @@ struct EulerSmem {
 
 // One line of the Eulerian stage, (v, p) as a packed pair of lines: q(p, v, r) gives the pair
 // (v_a, p) and rho at the positions p = -3..18 (called in order, each once).  emit(c, dm, dpv,
-// dv) as in sweep_eulerian_dev.  ahead(): before the last four steps.
+// dv) for the cells c = 0 .. 15 as sweep_eulerian_faces describes.  ahead(): before the last four steps.
 template <bool FLAT, typename QF, typename EF, typename AF>
 __device__ __forceinline__ void euler_line_pair(QF q, float gamma, float th, EF emit, AF ahead) {
   LinePair<FLAT> ln;
