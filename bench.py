@@ -41,16 +41,19 @@ N_CELLS_SIDE = 256
 BYTES_EUL = {4: 44, 8: 88}
 BYTES_LAG = {4: 48, 8: 96}
 # algorithmic FP32 operations per cell (add, mul, fma, min, compare, select, sqrt and
-# divide each counted once) of the Lagrangian stage: 18 (field, axis) line updates of
-# 62 (slope 12, face 4, parabola 26, upwind average 17, update 3), the velocity template
-# and face velocities 57, energy correction 30, CFL terms 12, compensated sums 42.
-OPS_LAG = 18 * 62 + 57 + 30 + 12 + 42
-# Eulerian stage: per axis v and p parabolas 84, face constants 15, four averages 32,
-# face solution 9, updates 8, v = m / rho 1; plus 6 for rho E and rho eps.
-OPS_EUL = 3 * (84 + 15 + 32 + 9 + 8 + 1) + 6
-# DRAM bytes of one Lagrangian launch measured by ncu (dram__bytes_read + write, one launch
-# of the 256^3 point blast, the timed workload itself; see profiles/).
-NCU_LAG_DRAM_BYTES_256 = 486.10e6 + 381.00e6
+# divide each counted once) of the minimal formulation (parabolas as face deviations) of the
+# Lagrangian stage: 18 (field, axis) line updates of 26 (slope 6, face 4, monotonicity 5,
+# upwind flux 7, update 2, a sixth of the face's weights, rounded up to 2), the velocity
+# template and face velocities 57, energy correction 30, CFL terms 12, compensated sums 42.
+OPS_LAG = 18 * 26 + 57 + 30 + 12 + 42
+# Eulerian stage: per axis the v and p parabolas 30, face constants 15, weights 4, four
+# averages 8, face solution 9, updates 8, v = m / rho 1; plus 6 for rho E and rho eps.
+OPS_EUL = 3 * (30 + 15 + 4 + 8 + 9 + 8 + 1) + 6
+# the same in face values, which FP64 takes (the bits of the oracle's expressions)
+OPS_LAG_FACES = 18 * 62 + 57 + 30 + 12 + 42
+# DRAM bytes of one FP32 Lagrangian stage measured by ncu (dram__bytes_read + write of its two
+# launches, of a 256^3 point blast like the timed workload; see profiles/).
+NCU_LAG_DRAM_BYTES_256 = (268.9e6 + 176.4e6) + (726.8e6 + 374.9e6)
 SMS, FP32_LANES = 152, 128
 
 
@@ -282,7 +285,7 @@ def gpu_configs(args, dev, stream, barrier, disk_steps):
                      "t": t}
     out["sod_1d_256"] = dict(res, unit="Mcell-updates/s",
                              workload="Sod (Table 2 row 1), 256 cells, CFL 0.4, outflow, run to "
-                                      "t = 0.2, through the grid path (three launches per step)")
+                                      "t = 0.2, through the grid path (two launches per step)")
     # the same run as a batch of one instance: the whole run in one persistent launch
     res = {}
     for dtype, name in kinds:
@@ -471,7 +474,7 @@ def slab_bench(args):
                        "global_batch": 1, "seq_len": 0,
                        "parallelism": f"z-slabs x{world}" if world > 1 else
                                       f"{nslab} slabs in one process (plane copies)"},
-            "gpu_launches": 4 * len(layouts) * args.steps,  # two stages, reduce, apply
+            "gpu_launches": 4 * len(layouts) * args.steps,  # Eulerian, velocities, sweeps, apply
             "clocks": cs.summary()}), flush=True)
     if world > 1:
         dist.destroy_process_group()
@@ -739,7 +742,7 @@ def main():
                        "tile_order_trial_ms": {str(k): v for k, v in r32["tile_tune"][1].items()},
                        "parallelism": "replicas" if world > 1 else "single GPU",
                        "l2": "no flush: state 403 MB x 2 + U* 336 MB > 129 MB L2"},
-            "roofline": {"bound": "alu", "kernel": "lagrangian_tile<float>",
+            "roofline": {"bound": "alu", "kernel": "face_velocity_f32 + lagrangian_sweep_f32",
                          "achieved": lag_ops, "peak": alu_peak, "unit": "TFLOP/s",
                          "frac": lag_ops / alu_peak,
                          "hbm_frac": lag_gbs / peak,
@@ -748,9 +751,10 @@ def main():
                                        "one operation per lane per clock (FMA counted once)",
                          "algorithmic_ops_per_cell": OPS_LAG,
                          "traffic": NCU_LAG_DRAM_BYTES_256 if args.n == 256 else None,
-                         "traffic_note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of one "
-                                         "launch of the 256^3 point blast (51.7 B/cell; 48 "
-                                         "algorithmic)",
+                         "traffic_note": "ncu dram__bytes_read.sum + dram__bytes_write.sum of the "
+                                         "stage's two launches on a 256^3 point blast (92.2 "
+                                         "B/cell; 48 algorithmic, 25.5 the face velocities "
+                                         "written and read)",
                          "kernel_ms": {"eulerian": keul, "lagrangian": klag, "finalize": kfin},
                          "eulerian": {"achieved": eul_ops, "frac": eul_ops / alu_peak,
                                       "algorithmic_ops_per_cell": OPS_EUL},
@@ -762,14 +766,17 @@ def main():
             "fp64": {"value": v64, "unit": "Mcell-updates/s", "ms_per_step": r64["ms"] / r64["steps"],
                      "steps": r64["steps"], "kernel_ms": r64["kernel_ms"],
                      "roofline": {"bound": "alu", "kernel": "lagrangian_tile<double>",
-                                  "achieved": OPS_LAG * cells / (r64["kernel_ms"][1] * 1e-3) / 1e12,
+                                  "achieved": OPS_LAG_FACES * cells / (r64["kernel_ms"][1] * 1e-3) / 1e12,
                                   "peak": fma_peak["f64"] / 1e12, "unit": "TFLOP/s",
-                                  "frac": OPS_LAG * cells / (r64["kernel_ms"][1] * 1e-3) / fma_peak["f64"],
+                                  "frac": OPS_LAG_FACES * cells / (r64["kernel_ms"][1] * 1e-3) / fma_peak["f64"],
                                   "peak_kind": "measured FP64 FMA throughput (ppml_fma_peak), "
                                                "an FMA counted once",
-                                  "algorithmic_ops_per_cell": OPS_LAG,
+                                  "algorithmic_ops_per_cell": OPS_LAG_FACES,
                                   "note": "IEEE division and square root are sequences of "
-                                          "several FP64 instructions but count once"}},
+                                          "several FP64 instructions but count once; cells "
+                                          "whose operands are equal or zero (most of the "
+                                          "ambient gas) issue none, so the fraction may "
+                                          "exceed 1"}},
             "fma_peak_measured": {"f32_tfma_s": fma_peak["f32"] / 1e12,
                                   "f64_tfma_s": fma_peak["f64"] / 1e12,
                                   "lagrangian_f32_frac_of_measured": lag_ops * 1e12 / fma_peak["f32"]},

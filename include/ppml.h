@@ -24,8 +24,8 @@
  *     mirror with the normal momentum negated; edges and corners as if ghosts were
  *     filled along x, then y, then z).
  *   - The caller owns every state array and the stream; the library owns its handle,
- *     the intermediate state U* and its reduction scratch (allocated by ppml_init_grid
- *     with cudaMalloc, freed by ppml_free_grid).
+ *     the intermediate state U* and its scratch (allocated by ppml_init_grid with
+ *     cudaMalloc, freed by ppml_free_grid).
  *   - `stream` is a cudaStream_t (NULL = legacy default stream).  Calls are asynchronous
  *     on that stream unless they return a host value (documented per call).
  *   - Return value: PPML_OK (0) or an error code; ppml_last_error() gives a message for
@@ -124,7 +124,8 @@ typedef struct {
 typedef struct ppml_grid ppml_grid;
 
 /* Create a handle for the grid in *d and allocate its scratch (U*: five fields of the
- * state's type, in FP32 also the four low parts of U*'s m and rho E; reduction partials).
+ * state's type, in FP32 also the four low parts of U*'s m and rho E and, with three active
+ * axes, the face velocities of every 16^3 tile, 52 KB each; reduction partials).
  * Reads u0 once on `stream` to fix the mean initial density (the vacuum threshold
  * reference, Sec. 1.4) and the first CFL step; synchronizes the stream.  u0 is not
  * modified.  On error *out is NULL. */
@@ -197,8 +198,9 @@ int ppml_fourier_amplitudes(ppml_grid* g, const void* rho, double r_f, int m_max
  * (k + 1/2 - nz/2) h); the grid is centred on the origin of the expansion.  Requires
  * h[0] = h[1] = h[2].  rho, phi: device arrays of nx*ny*nz cells of the grid's type (may
  * not alias; phi is also the work array).  Moments and shell values are formed in FP64; the
- * transforms run in the grid's type.  The first call creates cuFFT plans and buffers of
- * about 2 (N+1)/N x 3 states' worth of the grid's type, kept in the handle.  Asynchronous.
+ * transforms run in the grid's type.  The first call creates buffers kept in the handle: on FP32
+ * grids of at most 256 points per axis sine matrices and tables, else cuFFT plans and about
+ * 2 (N+1)/N x 3 states' worth of the grid's type.  Asynchronous.
  * PPML_E_INVAL for bad arguments or unknown flags. */
 int ppml_poisson_isolated(ppml_grid* g, const void* rho, void* phi, double G, unsigned flags,
                           void* stream);
@@ -277,13 +279,14 @@ int ppml_read_diag(ppml_grid* g, ppml_diag* out, void* stream);
 const double* ppml_dt_device(const ppml_grid* g);
 
 /* Measurement hook (not part of the paper's method).  enable != 0: every following
- * ppml_step records CUDA events on its stream around each of its kernels (Eulerian,
- * Lagrangian, finalize) and accumulates their durations; enable == 0 stops recording.
+ * ppml_step records CUDA events on its stream around each of its stages (Eulerian,
+ * Lagrangian) and accumulates their durations; enable == 0 stops recording.
  * Do not enable while capturing a CUDA graph.  Resets the accumulated times. */
 int ppml_profile(ppml_grid* g, int enable);
 
-/* Accumulated kernel durations in milliseconds (ms[0] Eulerian, ms[1] Lagrangian,
- * ms[2] finalize) and the number of profiled steps.  Synchronizes the device. */
+/* Accumulated stage durations in milliseconds (ms[0] Eulerian, ms[1] Lagrangian with the
+ * reduction of its partials, ms[2] what lies between that and the step's end: the event
+ * resolution) and the number of profiled steps.  Synchronizes the device. */
 int ppml_kernel_times(ppml_grid* g, double ms[3], long long* steps);
 
 /* ------------------------------------------------------------ step without allocation
@@ -293,7 +296,7 @@ int ppml_kernel_times(ppml_grid* g, double ms[3], long long* steps);
  * memory budget, real-time loops that must not allocate.  It performs the same step as
  * ppml_step (same kernels) without a handle: U*, the reduction partials and the step
  * scalars live in a fixed device buffer inside libppml.so sized for grids of at most
- * PPML_NOALLOC_MAX_CELLS cells (about 12 MB, held on every GPU that loads the library
+ * PPML_NOALLOC_MAX_CELLS cells (about 15 MB, held on every GPU that loads the library
  * until the process exits).  Nothing is allocated by the call (no cudaMalloc/cudaFree).
  *   d         the problem statement (as for ppml_init_grid); nx*ny*nz above the limit
  *             returns PPML_E_INVAL; d->t_end must be 0 (the call keeps no simulated time,
