@@ -1,7 +1,7 @@
 // Device building blocks of the PPML step (Kulikov & Vorobyov, arXiv:1607.01105),
 // templated on the arithmetic type T (float or double).  Each helper states the passage
 // it implements.  Readings of garbled or silent passages (identical to the ones the
-// project's independent CPU checker takes):
+// project's independent CPU oracle takes):
 //   * Delta q = q^R - q^L (Appendix prints q^L - q^R, contradicting eq. A1 and the
 //     characteristic averages);
 //   * rho_L, rho_R, p_L, p_R inside the Roe averages, lambda and the impedance are the
@@ -9,7 +9,7 @@
 //   * the monotonicity step tests "flat" first, then applies at most one overshoot fix.
 //
 // Precision policy.  The double instantiation is compiled without FMA contraction and
-// evaluates every expression in the same order as the FP64 checker (x/6, 2y/3,
+// evaluates every expression in the same order as the FP64 oracle (x/6, 2y/3,
 // (speed * tau) / h), so the FP64 path reproduces it bit for bit.  The float
 // instantiation uses the cheaper forms (doubled slopes, x * (1/12), y * (2/3),
 // speed * (tau/h)) and FMAs.

@@ -49,6 +49,9 @@ __global__ void apply_reduced_kernel(const double* __restrict__ red, DevScalars*
 
 }  // namespace
 
+// The fewest tiles a launch of the FP32 Lagrangian stage is cut into: one wave of its CTAs.
+constexpr int kFaceTilesMin = 304;
+
 static int launch_finalize(const Partial* P, int nblk, const Finalize& f, cudaStream_t st) {
   finalize_kernel<<<1, kFinThreads, 0, st>>>(P, nblk, f);
   return ppml_check_launch("finalize_kernel");
@@ -61,7 +64,8 @@ struct ppml_grid {
   void* ustar[6];  // [0] unused (rho is not changed by the Eulerian stage)
   void* ustar_lo[5];  // FP32: low parts of U*'s m and rho E ([0] unused)
   Partial* partials;
-  float* face;   // FP32 with three active axes: face velocities of every tile
+  float* face;   // FP32 with three active axes: face velocities of face_tiles tiles
+  int face_tiles;
   void* inflow;  // 36 values of the state's type: the inflow faces' ghost states [face][field]
   int nblk_march, nblk_diag, npartials;  // tiles (partials of a step), diagnostics blocks
   int tiles_x, tiles_y, tiles_z;
@@ -215,7 +219,7 @@ MarchArgs<T> make_args(const ppml_grid* g, double dt_host, const double* dt_dev)
   A.inflow = (const T*)g->inflow;
   A.fin = make_finalize(g, 0, nullptr);
   A.face = (T*)g->face;
-  A.face_tiles = g->nblk_march;
+  A.face_tiles = g->face_tiles;
   A.any_inflow = 0;
   for (int q = 0; q < 6; q++) A.any_inflow |= g->d.bc[q] == PPML_BC_INFLOW;
   return A;
@@ -357,11 +361,19 @@ extern "C" int ppml_init_grid(const ppml_grid_desc* d, const ppml_state* u0, voi
       return ppml_fail(PPML_E_NOMEM, "cudaMalloc of U* low parts (%zu bytes) failed", fbytes);
     }
   }
-  if (d->dtype == PPML_F32 && d->nx > 1 && d->ny > 1 && d->nz > 1 &&
-      cudaMalloc(&g->face, kFaceBytes * (size_t)g->nblk_march) != cudaSuccess) {
-    ppml_free_grid(g);
-    return ppml_fail(PPML_E_NOMEM, "cudaMalloc of the face velocities (%zu bytes) failed",
-                     kFaceBytes * (size_t)g->nblk_march);
+  if (d->dtype == PPML_F32 && d->nx > 1 && d->ny > 1 && d->nz > 1) {
+    // face velocities of every tile, or of as many as fit (then a step takes several launches)
+    g->face_tiles = g->nblk_march;
+    while (cudaMalloc(&g->face, kFaceBytes * (size_t)g->face_tiles) != cudaSuccess) {
+      cudaGetLastError();
+      g->face = nullptr;
+      if (g->face_tiles <= kFaceTilesMin) {
+        ppml_free_grid(g);
+        return ppml_fail(PPML_E_NOMEM, "cudaMalloc of the face velocities (%zu bytes) failed",
+                         kFaceBytes * (size_t)kFaceTilesMin);
+      }
+      g->face_tiles = std::max(kFaceTilesMin, g->face_tiles / 8);
+    }
   }
   if (cudaMalloc(&g->partials, sizeof(Partial) * (size_t)g->npartials) != cudaSuccess ||
       cudaMalloc(&g->dev, sizeof(DevScalars)) != cudaSuccess ||

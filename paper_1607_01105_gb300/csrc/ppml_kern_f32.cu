@@ -23,13 +23,14 @@ cudaError_t prepare_sweeps(float) {
   return e;
 }
 
-bool three_axes(const MarchArgs<float>& A) {
-  return A.g.n[0] > 1 && A.g.n[1] > 1 && A.g.n[2] > 1;
+// Three active axes, and offsets (three halo planes beyond the grid included) of 32 bits.
+bool sweep_grid(const MarchArgs<float>& A) {
+  return A.g.n[0] > 1 && A.g.n[1] > 1 && A.g.n[2] > 1 && offsets_fit(A.g);
 }
 
 // Eulerian stage of plain float states with three active axes.  False: not such a state.
 bool launch_euler_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
-  if (!three_axes(A)) return false;
+  if (!sweep_grid(A)) return false;
   constexpr size_t SM = sizeof(EulerSmem);
   const bool flat = (A.flags & PPML_FIRST_ORDER) != 0;
   if (A.phi) {
@@ -48,11 +49,18 @@ bool launch_euler_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
 
 // Lagrangian stage of plain float states with three active axes: face velocities, then the
 // sweeps; in several launches where the face array does not hold every tile (the
-// allocation-free step).  False: not such a state, nothing launched.
+// allocation-free step, or a handle on a nearly full device), then in x-major order (the
+// results do not depend on it).  False: not such a state, nothing launched.
 bool launch_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
-  if (!A.face || !three_axes(A)) return false;
+  if (!A.face || !sweep_grid(A)) return false;
   MarchArgs<float> B = A;
-  const int per = A.face_tiles >= nblk || A.tile_order != 0 ? nblk : A.face_tiles;
+  const int tiles = A.tiles_x * A.tiles_y * A.tiles_z;
+  int per = nblk;  // (padded orders launch more blocks than there are tiles)
+  if (A.face_tiles < tiles) {
+    B.tile_order = 0;
+    nblk = tiles;
+    per = A.face_tiles;
+  }
   for (int first = 0; first < nblk; first += per) {
     const int n = nblk - first < per ? nblk - first : per;
     B.tile_first = first;

@@ -51,7 +51,7 @@ __device__ __forceinline__ double centre(int i, int n, double h) {
 // fixed-shape tree, so the result does not depend on scheduling.  A warp takes one row
 // (j, k) at a time and sums rho, rho x, rho x^2 over it (each lane its own cells); y and z
 // are the same for the whole row, so the seven moments cost seven more operations per lane
-// and row instead of about 25 FP64 operations per cell (128^3: 136 us before).
+// and row instead of about 25 FP64 operations per cell (128^3 FP32: 136 us before, 75 so).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ rho, Dims D,
                                                           double h, double* __restrict__ part) {
@@ -99,6 +99,7 @@ __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ 
 // half integers times h, so x', y' and their products are exact floats there, each term is a
 // product with its exact error, and the sums are TwoSum pairs (about 2^-45, far below the
 // float potential).  Blocks take planes; z enters once per plane and lane, in double.
+// 128^3: 42 us (75 with FP64 sums).
 constexpr int kPairMax = 2048;
 struct PairSum {
   float hi, lo;
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho
 }
 
 // The cells of the grid's boundary, a thread each (inside the rows of rhs_kernel they would
-// hold up warps of interior cells): the source as above with rho = 0 outside, in FP64, minus
+// hold up warps of interior cells; 128^3 FP32: 125 us then, 21 + 16 apart): the source as above with rho = 0 outside, in FP64, minus
 // the stencil weights times the shell values next to the cell.
 __host__ __device__ __forceinline__ long long edge_cells(const Dims& D) {
   const long long nx = D.n[0], ny = D.n[1], nz = D.n[2];
@@ -440,7 +441,7 @@ __global__ void __launch_bounds__(kThreads) dst_unpack_kernel(const T* __restric
 // on packed FMAs, summing blocks of 16 terms before adding them up (the rounding error of a
 // fast transform).  128^3: 134 M FMAs a pass, 3.4 us at the FMA peak, beside 16.8 MB of
 // traffic; the odd extension, the real transform of 2 (N + 1) points and the unpacking took
-// about 100 us a pass (258 = 2 3 43 is a poor length).  N^2 work: beyond kDenseMax the
+// about 100 us a pass (258 = 2 3 43 is a poor length), this takes 25.  N^2 work: beyond kDenseMax the
 // matrix does not fit and the transform of the extension is used.
 constexpr int kDenseMax = 256;
 constexpr int kDenseCols = 64;

@@ -43,6 +43,12 @@ using IntC = std::integral_constant<int, V>;
 template <bool V>
 using BoolC = std::integral_constant<bool, V>;
 
+// Whether element offsets of the grid, three halo planes beyond it included, fit 32 bits (what
+// the kernels of plain FP32 states and of thin grids address with; the tile kernels take any).
+__host__ __device__ __forceinline__ bool offsets_fit(const GridGeom& g) {
+  return g.ncell + TH * g.nxy < (1ll << 31);
+}
+
 struct TileGeom {
   int i0, j0, k0;
   int id;      // x-major index of the tile (its slot in the per-tile partials)
@@ -294,7 +300,7 @@ __device__ __forceinline__ void sweep_eulerian_faces(VF v, PF pr, RF r, float ga
   hook(TB + 3);
 }
 
-// FP64 line pipeline, every expression in the checker's order: push(q) takes the next
+// FP64 line pipeline, every expression in the oracle's order: push(q) takes the next
 // position p; then q2 is the value and L, R, D, S the parabola of cell p - 2.  FLAT: the
 // first-order variant.
 template <bool FLAT>
@@ -338,7 +344,7 @@ struct LineF64 {
   }
 };
 
-// The Eulerian sweep in FP64, every expression in the checker's order.  Where neither side of
+// The Eulerian sweep in FP64, every expression in the oracle's order.  Where neither side of
 // a face varies, the face solution is the cells' own (v, p) and the impedance and the wave
 // speed, three square roots and two divisions, are not needed.  Rolled: the FP64 pipe binds
 // it and the branches make a long body.
@@ -520,7 +526,7 @@ __device__ __forceinline__ void stage_box_fast(T* box, const T* __restrict__ src
 }
 
 // Face velocities as the sweeps read them.  FP64: v^ itself (the flux and the Courant
-// number are formed as the checker forms them).  FP32: w = v^ th / 2 (th = tau / h), so
+// number are formed as the oracle forms them).  FP32: w = v^ th / 2 (th = tau / h), so
 // that |w| is half the Courant number y and w times the upwind state is half of th times
 // the flux (both exact rescalings of v^ th): the per-field products by th disappear, the
 // sweeps accumulate half divergences and the update subtracts twice their sum.
@@ -656,7 +662,7 @@ __device__ __forceinline__ void lag_line_faces(const float* core, const float* h
 }
 
 // One line of the FP64 Lagrangian stage (arguments as lag_line_faces'; th = tau / h, fw the
-// faces' weights of the characteristic averages), every expression in the checker's order.
+// faces' weights of the characteristic averages), every expression in the oracle's order.
 template <int MODE, bool FLAT, int CS>
 __device__ __forceinline__ void lag_line_f64(const double* core, const double* halo,
                                              const double* vh, const f64::Weights* fw, double th,
@@ -1139,7 +1145,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
 // ====================================================================== Eulerian stage
 
 // eq. SCHintenEulerian: rho eps - (gamma - 1) rho eps th (V+ - V-), one rounding order for
-// every code path (FP32: one FMA; FP64: as written, the checker's order).
+// every code path (FP32: one FMA; FP64: as written, the oracle's order).
 __device__ __forceinline__ float eps_update(float ei, float gm1, float dv) {
   return fmaf(-(gm1 * ei), dv, ei);
 }

@@ -17,6 +17,11 @@
 // time, so three CTAs share an SM, the weights of a face are formed once for two fields, and
 // no staging phase is left: the z sweep reads its columns from global memory itself, a few
 // positions ahead, and leaves them in shared memory for the x and y sweeps.
+//
+// Bound by instruction issue (about half of the slots busy with 16 warps an SM) and the ALU
+// pipe that the minima and selects share; 128 registers a thread rule out a third CTA (at 80:
+// 2844 us for two 256^3 steps against 2685).  256^3, one step, before and after: Eulerian
+// 580 -> 315 us, Lagrangian 1325 -> 592 + 166 us; DRAM traffic 41.7 B/cell, 26.5 + 65.7.
 #pragma once
 #include "ppml_pair.cuh"
 #include "ppml_tile.cuh"
@@ -59,7 +64,8 @@ constexpr int FV_PLANE = FV_W * FV_W;
 // is summed from shared memory and the z part from the thread's last planes; v_z takes nine
 // values of its plane.  Products with the Roe weight sqrt(rho) of plane k - 1 then meet their
 // neighbours through shared memory, remapped so that each face row is stored contiguously.
-// One plane of loads is in flight ahead.
+// One plane of loads is in flight ahead.  Bound by its two barriers a plane (286 instructions
+// a cell, issue 66 % busy); 166 us at 256^3.
 template <bool SPECIAL>  // mirrored or prescribed ghosts may occur
 __device__ __forceinline__ void face_velocity_tile(const MarchArgs<float>& A, const TileGeom& tg,
                                                    const TileMaps32& M, const float th[3],
