@@ -17,6 +17,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 #include "ppml_f64.cuh"
 
 namespace ppml {
@@ -340,6 +342,14 @@ template <>
 struct TableOf<float> {
   using type = FloatPair;
 };
+// A table value in the arithmetic V of the kernel that reads it.
+template <typename V, typename U>
+__device__ __forceinline__ V table_as(U t) {
+  if constexpr (std::is_same_v<V, U>)
+    return t;
+  else
+    return (double)t.x + (double)t.y;
+}
 
 // c / (1 - p t) of the Poisson symbols: p the product of two tables, t the third.  In float
 // pairs every product and the difference keep about 2^-46, so 1 - p t of the smoothest mode
@@ -373,6 +383,7 @@ __device__ __forceinline__ FloatPair over_one_minus(FloatPair c, FloatPair p, Fl
 }
 __device__ __forceinline__ double scaled(double v, double f) { return v * f; }
 __device__ __forceinline__ float scaled(float v, FloatPair f) { return fmaf(v, f.x, v * f.y); }
+__device__ __forceinline__ float scaled(float v, double f) { return (float)((double)v * f); }
 
 // rho eps = (eh + el) - |m|^2 / (2 rho) with rho = rh + rl and m_a = mh_a + ml_a, in
 // double-float (about 44 significant bits), rounded once to float.  Sec. 1.4 (dense

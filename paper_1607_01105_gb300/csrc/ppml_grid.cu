@@ -451,6 +451,11 @@ double ppml_table_value(double x, bool f64) {
   return r;
 }
 
+bool ppml_pair_range(double c, double factor) {
+  const double a = fabs(c);
+  return a == 0.0 || (a >= 0x1p-90 && a * std::max(factor, 1.0) <= 0x1p120);
+}
+
 extern "C" int ppml_poisson_periodic(ppml_grid* g, const void* rho, void* phi, double G,
                                      void* stream) {
   ppml_clear_error();
@@ -492,9 +497,13 @@ extern "C" int ppml_poisson_periodic(ppml_grid* g, const void* rho, void* phi, d
   if (r != CUFFT_SUCCESS) return ppml_fail(PPML_E_CUDA, "cuFFT forward failed (%d)", (int)r);
   const double h = g->d.h[0];
   const double coef = -(2.0 / 3.0) * M_PI * G * h * h / ((double)n[0] * n[1] * n[2]);
-  const double c = ppml_table_value(coef, f64);
-  int rc = f64 ? launch_poisson_symbol<double>(g->spec, g->tables, mx, n[1], n[2], c, st)
-               : launch_poisson_symbol<float>(g->spec, g->tables, mx, n[1], n[2], c, st);
+  // float pairs take any coefficient whose quotients stay floats: the largest is that of the
+  // smoothest mode, (3/2) (N / pi)^2 times it.  Others (cells of 1e24 cm with G in CGS units)
+  // are formed in double, as on FP64 grids.
+  const double longest = std::max(n[0], std::max(n[1], n[2]));
+  const bool pairs = ppml_pair_range(coef, 1.5 * (longest / M_PI) * (longest / M_PI));
+  int rc = f64 ? launch_poisson_symbol<double>(g->spec, g->tables, mx, n[1], n[2], coef, false, st)
+               : launch_poisson_symbol<float>(g->spec, g->tables, mx, n[1], n[2], coef, pairs, st);
   if (rc) return rc;
   r = f64 ? cufftExecZ2D(g->fft_inv, (cufftDoubleComplex*)g->spec, (cufftDoubleReal*)phi)
           : cufftExecC2R(g->fft_inv, (cufftComplex*)g->spec, (cufftReal*)phi);

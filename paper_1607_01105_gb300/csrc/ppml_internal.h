@@ -34,3 +34,6 @@ void ppml_fourier_free(FourierState* s);
 // x as a kernel's table holds it (TableOf in ppml_device.cuh): a double (f64), or its float
 // pair (hi, lo) in a double's storage.
 double ppml_table_value(double x, bool f64);
+// Whether a kernel can take the constant c, and quotients of up to `factor` times it, as float
+// pairs: neither overflows, and the low part keeps its bits.
+bool ppml_pair_range(double c, double factor);

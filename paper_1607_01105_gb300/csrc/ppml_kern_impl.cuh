@@ -159,27 +159,27 @@ int launch_diag<PPML_REAL>(const MarchArgs<PPML_REAL>& A, int nblk, cudaStream_t
 namespace {
 // Multiply the half spectrum (R2C layout: kx in [0, nx/2], ky, kz) by the inverse symbol of
 // the 27-point stencil, coef / (1 - tx ty tz); tables hold 1 - (2/3) sin^2(pi k / N) per axis
-// (FP32 grids: as float pairs, coef too).  A warp takes one row of kx at a time, so tz ty is
-// formed once per row.  512^3 FP32: 1986 us with an FP64 division per value, 204 us in pairs.
-template <typename T>
+// (FP32 grids: as float pairs).  A warp takes one row of kx at a time, so tz ty is formed once
+// per row.  V: the arithmetic, double or (FP32 grids) float pairs: 512^3 FP32: 1986 us with an
+// FP64 division per value, 204 us in pairs.
+template <typename T, typename V>
 __global__ void __launch_bounds__(256) poisson_symbol_kernel(T* spec, const double* __restrict__ tab,
-                                                             int mx, int ny, int nz, double coef) {
-  using V = typename TableOf<T>::type;
+                                                             int mx, int ny, int nz, V coef) {
+  using U = typename TableOf<T>::type;
   using T2 = std::conditional_t<sizeof(T) == 8, double2, float2>;
-  static_assert(sizeof(V) == sizeof(double), "a table value fills a double's storage");
+  static_assert(sizeof(U) == sizeof(double), "a table value fills a double's storage");
   T2* const s = reinterpret_cast<T2*>(spec);
-  const V* const tx = reinterpret_cast<const V*>(tab);
-  const V* const ty = tx + mx;
-  const V* const tz = ty + ny;
-  const V c = *reinterpret_cast<const V*>(&coef);
+  const U* const tx = reinterpret_cast<const U*>(tab);
+  const U* const ty = tx + mx;
+  const U* const tz = ty + ny;
   const int lane = threadIdx.x & 31;
   const long long rows = (long long)ny * nz;
   const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
   for (long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < rows;
        row += warps) {
-    const V tzy = table_product(tz[row / ny], ty[row % ny]);
+    const V tzy = table_product(table_as<V>(tz[row / ny]), table_as<V>(ty[row % ny]));
     for (int kx = lane; kx < mx; kx += 32) {
-      const V f = over_one_minus(c, tzy, tx[kx]);
+      const V f = over_one_minus(coef, tzy, table_as<V>(tx[kx]));
       T2 v = s[row * mx + kx];
       v.x = scaled(v.x, f);
       v.y = scaled(v.y, f);
@@ -188,14 +188,28 @@ __global__ void __launch_bounds__(256) poisson_symbol_kernel(T* spec, const doub
     }
   }
 }
+
+template <typename T>
+void launch_symbol(T* spec, const double* tab, int mx, int ny, int nz, double coef, bool pairs,
+                   cudaStream_t st) {
+  const long long rows = (long long)ny * nz;
+  const int blocks = (int)((rows + 7) / 8 < 152 * 8 ? (rows + 7) / 8 : 152 * 8);
+  if constexpr (sizeof(T) == 4) {
+    if (pairs) {
+      const float hi = (float)coef;
+      const FloatPair c = {hi, (float)(coef - (double)hi)};
+      poisson_symbol_kernel<T, FloatPair><<<blocks, 256, 0, st>>>(spec, tab, mx, ny, nz, c);
+      return;
+    }
+  }
+  poisson_symbol_kernel<T, double><<<blocks, 256, 0, st>>>(spec, tab, mx, ny, nz, coef);
+}
 }  // namespace
 
 template <>
 int launch_poisson_symbol<PPML_REAL>(void* spec, const double* tab, int mx, int ny, int nz,
-                                     double coef, cudaStream_t st) {
-  const long long rows = (long long)ny * nz;
-  const int blocks = (int)((rows + 7) / 8 < 152 * 8 ? (rows + 7) / 8 : 152 * 8);
-  poisson_symbol_kernel<PPML_REAL><<<blocks, 256, 0, st>>>((PPML_REAL*)spec, tab, mx, ny, nz, coef);
+                                     double coef, bool pairs, cudaStream_t st) {
+  launch_symbol<PPML_REAL>((PPML_REAL*)spec, tab, mx, ny, nz, coef, pairs, st);
   return ppml_check_launch("poisson_symbol_kernel");
 }
 

@@ -21,9 +21,10 @@ template <typename T>
 int launch_lagrangian(const MarchArgs<T>& A, int nblk, cudaStream_t st);
 template <typename T>
 int launch_diag(const MarchArgs<T>& A, int nblk, cudaStream_t st);
+// pairs: FP32 grids, in float pairs (the coefficient within their range), else in double.
 template <typename T>
 int launch_poisson_symbol(void* spec, const double* tab, int mx, int ny, int nz, double coef,
-                          cudaStream_t st);
+                          bool pairs, cudaStream_t st);
 // Batched 1D problems: the vacuum thresholds of all ninst instances (instance = CTA index),
 // then one CTA per instance of order[0 .. ninst), or one cluster of two CTAs per work item
 // of items[0 .. nitems) (nlmax: the largest half of a split instance, nmax: the largest
@@ -51,7 +52,7 @@ int launch_batch_cluster(T* rho, T* m, T* en, T* ei, BatchLo<T> lo, InstDev* ins
   int launch_diag<R>(const MarchArgs<R>& A, int nblk, cudaStream_t st);                       \
   template <>                                                                                \
   int launch_poisson_symbol<R>(void* spec, const double* tab, int mx, int ny, int nz,          \
-                               double coef, cudaStream_t st);                                  \
+                               double coef, bool pairs, cudaStream_t st);                      \
   template <>                                                                                \
   int launch_batch_vacuum<R>(const R* rho, InstDev* inst, int ninst, cudaStream_t st);        \
   template <>                                                                                \
