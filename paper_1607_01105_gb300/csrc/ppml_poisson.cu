@@ -246,8 +246,9 @@ __device__ __forceinline__ void pair_add(SourcePair& s, float x) {
 
 // Right-hand side 4 pi G h^2 (rho [+ D7 rho / 12]) of the cells away from the boundary, written
 // into the potential array (the work array); boundary cells are left to rhs_edge_kernel.  One
-// row of x per warp pass.
-template <typename T>
+// row of x per warp pass.  PAIRS: FP32 grids in float pairs, for constants in their range
+// (ppml_pair_range).
+template <typename T, bool PAIRS>
 __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho, T* __restrict__ out,
                                                        Dims D, double h, double G, int printed) {
   const double c = 4.0 * M_PI * G * h * h;
@@ -263,29 +264,39 @@ __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho
     for (int i = 1 + lane; i < nx - 1; i += 32) {
       const long long idx = row * nx + i;
       const T rc = rho[idx];
-      if (printed) {
-        if constexpr (sizeof(T) == 4)
-          out[idx] = fmaf(rc, ch, rc * cl);
-        else
-          out[idx] = c * rc;
-        continue;
+      T nb[6] = {};
+      if (!printed) {
+        nb[0] = rho[idx - 1];
+        nb[1] = rho[idx + 1];
+        nb[2] = rho[idx - nx];
+        nb[3] = rho[idx + nx];
+        nb[4] = rho[idx - D.nxy];
+        nb[5] = rho[idx + D.nxy];
       }
-      const T nb[6] = {rho[idx - 1],  rho[idx + 1],     rho[idx - nx],
-                       rho[idx + nx], rho[idx - D.nxy], rho[idx + D.nxy]};
-      if constexpr (sizeof(T) == 4) {
-        // c / 12 (6 rho + sum), the products to 2^-46
-        SourcePair s = {6.0f * rc, 0.0f};
-        s.lo = fmaf(6.0f, rc, -s.hi);
+      auto in_double = [&]() -> T {
+        if (printed) return (T)(c * (double)rc);
+        double lap = -6.0 * (double)rc;
 #pragma unroll
-        for (int q = 0; q < 6; q++) pair_add(s, nb[q]);
-        const float p = s.hi * c12h;
-        out[idx] = p + (fmaf(s.hi, c12h, -p) + fmaf(s.hi, c12l, s.lo * c12h));
+        for (int q = 0; q < 6; q++) lap += (double)nb[q];
+        return (T)(c * ((double)rc + lap / 12.0));
+      };
+      T v;
+      if constexpr (PAIRS) {
+        if (printed) {
+          v = fmaf(rc, ch, rc * cl);
+        } else {
+          // c / 12 (6 rho + sum), the products to 2^-46
+          SourcePair s = {6.0f * rc, 0.0f};
+          s.lo = fmaf(6.0f, rc, -s.hi);
+#pragma unroll
+          for (int q = 0; q < 6; q++) pair_add(s, nb[q]);
+          const float p = s.hi * c12h;
+          v = p + (fmaf(s.hi, c12h, -p) + fmaf(s.hi, c12l, s.lo * c12h));
+        }
       } else {
-        double lap = -6.0 * rc;
-#pragma unroll
-        for (int q = 0; q < 6; q++) lap += nb[q];
-        out[idx] = c * (rc + lap / 12.0);
+        v = in_double();
       }
+      out[idx] = v;
     }
   }
 }
@@ -736,7 +747,12 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   if ((rc = ppml_check_launch("moment_final_kernel"))) return rc;
   shell_kernel<<<blocks_for(shell_cells(D)), kThreads, 0, st>>>(D, h, G, s->mom, s->shell);
   if ((rc = ppml_check_launch("shell_kernel"))) return rc;
-  rhs_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, h, G, printed);
+  const double source = 4.0 * M_PI * G * h * h;
+  if (sizeof(T) == sizeof(float) && ppml_pair_range(source, 1.0) && ppml_pair_range(source / 12.0, 1.0))
+    rhs_kernel<float, true><<<blocks_for(D.ncell), kThreads, 0, st>>>((const float*)rho, (float*)phi,
+                                                                      D, h, G, printed);
+  else
+    rhs_kernel<T, false><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, h, G, printed);
   if ((rc = ppml_check_launch("rhs_kernel"))) return rc;
   rhs_edge_kernel<T><<<blocks_for(edge_cells(D)), kThreads, 0, st>>>(rho, phi, D, h, G, s->shell,
                                                                      printed);

@@ -50,3 +50,20 @@ def test_periodic_potential_in_any_units(n, h, scale, G):
     ref = poisson.solve_periodic(rho, h, G)
     assert np.all(np.isfinite(got))
     assert np.max(np.abs(got - ref)) <= TOL * np.max(np.abs(ref))
+
+
+def _blob(n):
+    x, y, z = [(np.arange(m) + 0.5) / m - 0.5 for m in n]
+    z, y, x = np.meshgrid(z, y, x, indexing="ij")
+    return np.exp(-(x * x + 1.5 * (y - 0.1) ** 2 + 2.0 * (z + 0.05) ** 2) / 0.05)
+
+
+# grids of the dense transforms and of the transforms of the odd extension
+@pytest.mark.parametrize("n", [(20, 24, 28), (300, 12, 10)])
+@pytest.mark.parametrize("printed", [False, True])
+@pytest.mark.parametrize("h,scale,G", UNITS)
+def test_isolated_potential_in_any_units(n, printed, h, scale, G):
+    rho, got = _solve(n, h, scale * _blob(n), G, True, printed)
+    ref = poisson.solve_isolated(rho, h, G, printed_rhs=printed)
+    assert np.all(np.isfinite(got))
+    assert np.max(np.abs(got - ref)) <= TOL * np.max(np.abs(ref))
