@@ -22,6 +22,7 @@
 // the half spectrum live in buffers kept by the solver state between calls.
 #include <cuda_runtime.h>
 #include <cufft.h>
+#include <float.h>
 #include <math.h>
 
 #include <vector>
@@ -98,7 +99,9 @@ __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ 
 // The same on FP32 grids of at most kPairMax cells per axis, in float pairs: the centres are
 // half integers times h, so x', y' and their products are exact floats there, each term is a
 // product with its exact error, and the sums are TwoSum pairs (about 2^-45, far below the
-// float potential).  Blocks take planes; z enters once per plane and lane, in double.
+// float potential).  Blocks take planes; z enters once per plane and lane, in double.  Sums
+// that overflow a float (densities of 1e26 and more) or lie where the products' errors
+// underflow are formed again in double.
 // 128^3: 42 us (75 with FP64 sums).
 constexpr int kPairMax = 2048;
 struct PairSum {
@@ -119,22 +122,44 @@ __global__ void __launch_bounds__(kThreads) moment_pair_kernel(const float* __re
   const double vol = h * h * h;
   for (int k = blockIdx.x; k < D.n[2]; k += gridDim.x) {
     PairSum s[6] = {};  // m, m x, m y, m x x, m y y, m x y
-    for (int j = warp; j < D.n[1]; j += kThreads / 32) {
-      const float y = (float)j + 0.5f - 0.5f * (float)D.n[1];
-      const float* row = rho + (long long)k * D.nxy + (long long)j * D.n[0];
-      for (int i = lane; i < D.n[0]; i += 32) {
-        const float x = (float)i + 0.5f - 0.5f * (float)D.n[0], m = row[i];
-        s[0].add(m, 1.0f);
-        s[1].add(m, x);
-        s[2].add(m, y);
-        s[3].add(m, x * x);
-        s[4].add(m, y * y);
-        s[5].add(m, x * y);
+    auto cells = [&](auto add) {  // add(m, x, y) for the thread's cells of the plane
+      for (int j = warp; j < D.n[1]; j += kThreads / 32) {
+        const float y = (float)j + 0.5f - 0.5f * (float)D.n[1];
+        const float* row = rho + (long long)k * D.nxy + (long long)j * D.n[0];
+        for (int i = lane; i < D.n[0]; i += 32)
+          add(row[i], (float)i + 0.5f - 0.5f * (float)D.n[0], y);
       }
+    };
+    cells([&](float m, float x, float y) {
+      s[0].add(m, 1.0f);
+      s[1].add(m, x);
+      s[2].add(m, y);
+      s[3].add(m, x * x);
+      s[4].add(m, y * y);
+      s[5].add(m, x * y);
+    });
+    double t[6];
+    bool in_range = s[0].hi == 0.0f || fabsf(s[0].hi) >= 0x1p-110f;
+#pragma unroll
+    for (int q = 0; q < 6; q++) {
+      t[q] = s[q].value();
+      in_range = in_range && fabs(t[q]) <= (double)FLT_MAX;
     }
-    const double z = centre(k, D.n[2], h), m0 = vol * s[0].value(), mx = vol * h * s[1].value(),
-                 my = vol * h * s[2].value(), mxx = vol * h * h * s[3].value(),
-                 myy = vol * h * h * s[4].value(), mxy = vol * h * h * s[5].value();
+    if (!in_range) {
+#pragma unroll
+      for (int q = 0; q < 6; q++) t[q] = 0.0;
+      cells([&](float m, float x, float y) {
+        const double dm = m, dx = dm * x, dy = dm * y;
+        t[0] += dm;
+        t[1] += dx;
+        t[2] += dy;
+        t[3] += dx * x;
+        t[4] += dy * y;
+        t[5] += dx * y;
+      });
+    }
+    const double z = centre(k, D.n[2], h), m0 = vol * t[0], mx = vol * h * t[1], my = vol * h * t[2],
+                 mxx = vol * h * h * t[3], myy = vol * h * h * t[4], mxy = vol * h * h * t[5];
     acc[0] += m0;
     acc[1] += z * z * m0 + myy;
     acc[2] += mxx + z * z * m0;
@@ -247,7 +272,8 @@ __device__ __forceinline__ void pair_add(SourcePair& s, float x) {
 // Right-hand side 4 pi G h^2 (rho [+ D7 rho / 12]) of the cells away from the boundary, written
 // into the potential array (the work array); boundary cells are left to rhs_edge_kernel.  One
 // row of x per warp pass.  PAIRS: FP32 grids in float pairs, for constants in their range
-// (ppml_pair_range).
+// (ppml_pair_range); a cell whose pair overflows (the sum of densities above 2.8e37) is formed
+// in double.
 template <typename T, bool PAIRS>
 __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho, T* __restrict__ out,
                                                        Dims D, double h, double G, int printed) {
@@ -293,6 +319,7 @@ __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho
           const float p = s.hi * c12h;
           v = p + (fmaf(s.hi, c12h, -p) + fmaf(s.hi, c12l, s.lo * c12h));
         }
+        if (!(fabsf(v) <= FLT_MAX)) v = in_double();
       } else {
         v = in_double();
       }

@@ -67,3 +67,14 @@ def test_isolated_potential_in_any_units(n, printed, h, scale, G):
     ref = poisson.solve_isolated(rho, h, G, printed_rhs=printed)
     assert np.all(np.isfinite(got))
     assert np.max(np.abs(got - ref)) <= TOL * np.max(np.abs(ref))
+
+
+# densities near the ends of the float range: second moments and neighbour sums beyond it,
+# products' errors below it
+@pytest.mark.parametrize("n", [(64, 64, 48), (300, 20, 12), (20, 40, 41)])
+@pytest.mark.parametrize("scale,G", [(3e38, 1e-23), (1e37, 1e-20), (1e35, 1e-37), (1e-37, 1e25)])
+def test_isolated_potential_of_any_density(n, scale, G):
+    rho, got = _solve(n, 0.03, scale * _blob(n), G, True)
+    ref = poisson.solve_isolated(rho, 0.03, G)
+    assert np.all(np.isfinite(got))
+    assert np.max(np.abs(got - ref)) <= TOL * np.max(np.abs(ref))
