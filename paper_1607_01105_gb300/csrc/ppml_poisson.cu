@@ -25,6 +25,7 @@
 #include <float.h>
 #include <math.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "../../include/ppml.h"
@@ -48,24 +49,46 @@ __device__ __forceinline__ double centre(int i, int n, double h) {
   return ((double)i + 0.5 - 0.5 * (double)n) * h;
 }
 
+// How rows of x are spread over threads: a group of `lanes` threads (a power of two: short
+// rows share a warp) takes a piece of at most `length` cells of one row, `pieces` to a row
+// (more than one where the rows are fewer than the groups that should be busy).
+struct RowPieces {
+  int lanes, pieces, length;
+};
+RowPieces row_pieces(int nx, long long rows, long long groups_wanted) {
+  RowPieces p;
+  p.lanes = 1;
+  while (p.lanes < nx && p.lanes < 32) p.lanes *= 2;
+  const long long most = (nx + 8LL * p.lanes - 1) / (8 * p.lanes);  // eight cells a thread
+  const long long want = std::max(1LL, groups_wanted / rows);
+  p.pieces = (int)std::min(want, most);
+  p.length = ((nx + p.pieces - 1) / p.pieces + p.lanes - 1) / p.lanes * p.lanes;
+  return p;
+}
+
 // Stage 1a: per-block FP64 partial moments of the masses rho h^3, fixed block count and a
-// fixed-shape tree, so the result does not depend on scheduling.  A warp takes one row
-// (j, k) at a time and sums rho, rho x, rho x^2 over it (each lane its own cells); y and z
-// are the same for the whole row, so the seven moments cost seven more operations per lane
-// and row instead of about 25 FP64 operations per cell (128^3 FP32: 136 us before, 75 so).
+// fixed-shape tree, so the result does not depend on scheduling.  A group of threads takes a
+// row (j, k), or a piece of it, at a time and sums rho, rho x, rho x^2 over it (each lane its
+// own cells); y and z are the same for the whole row, so the seven moments cost seven more
+// operations per lane and row instead of about 25 FP64 operations per cell (128^3 FP32: 136 us
+// before, 75 so).  A warp to every row, short or not: 1024 x 1024 cells in the y-z plane took
+// 2.26 ms (81 us so), 65536 x 4 x 4 1.20 ms (42).
 template <typename T>
 __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ rho, Dims D,
-                                                          double h, double* __restrict__ part) {
+                                                          RowPieces R, double h,
+                                                          double* __restrict__ part) {
   double acc[kMoments] = {0, 0, 0, 0, 0, 0, 0};
   const double vol = h * h * h;
-  const int lane = threadIdx.x & 31;
-  const long long rows = (long long)D.n[1] * D.n[2];
-  const long long warps = (long long)gridDim.x * (kThreads / 32);
-  for (long long r = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); r < rows;
-       r += warps) {
+  const int lane = threadIdx.x & (R.lanes - 1), per_block = kThreads / R.lanes;
+  const long long items = (long long)D.n[1] * D.n[2] * R.pieces;
+  const long long groups = (long long)gridDim.x * per_block;
+  for (long long q = (long long)blockIdx.x * per_block + threadIdx.x / R.lanes; q < items;
+       q += groups) {
+    const long long r = q / R.pieces;
+    const int i0 = (int)(q % R.pieces) * R.length, i1 = min(i0 + R.length, D.n[0]);
     const int j = (int)(r % D.n[1]), k = (int)(r / D.n[1]);
     double m0 = 0.0, m1 = 0.0, m2 = 0.0;
-    for (int i = lane; i < D.n[0]; i += 32) {
+    for (int i = i0 + lane; i < i1; i += R.lanes) {
       const double x = centre(i, D.n[0], h), m = (double)rho[r * D.n[0] + i], mx = m * x;
       m0 += m;
       m1 += mx;
@@ -96,14 +119,19 @@ __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ 
   if (threadIdx.x < kMoments) part[(size_t)blockIdx.x * kMoments + threadIdx.x] = s[threadIdx.x][0];
 }
 
-// The same on FP32 grids of at most kPairMax cells per axis, in float pairs: the centres are
-// half integers times h, so x', y' and their products are exact floats there, each term is a
-// product with its exact error, and the sums are TwoSum pairs (about 2^-45, far below the
-// float potential).  Blocks take planes; z enters once per plane and lane, in double.  Sums
-// that overflow a float (densities of 1e26 and more) or lie where the products' errors
-// underflow are formed again in double.
-// 128^3: 42 us (75 with FP64 sums).
+// The same on FP32 grids of at most kPairMax cells along x and y, in float pairs: the centres
+// are half integers times h, so x', y' and their products are exact floats there, each term is
+// a product with its exact error, and the sums are TwoSum pairs (about 2^-45, far below the
+// float potential).  A block takes some rows of one plane at a time; z enters once per thread
+// and item, in double: about 60 FP64 instructions a warp, so an item has at least kPairItem
+// cells (eight a thread), and grids of smaller planes take moment_kernel.  Planes are cut
+// where they are fewer than kPairBlocks (two CTAs an SM): 2048 x 2048 x 1 takes 8.0 ms on one
+// CTA, 44 us so, 128 planes of 128 x 256 cells 39 and 29 us.  Sums that overflow a float
+// (densities of 1e26 and more) or lie where the products' errors underflow are formed again in
+// double.
 constexpr int kPairMax = 2048;
+constexpr int kPairItem = 2048;
+constexpr int kPairBlocks = 304;
 struct PairSum {
   float hi, lo;
   __device__ __forceinline__ void add(float m, float c) {  // += m c
@@ -116,17 +144,23 @@ struct PairSum {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 __global__ void __launch_bounds__(kThreads) moment_pair_kernel(const float* __restrict__ rho, Dims D,
-                                                               double h, double* __restrict__ part) {
+                                                               RowPieces R, int cuts, double h,
+                                                               double* __restrict__ part) {
   double acc[kMoments] = {0, 0, 0, 0, 0, 0, 0};
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int lane = threadIdx.x & (R.lanes - 1), groups = kThreads / R.lanes;
+  const int rows = (D.n[1] + cuts - 1) / cuts;  // of an item
   const double vol = h * h * h;
-  for (int k = blockIdx.x; k < D.n[2]; k += gridDim.x) {
+  for (long long item = blockIdx.x; item < (long long)D.n[2] * cuts; item += gridDim.x) {
+    const int k = (int)(item / cuts), j0 = (int)(item % cuts) * rows;
+    const int pieces = max(min(rows, D.n[1] - j0), 0) * R.pieces;
     PairSum s[6] = {};  // m, m x, m y, m x x, m y y, m x y
-    auto cells = [&](auto add) {  // add(m, x, y) for the thread's cells of the plane
-      for (int j = warp; j < D.n[1]; j += kThreads / 32) {
+    auto cells = [&](auto add) {  // add(m, x, y) for the thread's cells of the item
+      for (int q = threadIdx.x / R.lanes; q < pieces; q += groups) {
+        const int j = j0 + q / R.pieces, i0 = q % R.pieces * R.length;
         const float y = (float)j + 0.5f - 0.5f * (float)D.n[1];
         const float* row = rho + (long long)k * D.nxy + (long long)j * D.n[0];
-        for (int i = lane; i < D.n[0]; i += 32)
+        const int i1 = min(i0 + R.length, D.n[0]);
+        for (int i = i0 + lane; i < i1; i += R.lanes)
           add(row[i], (float)i + 0.5f - 0.5f * (float)D.n[0], y);
       }
     };
@@ -760,13 +794,19 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   for (int a = 0; a < 3; a++) D.n[a] = s->n[a];
   D.nxy = (long long)D.n[0] * D.n[1];
   D.ncell = D.nxy * D.n[2];
-  const int nb = blocks_for(D.ncell) < kMaxMomentBlocks ? blocks_for(D.ncell) : kMaxMomentBlocks;
-  int blocks = nb;
-  if (sizeof(T) == sizeof(float) && D.n[0] <= kPairMax && D.n[1] <= kPairMax) {
-    blocks = D.n[2] < kMaxMomentBlocks ? D.n[2] : kMaxMomentBlocks;
-    moment_pair_kernel<<<blocks, kThreads, 0, st>>>((const float*)rho, D, h, s->part);
+  int blocks;
+  if (sizeof(T) == sizeof(float) && D.n[0] <= kPairMax && D.n[1] <= kPairMax && D.nxy >= kPairItem) {
+    const int most = (int)std::min<long long>(D.nxy / kPairItem, D.n[1]);
+    const int cuts = std::min((kPairBlocks + D.n[2] - 1) / D.n[2], most);
+    const int rows = (D.n[1] + cuts - 1) / cuts;
+    RowPieces R = row_pieces(D.n[0], rows, 1);
+    R = row_pieces(D.n[0], rows, kThreads / R.lanes);
+    blocks = (int)std::min<long long>((long long)D.n[2] * cuts, kMaxMomentBlocks);
+    moment_pair_kernel<<<blocks, kThreads, 0, st>>>((const float*)rho, D, R, cuts, h, s->part);
   } else {
-    moment_kernel<T><<<nb, kThreads, 0, st>>>(rho, D, h, s->part);
+    blocks = std::min(blocks_for(D.ncell), kMaxMomentBlocks);
+    const RowPieces R = row_pieces(D.n[0], D.nxy / D.n[0] * D.n[2], (long long)blocks * (kThreads / 32));
+    moment_kernel<T><<<blocks, kThreads, 0, st>>>(rho, D, R, h, s->part);
   }
   int rc = ppml_check_launch("moment_kernel");
   if (rc) return rc;

@@ -1,0 +1,75 @@
+"""The Poisson solves on grids far from a cube (planes, columns, few or short rows): values
+against the oracle, and no kernel that such a shape leaves to a few threads.  The latter compares
+a kernel's device time on the shape with its time on a near-cube of as many cells: the work is
+the same, so a ratio over the bar means that most of the device idles."""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+if not torch.cuda.is_available():
+    pytest.skip("needs a CUDA device", allow_module_level=True)
+
+from oracle import poisson  # noqa: E402
+from paper_1607_01105_gb300 import ppml  # noqa: E402
+
+pytestmark = pytest.mark.gpu
+
+F32, F64 = ppml.PPML_F32, ppml.PPML_F64
+O, P = ppml.OUTFLOW, ppml.PERIODIC
+TOL = {F32: 2e-5, F64: 1e-11}  # of the largest potential
+
+
+def _solver(n, dtype, isolated):
+    x, y, z = [(np.arange(m) + 0.5) / m - 0.5 for m in n]
+    z, y, x = np.meshgrid(z, y, x, indexing="ij")
+    rho = np.exp(-(x * x + 1.5 * (y - 0.1) ** 2 + 2.0 * (z + 0.05) ** 2) / 0.05).astype(np.float32)
+    r = torch.as_tensor(rho.ravel()).to("cuda", ppml.torch_dtype(dtype))
+    grid = ppml.Grid(n, (0.05,) * 3, 1.4, 0.2, (O if isolated else P,) * 6, dtype,
+                     u0=[torch.ones_like(r) for _ in range(6)])
+    phi = torch.empty_like(r)
+    solve = grid.poisson_isolated if isolated else grid.poisson_periodic
+    return rho.astype(np.float64), phi, lambda: solve(r, phi, 1.1)
+
+
+SHAPES = [(256, 256, 1), (300, 1, 40), (1, 300, 40), (4, 3, 700), (700, 4, 3), (3, 600, 5), (2049, 8, 1),
+          (1, 1, 500), (64, 48, 40)]
+
+
+@pytest.mark.parametrize("dtype", [F32, F64])
+@pytest.mark.parametrize("n", SHAPES)
+def test_isolated_shapes(n, dtype):
+    rho, phi, solve = _solver(n, dtype, True)
+    solve()
+    ref = poisson.solve_isolated(rho, 0.05, 1.1)
+    got = phi.double().cpu().numpy().reshape(ref.shape)
+    assert np.max(np.abs(got - ref)) <= TOL[dtype] * np.max(np.abs(ref))
+
+
+def _kernel_us(solve, names):
+    """Device time per call of the kernels whose names contain one of `names`."""
+    from torch.profiler import ProfilerActivity, profile
+    for _ in range(3):
+        solve()
+    for _ in range(3):  # (a process's first session may record nothing)
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            for _ in range(5):
+                solve()
+            torch.cuda.synchronize()
+        us = [e.device_time_total for e in prof.key_averages() if any(n in e.key for n in names)]
+        if us:
+            break
+    assert us, names
+    return sum(us) / 5
+
+
+BAR = 3.0  # the shapes' kernels take 1 to 2 times the near-cube's; on a few threads 5 to 20
+
+
+@pytest.mark.parametrize("dtype,n,cube", [
+    (F32, (2048, 2048, 1), (128, 256, 128)), (F32, (1024, 1024, 4), (128, 256, 128)),
+    (F32, (2048, 1, 2048), (128, 256, 128)), (F64, (65536, 4, 4), (128, 128, 64)),
+    (F64, (1, 1024, 1024), (128, 128, 64))])
+def test_moments_of_any_shape_fill_the_device(dtype, n, cube):
+    t = [_kernel_us(_solver(m, dtype, True)[2], ("moment_kernel", "moment_pair_kernel")) for m in (n, cube)]
+    assert t[0] <= BAR * t[1], t
