@@ -329,6 +329,24 @@ __device__ __forceinline__ void df_split(double x, float& hi, float& lo) {
   lo = (float)(x - (double)hi);
 }
 
+// Quotients by a divisor known at launch, for 0 <= n < 2^31 (any cell index): n m >> s with
+// m = 2^s / d rounded up and s = 31 + ceil(log2 d), whose error n (m d - 2^s) < 2^s leaves the
+// quotient's integer part (Granlund and Montgomery, "Division by invariant integers using
+// multiplication", 1994).  A 64-bit division takes some 60 instructions, this three.
+struct IndexDivisor {
+  unsigned m;
+  int s;
+  explicit IndexDivisor(int d) {
+    int l = 0;
+    while ((1ll << l) < d) l++;
+    s = 31 + l;
+    m = (unsigned)((1ull << s) / (unsigned)d + 1u);
+  }
+  __host__ __device__ unsigned quotient(unsigned n) const {
+    return (unsigned)(((unsigned long long)n * m) >> s);
+  }
+};
+
 // A value of a host-formed table as a kernel of either precision reads it: the double
 // itself, or its float pair (hi, lo).
 struct FloatPair {

@@ -51,19 +51,49 @@ __device__ __forceinline__ double centre(int i, int n, double h) {
 
 // How rows of x are spread over threads: a group of `lanes` threads (a power of two: short
 // rows share a warp) takes a piece of at most `length` cells of one row, `pieces` to a row
-// (more than one where the rows are fewer than the groups that should be busy).
+// (more than one where the rows are fewer than the groups that should be busy, of at least
+// `cells` cells a thread).
 struct RowPieces {
-  int lanes, pieces, length;
+  int log_lanes, pieces, length;
+  IndexDivisor by_pieces, by_ny;
+  unsigned items;  // pieces of all rows
 };
-RowPieces row_pieces(int nx, long long rows, long long groups_wanted) {
-  RowPieces p;
-  p.lanes = 1;
-  while (p.lanes < nx && p.lanes < 32) p.lanes *= 2;
-  const long long most = (nx + 8LL * p.lanes - 1) / (8 * p.lanes);  // eight cells a thread
-  const long long want = std::max(1LL, groups_wanted / rows);
-  p.pieces = (int)std::min(want, most);
-  p.length = ((nx + p.pieces - 1) / p.pieces + p.lanes - 1) / p.lanes * p.lanes;
-  return p;
+RowPieces row_pieces(int nx, int ny, long long rows, long long threads, int cells) {
+  int log_lanes = 0;
+  while ((1 << log_lanes) < nx && log_lanes < 5) log_lanes++;
+  const long long lanes = 1 << log_lanes;
+  const long long most = (nx + cells * lanes - 1) / (cells * lanes);
+  const int pieces = (int)std::min(std::max(1LL, threads / lanes / rows), most);
+  const int length = (int)(((nx + pieces - 1) / pieces + lanes - 1) / lanes * lanes);
+  return {log_lanes, pieces, length, IndexDivisor(pieces), IndexDivisor(ny), (unsigned)(rows * pieces)};
+}
+// The rows of a kernel's threads: WARP, rows of a warp each (a constant step).
+template <bool WARP>
+struct RowWalk {
+  int step, lane;
+  unsigned first, groups;
+  __device__ __forceinline__ explicit RowWalk(const RowPieces& R) {
+    const int log_lanes = WARP ? 5 : R.log_lanes;
+    const unsigned per_block = kThreads >> log_lanes;
+    step = 1 << log_lanes;
+    lane = threadIdx.x & (step - 1);
+    first = blockIdx.x * per_block + (threadIdx.x >> log_lanes);
+    groups = gridDim.x * per_block;
+  }
+};
+// The copies of the sine transform load kBatch cells before they store any (one float a thread
+// in flight is half of what the memory takes).
+constexpr int kBatch = 4;
+// Item q: the cells i0, i0 + step, .. < i1 of row (j, k) for this lane.
+struct RowItem {
+  long long row;
+  int j, k, i0, i1;
+};
+__device__ __forceinline__ RowItem row_item(const Dims& D, const RowPieces& R, unsigned q, int lane) {
+  const unsigned row = R.by_pieces.quotient(q), k = R.by_ny.quotient(row);
+  const int i = (int)(q - row * (unsigned)R.pieces) * R.length;
+  return {(long long)row, (int)(row - k * (unsigned)D.n[1]), (int)k, i + lane,
+          min(i + R.length, D.n[0])};
 }
 
 // Stage 1a: per-block FP64 partial moments of the masses rho h^3, fixed block count and a
@@ -73,28 +103,23 @@ RowPieces row_pieces(int nx, long long rows, long long groups_wanted) {
 // operations per lane and row instead of about 25 FP64 operations per cell (128^3 FP32: 136 us
 // before, 75 so).  A warp to every row, short or not: 1024 x 1024 cells in the y-z plane took
 // 2.26 ms (81 us so), 65536 x 4 x 4 1.20 ms (42).
-template <typename T>
+template <typename T, bool WARP>
 __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ rho, Dims D,
                                                           RowPieces R, double h,
                                                           double* __restrict__ part) {
   double acc[kMoments] = {0, 0, 0, 0, 0, 0, 0};
   const double vol = h * h * h;
-  const int lane = threadIdx.x & (R.lanes - 1), per_block = kThreads / R.lanes;
-  const long long items = (long long)D.n[1] * D.n[2] * R.pieces;
-  const long long groups = (long long)gridDim.x * per_block;
-  for (long long q = (long long)blockIdx.x * per_block + threadIdx.x / R.lanes; q < items;
-       q += groups) {
-    const long long r = q / R.pieces;
-    const int i0 = (int)(q % R.pieces) * R.length, i1 = min(i0 + R.length, D.n[0]);
-    const int j = (int)(r % D.n[1]), k = (int)(r / D.n[1]);
+  const RowWalk<WARP> W(R);
+  for (unsigned q = W.first; q < R.items; q += W.groups) {
+    const RowItem t = row_item(D, R, q, W.lane);
     double m0 = 0.0, m1 = 0.0, m2 = 0.0;
-    for (int i = i0 + lane; i < i1; i += R.lanes) {
-      const double x = centre(i, D.n[0], h), m = (double)rho[r * D.n[0] + i], mx = m * x;
+    for (int i = t.i0; i < t.i1; i += W.step) {
+      const double x = centre(i, D.n[0], h), m = (double)rho[t.row * D.n[0] + i], mx = m * x;
       m0 += m;
       m1 += mx;
       m2 += mx * x;
     }
-    const double y = centre(j, D.n[1], h), z = centre(k, D.n[2], h);
+    const double y = centre(t.j, D.n[1], h), z = centre(t.k, D.n[2], h);
     m0 *= vol;
     m1 *= vol;
     m2 *= vol;
@@ -123,13 +148,14 @@ __global__ void __launch_bounds__(kThreads) moment_kernel(const T* __restrict__ 
 // are half integers times h, so x', y' and their products are exact floats there, each term is
 // a product with its exact error, and the sums are TwoSum pairs (about 2^-45, far below the
 // float potential).  A block takes some rows of one plane at a time; z enters once per thread
-// and item, in double: about 60 FP64 instructions a warp, so an item has at least kPairItem
-// cells (eight a thread), and grids of smaller planes take moment_kernel.  Planes are cut
-// where they are fewer than kPairBlocks (two CTAs an SM): 2048 x 2048 x 1 takes 8.0 ms on one
+// and item, in double: about 60 FP64 instructions a warp, so grids of small planes (below
+// kPairPlane) take moment_kernel unless every block has one plane only.  Planes are cut, into
+// items of at least kPairItem cells, where they are fewer than kPairBlocks (two CTAs an SM): 2048 x 2048 x 1 takes 8.0 ms on one
 // CTA, 44 us so, 128 planes of 128 x 256 cells 39 and 29 us.  Sums that overflow a float
 // (densities of 1e26 and more) or lie where the products' errors underflow are formed again in
 // double.
 constexpr int kPairMax = 2048;
+constexpr int kPairPlane = 512;
 constexpr int kPairItem = 2048;
 constexpr int kPairBlocks = 304;
 struct PairSum {
@@ -144,23 +170,26 @@ struct PairSum {
   __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 __global__ void __launch_bounds__(kThreads) moment_pair_kernel(const float* __restrict__ rho, Dims D,
-                                                               RowPieces R, int cuts, double h,
+                                                               RowPieces R, int cuts,
+                                                               IndexDivisor by_cuts, double h,
                                                                double* __restrict__ part) {
   double acc[kMoments] = {0, 0, 0, 0, 0, 0, 0};
-  const int lane = threadIdx.x & (R.lanes - 1), groups = kThreads / R.lanes;
-  const int rows = (D.n[1] + cuts - 1) / cuts;  // of an item
+  const int step = 1 << R.log_lanes, lane = threadIdx.x & (step - 1);
+  const unsigned groups = kThreads >> R.log_lanes;
+  const int rows = (int)by_cuts.quotient(D.n[1] + cuts - 1);  // of an item
   const double vol = h * h * h;
-  for (long long item = blockIdx.x; item < (long long)D.n[2] * cuts; item += gridDim.x) {
-    const int k = (int)(item / cuts), j0 = (int)(item % cuts) * rows;
-    const int pieces = max(min(rows, D.n[1] - j0), 0) * R.pieces;
+  for (unsigned item = blockIdx.x; item < (unsigned)(D.n[2] * cuts); item += gridDim.x) {
+    const int k = (int)by_cuts.quotient(item), j0 = (int)(item - (unsigned)(k * cuts)) * rows;
+    const unsigned pieces = max(min(rows, D.n[1] - j0), 0) * R.pieces;
     PairSum s[6] = {};  // m, m x, m y, m x x, m y y, m x y
     auto cells = [&](auto add) {  // add(m, x, y) for the thread's cells of the item
-      for (int q = threadIdx.x / R.lanes; q < pieces; q += groups) {
-        const int j = j0 + q / R.pieces, i0 = q % R.pieces * R.length;
+      for (unsigned q = threadIdx.x >> R.log_lanes; q < pieces; q += groups) {
+        const unsigned r = R.by_pieces.quotient(q);
+        const int j = j0 + (int)r, i0 = (int)(q - r * (unsigned)R.pieces) * R.length;
         const float y = (float)j + 0.5f - 0.5f * (float)D.n[1];
         const float* row = rho + (long long)k * D.nxy + (long long)j * D.n[0];
         const int i1 = min(i0 + R.length, D.n[0]);
-        for (int i = i0 + lane; i < i1; i += R.lanes)
+        for (int i = i0 + lane; i < i1; i += step)
           add(row[i], (float)i + 0.5f - 0.5f * (float)D.n[0], y);
       }
     };
@@ -303,26 +332,32 @@ __device__ __forceinline__ void pair_add(SourcePair& s, float x) {
   s.hi = t;
 }
 
+// 4 pi G h^2 and, as pairs, it and its twelfth (formed once on the host: a division in each
+// thread's prologue took as long as a 128^3 grid's cells).
+struct Source {
+  double c;
+  float ch, cl, c12h, c12l;
+  explicit Source(double c_) : c(c_), ch((float)c_), cl((float)(c_ - (double)ch)) {
+    c12h = (float)(c / 12.0);
+    c12l = (float)(c / 12.0 - (double)c12h);
+  }
+};
+
 // Right-hand side 4 pi G h^2 (rho [+ D7 rho / 12]) of the cells away from the boundary, written
-// into the potential array (the work array); boundary cells are left to rhs_edge_kernel.  One
-// row of x per warp pass.  PAIRS: FP32 grids in float pairs, for constants in their range
-// (ppml_pair_range); a cell whose pair overflows (the sum of densities above 2.8e37) is formed
-// in double.
-template <typename T, bool PAIRS>
+// into the potential array (the work array); boundary cells are left to rhs_edge_kernel.
+// PAIRS: FP32 grids in float pairs, for constants in their range (ppml_pair_range); a cell
+// whose pair overflows (the sum of densities above 2.8e37) is formed in double.
+template <typename T, bool PAIRS, bool WARP>
 __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho, T* __restrict__ out,
-                                                       Dims D, double h, double G, int printed) {
-  const double c = 4.0 * M_PI * G * h * h;
-  const float ch = (float)c, cl = (float)(c - (double)ch);
-  const float c12h = (float)(c / 12.0), c12l = (float)(c / 12.0 - (double)c12h);
-  const int lane = threadIdx.x & 31, nx = D.n[0];
-  const long long rows = (long long)D.n[1] * D.n[2];
-  const long long warps = (long long)gridDim.x * (kThreads / 32);
-  for (long long row = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows;
-       row += warps) {
-    const int j = (int)(row % D.n[1]), k = (int)(row / D.n[1]);
-    if (j == 0 || k == 0 || j == D.n[1] - 1 || k == D.n[2] - 1) continue;
-    for (int i = 1 + lane; i < nx - 1; i += 32) {
-      const long long idx = row * nx + i;
+                                                       Dims D, RowPieces R, Source S, int printed) {
+  const int nx = D.n[0];
+  const RowWalk<WARP> W(R);
+  for (unsigned q = W.first; q < R.items; q += W.groups) {
+    const RowItem t = row_item(D, R, q, W.lane);
+    if (t.j == 0 || t.k == 0 || t.j == D.n[1] - 1 || t.k == D.n[2] - 1) continue;
+    for (int i = t.i0; i < t.i1; i += W.step) {
+      if (i == 0 || i == nx - 1) continue;
+      const long long idx = t.row * nx + i;
       const T rc = rho[idx];
       T nb[6] = {};
       if (!printed) {
@@ -334,24 +369,24 @@ __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho
         nb[5] = rho[idx + D.nxy];
       }
       auto in_double = [&]() -> T {
-        if (printed) return (T)(c * (double)rc);
+        if (printed) return (T)(S.c * (double)rc);
         double lap = -6.0 * (double)rc;
 #pragma unroll
         for (int q = 0; q < 6; q++) lap += (double)nb[q];
-        return (T)(c * ((double)rc + lap / 12.0));
+        return (T)(S.c * ((double)rc + lap / 12.0));
       };
       T v;
       if constexpr (PAIRS) {
         if (printed) {
-          v = fmaf(rc, ch, rc * cl);
+          v = fmaf(rc, S.ch, rc * S.cl);
         } else {
           // c / 12 (6 rho + sum), the products to 2^-46
           SourcePair s = {6.0f * rc, 0.0f};
           s.lo = fmaf(6.0f, rc, -s.hi);
 #pragma unroll
           for (int q = 0; q < 6; q++) pair_add(s, nb[q]);
-          const float p = s.hi * c12h;
-          v = p + (fmaf(s.hi, c12h, -p) + fmaf(s.hi, c12l, s.lo * c12h));
+          const float p = s.hi * S.c12h;
+          v = p + (fmaf(s.hi, S.c12h, -p) + fmaf(s.hi, S.c12l, s.lo * S.c12h));
         }
         if (!(fabsf(v) <= FLT_MAX)) v = in_double();
       } else {
@@ -433,38 +468,57 @@ __global__ void __launch_bounds__(kThreads) rhs_edge_kernel(const T* __restrict_
 // Odd extension of every line along `axis` to M = 2 (N + 1) points:
 // (0, w_0 .. w_{N-1}, 0, -w_{N-1} .. -w_0).  Layout of the extension: axis 0 line-major
 // (line * M + p); axes 1 and 2 position-major (p * B + b), b the line's index over the
-// other two axes in memory order, so both the gather and the store are coalesced.  A warp
-// takes one contiguous row of the extension at a time (axis 0: a line; else, of position p,
-// the lines of one row of x), so no per-value index division is left (128^3: 16 us with
-// them, three quarters of it the divisions).
-template <typename T>
+// other two axes in memory order, so both the reads and the stores are coalesced.  A thread
+// stores the two images of each of its cells, those of a line's ends also the zeros before them.
+template <typename T, bool WARP>
 __global__ void __launch_bounds__(kThreads) dst_pack_kernel(const T* __restrict__ w, T* __restrict__ ext,
-                                                            Dims D, int axis) {
-  const int N = D.n[axis], nx = D.n[0];
-  const int M = 2 * (N + 1);
-  const int lane = threadIdx.x & 31;
-  const int other = axis == 0 ? 0 : D.n[axis == 1 ? 2 : 1];  // rows of x per position
-  const long long rows = axis == 0 ? (long long)D.n[1] * D.n[2] : (long long)M * other;
-  const long long warps = (long long)gridDim.x * (kThreads / 32);
-  for (long long row = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows;
-       row += warps) {
+                                                            Dims D, RowPieces R, int axis) {
+  const int N = D.n[axis], nx = D.n[0], M = 2 * (N + 1);
+  const long long B = D.ncell / N;
+  const RowWalk<WARP> W(R);
+  for (unsigned r = W.first; r < R.items; r += W.groups) {
+    const RowItem t = row_item(D, R, r, W.lane);
+    const T* const src = w + t.row * nx;
     if (axis == 0) {
-      for (int p = lane; p < M; p += 32) {
-        const int q = p <= N ? p - 1 : 2 * N + 1 - p;  // position along the axis, 0..N-1
-        const T v = p == 0 || p == N + 1 ? T(0) : w[row * N + q];
-        ext[row * M + p] = p <= N ? v : -v;
+      T* const line = ext + t.row * M;
+      for (int i0 = t.i0; i0 < t.i1; i0 += kBatch * W.step) {
+        T v[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; u++)
+          if (i0 + u * W.step < t.i1) v[u] = src[i0 + u * W.step];
+#pragma unroll
+        for (int u = 0; u < kBatch; u++) {
+          const int i = i0 + u * W.step;
+          if (i < t.i1) {
+            line[i + 1] = v[u];
+            line[M - 1 - i] = -v[u];
+          }
+        }
       }
+      if (t.i0 == 0) line[0] = line[N + 1] = T(0);
     } else {
-      const int p = (int)(row / other), r = (int)(row % other);
-      const int q = p <= N ? p - 1 : 2 * N + 1 - p;
-      const bool zero = p == 0 || p == N + 1;
-      const T* src = w + (axis == 1 ? (long long)r * D.nxy + (long long)q * nx
-                                    : (long long)q * D.nxy + (long long)r * nx);
-      T* dst = ext + row * nx;
-      for (int i = lane; i < nx; i += 32) {
-        const T v = zero ? T(0) : src[i];
-        dst[i] = p <= N ? v : -v;
+      const int q = axis == 1 ? t.j : t.k;  // position along the axis
+      T* const lines = ext + (long long)(axis == 1 ? t.k : t.j) * nx;
+      T* const dst = lines + (q + 1) * B;
+      T* const image = lines + (M - 1 - q) * B;
+      for (int i0 = t.i0; i0 < t.i1; i0 += kBatch * W.step) {
+        T v[kBatch];
+#pragma unroll
+        for (int u = 0; u < kBatch; u++)
+          if (i0 + u * W.step < t.i1) v[u] = src[i0 + u * W.step];
+#pragma unroll
+        for (int u = 0; u < kBatch; u++) {
+          const int i = i0 + u * W.step;
+          if (i < t.i1) {
+            dst[i] = v[u];
+            image[i] = -v[u];
+          }
+        }
       }
+      if (q == 0)
+        for (int i = t.i0; i < t.i1; i += W.step) lines[i] = T(0);
+      if (q == N - 1)
+        for (int i = t.i0; i < t.i1; i += W.step) lines[(N + 1) * B + i] = T(0);
     }
   }
 }
@@ -472,10 +526,11 @@ __global__ void __launch_bounds__(kThreads) dst_pack_kernel(const T* __restrict_
 // Sine amplitudes back into the work array: S_k = -Im(Y_k) / 2, k = q + 1 (the halving is
 // exact).  `tab` non-NULL (the last axis of the forward transform): also divided by the
 // eigenvalue 6 (prod - 1), with the inverse transform's scale folded in: times
-// c / (1 - tz ty tx), c = -scale / 6 (a table value, as tab's).  A warp takes one row of x.
-template <typename T>
+// c / (1 - tz ty tx), c = -scale / 6 (a table value, as tab's).
+template <typename T, bool WARP>
 __global__ void __launch_bounds__(kThreads) dst_unpack_kernel(const T* __restrict__ spec,
-                                                              T* __restrict__ w, Dims D, int axis,
+                                                              T* __restrict__ w, Dims D,
+                                                              RowPieces R, int axis,
                                                               const double* __restrict__ tab,
                                                               double coef) {
   using V = typename TableOf<T>::type;
@@ -486,21 +541,26 @@ __global__ void __launch_bounds__(kThreads) dst_unpack_kernel(const T* __restric
   const int nx = D.n[0], N = D.n[axis];
   const long long B = D.ncell / N;
   const long long half = N + 2;  // M / 2 + 1 complex values per line
-  const int lane = threadIdx.x & 31;
-  const long long rows = (long long)D.n[1] * D.n[2];
-  const long long warps = (long long)gridDim.x * (kThreads / 32);
-  for (long long row = (long long)blockIdx.x * (kThreads / 32) + (threadIdx.x >> 5); row < rows;
-       row += warps) {
-    const int j = (int)(row % D.n[1]), k = (int)(row / D.n[1]);
-    const long long ci = axis == 0 ? row * half + 1
-                                   : (axis == 1 ? (long long)(j + 1) * B + (long long)k * nx
-                                                : (long long)(k + 1) * B + (long long)j * nx);
+  const RowWalk<WARP> W(R);
+  for (unsigned q = W.first; q < R.items; q += W.groups) {
+    const RowItem t = row_item(D, R, q, W.lane);
+    const long long ci = axis == 0 ? t.row * half + 1
+                                   : (axis == 1 ? (long long)(t.j + 1) * B + (long long)t.k * nx
+                                                : (long long)(t.k + 1) * B + (long long)t.j * nx);
     V tzy = V();
-    if (tab) tzy = table_product(tz[k], ty[j]);
-    for (int i = lane; i < nx; i += 32) {
-      T v = T(-0.5) * spec[2 * (ci + i) + 1];
-      if (tab) v = scaled(v, over_one_minus(c, tzy, tx[i]));
-      w[row * nx + i] = v;
+    if (tab) tzy = table_product(tz[t.k], ty[t.j]);
+    for (int i0 = t.i0; i0 < t.i1; i0 += kBatch * W.step) {
+      T v[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; u++)
+        if (i0 + u * W.step < t.i1) v[u] = T(-0.5) * spec[2 * (ci + i0 + u * W.step) + 1];
+#pragma unroll
+      for (int u = 0; u < kBatch; u++) {
+        const int i = i0 + u * W.step;
+        if (i >= t.i1) break;
+        if (tab) v[u] = scaled(v[u], over_one_minus(c, tzy, tx[i]));
+        w[t.row * nx + i] = v[u];
+      }
     }
   }
 }
@@ -787,7 +847,7 @@ static int iso_create(const ppml_grid_desc* d, PoissonIso** out) {
   return PPML_OK;
 }
 
-template <typename T>
+template <typename T, bool WARP>
 static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int printed,
                    cudaStream_t st) {
   Dims D;
@@ -795,18 +855,19 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   D.nxy = (long long)D.n[0] * D.n[1];
   D.ncell = D.nxy * D.n[2];
   int blocks;
-  if (sizeof(T) == sizeof(float) && D.n[0] <= kPairMax && D.n[1] <= kPairMax && D.nxy >= kPairItem) {
-    const int most = (int)std::min<long long>(D.nxy / kPairItem, D.n[1]);
+  const long long rows = D.ncell / D.n[0];
+  if (sizeof(T) == sizeof(float) && D.n[0] <= kPairMax && D.n[1] <= kPairMax &&
+      (D.nxy >= kPairPlane || D.n[2] <= kMaxMomentBlocks)) {
+    const int most = (int)std::max(1LL, std::min<long long>(D.nxy / kPairItem, D.n[1]));
     const int cuts = std::min((kPairBlocks + D.n[2] - 1) / D.n[2], most);
-    const int rows = (D.n[1] + cuts - 1) / cuts;
-    RowPieces R = row_pieces(D.n[0], rows, 1);
-    R = row_pieces(D.n[0], rows, kThreads / R.lanes);
     blocks = (int)std::min<long long>((long long)D.n[2] * cuts, kMaxMomentBlocks);
-    moment_pair_kernel<<<blocks, kThreads, 0, st>>>((const float*)rho, D, R, cuts, h, s->part);
+    moment_pair_kernel<<<blocks, kThreads, 0, st>>>(
+        (const float*)rho, D, row_pieces(D.n[0], D.n[1], (D.n[1] + cuts - 1) / cuts, kThreads, 8), cuts,
+        IndexDivisor(cuts), h, s->part);
   } else {
     blocks = std::min(blocks_for(D.ncell), kMaxMomentBlocks);
-    const RowPieces R = row_pieces(D.n[0], D.nxy / D.n[0] * D.n[2], (long long)blocks * (kThreads / 32));
-    moment_kernel<T><<<blocks, kThreads, 0, st>>>(rho, D, R, h, s->part);
+    moment_kernel<T, WARP><<<blocks, kThreads, 0, st>>>(
+        rho, D, row_pieces(D.n[0], D.n[1], rows, (long long)blocks * kThreads, 8), h, s->part);
   }
   int rc = ppml_check_launch("moment_kernel");
   if (rc) return rc;
@@ -814,12 +875,13 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   if ((rc = ppml_check_launch("moment_final_kernel"))) return rc;
   shell_kernel<<<blocks_for(shell_cells(D)), kThreads, 0, st>>>(D, h, G, s->mom, s->shell);
   if ((rc = ppml_check_launch("shell_kernel"))) return rc;
-  const double source = 4.0 * M_PI * G * h * h;
-  if (sizeof(T) == sizeof(float) && ppml_pair_range(source, 1.0) && ppml_pair_range(source / 12.0, 1.0))
-    rhs_kernel<float, true><<<blocks_for(D.ncell), kThreads, 0, st>>>((const float*)rho, (float*)phi,
-                                                                      D, h, G, printed);
+  const Source source(4.0 * M_PI * G * h * h);
+  const RowPieces R = row_pieces(D.n[0], D.n[1], rows, (long long)blocks_for(D.ncell) * kThreads, 1);
+  if (sizeof(T) == sizeof(float) && ppml_pair_range(source.c, 1.0) && ppml_pair_range(source.c / 12.0, 1.0))
+    rhs_kernel<float, true, WARP><<<blocks_for(D.ncell), kThreads, 0, st>>>((const float*)rho, (float*)phi,
+                                                                      D, R, source, printed);
   else
-    rhs_kernel<T, false><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, h, G, printed);
+    rhs_kernel<T, false, WARP><<<blocks_for(D.ncell), kThreads, 0, st>>>(rho, phi, D, R, source, printed);
   if ((rc = ppml_check_launch("rhs_kernel"))) return rc;
   rhs_edge_kernel<T><<<blocks_for(edge_cells(D)), kThreads, 0, st>>>(rho, phi, D, h, G, s->shell,
                                                                      printed);
@@ -843,8 +905,7 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
   }
   for (int pass = 0; pass < 2; pass++) {
     for (int a = 0; a < 3; a++) {
-      const long long total = 2LL * (D.n[a] + 1) * (D.ncell / D.n[a]);
-      dst_pack_kernel<T><<<blocks_for(total), kThreads, 0, st>>>(phi, (T*)s->ext, D, a);
+      dst_pack_kernel<T, WARP><<<blocks_for(D.ncell), kThreads, 0, st>>>(phi, (T*)s->ext, D, R, a);
       if ((rc = ppml_check_launch("dst_pack_kernel"))) return rc;
       if (cufftSetStream(s->plan[a], st) != CUFFT_SUCCESS)
         return ppml_fail(PPML_E_CUDA, "cufftSetStream failed");
@@ -854,8 +915,8 @@ static int iso_run(PoissonIso* s, const T* rho, T* phi, double h, double G, int 
       else
         r = cufftExecR2C(s->plan[a], (cufftReal*)s->ext, (cufftComplex*)s->spec);
       if (r != CUFFT_SUCCESS) return ppml_fail(PPML_E_CUDA, "cuFFT sine transform failed (%d)", (int)r);
-      dst_unpack_kernel<T><<<blocks_for(D.ncell), kThreads, 0, st>>>(
-          (const T*)s->spec, phi, D, a, pass == 0 && a == 2 ? s->tab : nullptr, symbol);
+      dst_unpack_kernel<T, WARP><<<blocks_for(D.ncell), kThreads, 0, st>>>(
+          (const T*)s->spec, phi, D, R, a, pass == 0 && a == 2 ? s->tab : nullptr, symbol);
       if ((rc = ppml_check_launch("dst_unpack_kernel"))) return rc;
     }
   }
@@ -870,7 +931,12 @@ int ppml_iso_solve(PoissonIso** state, const ppml_grid_desc* d, const void* rho,
   }
   PoissonIso* s = *state;
   const int printed = (flags & PPML_POISSON_PRINTED_RHS) != 0;
-  if (d->dtype == PPML_F64)
-    return iso_run<double>(s, (const double*)rho, (double*)phi, d->h[0], G, printed, st);
-  return iso_run<float>(s, (const float*)rho, (float*)phi, d->h[0], G, printed, st);
+  auto run = [&](auto warp) {
+    constexpr bool W = decltype(warp)::value;
+    if (d->dtype == PPML_F64)
+      return iso_run<double, W>(s, (const double*)rho, (double*)phi, d->h[0], G, printed, st);
+    return iso_run<float, W>(s, (const float*)rho, (float*)phi, d->h[0], G, printed, st);
+  };
+  // rows of at least a warp's half have a warp each, shorter ones share it
+  return s->n[0] > 16 ? run(std::true_type()) : run(std::false_type());
 }

@@ -73,3 +73,11 @@ BAR = 3.0  # the shapes' kernels take 1 to 2 times the near-cube's; on a few thr
 def test_moments_of_any_shape_fill_the_device(dtype, n, cube):
     t = [_kernel_us(_solver(m, dtype, True)[2], ("moment_kernel", "moment_pair_kernel")) for m in (n, cube)]
     assert t[0] <= BAR * t[1], t
+
+
+@pytest.mark.parametrize("dtype,n,cube", [
+    (F64, (1, 1024, 1024), (128, 128, 64)), (F64, (3, 600, 600), (128, 128, 66)),
+    (F32, (1, 1024, 1024), (300, 70, 50)), (F32, (4, 4, 65536), (300, 70, 50))])
+def test_sine_transform_copies_of_any_shape_fill_the_device(dtype, n, cube):
+    t = [_kernel_us(_solver(m, dtype, True)[2], ("dst_pack_kernel", "dst_unpack_kernel")) for m in (n, cube)]
+    assert t[0] <= BAR * t[1], t
