@@ -1,5 +1,7 @@
 // Definitions of the launchers for one precision PPML_REAL (included by
 // ppml_kern_f32.cu / ppml_kern_f64.cu).
+#include <algorithm>
+
 #include "../../include/ppml.h"
 #include "ppml_internal.h"
 #include "ppml_launch.h"
@@ -159,32 +161,44 @@ int launch_diag<PPML_REAL>(const MarchArgs<PPML_REAL>& A, int nblk, cudaStream_t
 namespace {
 // Multiply the half spectrum (R2C layout: kx in [0, nx/2], ky, kz) by the inverse symbol of
 // the 27-point stencil, coef / (1 - tx ty tz); tables hold 1 - (2/3) sin^2(pi k / N) per axis
-// (FP32 grids: as float pairs).  A warp takes one row of kx at a time, so tz ty is formed once
-// per row.  V: the arithmetic, double or (FP32 grids) float pairs: 512^3 FP32: 1986 us with an
-// FP64 division per value, 204 us in pairs.
+// (FP32 grids: as float pairs).  A thread per value, whatever the grid's shape (a warp per row
+// of kx: 65536 x 4 x 4 in FP64 903 us, 14.6 so; 128^3, rows of 65 values, 41 and 27.5).  V: the
+// arithmetic, double or (FP32 grids) float pairs, which the memory bounds: 512^3 201 us for
+// 1.07 GB, 1986 with an FP64 division per value.
+struct SymbolIndex {
+  int mx, ny;
+  unsigned n;  // values
+  IndexDivisor by_mx, by_ny;
+};
 template <typename T, typename V>
 __global__ void __launch_bounds__(256) poisson_symbol_kernel(T* spec, const double* __restrict__ tab,
-                                                             int mx, int ny, int nz, V coef) {
+                                                             SymbolIndex X, V coef) {
   using U = typename TableOf<T>::type;
   using T2 = std::conditional_t<sizeof(T) == 8, double2, float2>;
   static_assert(sizeof(U) == sizeof(double), "a table value fills a double's storage");
   T2* const s = reinterpret_cast<T2*>(spec);
   const U* const tx = reinterpret_cast<const U*>(tab);
-  const U* const ty = tx + mx;
-  const U* const tz = ty + ny;
-  const int lane = threadIdx.x & 31;
-  const long long rows = (long long)ny * nz;
-  const long long warps = (long long)gridDim.x * (blockDim.x >> 5);
-  for (long long row = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < rows;
-       row += warps) {
-    const V tzy = table_product(table_as<V>(tz[row / ny]), table_as<V>(ty[row % ny]));
-    for (int kx = lane; kx < mx; kx += 32) {
-      const V f = over_one_minus(coef, tzy, table_as<V>(tx[kx]));
-      T2 v = s[row * mx + kx];
-      v.x = scaled(v.x, f);
-      v.y = scaled(v.y, f);
-      if (row == 0 && kx == 0) v.x = v.y = T(0);  // the k = 0 mode
-      s[row * mx + kx] = v;
+  const U* const ty = tx + X.mx;
+  const U* const tz = ty + X.ny;
+  constexpr int B = sizeof(V) == sizeof(T) ? 1 : 2;  // values in flight (float pairs: memory-bound)
+  const unsigned stride = gridDim.x * 256 * B;
+  for (unsigned first = blockIdx.x * 256 * B + threadIdx.x; first < X.n; first += stride) {
+    T2 v[B];
+#pragma unroll
+    for (int u = 0; u < B; u++)
+      if (first + u * 256 < X.n) v[u] = s[first + u * 256];
+#pragma unroll
+    for (int u = 0; u < B; u++) {
+      const unsigned idx = first + u * 256;
+      if (idx >= X.n) break;
+      const unsigned row = X.by_mx.quotient(idx), kx = idx - row * (unsigned)X.mx;
+      const unsigned kz = X.by_ny.quotient(row), ky = row - kz * (unsigned)X.ny;
+      const V f = over_one_minus(coef, table_product(table_as<V>(tz[kz]), table_as<V>(ty[ky])),
+                                 table_as<V>(tx[kx]));
+      v[u].x = scaled(v[u].x, f);
+      v[u].y = scaled(v[u].y, f);
+      if (idx == 0) v[u].x = v[u].y = T(0);  // the k = 0 mode
+      s[idx] = v[u];
     }
   }
 }
@@ -192,17 +206,18 @@ __global__ void __launch_bounds__(256) poisson_symbol_kernel(T* spec, const doub
 template <typename T>
 void launch_symbol(T* spec, const double* tab, int mx, int ny, int nz, double coef, bool pairs,
                    cudaStream_t st) {
-  const long long rows = (long long)ny * nz;
-  const int blocks = (int)((rows + 7) / 8 < 152 * 8 ? (rows + 7) / 8 : 152 * 8);
+  const long long n = (long long)mx * ny * nz;
+  const SymbolIndex X = {mx, ny, (unsigned)n, IndexDivisor(mx), IndexDivisor(ny)};
+  const int blocks = (int)std::min((n + 255) / 256, 152LL * 16);
   if constexpr (sizeof(T) == 4) {
     if (pairs) {
       const float hi = (float)coef;
       const FloatPair c = {hi, (float)(coef - (double)hi)};
-      poisson_symbol_kernel<T, FloatPair><<<blocks, 256, 0, st>>>(spec, tab, mx, ny, nz, c);
+      poisson_symbol_kernel<T, FloatPair><<<blocks, 256, 0, st>>>(spec, tab, X, c);
       return;
     }
   }
-  poisson_symbol_kernel<T, double><<<blocks, 256, 0, st>>>(spec, tab, mx, ny, nz, coef);
+  poisson_symbol_kernel<T, double><<<blocks, 256, 0, st>>>(spec, tab, X, coef);
 }
 }  // namespace
 

@@ -81,3 +81,21 @@ def test_moments_of_any_shape_fill_the_device(dtype, n, cube):
 def test_sine_transform_copies_of_any_shape_fill_the_device(dtype, n, cube):
     t = [_kernel_us(_solver(m, dtype, True)[2], ("dst_pack_kernel", "dst_unpack_kernel")) for m in (n, cube)]
     assert t[0] <= BAR * t[1], t
+
+
+@pytest.mark.parametrize("dtype", [F32, F64])
+@pytest.mark.parametrize("n", [s for s in SHAPES if min(s) != 2])
+def test_periodic_shapes(n, dtype):
+    rho, phi, solve = _solver(n, dtype, False)
+    solve()
+    ref = poisson.solve_periodic(rho, 0.05, 1.1)
+    got = phi.double().cpu().numpy().reshape(ref.shape)
+    tol = 2e-5 if dtype == F32 else 1e-12  # of the largest potential
+    assert np.max(np.abs(got - ref)) <= tol * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("dtype", [F32, F64])
+@pytest.mark.parametrize("n", [(65536, 4, 4), (4, 4, 65536), (1, 1024, 1024), (1048576, 1, 1)])
+def test_symbol_of_any_shape_fills_the_device(dtype, n):
+    t = [_kernel_us(_solver(m, dtype, False)[2], ("poisson_symbol_kernel",)) for m in (n, (128, 128, 64))]
+    assert t[0] <= BAR * t[1], t
