@@ -124,8 +124,9 @@ typedef struct {
 typedef struct ppml_grid ppml_grid;
 
 /* Create a handle for the grid in *d and allocate its scratch (U*: five fields of the
- * state's type, in FP32 also the four low parts of U*'s m and rho E and, with three active
- * axes, the face velocities of every 16^3 tile, 52 KB each; reduction partials).
+ * state's type, in FP32 also the four low parts of U*'s m and rho E, whose space plain states
+ * of three active axes use for the face velocities of their 16^3 tiles: 256 MB at most where the
+ * tiles are mostly padding and that space is less; reduction partials).
  * Reads u0 once on `stream` to fix the mean initial density (the vacuum threshold
  * reference, Sec. 1.4) and the first CFL step; synchronizes the stream.  u0 is not
  * modified.  On error *out is NULL. */

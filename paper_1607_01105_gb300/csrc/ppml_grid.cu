@@ -49,8 +49,10 @@ __global__ void apply_reduced_kernel(const double* __restrict__ red, DevScalars*
 
 }  // namespace
 
-// The fewest tiles a launch of the FP32 Lagrangian stage is cut into: one wave of its CTAs.
-constexpr int kFaceTilesMin = 304;
+// What the face velocities of an FP32 grid whose tiles are mostly padding may take where the low
+// parts' space is less: 5140 tiles, 17 waves of the Lagrangian stage's CTAs.  (1024 x 1024 x 4
+// cells, 4096 tiles: a step of 890 us in one launch each of the two kernels, 980 in five.)
+constexpr size_t kFaceBytesMax = 256ull << 20;
 
 static int launch_finalize(const Partial* P, int nblk, const Finalize& f, cudaStream_t st) {
   finalize_kernel<<<1, kFinThreads, 0, st>>>(P, nblk, f);
@@ -62,9 +64,11 @@ struct ppml_grid {
   GridGeom geom;
   size_t elt;
   void* ustar[6];  // [0] unused (rho is not changed by the Eulerian stage)
-  void* ustar_lo[5];  // FP32: low parts of U*'s m and rho E ([0] unused)
+  // FP32: low parts of U*'s m and rho E ([0] unused), all in one allocation (ustar_lo[1]),
+  // whose space plain states of three active axes use for the face velocities of face_tiles
+  // tiles at a time: a step is of one kind or the other
+  void* ustar_lo[5];
   Partial* partials;
-  float* face;   // FP32 with three active axes: face velocities of face_tiles tiles
   int face_tiles;
   void* inflow;  // 36 values of the state's type: the inflow faces' ghost states [face][field]
   int nblk_march, nblk_diag, npartials;  // tiles (partials of a step), diagnostics blocks
@@ -218,7 +222,7 @@ MarchArgs<T> make_args(const ppml_grid* g, double dt_host, const double* dt_dev)
   A.flags = g->d.flags;
   A.inflow = (const T*)g->inflow;
   A.fin = make_finalize(g, 0, nullptr);
-  A.face = (T*)g->face;
+  A.face = g->face_tiles ? (T*)g->ustar_lo[1] : nullptr;
   A.face_tiles = g->face_tiles;
   A.any_inflow = 0;
   for (int q = 0; q < 6; q++) A.any_inflow |= g->d.bc[q] == PPML_BC_INFLOW;
@@ -355,25 +359,30 @@ extern "C" int ppml_init_grid(const ppml_grid_desc* d, const ppml_state* u0, voi
       return ppml_fail(PPML_E_NOMEM, "cudaMalloc of U* (%zu bytes) failed", fbytes);
     }
   }
-  for (int f = 1; f < 5 && d->dtype == PPML_F32; f++) {
-    if (cudaMalloc(&g->ustar_lo[f], fbytes) != cudaSuccess) {
-      ppml_free_grid(g);
-      return ppml_fail(PPML_E_NOMEM, "cudaMalloc of U* low parts (%zu bytes) failed", fbytes);
+  if (d->dtype == PPML_F32) {
+    const size_t part = (fbytes + 255) / 256 * 256, lo_bytes = 4 * part;
+    // the face velocities of whole tiles, 12.75 B a cell, lie within the 16 B of the low parts;
+    // small grids with much padding may take up to kFaceBytesMax in all, larger ones (and all
+    // if the device has no room for more) several launches a step
+    size_t bytes = lo_bytes;
+    const bool faces = d->nx > 1 && d->ny > 1 && d->nz > 1;
+    if (faces) {
+      const size_t need = kFaceBytes * (size_t)g->nblk_march;
+      bytes = std::max(lo_bytes, std::min(need, kFaceBytesMax));
     }
-  }
-  if (d->dtype == PPML_F32 && d->nx > 1 && d->ny > 1 && d->nz > 1) {
-    // face velocities of every tile, or of as many as fit (then a step takes several launches)
-    g->face_tiles = g->nblk_march;
-    while (cudaMalloc(&g->face, kFaceBytes * (size_t)g->face_tiles) != cudaSuccess) {
+    cudaError_t e = cudaMalloc(&g->ustar_lo[1], bytes);
+    if (e != cudaSuccess && bytes > lo_bytes && lo_bytes >= kFaceBytes) {
       cudaGetLastError();
-      g->face = nullptr;
-      if (g->face_tiles <= kFaceTilesMin) {
-        ppml_free_grid(g);
-        return ppml_fail(PPML_E_NOMEM, "cudaMalloc of the face velocities (%zu bytes) failed",
-                         kFaceBytes * (size_t)kFaceTilesMin);
-      }
-      g->face_tiles = std::max(kFaceTilesMin, g->face_tiles / 8);
+      bytes = lo_bytes;
+      e = cudaMalloc(&g->ustar_lo[1], bytes);
     }
+    if (e != cudaSuccess) {
+      cudaGetLastError();
+      ppml_free_grid(g);
+      return ppml_fail(PPML_E_NOMEM, "cudaMalloc of U* low parts (%zu bytes) failed", bytes);
+    }
+    for (int f = 2; f < 5; f++) g->ustar_lo[f] = (char*)g->ustar_lo[1] + (f - 1) * part;
+    if (faces) g->face_tiles = (int)std::min((size_t)g->nblk_march, bytes / kFaceBytes);
   }
   if (cudaMalloc(&g->partials, sizeof(Partial) * (size_t)g->npartials) != cudaSuccess ||
       cudaMalloc(&g->dev, sizeof(DevScalars)) != cudaSuccess ||
@@ -420,10 +429,8 @@ extern "C" int ppml_free_grid(ppml_grid* g) {
   cudaDeviceSynchronize();
   for (int f = 0; f < 6; f++)
     if (g->ustar[f]) cudaFree(g->ustar[f]);
-  for (int f = 0; f < 5; f++)
-    if (g->ustar_lo[f]) cudaFree(g->ustar_lo[f]);
+  if (g->ustar_lo[1]) cudaFree(g->ustar_lo[1]);
   if (g->partials) cudaFree(g->partials);
-  if (g->face) cudaFree(g->face);
   if (g->inflow) cudaFree(g->inflow);
   if (g->dev) cudaFree(g->dev);
   if (g->ev) {

@@ -48,9 +48,9 @@ bool launch_euler_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
 }
 
 // Lagrangian stage of plain float states with three active axes: face velocities, then the
-// sweeps; in several launches where the face array does not hold every tile (the
-// allocation-free step, or a handle on a nearly full device), then in x-major order (the
-// results do not depend on it).  False: not such a state, nothing launched.
+// sweeps; in several launches of about as many tiles each where the face array does not hold
+// every tile (the allocation-free step, or a grid whose tiles are mostly padding), then in
+// x-major order (the results do not depend on it).  False: not such a state, nothing launched.
 bool launch_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
   if (!A.face || !sweep_grid(A)) return false;
   MarchArgs<float> B = A;
@@ -59,7 +59,8 @@ bool launch_sweeps(const MarchArgs<float>& A, int nblk, cudaStream_t st) {
   if (A.face_tiles < tiles) {
     B.tile_order = 0;
     nblk = tiles;
-    per = A.face_tiles;
+    const int launches = (tiles + A.face_tiles - 1) / A.face_tiles;
+    per = (tiles + launches - 1) / launches;
   }
   for (int first = 0; first < nblk; first += per) {
     const int n = nblk - first < per ? nblk - first : per;
