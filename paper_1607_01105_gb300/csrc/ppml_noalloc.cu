@@ -25,18 +25,20 @@ using namespace ppml;
 
 namespace {
 
-// U* (five fields) in the widest element type, then the partials, then the scalars.
+// U* (five fields) in the widest element type, more face velocities, the partials, the scalars.
 constexpr size_t kUstarBytes = 5ull * PPML_NOALLOC_MAX_CELLS * sizeof(double);
 // A tile of 16^3 cells covers at least 16 cells of any grid, so the tile count of a grid
 // of at most PPML_NOALLOC_MAX_CELLS cells is at most PPML_NOALLOC_MAX_CELLS / 16 + a few
 // partial tiles per axis.
 constexpr size_t kMaxPartials = PPML_NOALLOC_MAX_CELLS / 16 + 4096;
 constexpr size_t kPartialBytes = kMaxPartials * sizeof(Partial);
-// FP32: the face velocities of a launch's tiles (64^3 cells are 64 tiles; thin grids of more
-// tiles take several launches).
-constexpr int kFaceTiles = 64;
-constexpr size_t kFaceOffset = (kUstarBytes + kPartialBytes + sizeof(DevScalars) + 255) / 256 * 256;
-constexpr size_t kScratchBytes = kFaceOffset + kFaceTiles * kFaceBytes;
+// FP32: the face velocities of a launch's tiles, from the end of U* in floats on: 64 tiles (64^3
+// cells) and the half of U* that doubles would fill, 164 to 265 tiles in all.  Thin grids of
+// more tiles (3 x 3 x 29127: 1821) take several launches.
+constexpr size_t kFaceMore = 64 * kFaceBytes;
+constexpr size_t kFieldsBytes = kUstarBytes + kFaceMore;
+constexpr size_t kScratchBytes = kFieldsBytes + kPartialBytes + sizeof(DevScalars);
+static_assert(kFieldsBytes % 256 == 0 && kPartialBytes % alignof(DevScalars) == 0, "alignment");
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
 
@@ -69,8 +71,8 @@ int step_noalloc(const ppml_grid_desc* d, const ppml_state* u_in, ppml_state* u_
   if (rc) return rc;
   const long long ncell = (long long)d->nx * d->ny * d->nz;
   T* ustar = (T*)scratch;
-  Partial* partials = (Partial*)(scratch + kUstarBytes);
-  DevScalars* S = (DevScalars*)(scratch + kUstarBytes + kPartialBytes);
+  Partial* partials = (Partial*)(scratch + kFieldsBytes);
+  DevScalars* S = (DevScalars*)(scratch + kFieldsBytes + kPartialBytes);
   MarchArgs<T> A;
   memset(&A, 0, sizeof(A));
   A.g.n[0] = d->nx;
@@ -95,8 +97,9 @@ int step_noalloc(const ppml_grid_desc* d, const ppml_state* u_in, ppml_state* u_
   A.tiles_z = tiles_z;
   A.tile_order = 0;
   if (sizeof(T) == 4) {
-    A.face = (T*)(scratch + kFaceOffset);
-    A.face_tiles = kFaceTiles;
+    const size_t fields = (5 * (size_t)ncell * sizeof(T) + 255) / 256 * 256;
+    A.face = (T*)(scratch + fields);
+    A.face_tiles = (int)((kFieldsBytes - fields) / kFaceBytes);
   }
   const int nblk = A.tiles_x * A.tiles_y * tiles_z;
   if ((size_t)nblk > kMaxPartials)

@@ -87,3 +87,29 @@ def test_plain_and_double_float_steps_share_a_handle():
     for _ in range(3):
         a, b = steps(g, a, 1), steps(g, b, 1)
     assert all(torch.equal(x, y) for x, y in zip(a + b, plain + double))
+
+
+@pytest.mark.parametrize("n,launches", [((3, 3, 29127), 12), ((17, 17, 907), 2), ((64, 64, 64), 1),
+                                        ((16, 16, 16 * 64), 1), ((3, 3, 3), 1)])
+def test_noalloc_step_uses_the_whole_buffer(n, launches):
+    """The allocation-free FP32 step: as many tiles a launch as its buffer holds, and the bits
+    of the handle's step."""
+    from torch.profiler import ProfilerActivity, profile
+    u = ppml.to_device(inputs.random_smooth(n=n, bc=(P,) * 6).u, F32)
+    a, b = [torch.empty_like(x) for x in u], [torch.empty_like(x) for x in u]
+    h, rho = (0.02,) * 3, float(u[0].double().mean())
+    grid = ppml.Grid(n, h, 1.4, 0.2, (P,) * 6, F32, u0=u, rho_ref=rho)
+    grid.step(u, a, 1e-3)
+    desc = ppml.make_desc(n, h, 1.4, 0.2, (P,) * 6, F32)
+    for _ in range(3):  # (a process's first session may record nothing)
+        torch.cuda.synchronize()
+        with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            out = ppml.step_noalloc(desc, u, b, 1e-3, rho)
+            torch.cuda.synchronize()
+        count = sum(e.count for e in prof.key_averages() if "face_velocity" in e.key)
+        if count:
+            break
+    assert count == launches
+    assert all(torch.equal(x, y) for x, y in zip(a, b))
+    d = grid.diag()
+    assert out[0] == d["dt_next"] and out[3] == d["sums"]
