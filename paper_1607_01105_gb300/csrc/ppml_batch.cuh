@@ -643,14 +643,15 @@ __device__ __forceinline__ void advance_part_f32(float* __restrict__ g_rho, floa
   }
 }
 
-// One CTA's part of an instance advanced for up to max_steps steps (Sec. 1 in 1D).  PAIR:
+// One CTA's part of an FP64 or a double-float instance (plain FP32 ones: advance_part_f32)
+// advanced for up to max_steps steps (Sec. 1 in 1D).  PAIR:
 // the part is half of an instance and the partner CTA of the cluster holds the other half
 // (halo exchange and common CFL step in pair_cfl_step); else the part is the instance.
 // Local arrays: four fields with G cells of padding on each side (the halo facing the
-// partner, outflow ghosts at the instance's ends), face arrays indexed f + FO, and (DF,
-// FP32 only) the low parts of rho, m, rho E padded like the fields, read from g_lo at the
-// start and written back at the end.
-template <typename T, int NTHREADS, bool PAIR, bool DF>
+// partner, outflow ghosts at the instance's ends), face arrays indexed f + FO, and (DF) the
+// low parts of rho, m, rho E padded like the fields, read from g_lo at the start and written
+// back at the end.
+template <typename T, int NTHREADS, bool PAIR>
 __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restrict__ g_m,
                                              T* __restrict__ g_en, T* __restrict__ g_ei,
                                              T* const* g_lo, InstDev& I, const Part P, T* smem,
@@ -658,7 +659,7 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
                                              int max_steps, double* red, T* xslot) {
   constexpr int G = PAIR ? kPairHalo : kBatchGhost;
   constexpr int FO = PAIR ? 3 : 0;
-  static_assert(!DF || sizeof(T) == 4, "double-float states are FP32 only");
+  constexpr bool DF = sizeof(T) == 4;
   const int nl = P.nl;
   T* R = smem;
   T* M = R + stride;
@@ -910,7 +911,7 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
       vm = T(0);
       cm = T(0);
       for (int c0 = tid; c0 < nl; c0 += kU * NTHREADS) {
-        // every field's update (DF: rho, m, rho E added to their double-float pairs)
+        // every field's update (rho, m, rho E added to their double-float pairs)
         float q[kU][4], ql[kU][3];
 #pragma unroll
         for (int u = 0; u < kU; u++) {
@@ -918,16 +919,9 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
           const float d0 = th * (FA[c + 1 + FO] - FA[c + FO]);
           const float d1 = th * (FB[c + 1 + FO] - FB[c + FO]);
           const float d2 = th * (FC[c + 1 + FO] - FC[c + FO]);
-          if constexpr (DF) {
-            df_sub(R[g], RL[g], d0, q[u][0], ql[u][0]);
-            df_sub(M[g], ML[g], d1, q[u][1], ql[u][1]);
-            df_sub(E[g], EL[g], d2, q[u][2], ql[u][2]);
-          } else {
-            q[u][0] = R[g] - d0;
-            q[u][1] = M[g] - d1;
-            q[u][2] = E[g] - d2;
-            ql[u][0] = ql[u][1] = ql[u][2] = 0.0f;
-          }
+          df_sub(R[g], RL[g], d0, q[u][0], ql[u][0]);
+          df_sub(M[g], ML[g], d1, q[u][1], ql[u][1]);
+          df_sub(E[g], EL[g], d2, q[u][2], ql[u][2]);
           q[u][3] = Ei[g] - th * (FD[c + 1 + FO] - FD[c + FO]);
         }
         // Sec. 1.4: the dense branch for all kU cells without control flow (so that
@@ -949,16 +943,13 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
           wl[u][4] = ql[u][2];
           vac[u] = vacuum_cell_f32(w[u], rho_vac_up);
           any_vac |= vac[u];
-          q[u][3] = DF ? dense_eps_df(w[u], wl[u]) : dense_eps_f32(w[u]);
+          q[u][3] = dense_eps_df(w[u], wl[u]);
         }
         if (any_vac) {
 #pragma unroll
           for (int u = 0; u < kU; u++)
             if (vac[u]) {
-              if constexpr (DF)
-                vacuum_correct_df(w[u], wl[u], I.rho_vac);
-              else
-                vacuum_correct_f32(w[u], I.rho_vac);
+              vacuum_correct_df(w[u], wl[u], I.rho_vac);
               q[u][1] = w[u][1];
               ql[u][1] = wl[u][1];
               q[u][3] = w[u][5];
@@ -972,11 +963,9 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
             M[g] = q[u][1];
             E[g] = q[u][2];
             Ei[g] = q[u][3];
-            if constexpr (DF) {
-              RL[g] = ql[u][0];
-              ML[g] = ql[u][1];
-              EL[g] = ql[u][2];
-            }
+            RL[g] = ql[u][0];
+            ML[g] = ql[u][1];
+            EL[g] = ql[u][2];
           }
         }
         // next step's CFL maxima over the valid cells (a clamped duplicate may have read
@@ -1063,7 +1052,7 @@ __global__ void __launch_bounds__(NTHREADS, kBatchCtas<T, NTHREADS>) batch_kerne
     advance_part_f32<NTHREADS, false>(g_rho, g_m, g_en, g_ei, I, P, (T*)smem_raw,
                                       nmax + 2 * kBatchGhost, gamma_d, cfl, max_steps, red, nullptr);
   else
-    advance_part<T, NTHREADS, false, DF>(g_rho, g_m, g_en, g_ei, lo.p, I, P, (T*)smem_raw,
+    advance_part<T, NTHREADS, false>(g_rho, g_m, g_en, g_ei, lo.p, I, P, (T*)smem_raw,
                                          nmax + 2 * kBatchGhost, nmax + 1, gamma_d, cfl, max_steps,
                                          red, nullptr);
   // the time keeper's copy holds the instance's time
@@ -1111,7 +1100,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, kBatchCtas
                                        nlmax + 2 * kPairHalo, gamma_d, cfl, max_steps, red,
                                        &xslot[0][0]);
     else
-      advance_part<T, NTHREADS, true, DF>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
+      advance_part<T, NTHREADS, true>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
                                           nlmax + 2 * kPairHalo, nlmax + 8, gamma_d, cfl, max_steps,
                                           red, &xslot[0][0]);
     if (rank == 0 && threadIdx.x == 0) {  // both CTAs hold the same time; rank 0 stores it
@@ -1128,7 +1117,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(NTHREADS, kBatchCtas
       advance_part_f32<NTHREADS, false>(g_rho, g_m, g_en, g_ei, I, P, (T*)smem_raw,
                                         nmax + 2 * kBatchGhost, gamma_d, cfl, max_steps, red, nullptr);
     else
-      advance_part<T, NTHREADS, false, DF>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
+      advance_part<T, NTHREADS, false>(g_rho, g_m, g_en, g_ei, g_lo, I, P, (T*)smem_raw,
                                            nmax + 2 * kBatchGhost, nmax + 1, gamma_d, cfl, max_steps,
                                            red, nullptr);
     if (sizeof(T) == 4 && !DF ? keeps_time<NTHREADS>() : threadIdx.x == 0) {

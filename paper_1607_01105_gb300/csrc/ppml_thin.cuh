@@ -17,13 +17,12 @@ namespace ppml {
 
 constexpr int THIN_NT = 256;
 
-// Cells of a CTA along the two axes and of a segment (the Eulerian and Lagrangian stages').
-// FP64 issues an instruction per 19 cycles and SM, so its chains are cut shortest.
+// Cells of a CTA along the two axes and of a segment.  (FP64 grids of one axis have a pass per
+// quantity in place of segments, below.)
 template <typename T, bool TWO>
 struct ThinShape {
   static constexpr int LA = TWO ? 16 : 32, LB = TWO ? 16 : 1;
-  static constexpr int SEG_E = TWO ? 4 : (sizeof(T) == 8 ? 1 : 2);
-  static constexpr int SEG_L = TWO ? 4 : (sizeof(T) == 8 ? 1 : 2);
+  static constexpr int SEG = TWO ? 4 : 2;
   static constexpr int GB = TWO ? TH : 0;                  // ghosts along the second axis
   static constexpr int WA = LA + 2 * TH, WB = LB + 2 * GB;  // box
   static constexpr int PA = WA + 1;                        // box pitch
@@ -244,15 +243,15 @@ __global__ void __launch_bounds__(THIN_NT) thin_eulerian(MarchArgs<T> A) {
   if (TWO) load_box<T, S>(M.u[2], A, 1 + t.axB, t, maps);
   load_box<T, S>(M.u[3], A, 5, t, maps);
   __syncthreads();
-  constexpr int TASKS = (TWO ? 2 : 1) * S::CELLS / S::SEG_E;
+  constexpr int TASKS = (TWO ? 2 : 1) * S::CELLS / S::SEG;
   for (int e = threadIdx.x; e < TASKS; e += THIN_NT) {
-    const ThinTask<S, S::SEG_E> k(e);
+    const ThinTask<S, S::SEG> k(e);
     const int ax = k.q == 0 ? t.axA : t.axB, b0 = k.box(), c0 = k.cell(), cs = k.cell_stride();
     const AxisStep<T> ks(stc[0], hdiv[ax], T(ax == 0 ? stc[1] : (ax == 1 ? stc[2] : stc[3])));
     const T* const r = M.u[0] + b0;
     const T* const m = M.u[1 + k.q] + b0;
     const T* const ei = M.u[3] + b0;
-    thin_euler_line<FLAT, S::SEG_E>(
+    thin_euler_line<FLAT, S::SEG>(
         [&](int p, T& rho, T& mv, T& pr) {
           const int o = p * k.stride;
           rho = r[o];
@@ -455,13 +454,13 @@ __global__ void __launch_bounds__(THIN_NT) thin_lagrangian(MarchArgs<T> A) {
   }
   __syncthreads();
   constexpr int GROUP = sizeof(T) == 4 ? 2 : 1;  // fields of a task
-  constexpr int SEGS = (TWO ? 2 : 1) * S::CELLS / S::SEG_L;
+  constexpr int SEGS = (TWO ? 2 : 1) * S::CELLS / S::SEG;
   for (int e = threadIdx.x; e < SEGS * (6 / GROUP); e += THIN_NT) {
-    const ThinTask<S, S::SEG_L> k(e % SEGS);
+    const ThinTask<S, S::SEG> k(e % SEGS);
     const int f = e / SEGS * GROUP;
     const int first = k.q == 0 ? k.i : k.j, line = k.q == 0 ? k.j : k.i;
     const int ax = k.q == 0 ? t.axA : t.axB;
-    thin_lag_line<FLAT, S::SEG_L>(
+    thin_lag_line<FLAT, S::SEG>(
         M.u[f] + k.box(), M.u[f + GROUP - 1] + k.box(), k.stride,
         &M.face[k.q][first * S::LB + line], S::LB, &M.d[k.q][f][k.cell()],
         &M.d[k.q][f + GROUP - 1][k.cell()], k.cell_stride(),
@@ -673,15 +672,13 @@ __global__ void __launch_bounds__(THIN_NT) thin1d_lagrangian_f64(MarchArgs<doubl
   __syncthreads();
   // slopes of the fields (38 threads each), and beside them the velocities and Roe weights
   // of the cells -1 .. L (the template of a cell whose transverse neighbours are itself)
-  for (int e = tid; e < 6 * E::W + (E::L + 2); e += THIN_NT) {
-    if (e < 6 * E::W) {
-      const int f = e / E::W, c = e % E::W;
-      const double* const q = M.u[f];
-      if (c >= 1 && c < E::W - 1)
-        M.s[f][c] = FLAT ? 0.0
-                         : f64::slope(f64::diff(q[c], q[c - 1]), f64::diff(q[c + 1], q[c]),
-                                      q[c - 1], q[c + 1]);
-    }
+  for (int e = tid; e < 6 * E::W; e += THIN_NT) {
+    const int f = e / E::W, c = e % E::W;
+    const double* const q = M.u[f];
+    if (c >= 1 && c < E::W - 1)
+      M.s[f][c] = FLAT ? 0.0
+                       : f64::slope(f64::diff(q[c], q[c - 1]), f64::diff(q[c + 1], q[c]),
+                                    q[c - 1], q[c + 1]);
   }
   if (tid >= THIN_NT - 64 && tid - (THIN_NT - 64) < E::L + 2) {
     const int c = tid - (THIN_NT - 64) + 2;
