@@ -949,7 +949,7 @@ __device__ __forceinline__ void advance_part(T* __restrict__ g_rho, T* __restric
 #pragma unroll
           for (int u = 0; u < kU; u++)
             if (vac[u]) {
-              vacuum_correct_df(w[u], wl[u], I.rho_vac);
+              vacuum_correct_df<true>(w[u], wl[u], I.rho_vac);
               q[u][1] = w[u][1];
               ql[u][1] = wl[u][1];
               q[u][3] = w[u][5];

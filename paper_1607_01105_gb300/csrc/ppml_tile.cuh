@@ -1063,7 +1063,7 @@ __global__ void __launch_bounds__(TN, MINB) lagrangian_tile(MarchArgs<T> A) {
         for (int q = 0; q < FB; q++)
           if (vac[q]) {
             if constexpr (DF)
-              vacuum_correct_df(u[q], ul[q], A.rho_vac);
+              vacuum_correct_df<false>(u[q], ul[q], A.rho_vac);
             else
               vacuum_correct_f32(u[q], A.rho_vac);
             nvac++;
