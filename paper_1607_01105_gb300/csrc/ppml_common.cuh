@@ -154,7 +154,7 @@ __device__ __forceinline__ void ff_add(float& hi, float& lo, float bh, float bl)
 
 // block_reduce_store for the FP32 stage kernels: the warp level of the sums runs in
 // double-float (FP32 operations only), the maxima in float (exact) and the counters in
-// 32 bits; warp leaders convert to double and thread 0 folds the warps in a fixed order.
+// 32 bits; warp leaders convert to double and fold_warps folds the warps in a fixed order.
 template <int NTHREADS>
 __device__ __forceinline__ void block_reduce_store_f32(const float hi_in[6], const float lo_in[6],
                                                        float vmax, float cmax, unsigned nvac,

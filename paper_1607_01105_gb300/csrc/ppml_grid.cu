@@ -2,13 +2,16 @@
 // grid (Kulikov & Vorobyov, arXiv:1607.01105, Sec. 1).
 //
 // Per step, on the caller's stream:
-//   eulerian_tile      Sec. 1.1/1.2: PPML parabolas of v and p, acoustic face solve,
+//   Eulerian stage     Sec. 1.1/1.2: PPML parabolas of v and p, acoustic face solve,
 //                      unsplit update of m, rho E, rho eps -> U* (library scratch)
-//   lagrangian_tile    Sec. 1.3/1.4: 9-point velocity template, Roe-weighted face velocity,
+//   Lagrangian stage   Sec. 1.3/1.4: 9-point velocity template, Roe-weighted face velocity,
 //                      upwind parabola fluxes of all six fields, unsplit update, energy
-//                      correction; per-CTA partial maxima and sums of U^{n+1}
-//                      the last CTA to finish reduces them in a fixed order -> device-resident
-//                      CFL step (Sec. 1.1), FP64 sums, time and flags (finalize_cta)
+//                      correction; per-CTA partial maxima and sums of U^{n+1}, which the last
+//                      CTA to finish reduces in a fixed order -> device-resident CFL step
+//                      (Sec. 1.1), FP64 sums, time and flags (finalize_cta)
+// Their kernels by the grid's active axes and the state's type (ppml_kern_impl.cuh): plain
+// FP32 with three axes in ppml_tile_f32.cuh, grids of one or two axes in ppml_thin.cuh, FP64
+// with three axes and double-float states in ppml_tile.cuh.
 // No host synchronization inside a step, so consecutive steps can be captured in a CUDA
 // graph (the step size stays on the device).
 #include <cuda_runtime.h>

@@ -7,8 +7,9 @@
 // the stencil of a boundary cell are moved to the right-hand side.  Stages 2-3: with
 // Dirichlet data on the shell the 27-point operator is diagonal in the sine basis
 // sin(pi j (i + 1) / (N + 1)), j = 1..N, so the exponential transform the paper prints is
-// replaced by a type-I sine transform along each axis (odd extension to 2 (N + 1) points and
-// a batched real-to-complex cuFFT), the amplitudes are divided by the operator's eigenvalue
+// replaced by a type-I sine transform along each axis (FP32 grids of at most 256 points per
+// axis: dense half-size matrix products; else odd extension to 2 (N + 1) points and a batched
+// real-to-complex cuFFT), the amplitudes are divided by the operator's eigenvalue
 // 6 (prod_a (1 - (2/3) sin^2(pi j_a / (2 (N_a + 1)))) - 1), and the same sine transform,
 // scaled by prod_a 2 / (N_a + 1), brings the potential back.  The right-hand side is
 // 4 pi G h^2 (rho + D7 rho / 12) (D7 the 7-point second difference, rho = 0 outside), which
@@ -18,8 +19,12 @@
 // Geometry: cell (i, j, k) has its centre at ((i + 1/2 - nx/2) h, (j + 1/2 - ny/2) h,
 // (k + 1/2 - nz/2) h), i.e. the grid is centred on the origin of the expansion.
 //
-// The potential array doubles as the work array of the transforms; the odd extension and
-// the half spectrum live in buffers kept by the solver state between calls.
+// The potential array doubles as the work array of the transforms; the sine matrices, or the
+// odd extension and the half spectrum, live in buffers kept by the solver state between calls.
+//
+// FP32 grids form the moments, the source and the symbol in float pairs (about 2^-45, below
+// the float potential's rounding), off the FP64 pipe, where the values lie in the pairs'
+// range, else in double.
 #include <cuda_runtime.h>
 #include <cufft.h>
 #include <float.h>
@@ -398,8 +403,9 @@ __global__ void __launch_bounds__(kThreads) rhs_kernel(const T* __restrict__ rho
 }
 
 // The cells of the grid's boundary, a thread each (inside the rows of rhs_kernel they would
-// hold up warps of interior cells; 128^3 FP32: 125 us then, 21 + 16 apart): the source as above with rho = 0 outside, in FP64, minus
-// the stencil weights times the shell values next to the cell.
+// hold up warps of interior cells; 128^3 FP32: 125 us then, 9 + 13 apart): the source as above
+// with rho = 0 outside, in FP64, minus the stencil weights times the shell values next to the
+// cell.
 __host__ __device__ __forceinline__ long long edge_cells(const Dims& D) {
   const long long nx = D.n[0], ny = D.n[1], nz = D.n[2];
   const long long in_x = nx > 2 ? nx - 2 : 0, in_y = ny > 2 ? ny - 2 : 0, in_z = nz > 2 ? nz - 2 : 0;
@@ -571,10 +577,10 @@ __global__ void __launch_bounds__(kThreads) dst_unpack_kernel(const T* __restric
 // j take the sums w_i + w_{N-1-i}, the even j the differences.  A CTA holds 64 lines and the
 // matrix in shared memory; a warp forms 16 outputs of one parity for two columns per lane,
 // on packed FMAs, summing blocks of 16 terms before adding them up (the rounding error of a
-// fast transform).  128^3: 134 M FMAs a pass, 3.4 us at the FMA peak, beside 16.8 MB of
+// fast transform).  128^3: 134 M FMAs a transform, 3.4 us at the FMA peak, beside 16.8 MB of
 // traffic; the odd extension, the real transform of 2 (N + 1) points and the unpacking took
-// about 100 us a pass (258 = 2 3 43 is a poor length), this takes 25.  N^2 work: beyond kDenseMax the
-// matrix does not fit and the transform of the extension is used.
+// about 100 us each (258 = 2 3 43 is a poor length), the six transforms of a solve take 103 so.
+// N^2 work: beyond kDenseMax the matrix does not fit and the transform of the extension is used.
 constexpr int kDenseMax = 256;
 constexpr int kDenseCols = 64;
 constexpr int kDenseOut = 16;

@@ -231,9 +231,11 @@ __device__ __forceinline__ Parab<T> flat_parabola(T q) {
 // reads position p, and with p = 19 after the last step; positions below p - 3 are no
 // longer read at that point (step p reads positions p, p - 2 and p - 3).
 //
-// FP32, the parabolas in face values: double-float states, whose low parts record the rounding
-// of exactly these expressions (and one- and two-axis grids with gravity; plain states of
-// three axes have eulerian_sweep_f32, of fewer thin_eulerian).
+// FP32, the parabolas in face values: double-float states, by choice: a low part holds what the
+// high part rounds off of value minus decrement, the deviation form's decrements, as good
+// against 64 bits, differ in their last bits, and states saved earlier go on with the same
+// bits (and one- and two-axis grids with gravity; plain states of three axes have
+// eulerian_sweep_f32, of fewer thin_eulerian).
 template <bool FLAT, typename VF, typename PF, typename RF, typename EF, typename HF>
 __device__ __forceinline__ void sweep_eulerian_faces(VF v, PF pr, RF r, float gamma, float th,
                                                      EF emit, HF hook) {
@@ -553,7 +555,7 @@ __device__ __forceinline__ float half_flux_f32(float w, float R_l, float D_l, fl
 }
 
 // One line of the Lagrangian stage for any axis with the parabola in face values, for
-// double-float states: their low parts record the rounding of exactly these expressions.
+// double-float states (the reason is at sweep_eulerian_faces).
 // Field values: core[p cs] for p in
 // [0, 16), halo[h SLP] for the positions -3..-1 (h = 0..2) and 16..18 (h = 3..5).  Face
 // velocities vh[c TN], c = 0..16 (face between cells c-1 and c).  MODE 0: acc = div;

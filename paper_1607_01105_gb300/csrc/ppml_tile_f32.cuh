@@ -11,16 +11,15 @@
 //                       Sec. 1.4, the CFL maxima and sums
 //
 // Why two: one kernel that holds the velocity boxes, the face velocities of its lines, a
-// field with its halos and an accumulator fills 105 KB of shared memory, two CTAs of eight
-// warps per SM, and waits for staging with nothing beside it (issue slots 52 % busy).  With
-// the velocities coming from L2 in coalesced rows the sweeps need 70 KB for two fields at a
-// time, so three CTAs share an SM, the weights of a face are formed once for two fields, and
-// no staging phase is left: the z sweep reads its columns from global memory itself, a few
-// positions ahead, and leaves them in shared memory for the x and y sweeps.
+// field with its halos and an accumulator fills 105 KB of shared memory and waits for staging
+// with nothing beside it (issue slots 52 % busy).  With the velocities coming from L2 in
+// coalesced rows the weights of a face are formed once for two fields, and no staging phase is
+// left: the z sweep reads its columns from global memory itself, a few positions ahead, and
+// leaves them in shared memory (70 KB for two fields) for the x and y sweeps.
 //
-// Bound by instruction issue (about half of the slots busy with 16 warps an SM) and the ALU
-// pipe that the minima and selects share; 128 registers a thread rule out a third CTA (at 80:
-// 2844 us for two 256^3 steps against 2685).  256^3, one step, before and after: Eulerian
+// Bound by instruction issue (about half of the slots busy) and the ALU pipe that the minima
+// and selects share, with two CTAs of eight warps an SM: the shared memory would hold three,
+// the 128 registers a thread do not (at 80: 2844 us for two 256^3 steps against 2685).  256^3, one step, before and after: Eulerian
 // 580 -> 315 us, Lagrangian 1325 -> 592 + 166 us; DRAM traffic 41.7 B/cell, 26.5 + 65.7.
 #pragma once
 #include "ppml_pair.cuh"
