@@ -576,10 +576,14 @@ __global__ void __launch_bounds__(kThreads) dst_unpack_kernel(const T* __restric
 // symmetry sin(pi j (N - i) / (N + 1)) = -+ sin(pi j (i + 1) / (N + 1)) halves it: the odd
 // j take the sums w_i + w_{N-1-i}, the even j the differences.  A CTA holds 64 lines and the
 // matrix in shared memory; a warp forms 16 outputs of one parity for two columns per lane,
-// on packed FMAs, summing blocks of 16 terms before adding them up (the rounding error of a
-// fast transform).  128^3: 134 M FMAs a transform, 3.4 us at the FMA peak, beside 16.8 MB of
-// traffic; the odd extension, the real transform of 2 (N + 1) points and the unpacking took
-// about 100 us each (258 = 2 3 43 is a poor length), the six transforms of a solve take 103 so.
+// on packed FMAs, in chains of four terms, two of which are added before they join the sum: the
+// rounding of the sums is what the solve's error is made of.  Against 64 bits (relative L2, mean
+// of six blobs) 47^3 1.57e-7, 53^3 1.51e-7, 64 x 64 x 40 1.36e-7, where the transform of the odd
+// extension has 1.57e-7, 1.72e-7 and 1.72e-7, and chains of sixteen 1.96e-7, 1.94e-7 and 1.95e-7
+// (2 % faster); on most larger sizes the fast transform has twice the error.
+// 128^3: 134 M FMAs a transform, 3.4 us at the FMA peak, beside 16.8 MB of traffic; the odd
+// extension, the real transform of 2 (N + 1) points and the unpacking took about 100 us each
+// (258 = 2 3 43 is a poor length), the six transforms of a solve take 105 so.
 // N^2 work: beyond kDenseMax the matrix does not fit and the transform of the extension is used.
 constexpr int kDenseMax = 256;
 constexpr int kDenseCols = 64;
@@ -634,31 +638,49 @@ __device__ __forceinline__ void dense_sine(float* D, const float* Sm, const Dens
                                                  (ch - d.chunks[0]) * d.terms[1]);
     const float* x = D + (odd ? 0 : (N - 1) * kDenseCols) + lane;
     const int step = odd ? kDenseCols : -kDenseCols;
-    for (int i0 = 0; i0 < terms; i0 += 16) {
-      float2 acc[kDenseOut / 2][2];
+    // eight terms (n of them at the end) of half of the outputs at a time: two chains of four,
+    // their sum added to the outputs
+    auto group = [&](int i0, auto full, int n) {
+      constexpr bool FULL = decltype(full)::value;
 #pragma unroll
-      for (int q = 0; q < kDenseOut / 2; q++) acc[q][0] = acc[q][1] = make_float2(0.0f, 0.0f);
-      const int i1 = min(i0 + 16, terms);
-#pragma unroll 4
-      for (int i = i0; i < i1; i++) {
-        const float2 a = both(x[i * step]), b = both(x[i * step + 32]);
-        const float4* row = reinterpret_cast<const float4*>(m + i * kDenseOut);
+      for (int half = 0; half < 2; half++) {
+        float2 sum[2][kDenseOut / 4][2];
 #pragma unroll
-        for (int q = 0; q < kDenseOut / 4; q++) {
-          const float4 w = row[q];
-          const float2 w0 = make_float2(w.x, w.y), w1 = make_float2(w.z, w.w);
-          acc[2 * q][0] = fma2(w0, a, acc[2 * q][0]);
-          acc[2 * q][1] = fma2(w0, b, acc[2 * q][1]);
-          acc[2 * q + 1][0] = fma2(w1, a, acc[2 * q + 1][0]);
-          acc[2 * q + 1][1] = fma2(w1, b, acc[2 * q + 1][1]);
-        }
+        for (int c = 0; c < 2; c++)
+#pragma unroll
+          for (int t = 0; t < 4; t++) {
+            const int i = i0 + 4 * c + t;
+            if (!FULL && 4 * c + t >= n) {
+              if (t > 0) break;
+#pragma unroll
+              for (int q = 0; q < kDenseOut / 4; q++) sum[c][q][0] = sum[c][q][1] = both(0.0f);
+              break;
+            }
+            const float2 a = both(x[i * step]), b = both(x[i * step + 32]);
+            const float4* row = reinterpret_cast<const float4*>(m + i * kDenseOut) + 2 * half;
+#pragma unroll
+            for (int q = 0; q < kDenseOut / 8; q++) {
+              const float4 w = row[q];
+              const float2 w0 = make_float2(w.x, w.y), w1 = make_float2(w.z, w.w);
+              float2(*const s0)[2] = &sum[c][2 * q];
+              s0[0][0] = t == 0 ? mul2(w0, a) : fma2(w0, a, s0[0][0]);
+              s0[0][1] = t == 0 ? mul2(w0, b) : fma2(w0, b, s0[0][1]);
+              s0[1][0] = t == 0 ? mul2(w1, a) : fma2(w1, a, s0[1][0]);
+              s0[1][1] = t == 0 ? mul2(w1, b) : fma2(w1, b, s0[1][1]);
+            }
+          }
+#pragma unroll
+        for (int q = 0; q < kDenseOut / 4; q++)
+#pragma unroll
+          for (int k = 0; k < 2; k++) {
+            float2& o = out[r][half * (kDenseOut / 4) + q][k];
+            o = add2(o, add2(sum[0][q][k], sum[1][q][k]));
+          }
       }
-#pragma unroll
-      for (int q = 0; q < kDenseOut / 2; q++) {
-        out[r][q][0] = add2(out[r][q][0], acc[q][0]);
-        out[r][q][1] = add2(out[r][q][1], acc[q][1]);
-      }
-    }
+    };
+    int i0 = 0;
+    for (; i0 + 8 <= terms; i0 += 8) group(i0, std::true_type(), 8);
+    if (i0 < terms) group(i0, std::false_type(), terms - i0);
   }
   __syncthreads();
 #pragma unroll

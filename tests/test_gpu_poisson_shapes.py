@@ -100,3 +100,27 @@ def test_periodic_shapes(n, dtype):
 def test_symbol_of_any_shape_fills_the_device(dtype, n):
     t = [_kernel_us(_solver(m, dtype, False)[2], ("poisson_symbol_kernel",)) for m in (n, (128, 128, 64))]
     assert t[0] <= BAR * t[1], t
+
+
+@pytest.mark.parametrize("n", [(47, 47, 47), (53, 53, 53), (64, 64, 40), (64, 65, 33), (127, 63, 47)])
+def test_dense_sine_transforms_are_as_accurate_as_fast_ones(n):
+    """The FP32 isolated solve against the FP64 one of the same stored densities, relative L2,
+    mean of six blobs: at most 1.85e-7, which is what transforms of the odd extension leave at
+    these sizes (1.57e-7 to 2.7e-7)."""
+    rng = np.random.default_rng(1607)
+    x, y, z = [(torch.arange(m, device="cuda", dtype=torch.float64) + 0.5) / m - 0.5 for m in n]
+    x, y, z = x.view(1, 1, -1), y.view(1, -1, 1), z.view(-1, 1, 1)
+    errs = []
+    for _ in range(6):
+        a = rng.uniform(size=5)
+        rho = torch.exp(-((x - 0.1 * a[0]) ** 2 + (1 + a[1]) * (y - 0.1 * a[2]) ** 2 + (1 + a[3]) * z * z)
+                        / (0.02 + 0.05 * a[4])) * (1 + 0.1 * torch.sin(20 * x + 15 * y + 9 * z))
+        r32 = rho.float().reshape(-1).contiguous()
+        out = []
+        for dtype, r in ((F32, r32), (F64, r32.double())):
+            grid = ppml.Grid(n, (0.01,) * 3, 1.4, 0.2, (O,) * 6, dtype, u0=[torch.ones_like(r) for _ in range(6)])
+            phi = torch.empty_like(r)
+            grid.poisson_isolated(r, phi, 1.0)
+            out.append(phi.double())
+        errs.append(float((out[0] - out[1]).norm() / out[1].norm()))
+    assert sum(errs) / 6 <= 1.85e-7, errs
